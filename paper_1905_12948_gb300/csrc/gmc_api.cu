@@ -45,7 +45,7 @@ struct gmc_ctx {
   // geometry
   int tile = 0;
   int64_t n_tiles = 0, ld = 0;
-  uint32_t ksel = 0, cap = 0, sample_rank = 0;
+  uint32_t ksel = 0, cap = 0, sample_rank = 0, sample_rank_hi = 0;
   int sample_chunks = 0;
   int64_t nb = 0, m = 0;
   uint32_t B_shift = 0xffffffffu;
@@ -62,7 +62,6 @@ struct gmc_ctx {
   uint32_t* ghist = nullptr;
   uint32_t* chist = nullptr;
   uint32_t* bucket = nullptr;  // K x 2*kBucketCap
-  int sel_shift = 20;
   uint32_t* sample_keys = nullptr;
   uint32_t* big_tiles = nullptr;
   uint32_t* rcount = nullptr;
@@ -266,6 +265,7 @@ TopkArgs topk_args_at(gmc_ctx* h, const float* grads, int64_t t) {
   A.ksel = h->ksel;
   A.cap = h->cap;
   A.sample_rank = h->sample_rank;
+  A.sample_rank_hi = h->sample_rank_hi;
   A.sample_chunks = h->sample_chunks;
   A.sample_blocks = h->sample_blocks;
   A.dense_prev = h->restored && t == h->t ? 1 : 0;
@@ -275,7 +275,6 @@ TopkArgs topk_args_at(gmc_ctx* h, const float* grads, int64_t t) {
   A.ghist = h->ghist;
   A.chist = h->chist;
   A.bucket = h->bucket;
-  A.sel_shift = h->sel_shift;
   A.sample_keys = h->sample_keys;
   A.n_sample = h->n_sample;
   A.sample_stride = h->sample_stride;
@@ -597,7 +596,7 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
       h->cap = (uint32_t)std::min<double>((double)d, capd);
     } else if (d <= kSampleAll) {
       h->sample_chunks = 0;
-      h->sample_rank = h->ksel;
+      h->sample_rank = h->sample_rank_hi = h->ksel;
       h->cap = (uint32_t)d;
     } else {
       h->sample_chunks = kSampleChunks;
@@ -605,6 +604,10 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
       const double mean = ns * (double)ks / (double)d;
       const double r = std::min(ns, std::ceil(mean + 5.0 * std::sqrt(mean) + 8.0));
       h->sample_rank = (uint32_t)r;
+      // the k-th key's rank in the sample is about `mean`: at a quarter of it
+      // the sampled key lies above the k-th (Poisson: 1e-7 at mean 33), and
+      // the relative histogram's bins need reach no further
+      h->sample_rank_hi = (uint32_t)std::max(1.0, std::floor(0.25 * mean));
       const double capd = std::ceil((double)d * (r + 8.0 * std::sqrt(r) + 16.0) / ns) + 4096.0;
       h->cap = (uint32_t)std::min<double>((double)d, capd);
     }
@@ -645,14 +648,6 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
     h->sample_blocks = (int)std::max<int64_t>(1, ((int64_t)h->n_sample + 2047) / 2048);
     h->theta_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(2 * h->num_sms / K + 1,
                                                                   ((int64_t)h->n_sample + 8191) / 8192));
-    // relative-histogram bin width 2^sel_shift keys: near the k-th key a key
-    // step of 2^23 is an octave of |v|, and a Gaussian-like tail puts about
-    // 11 ln2 * k * 2^s / 2^23 candidates in one bin; aim at 2048 (the bin is
-    // ranked in shared memory when it holds at most kBucketCap)
-    {
-      const double w = 2048.0 * 8388608.0 / (11.0 * std::log(2.0) * (double)h->ksel);
-      h->sel_shift = (int)std::min(20.0, std::max(0.0, std::floor(std::log2(w))));
-    }
     const int64_t Kt = (int64_t)K * h->n_tiles;
     if ((err = dalloc(h, &h->e, (size_t)K * h->ld)) != cudaSuccess ||
         (err = dalloc(h, &h->w, (size_t)h->ld)) != cudaSuccess ||

@@ -38,7 +38,7 @@ struct WorkerSel {
                      // top-s threshold, and (worker 0's) the dense select's blocks
   uint32_t count_bucket;  // candidates collected from the k-th key's bin
   uint32_t nsel;     // approximate top-s: components sent (the count varies by step)
-  uint32_t pad;
+  uint32_t shift;    // log2 of the relative histogram's bin width, in keys (from the sample)
 };
 
 // Step counters (see GMC_STAT_* in gmc.h), unsigned 64-bit slots.
@@ -209,6 +209,35 @@ __device__ __forceinline__ void block_find_from_top(const uint32_t* hist, int nb
         break;
       }
       above += h;
+    }
+  }
+  __syncthreads();
+}
+
+// The same for two ranks at once (one scan): out[0], out[1] = bin and rank of
+// the r0-th, out[2], out[3] of the r1-th largest key (out: shared memory).
+__device__ __forceinline__ void block_find2_from_top(const uint32_t* hist, int nbins, uint32_t r0, uint32_t r1,
+                                                     uint32_t* ws, uint32_t* out) {
+  const int per = nbins / blockDim.x;
+  const int hi = nbins - threadIdx.x * per;
+  uint32_t mine = 0;
+  for (int i = 1; i <= per; ++i) mine += hist[hi - i];
+  uint32_t total;
+  const uint32_t incl = block_inclusive_scan<uint32_t>(mine, ws, &total);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const uint32_t r = q ? r1 : r0;
+    uint32_t above = incl - mine;
+    if (above < r && r <= incl) {
+      for (int i = 1; i <= per; ++i) {
+        const uint32_t h = hist[hi - i];
+        if (r <= above + h) {
+          out[2 * q] = uint32_t(hi - i);
+          out[2 * q + 1] = r - above;
+          break;
+        }
+        above += h;
+      }
     }
   }
   __syncthreads();

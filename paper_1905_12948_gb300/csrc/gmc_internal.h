@@ -56,6 +56,7 @@ struct TopkArgs {
   uint32_t cap_part;         // slots per warp part (a multiple of 32: whole 128-byte lines)
   uint32_t* rcount;          // K x regions x kChunksPerTile: candidates written in each part
   uint32_t sample_rank;      // rank of the sampled threshold
+  uint32_t sample_rank_hi;   // rank of the sampled key the relative histogram reaches up to
   int sample_chunks;         // 0 = sample every element (or the approximate top-s sample)
   int sample_blocks;         // blocks per worker of the approximate top-s sample (k_sample)
   uint32_t n_sample;         // sampled positions per worker
@@ -76,7 +77,6 @@ struct TopkArgs {
   uint32_t* ghist;           // K x kHistBins: the approximate top-s sample's histogram (zero between uses)
   uint32_t* chist;           // K x kRelBins: the candidates' relative histogram (zeroed by the sample)
   uint32_t* bucket;          // K x 2*kBucketCap: keys, then indices of the k-th key's bin
-  int sel_shift;             // log2 of the relative-histogram bin width (in keys)
   uint32_t* sample_keys;     // K x sample_stride
   uint32_t* big_tiles;       // [0]: count, then tile ids left to the block aggregate
   uint32_t* cand_idx;        // current chunks: K x cap

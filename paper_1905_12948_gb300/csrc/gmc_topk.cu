@@ -446,9 +446,9 @@ __global__ void __cluster_dims__(scl::kCtas, 1, 1) __launch_bounds__(scl::kThrea
   cg::cluster_group cl = cg::this_cluster();
   __shared__ uint32_t hist[kHistBins];  // this CTA's counts
   __shared__ uint32_t red1[kHistBins];  // first CTA: the cluster's first-digit counts
-  __shared__ uint32_t red2[1024];       // first CTA: the cluster's second digits in the bin b1
+  __shared__ uint32_t red2[2048];       // first CTA: the cluster's second digits in the bins b1 and bh
   __shared__ uint32_t ws[32];
-  __shared__ uint32_t s_bin, s_rank;
+  __shared__ uint32_t s_find[4];
   const int k = blockIdx.y;
   const unsigned crank = cl.block_rank();
   WorkerSel& S = A.sel[k];
@@ -473,7 +473,7 @@ __global__ void __cluster_dims__(scl::kCtas, 1, 1) __launch_bounds__(scl::kThrea
     hist[b] = 0;
     red1[b] = 0;
   }
-  for (int b = threadIdx.x; b < 1024; b += blockDim.x) red2[b] = 0;
+  for (int b = threadIdx.x; b < 2048; b += blockDim.x) red2[b] = 0;
   const float* ek = A.e + (int64_t)k * A.ld;
   const float* gk = A.grads + (int64_t)k * A.d;
   const uint16_t* gk16 = A.grads16 + (int64_t)k * A.d;
@@ -536,37 +536,50 @@ __global__ void __cluster_dims__(scl::kCtas, 1, 1) __launch_bounds__(scl::kThrea
   for (int b = threadIdx.x; b < kHistBins; b += blockDim.x)
     if (hist[b]) atomicAdd(&r1[b], hist[b]);
   cl.sync();
-  // the bin of the r-th largest key and its rank there (every CTA alike)
+  // the bins of the r-th and of the rh-th largest key and their ranks there (every CTA alike)
   for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) hist[b] = r1[b];
-  if (threadIdx.x == 0) {
-    s_bin = 0;
-    s_rank = 0;
-  }
+  if (threadIdx.x < 4) s_find[threadIdx.x] = 0;
   __syncthreads();
   const uint32_t r = A.sample_rank < (uint32_t)n_s ? A.sample_rank : (uint32_t)n_s;
-  block_find_from_top(hist, kHistBins, r, ws, &s_bin, &s_rank);
-  const uint32_t b1 = s_bin, rr = s_rank;
-  for (int b = threadIdx.x; b < 1024; b += blockDim.x) hist[b] = 0;
+  const uint32_t rh = A.sample_rank_hi < r ? A.sample_rank_hi : r;
+  block_find2_from_top(hist, kHistBins, r, rh, ws, s_find);
+  const uint32_t b1 = s_find[0], rr = s_find[1], bh = s_find[2], rrh = s_find[3];
+  const uint32_t n_h = bh != b1 ? hist[bh] : 0u;  // keys of a bin of its own above b1
+  __syncthreads();
+  // second digits: bin b1's in the lower half, bin bh's (when it is another) in the upper
+  for (int b = threadIdx.x; b < 2048; b += blockDim.x) hist[b] = 0;
+  if (threadIdx.x < 4) s_find[threadIdx.x] = 0;
   __syncthreads();
 #pragma unroll
-  for (int q = 0; q < kSlots; ++q)
-    if (key[q] != 0xffffffffu && (key[q] >> 20) == b1) atomicAdd(&hist[(key[q] >> 10) & 1023u], 1u);
+  for (int q = 0; q < kSlots; ++q) {
+    if (key[q] == 0xffffffffu) continue;
+    const uint32_t bin = key[q] >> 20, dig = (key[q] >> 10) & 1023u;
+    if (bin == b1) atomicAdd(&hist[dig], 1u);
+    else if (bin == bh) atomicAdd(&hist[1024u + dig], 1u);
+  }
   __syncthreads();
   uint32_t* r2 = cl.map_shared_rank(red2, 0);
-  for (int b = threadIdx.x; b < 1024; b += blockDim.x)
+  for (int b = threadIdx.x; b < 2048; b += blockDim.x)
     if (hist[b]) atomicAdd(&r2[b], hist[b]);
   // after this barrier no CTA touches another's shared memory
   cl.sync();
   if (crank != 0) return;
-  if (threadIdx.x == 0) {
-    s_bin = 0;
-    s_rank = 0;
-  }
-  __syncthreads();
-  block_find_from_top(red2, 1024, rr, ws, &s_bin, &s_rank);
+  block_find2_from_top(red2, 2048, n_h + rr, rrh, ws, s_find);
   if (threadIdx.x == 0) {
     // capped at the Inf key: every non-finite value is a candidate (and counted there)
-    S.theta = min((b1 << 20) | (s_bin << 10), 0x7f800000u);
+    const uint32_t theta = min((b1 << 20) | ((s_find[0] & 1023u) << 10), 0x7f800000u);
+    // The candidates' relative histogram spans [theta, the last key of the
+    // rh-th sampled key's digits]: its bins follow the data. (Bins of a width
+    // fixed for a Gaussian tail were wide enough for 2,048 candidates at
+    // first, but residuals pile up below the level at which they are sent:
+    // after some 500 steps at d = 11.2 M one bin held more than kBucketCap and
+    // the worker went to the dense path, 25 ms instead of 0.46 ms a step.)
+    const uint32_t top = (bh << 20) | ((s_find[2] & 1023u) << 10) | 1023u;
+    const uint32_t range = top > theta ? top - theta : 0u;
+    uint32_t sh = 0;
+    while ((range >> sh) >= (uint32_t)kRelBins - 1) ++sh;
+    S.theta = theta;
+    S.shift = sh;
     S.count = 0;
     S.dense = 0;
   }
@@ -677,6 +690,7 @@ __global__ void __launch_bounds__(kThreads) k_sample_theta(TopkArgs A) {
   if (threadIdx.x == 0) {
     // capped at the Inf key: every non-finite value is a candidate (and counted there)
     S.theta = min(theta, 0x7f800000u);
+    S.shift = 20;  // the relative histogram is not used
     S.count = 0;
     S.dense = 0;
     S.nsel = 0;
@@ -1035,7 +1049,7 @@ struct Smem {
   uint64_t full[kStages];                  // e, g landed (1 arrival + tx bytes)
   uint64_t empty[kStages];                 // all consumer warps read the stage (8 arrivals)
   int32_t gmeta[kStages];                  // leading floats in the g stage, -1 = not copied
-  uint32_t theta[kMaxK];
+  uint32_t theta[kMaxK], shift[kMaxK];     // candidate threshold and relative histogram of each worker
   uint32_t Tp[kMaxK], tip[kMaxK];          // the previous step's selection (T, t_idx) per worker
   uint32_t tq[16];                         // claimed tiles (tile_at)
   uint32_t next[kSubTiles];                // per sub-tile: the next tile of its two warps
@@ -1191,6 +1205,7 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
   }
   for (int kk = threadIdx.x; kk < kMaxK; kk += blockDim.x) {
     sm.theta[kk] = kk < A.K ? A.sel[kk].theta : kNoCandidate;
+    sm.shift[kk] = kk < A.K ? A.sel[kk].shift : 0u;
     sm.Tp[kk] = kk < A.K ? A.sel[kk].T : 0u;  // this step's select runs after this pass
     sm.tip[kk] = kk < A.K ? A.sel[kk].t_idx : 0u;
   }
@@ -1485,7 +1500,7 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
             ci[line * 32 + lane] = si[lane];
             cv[line * 32 + lane] = x;
             nonfinite += is_nonfinite(x) ? 1u : 0u;
-            atomicAdd(&A.chist[(int64_t)k * kRelBins + rel_bin(mag_key(x), th, A.sel_shift)], 1u);
+            atomicAdd(&A.chist[(int64_t)k * kRelBins + rel_bin(mag_key(x), th, sm.shift[k])], 1u);
           }
           __syncwarp();
         }
@@ -1534,7 +1549,7 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
       A.cand_idx[(int64_t)k * A.cap + part0 + line * 32 + lane] = si[lane];
       A.cand_val[(int64_t)k * A.cap + part0 + line * 32 + lane] = x;
       nonfinite += is_nonfinite(x) ? 1u : 0u;
-      atomicAdd(&A.chist[(int64_t)k * kRelBins + rel_bin(mag_key(x), sm.theta[k], A.sel_shift)], 1u);
+      atomicAdd(&A.chist[(int64_t)k * kRelBins + rel_bin(mag_key(x), sm.theta[k], sm.shift[k])], 1u);
     }
   }
   if (nonfinite) {
@@ -1573,9 +1588,9 @@ __device__ __forceinline__ void candidate_part(const TopkArgs& A, int k, int p, 
 // ---------------------------------------------------------------------------
 // exact select among candidates, two passes:
 //   hist    a kRelBins-bin histogram of the candidates' keys above theta, in
-//           bins of 2^sel_shift keys (sel_shift is chosen from k so that the
-//           k-th key's bin holds about 2048 candidates on smooth data); the
-//           last block finds the bin holding the k-th key
+//           bins of 2^shift keys that span the sampled keys around the k-th
+//           (k_sample_cluster), so that they follow the data; every block of
+//           the next launch finds the bin holding the k-th key
 //   finish  the candidates of that bin are collected (key, index); the last
 //           block ranks them in shared memory: the k-th key T, how many keys
 //           equal T are kept, and -- when fewer are kept than there are -- the
@@ -1590,6 +1605,7 @@ __global__ void __launch_bounds__(kThreads) k_select_hist(TopkArgs A) {
   WorkerSel& S = A.sel[k];
   if (needs_dense(S, A.ksel, A.cap)) return;
   const uint32_t theta = S.theta;
+  const int shift = (int)S.shift;
   for (int b = threadIdx.x; b < kRelBins; b += blockDim.x) h[b] = 0;
   __syncthreads();
   const float* cv = A.cand_val + (int64_t)k * A.cap;
@@ -1606,7 +1622,7 @@ __global__ void __launch_bounds__(kThreads) k_select_hist(TopkArgs A) {
         kv[q] = i < hi ? mag_key(cv[i]) : 0xffffffffu;
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) warp_hist_add(h, kv[q] != 0xffffffffu ? rel_bin(kv[q], theta, A.sel_shift) : -1);
+      for (int q = 0; q < 4; ++q) warp_hist_add(h, kv[q] != 0xffffffffu ? rel_bin(kv[q], theta, shift) : -1);
     }
   }
   __syncthreads();
@@ -1627,6 +1643,7 @@ __global__ void __launch_bounds__(kThreads) k_select_finish(TopkArgs A) {
   WorkerSel& S = A.sel[k];
   if (needs_dense(S, A.ksel, A.cap)) return;
   const uint32_t theta = S.theta;
+  const int shift = (int)S.shift;
   // the bin holding the k-th key, and its rank there (every block, from the histogram)
   for (int b = threadIdx.x; b < kRelBins; b += blockDim.x) h[b] = __ldcg(&A.chist[(int64_t)k * kRelBins + b]);
   if (threadIdx.x == 0) {
@@ -1659,7 +1676,7 @@ __global__ void __launch_bounds__(kThreads) k_select_finish(TopkArgs A) {
     // the bytes of loading every candidate's index
 #pragma unroll
     for (int q = 0; q < kQ; ++q) {
-      const bool mine = in[q] && rel_bin(key[q], theta, A.sel_shift) == want;
+      const bool mine = in[q] && rel_bin(key[q], theta, shift) == want;
       idx[q] = mine ? ci[slot[q]] : 0u;
       m[q] = __ballot_sync(0xffffffffu, mine);
       n += __popc(m[q]);
@@ -1758,8 +1775,8 @@ __global__ void __launch_bounds__(kThreads) k_select_finish(TopkArgs A) {
   // every key of the bucket lies in the bin `want`: below the top bin its
   // keys are theta + want * 2^s + [0, 2^s), and only those low s bits are ranked
   const bool bounded = want < kRelBins - 1;
-  const uint32_t T = bounded ? smem_select_bits(keys, n, want_rank, A.sel_shift,
-                                                theta + ((uint32_t)want << A.sel_shift), h, ws, &s_bin,
+  const uint32_t T = bounded ? smem_select_bits(keys, n, want_rank, shift,
+                                                theta + ((uint32_t)want << shift), h, ws, &s_bin,
                                                 &s_rank, &n_tie)
                              : smem_select(keys, n, want_rank, h, ws, &s_bin, &s_rank, &n_tie);
   // ties: gather the indices of the keys equal to T over the keys, in place;
