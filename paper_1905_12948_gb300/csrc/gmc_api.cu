@@ -333,6 +333,11 @@ uint32_t golden_stride(int64_t nb) {
 }
 
 
+// Union flags (one byte a block) that one warp clears at the end of a step:
+// 64 KB take it a few microseconds, hidden behind nothing; more are cleared by
+// a memset before the step.
+constexpr int64_t kFlagsByWarp = 65536;
+
 RbgsArgs rbgs_args(gmc_ctx* h, const float* grads) {
   RbgsArgs A;
   std::memset(&A, 0, sizeof(A));
@@ -362,7 +367,12 @@ RbgsArgs rbgs_args(gmc_ctx* h, const float* grads) {
   A.uflag_cur = h->uflag[cur];
   A.slab = h->slab;
   A.has_prev = h->t > 0;
+  A.clear_flags = h->nb <= kFlagsByWarp ? 1 : 0;
+  A.det = h->detach_out;
+  A.det_ld = h->detach_ld;
+  A.det_b = detach_b(h);
   A.step_ctr = h->step_ctr;
+  A.total_ctr = h->total_ctr;
   A.tile_ctr = h->tile_ctr;
   A.wait_ns = kWaitLimitNs;
   A.hold_tile = -1;
@@ -397,9 +407,9 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
   const uint16_t* grads16 = bf16 ? static_cast<const uint16_t*>(grads_any) : nullptr;
   const double Kd = (double)h->K * (double)h->d;
   GMC_TRY(order_after_flush(h, s, true));
-  // the exact top-k's sample kernel clears the step's counters itself (a
-  // memset between two kernels would keep the second from starting early)
-  if (h->compressor != GMC_TOPK) GMC_TRY(cudaMemsetAsync(h->step_ctr, 0, sizeof(Counters), s));
+  // the exact top-k's sample kernel and the RBGS pick clear the step's counters
+  // themselves (a memset between two kernels would keep the second from starting early)
+  if (h->compressor == GMC_TOPK_APPROX) GMC_TRY(cudaMemsetAsync(h->step_ctr, 0, sizeof(Counters), s));
   unsigned long long pairs_add = 0;
   bool finalized = false;  // the step's counters already added up by its last kernel
   if (h->compressor != GMC_RBGS) {
@@ -463,12 +473,14 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     // restored state: w_t - w_{t-1} may be non-zero in any block (zero outside
     // the last union, where dlt holds it): flag every block as the last union's
     if (h->restored && h->t > 0) GMC_TRY(cudaMemsetAsync(A.uflag_prev, 1, (size_t)h->nb, s));
-    GMC_TRY(cudaMemsetAsync(A.uflag_cur, 0, (size_t)h->nb, s));
+    if (!A.clear_flags) GMC_TRY(cudaMemsetAsync(A.uflag_cur, 0, (size_t)h->nb, s));
     GMC_TRY(timed(h, GMC_KERNEL_RBGS_PICK, 0.0, s, [&] { return launch_rbgs_pick(A, s); }));
-    GMC_TRY(timed(h, GMC_KERNEL_RBGS_STEP, (bf16 ? 10.0 : 12.0) * Kd, s,
+    const double det_bytes = A.det ? 4.0 * Kd + 4.0 * h->d : 0.0;  // the detached rows, and w
+    GMC_TRY(timed(h, GMC_KERNEL_RBGS_STEP, (bf16 ? 10.0 : 12.0) * Kd + det_bytes, s,
                   [&] { return launch_rbgs_step(A, h->grid_rbgs, s); }));
+    finalized = true;
   }
-  if (h->detach_out) {
+  if (h->detach_out && h->compressor != GMC_RBGS) {
     DetachArgs D{h->w, h->e, h->ld, h->d, detach_b(h), h->detach_out, h->detach_ld, 0, h->K};
     GMC_TRY(timed(h, GMC_KERNEL_DETACH, 8.0 * Kd + 4.0 * h->d, s, [&] { return launch_detach(D, s); }));
   }
@@ -689,8 +701,8 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
     }
     // enough tiles for one per SM: the bulk-copy kernel (one persistent CTA per SM)
     h->rbgs_bulk = h->n_tiles >= h->num_sms;
-    h->grid_rbgs = h->rbgs_bulk ? h->num_sms
-                                : (int)std::min<int64_t>(h->n_tiles, (int64_t)h->num_sms * rbgs_blocks_per_sm());
+    h->grid_rbgs = h->rbgs_bulk ? h->num_sms  // (the load/store pass: 1,024 elements a block)
+                                : (int)std::min<int64_t>((d + 1023) / 1024, (int64_t)h->num_sms * rbgs_blocks_per_sm());
     const int64_t nbw = (h->nb + 31) / 32;
     if ((err = dalloc(h, &h->e, (size_t)K * h->ld)) != cudaSuccess ||
         (err = dalloc(h, &h->w, (size_t)h->ld)) != cudaSuccess ||
@@ -698,13 +710,13 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
         (err = dalloc(h, &h->bitmap, (size_t)K * nbw)) != cudaSuccess ||
         (err = dalloc(h, &h->rank, (size_t)K * h->nb)) != cudaSuccess ||
         (err = dalloc(h, &h->blocks, (size_t)K * h->m)) != cudaSuccess ||
-        (err = dalloc(h, &h->uflag[0], (size_t)h->nb)) != cudaSuccess ||
-        (err = dalloc(h, &h->uflag[1], (size_t)h->nb)) != cudaSuccess ||
+        (err = dalloc(h, &h->uflag[0], (size_t)h->nb + 3)) != cudaSuccess ||  // cleared in whole words
+        (err = dalloc(h, &h->uflag[1], (size_t)h->nb + 3)) != cudaSuccess ||
         (err = dalloc(h, &h->slab, (size_t)K * h->m * block)) != cudaSuccess)
       return fail(err);
   }
   if ((err = dalloc(h, &h->step_ctr, 1)) != cudaSuccess ||
-      (err = dalloc(h, &h->tile_ctr, 1)) != cudaSuccess ||
+      (err = dalloc(h, &h->tile_ctr, 2)) != cudaSuccess ||
       (err = dalloc(h, &h->total_ctr, 1)) != cudaSuccess ||
       (err = dalloc(h, &h->status, 1)) != cudaSuccess)
     return fail(err);
@@ -888,8 +900,7 @@ int gmc_get_params(gmc_t h, float* w_dev_out, void* stream) {
   DeviceGuard g(h->device);
   GMC_TRY_ST(flush(h, static_cast<cudaStream_t>(stream)));
   GMC_TRY(order_after_flush(h, static_cast<cudaStream_t>(stream), false));
-  GMC_TRY(cudaMemcpyAsync(w_dev_out, h->w, (size_t)h->d * sizeof(float), cudaMemcpyDeviceToDevice,
-                          static_cast<cudaStream_t>(stream)));
+  GMC_TRY(launch_copy_row(h->w, w_dev_out, h->d, static_cast<cudaStream_t>(stream)));
   return GMC_OK;
 }
 
@@ -899,8 +910,7 @@ int gmc_get_residual(gmc_t h, int32_t k, float* e_dev_out, void* stream) {
   DeviceGuard g(h->device);
   GMC_TRY_ST(flush(h, static_cast<cudaStream_t>(stream)));
   GMC_TRY(order_after_flush(h, static_cast<cudaStream_t>(stream), false));
-  GMC_TRY(cudaMemcpyAsync(e_dev_out, h->e + (int64_t)k * h->ld, (size_t)h->d * sizeof(float),
-                          cudaMemcpyDeviceToDevice, static_cast<cudaStream_t>(stream)));
+  GMC_TRY(launch_copy_row(h->e + (int64_t)k * h->ld, e_dev_out, h->d, static_cast<cudaStream_t>(stream)));
   return GMC_OK;
 }
 

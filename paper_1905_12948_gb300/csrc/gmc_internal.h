@@ -145,16 +145,21 @@ struct RbgsArgs {
   int32_t* rank;             // streams x nb: slot of a chosen block, -1 otherwise
   int32_t* blocks;           // streams x m: chosen blocks ascending
   uint8_t* uflag_prev;       // nb: union of the previous step's blocks
-  uint8_t* uflag_cur;        // nb: union of this step's blocks
+  uint8_t* uflag_cur;        // nb: union of this step's blocks (zero before the pick)
+  int clear_flags;           // the step's last warp clears uflag_prev, the next step's uflag_cur
   float* slab;               // K x (m*B): C(e_{t+1/2,k}) values, block slot major
   int has_prev;
   int bulk;                  // k_rbgs_bulk (bulk copies through shared memory), else k_rbgs_step
   int g_direct;              // grads is mapped host memory: read it with loads, not bulk copies
-  uint32_t* tile_ctr;        // tiles claimed by k_rbgs_bulk (zeroed by k_rbgs_pick)
+  uint32_t* tile_ctr;        // tiles claimed by k_rbgs_bulk, warps that ended the step (zeroed by k_rbgs_pick)
   uint64_t wait_ns;          // bound of the bulk pass's mbarrier waits (kWaitLimitNs)
   int64_t hold_tile;         // test hook, as in TopkArgs: no copy for item (hold_tile, hold_k)
   int hold_k;
+  float* det;                // detach output (Alg. 2): w_{t+1} - det_b*e_{t+1,k}, K rows of det_ld, or NULL
+  int64_t det_ld;
+  float det_b;
   Counters* step_ctr;
+  Counters* total_ctr;       // the step's last warp adds step_ctr to them
   unsigned* status;
 };
 
@@ -212,6 +217,8 @@ cudaError_t launch_rbgs_step(const RbgsArgs& A, int grid, cudaStream_t s);
 cudaError_t launch_rbgs_expand(const RbgsArgs& A, int k, uint32_t* idx_out, float* val_out,
                                cudaStream_t s);
 cudaError_t launch_detach(const DetachArgs& A, cudaStream_t s);
+// dst = src over n floats; src 16-byte aligned, allocated to a whole tile past n.
+cudaError_t launch_copy_row(const float* src, float* dst, int64_t n, cudaStream_t s);
 cudaError_t launch_finalize(Counters* step, Counters* total, unsigned long long pairs_add,
                             cudaStream_t s);
 

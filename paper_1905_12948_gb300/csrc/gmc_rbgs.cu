@@ -5,12 +5,18 @@
 //   pick   per block-choice stream (one shared by all workers, or one per
 //          worker): m distinct blocks out of nb by Floyd's sampling driven by a
 //          SplitMix64 counter stream keyed by (seed, t[, k]); writes the sorted
-//          block list, a block -> slot map and the union flags
+//          block list, a block -> slot map and the union flags, and clears the
+//          step's counters
 //   step   ONE dense pass per tile for all K workers in ascending order:
 //          v = (e + g) - c*(w_t - w_{t-1}); inside chosen blocks v is sent
 //          (copied to the worker's slab), summed into the aggregate and its
 //          residual set to +0, elsewhere v is the residual; then, on the union,
 //          w -= (eta/K) * sum and w_{t+1} - w_t is stored for the next step.
+//          With a detach output (Alg. 2) the same pass writes the rows
+//          w_{t+1} - b*e_{t+1,k}: 4 bytes a value on top of the step's 12,
+//          where a pass of its own read e back as well (d = 25.6 M, K = 32:
+//          step and rows 3,249 -> 2,040 us). The last block ends the step
+//          (end_step): two launches a step in all, where there were five.
 #include "gmc_internal.h"
 
 namespace gmc {
@@ -46,178 +52,289 @@ __device__ __forceinline__ uint32_t block_of(int64_t j, const RbgsArgs& A) {
 }
 
 // ---------------------------------------------------------------------------
-// pick: one block per stream
+// pick: one block per stream.
+//
+// Floyd's sampling takes, for i = 0 .. m-1 with top_i = nb-m+i, the draw r_i
+// uniform on [0, top_i], or top_i when r_i was taken before. It need not run
+// one draw after another: r_i was taken iff an earlier draw was the same block,
+// or r_i is an earlier step's top (r_i = top_i', i' < i) and that step took its
+// top, i.e. collided itself. The first is a table of each block's first draw
+// (atomicMin), the second a walk to smaller i. So every draw is decided by a
+// thread of its own: a chain of a few shared-memory reads, where the serial
+// form cost about 50 ns a draw (m = 62: 9.9 us, m = 3,906: 200 us).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_rbgs_pick(RbgsArgs A) {
+constexpr int kPickThreads = 1024;
+constexpr int kFirstWords = 16384;  // first-draw table kept in shared memory up to this many blocks
+
+__global__ void __launch_bounds__(kPickThreads) k_rbgs_pick(RbgsArgs A) {
   griddep_wait();
-  if (blockIdx.x == 0 && threadIdx.x == 0) *A.tile_ctr = 0u;  // the fused pass claims its tiles from it
-  extern __shared__ uint32_t bm_s[];
+  if (blockIdx.x == 0) {
+    if (threadIdx.x < 2) A.tile_ctr[threadIdx.x] = 0u;  // tiles claimed by the fused pass, its warps done
+    if (threadIdx.x < 8) A.step_ctr->v[threadIdx.x] = 0ull;
+  }
+  extern __shared__ uint32_t pick_s[];
   __shared__ uint32_t ws[32];
   const int s = blockIdx.x;
   const int64_t nbw = (A.nb + 31) / 32;
   const bool in_smem = nbw <= kPickSmemWords;
-  uint32_t* bm = in_smem ? bm_s : A.bitmap + (int64_t)s * nbw;
-  if (in_smem) {
-    for (int64_t i = threadIdx.x; i < nbw; i += blockDim.x) bm_s[i] = 0;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    // Floyd: for j = nb-m .. nb-1, r = uniform[0, j]; keep j if r was taken, else r
-    const uint64_t key = stream_key(A.seed, A.t, A.per_worker ? (uint64_t)s + 1 : 0ull);
-    uint64_t i = 0;
-    for (int64_t jj = A.nb - A.m; jj < A.nb; ++jj, ++i) {
-      const uint32_t r = below(draw(key, i), (uint64_t)jj + 1);
-      const uint32_t pick = ((bm[r >> 5] >> (r & 31)) & 1u) ? (uint32_t)jj : r;
-      bm[pick >> 5] |= 1u << (pick & 31);
-    }
-  }
-  __syncthreads();
+  const bool first_smem = A.nb <= kFirstWords;
   int32_t* rank = A.rank + (int64_t)s * A.nb;
   int32_t* blk = A.blocks + (int64_t)s * A.m;
+  uint32_t* bm = in_smem ? pick_s : A.bitmap + (int64_t)s * nbw;
+  // a block's first draw (the slot map's memory holds it until the map is written)
+  int32_t* first = first_smem ? reinterpret_cast<int32_t*>(pick_s + nbw) : rank;
+  if (in_smem)
+    for (int64_t i = threadIdx.x; i < nbw; i += blockDim.x) bm[i] = 0u;
+  for (int64_t b = threadIdx.x; b < A.nb; b += blockDim.x) first[b] = 0x7fffffff;
+  __syncthreads();
+  const uint64_t key = stream_key(A.seed, A.t, A.per_worker ? (uint64_t)s + 1 : 0ull);
+  const int64_t top0 = A.nb - A.m;
+  auto drawn = [&](int64_t i) { return below(draw(key, (uint64_t)i), (uint64_t)(top0 + i) + 1); };
+  for (int64_t i = threadIdx.x; i < A.m; i += blockDim.x) atomicMin(&first[drawn(i)], (int32_t)i);
+  __syncthreads();
+  for (int64_t i = threadIdx.x; i < A.m; i += blockDim.x) {
+    const uint32_t r0 = drawn(i);
+    bool taken = false;
+    int64_t at = i, x = r0;
+    for (;;) {  // `at` decreases at every turn
+      if ((first_smem ? first[x] : __ldcg(first + x)) < (int32_t)at) {
+        taken = true;
+        break;
+      }
+      if (x < top0 || x - top0 >= at) break;
+      at = x - top0;  // taken iff that step took its top
+      x = drawn(at);
+    }
+    const uint32_t pick = taken ? (uint32_t)(top0 + i) : r0;
+    atomicOr(&bm[pick >> 5], 1u << (pick & 31));
+  }
+  __syncthreads();
   uint32_t carry = 0;
   for (int64_t w0 = 0; w0 < nbw; w0 += blockDim.x) {
     const int64_t wi = w0 + threadIdx.x;
-    const uint32_t word = wi < nbw ? bm[wi] : 0u;
+    const uint32_t word = wi < nbw ? (in_smem ? bm[wi] : __ldcg(bm + wi)) : 0u;
     uint32_t tot;
     const uint32_t inc = block_inclusive_scan<uint32_t>((uint32_t)__popc(word), ws, &tot);
-    uint32_t q = carry + inc - (uint32_t)__popc(word);
-    if (wi < nbw) {
-      for (int bit = 0; bit < 32; ++bit) {
-        const int64_t b = wi * 32 + bit;
-        if (b >= A.nb) break;
-        if ((word >> bit) & 1u) {
-          rank[b] = (int32_t)q;
+    const uint32_t q0 = carry + inc - (uint32_t)__popc(word);
+    if (!in_smem && wi < nbw) bm[wi] = 0u;  // the global bitmap stays zero between steps
+    // a warp's 32 words, one after another: lane l takes block 32 * word + l
+    const int lane = threadIdx.x & 31;
+#pragma unroll 4
+    for (int i = 0; i < 32; ++i) {
+      const uint32_t wd = __shfl_sync(0xffffffffu, word, i);
+      const uint32_t qd = __shfl_sync(0xffffffffu, q0, i);
+      const int64_t b = (wi - lane + i) * 32 + lane;
+      if (b < A.nb) {
+        const bool on = (wd >> lane) & 1u;
+        const uint32_t q = qd + __popc(wd & lanemask_lt());
+        rank[b] = on ? (int32_t)q : -1;
+        if (on) {
           blk[q] = (int32_t)b;
           A.uflag_cur[b] = 1;
-          ++q;
-        } else {
-          rank[b] = -1;
         }
       }
-      if (!in_smem) bm[wi] = 0u;  // the global bitmap stays zero between steps
     }
     carry += tot;
   }
 }
 
 // ---------------------------------------------------------------------------
-// fused step: persistent blocks walk tiles of kRbgsTile elements
+// The end of the fused step, by the `warps` consumer warps of every block (red:
+// shared memory, 5 words a warp; they meet at named barrier 1): the block's
+// counts into step_ctr with one atomic each, and the last block out adds them
+// to the totals and clears the flags of the step before, which the next step's
+// pick sets again. (With a set of atomics per warp the d = 272 k step's 2,129
+// warps queued at one line.)
 // ---------------------------------------------------------------------------
-template <bool kBf16>
+constexpr int kEndWords = 5;
+__device__ __forceinline__ void end_step(const RbgsArgs& A, unsigned long long* red, int warp, int warps, int lane,
+                                         unsigned long long nonfinite, unsigned long long pairs,
+                                         unsigned long long nnz, unsigned long long uni,
+                                         unsigned long long changed) {
+  const unsigned long long c[kEndWords] = {warp_sum(pairs), warp_sum(nnz), warp_sum(uni), warp_sum(changed),
+                                           warp_sum(nonfinite)};
+  if (lane == 0)
+#pragma unroll
+    for (int i = 0; i < kEndWords; ++i) red[warp * kEndWords + i] = c[i];
+  asm volatile("bar.sync 1, %0;" ::"r"(warps * 32) : "memory");
+  if (warp != 0) return;
+  if (lane < kEndWords) {
+    constexpr int slot[kEndWords] = {kPairs, kNnz, kUnion, kChanged, kNonfinite};
+    unsigned long long x = 0;
+    for (int w = 0; w < warps; ++w) x += red[w * kEndWords + lane];
+    int at = slot[0];
+#pragma unroll
+    for (int i = 1; i < kEndWords; ++i) at = lane == i ? slot[i] : at;
+    if (x) {
+      atomicAdd(&A.step_ctr->v[at], x);
+      if (lane == kEndWords - 1) atomicOr(A.status, kStatusNonfinite);
+    }
+    __threadfence();
+  }
+  __syncwarp();
+  uint32_t last = 0;
+  if (lane == 0) {
+    __threadfence();
+    last = atomicAdd(A.tile_ctr + 1, 1u) == gridDim.x - 1 ? 1u : 0u;
+    if (last) {
+      __threadfence();
+      finalize_counters(A.step_ctr, A.total_ctr, 0ull);
+    }
+  }
+  last = __shfl_sync(0xffffffffu, last, 0);
+  if (last && A.clear_flags)
+    for (int64_t b = lane * 4; b < A.nb; b += 128)  // allocated in whole words
+      *reinterpret_cast<uint32_t*>(A.uflag_prev + b) = 0u;
+}
+
+// One group of 128 consecutive floats of a warp (lane l: elements 4l .. 4l+3)
+// stored at p, any 4-byte alignment: 16-byte stores of the aligned quads, each
+// made of its own and the next lane's values, and single floats at both ends.
+// mis: floats from p to the next 16-byte boundary (uniform over the warp).
+__device__ __forceinline__ void store_row128(float* p, float4 x, int mis, int lane) {
+  if (mis == 0) {
+    __stcs(reinterpret_cast<float4*>(p + lane * 4), x);
+    return;
+  }
+  float4 n;  // the next lane's values
+  n.x = __shfl_down_sync(0xffffffffu, x.x, 1);
+  n.y = __shfl_down_sync(0xffffffffu, x.y, 1);
+  n.z = __shfl_down_sync(0xffffffffu, x.z, 1);
+  const float4 q = mis == 1 ? make_float4(x.y, x.z, x.w, n.x)
+                            : (mis == 2 ? make_float4(x.z, x.w, n.x, n.y) : make_float4(x.w, n.x, n.y, n.z));
+  if (lane < 31) __stcs(reinterpret_cast<float4*>(p + lane * 4 + mis), q);
+  if (lane == 0) {
+    p[0] = x.x;
+    if (mis > 1) p[1] = x.y;
+    if (mis > 2) p[2] = x.z;
+  }
+  if (lane == 31) {  // the elements past the last whole quad
+    p[127] = x.w;
+    if (mis < 3) p[126] = x.z;
+    if (mis < 2) p[125] = x.y;
+  }
+}
+__device__ __forceinline__ int row_mis(const float* p) {
+  return (int)((4u - (uint32_t)(reinterpret_cast<uintptr_t>(p) >> 2)) & 3u);
+}
+// GMC+ detach (Alg. 2): w_{t+1} - b*e_{t+1,k} of 4 elements.
+__device__ __forceinline__ float4 detached4(float4 w, float b, float4 e) {
+  return make_float4(__fsub_rn(w.x, __fmul_rn(b, e.x)), __fsub_rn(w.y, __fmul_rn(b, e.y)),
+                     __fsub_rn(w.z, __fmul_rn(b, e.z)), __fsub_rn(w.w, __fmul_rn(b, e.w)));
+}
+// A lane's 4 elements at offset l of a sub-tile with lim valid elements, at row.
+__device__ __forceinline__ void store_row(float* row, int l, int lim, float4 x, int lane) {
+  // l - lane*4: the start of the warp's 128 elements
+  const int g0 = l - lane * 4;
+  if (g0 + 128 <= lim) {
+    store_row128(row + g0, x, row_mis(row + g0), lane);
+    return;
+  }
+  if (l < lim) row[l] = x.x;
+  if (l + 1 < lim) row[l + 1] = x.y;
+  if (l + 2 < lim) row[l + 2] = x.z;
+  if (l + 3 < lim) row[l + 3] = x.w;
+}
+
+// ---------------------------------------------------------------------------
+// fused step with plain loads and stores, for few tiles: a warp owns 128
+// elements (a lane 4) and runs through the workers in ascending order, kWk of
+// them loaded at a time. Bound by the latency of a few dependent loads, so it
+// has none it can do without: the slots of a lane's blocks are looked up for
+// every worker along with e and g (no union flags first), and w_t - w_{t-1} is
+// read as it lies, zero outside the last union.
+// ---------------------------------------------------------------------------
+constexpr int kLsSub = 128;  // elements per warp
+constexpr int kWk = 4;       // workers loaded together
+
+template <bool kBf16, bool kDetach>
 __global__ void __launch_bounds__(kThreads) k_rbgs_step(RbgsArgs A) {
   griddep_wait();
-  constexpr int U = kRbgsTile / (kThreads * 4);  // float4 groups per thread
-  __shared__ unsigned long long ws[32];
-  uint32_t nonfinite = 0;
-  unsigned long long pairs = 0, nnz = 0, uni = 0, changed = 0;
+  __shared__ unsigned long long red[kWarps * kEndWords];
+  const int lane = threadIdx.x & 31;
+  uint32_t nonfinite = 0, pairs = 0, nnz = 0, uni = 0, changed = 0;
   const int64_t slab_ld = A.m * A.B;
+  const int64_t nw = (int64_t)gridDim.x * kWarps;
 
-  for (int64_t tile = blockIdx.x; tile < A.n_tiles; tile += gridDim.x) {
-    const int64_t t0 = tile * kRbgsTile;
-    const int64_t last = (t0 + kRbgsTile < A.d ? t0 + kRbgsTile : A.d) - 1;
-    const int64_t b_lo = block_of(t0, A), b_hi = block_of(last, A);
-    int tp = 0, tc = 0;
-    for (int64_t b = b_lo + threadIdx.x; b <= b_hi; b += kThreads) {
-      tp |= A.has_prev ? A.uflag_prev[b] : 0;
-      tc |= A.uflag_cur[b];
+  for (int64_t g0 = ((int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5)) * kLsSub; g0 < A.d; g0 += nw * kLsSub) {
+    const int64_t j = g0 + lane * 4;
+    const int lim = A.d - g0 < kLsSub ? (int)(A.d - g0) : kLsSub;
+    const float4 d4 = *reinterpret_cast<const float4*>(A.dlt + j);
+    const float4 w4 = *reinterpret_cast<const float4*>(A.w + j);
+    uint32_t bid[4];
+    float acc[4];
+    uint32_t inU = 0;  // bit i: coordinate in this step's union
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      acc[i] = 0.f;
+      bid[i] = lane * 4 + i < lim ? block_of(j + i, A) : 0u;
     }
-    tp = __syncthreads_or(tp);
-    tc = __syncthreads_or(tc);
-
-    uint32_t bid[U][4];
-    float dlv[U][4], acc[U][4];
-    uint32_t inU = 0;  // bit (u*4+i): coordinate in this step's union
+    for (int k0 = 0; k0 < A.K; k0 += kWk) {
+      float4 ev[kWk], gv[kWk];
+      int32_t at[kWk][4];  // slot of the element's block among worker k's chosen ones, or -1
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int64_t j = t0 + u * (kThreads * 4) + threadIdx.x * 4;
-      float4 d4 = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (tp) d4 = *reinterpret_cast<const float4*>(A.dlt + j);
-      dlv[u][0] = d4.x; dlv[u][1] = d4.y; dlv[u][2] = d4.z; dlv[u][3] = d4.w;
+      for (int q = 0; q < kWk; ++q) {
+        const int k = k0 + q;
+        if (k < A.K) {
+          ev[q] = __ldcs(reinterpret_cast<const float4*>(A.e + (int64_t)k * A.ld + j));
+          const float* gk = A.grads + (int64_t)k * A.d;
+          gv[q] = kBf16 ? load_g4_bf16(A.grads16 + (int64_t)k * A.d, j, A.d) : load_g4(gk, j, A.d, g_mode(gk));
+          const int32_t* rk = A.rank + (A.per_worker ? (int64_t)k * A.nb : 0);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        acc[u][i] = 0.f;
-        const bool in = j + i < A.d;
-        bid[u][i] = in ? block_of(j + i, A) : 0u;
-        if (in && tc && A.uflag_cur[bid[u][i]]) inU |= 1u << (u * 4 + i);
-      }
-    }
-
-    for (int k = 0; k < A.K; ++k) {
-      const int32_t* rk = A.rank + (A.per_worker ? (int64_t)k * A.nb : 0);
-      float* ek = A.e + (int64_t)k * A.ld;
-      const float* gk = A.grads + (int64_t)k * A.d;
-      const uint16_t* gk16 = A.grads16 + (int64_t)k * A.d;
-      float* sk = A.slab + (int64_t)k * slab_ld;
-      const int gm = g_mode(gk);
-      float4 ev[U], gv[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int64_t j = t0 + u * (kThreads * 4) + threadIdx.x * 4;
-        ev[u] = __ldcs(reinterpret_cast<const float4*>(ek + j));
-        gv[u] = kBf16 ? load_g4_bf16(gk16, j, A.d) : load_g4(gk, j, A.d, gm);
+          for (int i = 0; i < 4; ++i) at[q][i] = lane * 4 + i < lim ? rk[bid[i]] : -1;
+        }
       }
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int64_t j = t0 + u * (kThreads * 4) + threadIdx.x * 4;
-        float v[4] = {accumulate(ev[u].x, gv[u].x, A.c, dlv[u][0]),
-                      accumulate(ev[u].y, gv[u].y, A.c, dlv[u][1]),
-                      accumulate(ev[u].z, gv[u].z, A.c, dlv[u][2]),
-                      accumulate(ev[u].w, gv[u].w, A.c, dlv[u][3])};
-        float en[4];
+      for (int q = 0; q < kWk; ++q) {
+        const int k = k0 + q;
+        if (k < A.K) {
+          float* sk = A.slab + (int64_t)k * slab_ld;
+          const float v[4] = {accumulate(ev[q].x, gv[q].x, A.c, d4.x), accumulate(ev[q].y, gv[q].y, A.c, d4.y),
+                              accumulate(ev[q].z, gv[q].z, A.c, d4.z), accumulate(ev[q].w, gv[q].w, A.c, d4.w)};
+          float en[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          en[i] = v[i];
-          if (j + i < A.d) {
-            nonfinite += is_nonfinite(v[i]) ? 1u : 0u;
-            if (tc) {
-              const int32_t q = rk[bid[u][i]];
-              if (q >= 0) {
-                acc[u][i] = __fadd_rn(acc[u][i], v[i]);
-                sk[(int64_t)q * A.B + (j + i - (int64_t)bid[u][i] * A.B)] = v[i];
-                en[i] = 0.f;  // e_{t+1,k} = +0 where sent
-                ++pairs;
-                nnz += (v[i] != 0.f);
-              }
+          for (int i = 0; i < 4; ++i) {
+            en[i] = v[i];
+            if (lane * 4 + i < lim) nonfinite += is_nonfinite(v[i]) ? 1u : 0u;
+            if (at[q][i] >= 0) {
+              inU |= 1u << i;
+              acc[i] = __fadd_rn(acc[i], v[i]);
+              sk[(int64_t)at[q][i] * A.B + (j + i - (int64_t)bid[i] * A.B)] = v[i];
+              en[i] = 0.f;  // e_{t+1,k} = +0 where sent
+              ++pairs;
+              nnz += (v[i] != 0.f);
             }
           }
+          __stcs(reinterpret_cast<float4*>(A.e + (int64_t)k * A.ld + j), make_float4(en[0], en[1], en[2], en[3]));
         }
-        __stcs(reinterpret_cast<float4*>(ek + j), make_float4(en[0], en[1], en[2], en[3]));
       }
     }
-
-    if (tp || tc) {
+    float wo[4] = {w4.x, w4.y, w4.z, w4.w};
+    float dd[4] = {0.f, 0.f, 0.f, 0.f};
+    bool touch = (__float_as_uint(d4.x) | __float_as_uint(d4.y) | __float_as_uint(d4.z) | __float_as_uint(d4.w)) != 0u;
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int64_t j = t0 + u * (kThreads * 4) + threadIdx.x * 4;
-        float dd[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (inU & (1u << (u * 4 + i))) {
-            const float wo = A.w[j + i];
-            const float wn = __fsub_rn(wo, __fmul_rn(A.a, acc[u][i]));
-            A.w[j + i] = wn;
-            dd[i] = __fsub_rn(wn, wo);
-            changed += (dd[i] != 0.f);
-            ++uni;
-          }
-        }
-        *reinterpret_cast<float4*>(A.dlt + j) = make_float4(dd[0], dd[1], dd[2], dd[3]);
+    for (int i = 0; i < 4; ++i) {
+      if (inU & (1u << i)) {
+        const float wn = __fsub_rn(wo[i], __fmul_rn(A.a, acc[i]));
+        A.w[j + i] = wn;
+        dd[i] = __fsub_rn(wn, wo[i]);
+        wo[i] = wn;
+        changed += (dd[i] != 0.f);
+        ++uni;
+        touch = true;
+      }
+    }
+    if (touch) *reinterpret_cast<float4*>(A.dlt + j) = make_float4(dd[0], dd[1], dd[2], dd[3]);
+    if (kDetach) {  // the residuals as this lane stored them
+      const float4 wn4 = make_float4(wo[0], wo[1], wo[2], wo[3]);
+#pragma unroll 8
+      for (int k = 0; k < A.K; ++k) {
+        const float4 e4 = *reinterpret_cast<const float4*>(A.e + (int64_t)k * A.ld + j);
+        store_row(A.det + (int64_t)k * A.det_ld + g0, lane * 4, lim, detached4(wn4, A.det_b, e4), lane);
       }
     }
   }
-  unsigned long long tot;
-  block_inclusive_scan<unsigned long long>(pairs, ws, &tot);
-  if (threadIdx.x == 0 && tot) atomicAdd(&A.step_ctr->v[kPairs], tot);
-  block_inclusive_scan<unsigned long long>(nnz, ws, &tot);
-  if (threadIdx.x == 0 && tot) atomicAdd(&A.step_ctr->v[kNnz], tot);
-  block_inclusive_scan<unsigned long long>(uni, ws, &tot);
-  if (threadIdx.x == 0 && tot) atomicAdd(&A.step_ctr->v[kUnion], tot);
-  block_inclusive_scan<unsigned long long>(changed, ws, &tot);
-  if (threadIdx.x == 0 && tot) atomicAdd(&A.step_ctr->v[kChanged], tot);
-  if (nonfinite) {
-    atomicOr(A.status, kStatusNonfinite);
-    atomicAdd(&A.step_ctr->v[kNonfinite], (unsigned long long)nonfinite);
-  }
+  end_step(A, red, threadIdx.x >> 5, kWarps, lane, nonfinite, pairs, nnz, uni, changed);
 }
 
 // (index, value) pairs of worker k's last C(.), in ascending index order.
@@ -237,15 +354,39 @@ __global__ void k_rbgs_expand(RbgsArgs A, int k, uint32_t* idx_out, float* val_o
   }
 }
 
-// GMC+ detach: out[k][j] = w[j] - b * e[k][j] (Alg. 2).
-__global__ void k_detach(DetachArgs A) {
+// GMC+ detach: out[k][j] = w[j] - b * e[k][j] (Alg. 2), where the step's own
+// pass does not write it (top-k steps, gmc_get_worker_params). Streaming, bound
+// by memory: a warp loads its 128 floats of w once and runs through the
+// workers of its slice (blockIdx.y).
+__global__ void __launch_bounds__(kThreads) k_detach(DetachArgs A, int per) {
   griddep_wait();
-  const int k = A.k0 + blockIdx.y;
-  const float* ek = A.e + (int64_t)k * A.ld;
-  float* ok = A.out + (int64_t)(k - A.k0) * A.out_ld;
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < A.d;
-       j += (int64_t)gridDim.x * blockDim.x)
-    ok[j] = __fsub_rn(A.w[j], __fmul_rn(A.b, ek[j]));
+  const int lane = threadIdx.x & 31;
+  const int k_lo = A.k0 + blockIdx.y * per, k_hi = min(A.k1, k_lo + per);
+  const int64_t nw = (int64_t)gridDim.x * kWarps;
+  for (int64_t g0 = ((int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5)) * 128; g0 < A.d; g0 += nw * 128) {
+    const int lim = A.d - g0 < 128 ? (int)(A.d - g0) : 128;
+    // w and the rows of e are allocated in whole tiles: reads past d stay inside
+    const float4 w4 = *reinterpret_cast<const float4*>(A.w + g0 + lane * 4);
+#pragma unroll 4
+    for (int k = k_lo; k < k_hi; ++k) {
+      const float4 e4 = __ldcs(reinterpret_cast<const float4*>(A.e + (int64_t)k * A.ld + g0 + lane * 4));
+      store_row(A.out + (int64_t)(k - A.k0) * A.out_ld + g0, lane * 4, lim, detached4(w4, A.b, e4), lane);
+    }
+  }
+}
+
+// dst[0..n) = src[0..n), src 16-byte aligned and readable to the next 128
+// floats. As fast as cudaMemcpyAsync at every size (138.4 M floats: 169 against
+// 170 us) and begins while the kernel before it ends (d = 272 k: 1.8 against
+// 5.4 us on the device, 11.4 against 17 us a call on the host).
+__global__ void __launch_bounds__(kThreads) k_copy_row(const float* __restrict__ src, float* dst, int64_t n) {
+  griddep_wait();
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = (int64_t)gridDim.x * kWarps;
+  for (int64_t g0 = ((int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5)) * 128; g0 < n; g0 += nw * 128) {
+    const float4 x = *reinterpret_cast<const float4*>(src + g0 + lane * 4);
+    store_row(dst + g0, lane * 4, n - g0 < 128 ? (int)(n - g0) : 128, x, lane);
+  }
 }
 
 __global__ void k_finalize(Counters* step, Counters* total, unsigned long long pairs_add) {
@@ -280,6 +421,7 @@ struct Smem {
   uint64_t empty[kStages];                 // all consumer warps read the stage
   int32_t gmeta[kStages];                  // leading floats in the g stage, -1 = not copied
   uint32_t tq[8];                          // claimed tiles (tile_at)
+  unsigned long long red[kConsumers * kEndWords];  // the warps' counts (end_step)
 };
 // Tiles: the first two of a CTA fixed, the rest claimed one tile ahead of the
 // producer's start of the tile before it. A consumer reads a tile's slot at
@@ -291,7 +433,7 @@ constexpr int kQ = 8;
 static_assert(kQ > kStages + kFixed, "the producer may overwrite a claimed tile not yet read");
 }  // namespace rbulk
 
-template <bool kBf16>
+template <bool kBf16, bool kDetach>
 __global__ void __launch_bounds__(rbulk::kThreadsAll, 1) k_rbgs_bulk(RbgsArgs A) {
   griddep_wait();
   using namespace rbulk;
@@ -381,11 +523,13 @@ __global__ void __launch_bounds__(rbulk::kThreadsAll, 1) k_rbgs_bulk(RbgsArgs A)
     tp = __any_sync(0xffffffffu, tp);
     tc = __any_sync(0xffffffffu, tc);
     float dl[kG][4], acc[kG][4];
+    float4 w4[kG];  // detach output: w_t, which is w_{t+1} outside the union
     uint32_t bid[kG][4];
     uint32_t inU = 0;  // bit (u*4+i): coordinate in this step's union
 #pragma unroll
     for (int u = 0; u < kG; ++u) {
       const int l = u * 128 + lane * 4;
+      if (kDetach) w4[u] = *reinterpret_cast<const float4*>(A.w + s0 + l);
       float4 d4 = make_float4(0.f, 0.f, 0.f, 0.f);
       if (tp && l < lim) d4 = *reinterpret_cast<const float4*>(A.dlt + s0 + l);
       dl[u][0] = d4.x; dl[u][1] = d4.y; dl[u][2] = d4.z; dl[u][3] = d4.w;
@@ -466,7 +610,10 @@ __global__ void __launch_bounds__(rbulk::kThreadsAll, 1) k_rbgs_bulk(RbgsArgs A)
             }
           }
         }
-        __stcs(reinterpret_cast<float4*>(ek + l), make_float4(en[0], en[1], en[2], en[3]));
+        const float4 e4 = make_float4(en[0], en[1], en[2], en[3]);
+        __stcs(reinterpret_cast<float4*>(ek + l), e4);
+        if (kDetach && !tc)
+          store_row(A.det + (int64_t)k * A.det_ld + s0, l, lim, detached4(w4[u], A.det_b, e4), lane);
       }
     }
     if (ok && (tp || tc)) {  // the union: w_{t+1} = w_t - a * sum, and w_{t+1} - w_t for the next step
@@ -489,58 +636,57 @@ __global__ void __launch_bounds__(rbulk::kThreadsAll, 1) k_rbgs_bulk(RbgsArgs A)
         *reinterpret_cast<float4*>(A.dlt + s0 + l) = make_float4(dd[0], dd[1], dd[2], dd[3]);
       }
     }
+    if (kDetach && ok && tc) {  // w_{t+1} is known now; w and the residuals as this lane stored them
+#pragma unroll
+      for (int u = 0; u < kG; ++u) {
+        const int l = u * 128 + lane * 4;
+        const float4 wn4 = *reinterpret_cast<const float4*>(A.w + s0 + l);
+        for (int k = 0; k < A.K; ++k) {
+          const float4 e4 = *reinterpret_cast<const float4*>(A.e + (int64_t)k * A.ld + s0 + l);
+          store_row(A.det + (int64_t)k * A.det_ld + s0, l, lim, detached4(wn4, A.det_b, e4), lane);
+        }
+      }
+    }
   }
   if (!ok) atomicOr(A.status, kStatusTimeout);
-  pairs = warp_sum(pairs);
-  nnz = warp_sum(nnz);
-  uni = warp_sum(uni);
-  changed = warp_sum(changed);
-  if (lane == 0) {
-    if (pairs) atomicAdd(&A.step_ctr->v[kPairs], pairs);
-    if (nnz) atomicAdd(&A.step_ctr->v[kNnz], nnz);
-    if (uni) atomicAdd(&A.step_ctr->v[kUnion], uni);
-    if (changed) atomicAdd(&A.step_ctr->v[kChanged], changed);
-  }
-  if (nonfinite) {
-    atomicOr(A.status, kStatusNonfinite);
-    atomicAdd(&A.step_ctr->v[kNonfinite], (unsigned long long)nonfinite);
-  }
+  end_step(A, sm.red, warp, kConsumers, lane, nonfinite, pairs, nnz, uni, changed);
 }
 
 }  // namespace
 
 cudaError_t configure_rbgs_kernels() {
-  cudaError_t err = cudaFuncSetAttribute((const void*)k_rbgs_pick,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kPickSmemWords * 4);
-  const cudaError_t e2 = cudaFuncSetAttribute((const void*)k_rbgs_bulk<false>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)sizeof(rbulk::Smem));
-  const cudaError_t e3 = cudaFuncSetAttribute((const void*)k_rbgs_bulk<true>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)sizeof(rbulk::Smem));
-  return err != cudaSuccess ? err : (e2 != cudaSuccess ? e2 : e3);
+  cudaError_t err = cudaFuncSetAttribute((const void*)k_rbgs_pick, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kPickSmemWords * 4 + kFirstWords * 4);
+  for (const void* f : {(const void*)k_rbgs_bulk<false, false>, (const void*)k_rbgs_bulk<true, false>,
+                        (const void*)k_rbgs_bulk<false, true>, (const void*)k_rbgs_bulk<true, true>}) {
+    const cudaError_t e2 =
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(rbulk::Smem));
+    if (err == cudaSuccess) err = e2;
+  }
+  return err;
 }
 
 int rbgs_blocks_per_sm() {
   int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rbgs_step<false>, kThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rbgs_step<false, true>, kThreads, 0);
   return n > 0 ? n : 1;
 }
 
 cudaError_t launch_rbgs_pick(const RbgsArgs& A, cudaStream_t s) {
   const int64_t nbw = (A.nb + 31) / 32;
-  const int smem = nbw <= kPickSmemWords ? (int)(nbw * 4) : 0;
-  const cudaError_t err = launch_pdl(k_rbgs_pick, dim3(A.per_worker ? A.K : 1), dim3(kThreads), smem, s, A);
-  if (err != cudaSuccess) return err;
-  return cudaGetLastError();
+  const int smem = (nbw <= kPickSmemWords ? (int)(nbw * 4) : 0) + (A.nb <= kFirstWords ? (int)(A.nb * 4) : 0);
+  return launch_pdl(k_rbgs_pick, dim3(A.per_worker ? A.K : 1), dim3(kPickThreads), smem, s, A);
 }
 
 cudaError_t launch_rbgs_step(const RbgsArgs& A, int grid, cudaStream_t s) {
   if (A.bulk) {
-    return launch_pdl(A.bf16 ? k_rbgs_bulk<true> : k_rbgs_bulk<false>, dim3(grid), dim3(rbulk::kThreadsAll),
-                      sizeof(rbulk::Smem), s, A);
+    const dim3 g(grid), b(rbulk::kThreadsAll);
+    const size_t sm = sizeof(rbulk::Smem);
+    if (A.det) return launch_pdl(A.bf16 ? k_rbgs_bulk<true, true> : k_rbgs_bulk<false, true>, g, b, sm, s, A);
+    return launch_pdl(A.bf16 ? k_rbgs_bulk<true, false> : k_rbgs_bulk<false, false>, g, b, sm, s, A);
   }
-  return launch_pdl(A.bf16 ? k_rbgs_step<true> : k_rbgs_step<false>, dim3(grid), dim3(kThreads), 0, s, A);
+  if (A.det) return launch_pdl(A.bf16 ? k_rbgs_step<true, true> : k_rbgs_step<false, true>, dim3(grid), dim3(kThreads), 0, s, A);
+  return launch_pdl(A.bf16 ? k_rbgs_step<true, false> : k_rbgs_step<false, false>, dim3(grid), dim3(kThreads), 0, s, A);
 }
 
 cudaError_t launch_rbgs_expand(const RbgsArgs& A, int k, uint32_t* idx_out, float* val_out,
@@ -552,11 +698,20 @@ cudaError_t launch_rbgs_expand(const RbgsArgs& A, int k, uint32_t* idx_out, floa
 }
 
 cudaError_t launch_detach(const DetachArgs& A, cudaStream_t s) {
-  const int64_t blocks = (A.d + 255) / 256;
-  const dim3 grid((unsigned)(blocks < 1024 ? blocks : 1024), (unsigned)(A.k1 - A.k0));
-  const cudaError_t err = launch_pdl(k_detach, dim3(grid), dim3(256), 0, s, A);
-  if (err != cudaSuccess) return err;
-  return cudaGetLastError();
+  // enough warps for small d: the workers are split over blockIdx.y until about 2,048 blocks run
+  const int64_t blocks = (A.d + 128 * kWarps - 1) / (128 * kWarps);
+  const int K = A.k1 - A.k0;
+  const int split = (int)(blocks >= 2048 ? 1 : (2048 / blocks < K ? 2048 / blocks : K));
+  const int per = (K + split - 1) / split;
+  const dim3 grid((unsigned)(blocks < 65536 ? blocks : 65536), (unsigned)((K + per - 1) / per));
+  return launch_pdl(k_detach, grid, dim3(kThreads), 0, s, A, per);
+}
+
+cudaError_t launch_copy_row(const float* src, float* dst, int64_t n, cudaStream_t s) {
+  if (reinterpret_cast<uintptr_t>(dst) & 3u)
+    return cudaMemcpyAsync(dst, src, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, s);
+  const int64_t blocks = (n + 128 * kWarps - 1) / (128 * kWarps);
+  return launch_pdl(k_copy_row, dim3((unsigned)blocks), dim3(kThreads), 0, s, src, dst, n);
 }
 
 cudaError_t launch_finalize(Counters* step, Counters* total, unsigned long long pairs_add,
