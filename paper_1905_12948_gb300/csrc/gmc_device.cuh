@@ -269,6 +269,76 @@ __device__ __forceinline__ void block_find_from_top_any(const uint32_t* hist, in
   __syncthreads();
 }
 
+// Radix select in shared memory over values below 2^bits (bits <= 31), taken
+// relative to `base` (x[i] - base): digits of at most 11 bits from the top.
+// Returns base + the r-th largest; rank_out = its rank among the values equal
+// to it. With bits = 31 and base = 0 this is a select over whole keys.
+__device__ __forceinline__ uint32_t smem_select_bits(const uint32_t* x, uint32_t n, uint32_t r, int bits,
+                                                     uint32_t base, uint32_t* h, uint32_t* ws,
+                                                     uint32_t* s_bin, uint32_t* s_rank, uint32_t* rank_out) {
+  uint32_t prefix = 0;  // the digits fixed so far
+  int done = 0;         // bits fixed so far (from the top)
+  while (done < bits) {
+    const int width = min(11, bits - done), shift = bits - done - width, nbins = 1 << width;
+    for (int b = threadIdx.x; b < nbins; b += blockDim.x) h[b] = 0;
+    if (threadIdx.x == 0) {
+      *s_bin = 0;
+      *s_rank = 0;
+    }
+    __syncthreads();
+    for (uint32_t i0 = 0; i0 < n; i0 += blockDim.x) {
+      const uint32_t i = i0 + threadIdx.x;
+      if (i < n) {
+        const uint32_t v = x[i] - base;
+        // the digits above this one must match the prefix (a shift by 32 is
+        // avoided: no digit is fixed before the first pass)
+        if (done == 0 || (v >> (shift + width)) == prefix) atomicAdd(&h[(v >> shift) & (uint32_t)(nbins - 1)], 1u);
+      }
+    }
+    __syncthreads();
+    block_find_from_top_any(h, nbins, r, ws, s_bin, s_rank);
+    prefix = (prefix << width) | *s_bin;
+    r = *s_rank;
+    done += width;
+    __syncthreads();
+  }
+  *rank_out = r;
+  return base + prefix;
+}
+
+// Radix select in shared memory: the r-th largest of n values (digits 11/10/10).
+__device__ __forceinline__ uint32_t smem_select(const uint32_t* x, uint32_t n, uint32_t r,
+                                                uint32_t* h, uint32_t* ws, uint32_t* s_bin,
+                                                uint32_t* s_rank, uint32_t* rank_out) {
+  uint32_t prefix = 0;
+  for (int pass = 0; pass < 3; ++pass) {
+    const int nbins = pass == 0 ? 2048 : 1024;
+    const int shift = pass == 0 ? 20 : (pass == 1 ? 10 : 0);
+    for (int b = threadIdx.x; b < nbins; b += blockDim.x) h[b] = 0;
+    if (threadIdx.x == 0) {
+      *s_bin = 0;
+      *s_rank = 0;
+    }
+    __syncthreads();
+    for (uint32_t i0 = 0; i0 < n; i0 += blockDim.x) {
+      const uint32_t i = i0 + threadIdx.x;
+      int bin = -1;
+      if (i < n) {
+        const uint32_t v = x[i];
+        if (pass == 0 || (v >> (shift + 10)) == prefix) bin = (int)((v >> shift) & (uint32_t)(nbins - 1));
+      }
+      if (bin >= 0) atomicAdd(&h[bin], 1u);  // plain atomics measured faster than match_any here
+    }
+    __syncthreads();
+    block_find_from_top(h, nbins, r, ws, s_bin, s_rank);
+    prefix = pass == 0 ? *s_bin : ((prefix << 10) | *s_bin);
+    r = *s_rank;
+    __syncthreads();
+  }
+  *rank_out = r;
+  return prefix;
+}
+
 // ---------------------------------------------------------------------------
 // mbarrier and bulk-copy primitives (inline PTX, sm_90+ / sm_103a)
 // ---------------------------------------------------------------------------
@@ -323,6 +393,60 @@ __device__ __forceinline__ bool wait_bounded(uint64_t* bar, uint32_t parity, uin
 // predecessor's writes are visible. Without that launch attribute it returns
 // at once.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// ---------------------------------------------------------------------------
+// Grid barrier of a cooperative launch (every block resident). `bar` is a word
+// that is zero when the launch begins; the blocks' arrivals of one barrier add
+// up to 2^31, so its top bit flips when the last one arrives. A wait is bounded
+// (limit_ns): false, for the whole block, when it gave up -- the block then
+// leaves. The word is put back to zero by the last block to leave (leave_grid),
+// also after a wait that gave up.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t* s_ok, uint64_t limit_ns) {
+  const uint32_t n = gridDim.x;
+  if (n == 1) {
+    __syncthreads();
+    return true;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const uint32_t old = atomicAdd(bar, blockIdx.x == 0 ? 0x80000000u - (n - 1) : 1u);
+    uint32_t ok = 1;
+    uint64_t t0 = 0;
+    for (uint32_t spins = 0; ((old ^ ld_acquire(bar)) & 0x80000000u) == 0; ++spins) {
+      if ((spins & 1023u) == 1023u) {
+        const uint64_t now = global_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > limit_ns) {
+          ok = 0;
+          break;
+        }
+      }
+    }
+    __threadfence();
+    *s_ok = ok;
+  }
+  __syncthreads();
+  return *s_ok != 0;
+}
+// Every block, as its last act: true for the last one of the grid to call it
+// (all its threads), which then resets what the next launch finds zeroed.
+__device__ __forceinline__ bool leave_grid(uint32_t* left, uint32_t* s_last) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    *s_last = atomicAdd(left, 1u) == gridDim.x - 1 ? 1u : 0u;
+    __threadfence();
+  }
+  __syncthreads();
+  return *s_last != 0;
+}
 
 // Tiles of a persistent streaming pass. A CTA's first kFixed tiles are fixed,
 // blockIdx.x + n * gridDim.x; every later one is claimed from a counter that

@@ -306,76 +306,6 @@ __global__ void __launch_bounds__(kThreads) k_sample(TopkArgs A) {
   // k_sample_theta fixes theta exactly from the keys and this histogram
 }
 
-// Radix select in shared memory over values below 2^bits (bits <= 31), taken
-// relative to `base` (x[i] - base): digits of at most 11 bits from the top.
-// Returns base + the r-th largest; rank_out = its rank among the values equal
-// to it. With bits = 31 and base = 0 this is a select over whole keys.
-__device__ __forceinline__ uint32_t smem_select_bits(const uint32_t* x, uint32_t n, uint32_t r, int bits,
-                                                     uint32_t base, uint32_t* h, uint32_t* ws,
-                                                     uint32_t* s_bin, uint32_t* s_rank, uint32_t* rank_out) {
-  uint32_t prefix = 0;  // the digits fixed so far
-  int done = 0;         // bits fixed so far (from the top)
-  while (done < bits) {
-    const int width = min(11, bits - done), shift = bits - done - width, nbins = 1 << width;
-    for (int b = threadIdx.x; b < nbins; b += blockDim.x) h[b] = 0;
-    if (threadIdx.x == 0) {
-      *s_bin = 0;
-      *s_rank = 0;
-    }
-    __syncthreads();
-    for (uint32_t i0 = 0; i0 < n; i0 += blockDim.x) {
-      const uint32_t i = i0 + threadIdx.x;
-      if (i < n) {
-        const uint32_t v = x[i] - base;
-        // the digits above this one must match the prefix (a shift by 32 is
-        // avoided: no digit is fixed before the first pass)
-        if (done == 0 || (v >> (shift + width)) == prefix) atomicAdd(&h[(v >> shift) & (uint32_t)(nbins - 1)], 1u);
-      }
-    }
-    __syncthreads();
-    block_find_from_top_any(h, nbins, r, ws, s_bin, s_rank);
-    prefix = (prefix << width) | *s_bin;
-    r = *s_rank;
-    done += width;
-    __syncthreads();
-  }
-  *rank_out = r;
-  return base + prefix;
-}
-
-// Radix select in shared memory: the r-th largest of n values (digits 11/10/10).
-__device__ __forceinline__ uint32_t smem_select(const uint32_t* x, uint32_t n, uint32_t r,
-                                                uint32_t* h, uint32_t* ws, uint32_t* s_bin,
-                                                uint32_t* s_rank, uint32_t* rank_out) {
-  uint32_t prefix = 0;
-  for (int pass = 0; pass < 3; ++pass) {
-    const int nbins = pass == 0 ? 2048 : 1024;
-    const int shift = pass == 0 ? 20 : (pass == 1 ? 10 : 0);
-    for (int b = threadIdx.x; b < nbins; b += blockDim.x) h[b] = 0;
-    if (threadIdx.x == 0) {
-      *s_bin = 0;
-      *s_rank = 0;
-    }
-    __syncthreads();
-    for (uint32_t i0 = 0; i0 < n; i0 += blockDim.x) {
-      const uint32_t i = i0 + threadIdx.x;
-      int bin = -1;
-      if (i < n) {
-        const uint32_t v = x[i];
-        if (pass == 0 || (v >> (shift + 10)) == prefix) bin = (int)((v >> shift) & (uint32_t)(nbins - 1));
-      }
-      if (bin >= 0) atomicAdd(&h[bin], 1u);  // plain atomics measured faster than match_any here
-    }
-    __syncthreads();
-    block_find_from_top(h, nbins, r, ws, s_bin, s_rank);
-    prefix = pass == 0 ? *s_bin : ((prefix << 10) | *s_bin);
-    r = *s_rank;
-    __syncthreads();
-  }
-  *rank_out = r;
-  return prefix;
-}
-
 // ---------------------------------------------------------------------------
 // The exact top-k's sample with one thread-block cluster per worker (its CTAs
 // are co-scheduled by the hardware). Each CTA forms v at its slots (up to 8 per
