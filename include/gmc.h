@@ -102,7 +102,9 @@ typedef struct gmc_ctx* gmc_t;
 #define GMC_STAT_NNZ        2 /* sum_k ||C_k||_0: sent components that are non-zero */
 #define GMC_STAT_UNION      3 /* |U_t|: coordinates sent by at least one worker */
 #define GMC_STAT_CHANGED    4 /* ||w_{t+1} - w_t||_0 */
-#define GMC_STAT_FALLBACKS  5 /* workers whose sampled filter fell back to the dense select */
+#define GMC_STAT_FALLBACKS  5 /* workers whose sampled filter fell back to the dense select (in the
+                                 one-launch step of small problems: whose k-th key had over 64
+                                 ties, or whose approximate top-s exceeded its limit) */
 #define GMC_STAT_NONFINITE  6 /* accumulator values that were NaN or Inf */
 #define GMC_STAT_COUNT      8 /* array length to pass */
 

@@ -51,6 +51,8 @@ struct gmc_ctx {
   uint32_t B_shift = 0xffffffffu;
   int grid_acc = 1, grid_agg = 1, grid_rbgs = 1, sel_blocks = 1;
   bool rbgs_bulk = false;
+  int grid_small = 0;                 // the one-launch top-k step's grid, 0: not taken
+  uint32_t* small_scratch = nullptr;
   // state
   int64_t t = 0;
   bool initialized = false;
@@ -407,12 +409,22 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
   const uint16_t* grads16 = bf16 ? static_cast<const uint16_t*>(grads_any) : nullptr;
   const double Kd = (double)h->K * (double)h->d;
   GMC_TRY(order_after_flush(h, s, true));
+  const bool small = h->grid_small && h->select_mode == GMC_SELECT_SAMPLED;
   // the exact top-k's sample kernel and the RBGS pick clear the step's counters
   // themselves (a memset between two kernels would keep the second from starting early)
-  if (h->compressor == GMC_TOPK_APPROX) GMC_TRY(cudaMemsetAsync(h->step_ctr, 0, sizeof(Counters), s));
+  if (h->compressor == GMC_TOPK_APPROX && !small) GMC_TRY(cudaMemsetAsync(h->step_ctr, 0, sizeof(Counters), s));
   unsigned long long pairs_add = 0;
   bool finalized = false;  // the step's counters already added up by its last kernel
-  if (h->compressor != GMC_RBGS) {
+  if (small) {
+    TopkArgs A = topk_args(h, grads);
+    A.grads16 = grads16;
+    A.bf16 = bf16 ? 1 : 0;
+    const DetachArgs D{h->w, h->e, h->ld, h->d, detach_b(h), h->detach_out, h->detach_ld, 0, h->K};
+    const double bytes = ((A.local_mom ? 20.0 : 12.0) - (bf16 ? 2.0 : 0.0)) * Kd + (D.out ? 4.0 * Kd : 0.0);
+    GMC_TRY(timed(h, GMC_KERNEL_ACCUMULATE, bytes, s,
+                  [&] { return launch_topk_step(A, D, h->grid_small, h->small_scratch, s); }));
+    finalized = true;
+  } else if (h->compressor != GMC_RBGS) {
     const bool approx = h->compressor == GMC_TOPK_APPROX;
     TopkArgs A = topk_args(h, grads);
     A.grads16 = grads16;
@@ -480,14 +492,14 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
                   [&] { return launch_rbgs_step(A, h->grid_rbgs, s); }));
     finalized = true;
   }
-  if (h->detach_out && h->compressor != GMC_RBGS) {
+  if (h->detach_out && h->compressor != GMC_RBGS && !small) {
     DetachArgs D{h->w, h->e, h->ld, h->d, detach_b(h), h->detach_out, h->detach_ld, 0, h->K};
     GMC_TRY(timed(h, GMC_KERNEL_DETACH, 8.0 * Kd + 4.0 * h->d, s, [&] { return launch_detach(D, s); }));
   }
   if (!finalized)
     GMC_TRY(timed(h, GMC_KERNEL_OTHER, 0.0, s,
                   [&] { return launch_finalize(h->step_ctr, h->total_ctr, pairs_add, s); }));
-  if (h->ev_step) GMC_TRY(cudaEventRecord(h->ev_step, s));
+  if (h->agg_pending) GMC_TRY(cudaEventRecord(h->ev_step, s));  // a flush on another stream waits for it
   h->t += 1;
   h->restored = false;
   return GMC_OK;
@@ -579,6 +591,7 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
   };
   cudaError_t err = configure_topk_kernels();
   if (err == cudaSuccess) err = configure_rbgs_kernels();
+  if (err == cudaSuccess) err = configure_small_kernels();
   if (err != cudaSuccess) return fail(err);
 
   const int64_t streams_wide = 2 * (int64_t)h->num_sms;
@@ -588,6 +601,10 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
     int U = K <= kBulkMaxK ? 4 : 2;
     if (d < 4096 * streams_wide) U = 2;
     if (d < 2048 * streams_wide) U = 1;
+    // a problem that fits in the SMs' shared memory takes the one-launch step,
+    // whose sub-chunks are groups of 128 coordinates (tiles of 1024)
+    h->grid_small = U < 4 || K > kBulkMaxK ? small_grid(d, K, h->num_sms) : 0;
+    if (h->grid_small) U = 1;
     h->tile = 1024 * U;
     h->n_tiles = (d + h->tile - 1) / h->tile;
     h->ld = h->n_tiles * h->tile;
@@ -674,6 +691,7 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
         (err = dalloc(h, &h->mask, (size_t)h->ld)) != cudaSuccess ||
         (err = dalloc(h, &h->sample_pend, (size_t)3 * h->sample_stride)) != cudaSuccess)
       return fail(err);
+    if (h->grid_small && (err = dalloc(h, &h->small_scratch, small_scratch_words(K))) != cudaSuccess) return fail(err);
     if (h->n_blk >= 8 && ((err = dalloc(h, &h->blk_cost, (size_t)h->n_blk)) != cudaSuccess ||
                           (err = dalloc(h, &h->blk_order, (size_t)h->n_blk)) != cudaSuccess))
       return fail(err);
@@ -815,6 +833,8 @@ int reset_state(gmc_ctx* h, cudaStream_t s) {
       GMC_TRY(cudaMemsetAsync(h->chunk[p], 0, (size_t)h->K * h->n_tiles * kChunksPerTile * sizeof(uint2), s));
     GMC_TRY(cudaMemsetAsync(h->sel, 0, (size_t)h->K * sizeof(WorkerSel), s));
     GMC_TRY(cudaMemsetAsync(h->mask, 0, (size_t)h->ld * sizeof(uint32_t), s));
+    if (h->small_scratch)
+      GMC_TRY(cudaMemsetAsync(h->small_scratch, 0, small_scratch_words(h->K) * sizeof(uint32_t), s));
     if (h->blk_cost) GMC_TRY(cudaMemsetAsync(h->blk_cost, 0, (size_t)h->n_blk * sizeof(uint32_t), s));
   } else {
     for (int p = 0; p < 2; ++p) GMC_TRY(cudaMemsetAsync(h->uflag[p], 0, (size_t)h->nb, s));

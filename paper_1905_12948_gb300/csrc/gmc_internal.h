@@ -230,6 +230,17 @@ int accumulate_smem_bytes(int tile, int K);
 cudaError_t configure_topk_kernels();
 cudaError_t configure_rbgs_kernels();
 
+// The one-launch top-k step (gmc_small.cu): up to kSmallItems (group of 128
+// coordinates, worker) accumulators of 512 bytes in a block's shared memory.
+constexpr int kSmallItems = 376;
+__host__ __device__ constexpr int kItemMaxBytes(int groups, int grid, int K) {
+  return (groups + grid - 1) / grid * K * 512;
+}
+int small_grid(int64_t d, int K, int num_sms);  // its grid, 0 when the problem does not fit
+size_t small_scratch_words(int K);
+cudaError_t configure_small_kernels();
+cudaError_t launch_topk_step(const TopkArgs& A, const DetachArgs& D, int grid, uint32_t* scratch, cudaStream_t s);
+
 constexpr int kRbgsTile = 4096;  // elements per tile of the fused RBGS kernel
 
 }  // namespace gmc

@@ -24,29 +24,6 @@ namespace {
 
 constexpr int kPickSmemWords = 12288;  // bitmap words kept in shared memory
 
-__device__ __forceinline__ float4 load_g4(const float* __restrict__ g, int64_t j, int64_t d,
-                                          int mode) {
-  if (j + 3 < d) {
-    if (mode == 4) return __ldcs(reinterpret_cast<const float4*>(g + j));
-    if (mode == 2) {
-      const float2 a = __ldcs(reinterpret_cast<const float2*>(g + j));
-      const float2 b = __ldcs(reinterpret_cast<const float2*>(g + j + 2));
-      return make_float4(a.x, a.y, b.x, b.y);
-    }
-    return make_float4(__ldcs(g + j), __ldcs(g + j + 1), __ldcs(g + j + 2), __ldcs(g + j + 3));
-  }
-  float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (j < d) r.x = g[j];
-  if (j + 1 < d) r.y = g[j + 1];
-  if (j + 2 < d) r.z = g[j + 2];
-  return r;
-}
-
-__device__ __forceinline__ int g_mode(const float* p) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-  return (a & 15) == 0 ? 4 : ((a & 7) == 0 ? 2 : 1);
-}
-
 __device__ __forceinline__ uint32_t block_of(int64_t j, const RbgsArgs& A) {
   return A.B_shift != 0xffffffffu ? (uint32_t)(j >> A.B_shift) : (uint32_t)(j / A.B);
 }
@@ -187,55 +164,11 @@ __device__ __forceinline__ void end_step(const RbgsArgs& A, unsigned long long* 
       *reinterpret_cast<uint32_t*>(A.uflag_prev + b) = 0u;
 }
 
-// One group of 128 consecutive floats of a warp (lane l: elements 4l .. 4l+3)
-// stored at p, any 4-byte alignment: 16-byte stores of the aligned quads, each
-// made of its own and the next lane's values, and single floats at both ends.
-// mis: floats from p to the next 16-byte boundary (uniform over the warp).
-__device__ __forceinline__ void store_row128(float* p, float4 x, int mis, int lane) {
-  if (mis == 0) {
-    __stcs(reinterpret_cast<float4*>(p + lane * 4), x);
-    return;
-  }
-  float4 n;  // the next lane's values
-  n.x = __shfl_down_sync(0xffffffffu, x.x, 1);
-  n.y = __shfl_down_sync(0xffffffffu, x.y, 1);
-  n.z = __shfl_down_sync(0xffffffffu, x.z, 1);
-  const float4 q = mis == 1 ? make_float4(x.y, x.z, x.w, n.x)
-                            : (mis == 2 ? make_float4(x.z, x.w, n.x, n.y) : make_float4(x.w, n.x, n.y, n.z));
-  if (lane < 31) __stcs(reinterpret_cast<float4*>(p + lane * 4 + mis), q);
-  if (lane == 0) {
-    p[0] = x.x;
-    if (mis > 1) p[1] = x.y;
-    if (mis > 2) p[2] = x.z;
-  }
-  if (lane == 31) {  // the elements past the last whole quad
-    p[127] = x.w;
-    if (mis < 3) p[126] = x.z;
-    if (mis < 2) p[125] = x.y;
-  }
-}
-__device__ __forceinline__ int row_mis(const float* p) {
-  return (int)((4u - (uint32_t)(reinterpret_cast<uintptr_t>(p) >> 2)) & 3u);
-}
 // GMC+ detach (Alg. 2): w_{t+1} - b*e_{t+1,k} of 4 elements.
 __device__ __forceinline__ float4 detached4(float4 w, float b, float4 e) {
   return make_float4(__fsub_rn(w.x, __fmul_rn(b, e.x)), __fsub_rn(w.y, __fmul_rn(b, e.y)),
                      __fsub_rn(w.z, __fmul_rn(b, e.z)), __fsub_rn(w.w, __fmul_rn(b, e.w)));
 }
-// A lane's 4 elements at offset l of a sub-tile with lim valid elements, at row.
-__device__ __forceinline__ void store_row(float* row, int l, int lim, float4 x, int lane) {
-  // l - lane*4: the start of the warp's 128 elements
-  const int g0 = l - lane * 4;
-  if (g0 + 128 <= lim) {
-    store_row128(row + g0, x, row_mis(row + g0), lane);
-    return;
-  }
-  if (l < lim) row[l] = x.x;
-  if (l + 1 < lim) row[l + 1] = x.y;
-  if (l + 2 < lim) row[l + 2] = x.z;
-  if (l + 3 < lim) row[l + 3] = x.w;
-}
-
 // ---------------------------------------------------------------------------
 // fused step with plain loads and stores, for few tiles: a warp owns 128
 // elements (a lane 4) and runs through the workers in ascending order, kWk of

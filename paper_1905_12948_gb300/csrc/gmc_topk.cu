@@ -32,24 +32,6 @@ namespace {
 
 constexpr int kMaxK = 32;  // workers supported by the top-k kernels (one lane or mask bit each)
 
-__device__ __forceinline__ float4 load_g4(const float* __restrict__ g, int64_t j, int64_t d,
-                                          int mode) {
-  if (j + 3 < d) {
-    if (mode == 4) return __ldcs(reinterpret_cast<const float4*>(g + j));
-    if (mode == 2) {
-      const float2 a = __ldcs(reinterpret_cast<const float2*>(g + j));
-      const float2 b = __ldcs(reinterpret_cast<const float2*>(g + j + 2));
-      return make_float4(a.x, a.y, b.x, b.y);
-    }
-    return make_float4(__ldcs(g + j), __ldcs(g + j + 1), __ldcs(g + j + 2), __ldcs(g + j + 3));
-  }
-  float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (j < d) r.x = g[j];
-  if (j + 1 < d) r.y = g[j + 1];
-  if (j + 2 < d) r.z = g[j + 2];
-  return r;
-}
-
 // The local momentum of worker k at sampled coordinate j, formed from g
 // (m_{t+1} = beta*m_t + eta*g, Sec. 2.3 eq. (3)) without storing it.
 __device__ __forceinline__ float local_m(const TopkArgs& A, int k, int64_t j, float g) {
@@ -78,12 +60,6 @@ __device__ __forceinline__ float4 scale_g(const TopkArgs& A, float4 g) {
   }
   return g;
 }
-
-__device__ __forceinline__ int g_mode(const float* p) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-  return (a & 15) == 0 ? 4 : ((a & 7) == 0 ? 2 : 1);
-}
-
 
 __device__ __forceinline__ uint32_t warp_excl_scan(uint32_t x, uint32_t* total) {
   const int lane = threadIdx.x & 31;

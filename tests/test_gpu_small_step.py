@@ -1,0 +1,90 @@
+"""The top-k step as one cooperative launch (problems that fit in the SMs' shared
+memory): edges of its split into groups of 128, its radix rounds, lists and ties,
+and steps of the other path before and after it. Bit for bit against the oracle."""
+import numpy as np
+import pytest
+
+from parity_util import Pair, assert_fp32_state
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("compressor", ["topk", "topk_approx"])
+@pytest.mark.parametrize("d,K,ratio", [
+    (1, 1, 1.0), (5, 2, 0.5), (127, 3, 0.1), (129, 32, 0.05), (1_000, 9, 1.0),
+    (128 * 152, 4, 0.01), (128 * 152 + 1, 5, 0.001), (210_001, 32, 0.01), (900_007, 8, 0.002),
+    (1_200_003, 1, 0.3), (1_244_159, 6, 0.001),   # the largest slices
+])
+def test_sizes(d, K, ratio, compressor):
+    rng = np.random.default_rng(d + K)
+    p = Pair(d, K, 0.9, 0.1, compressor=compressor, ratio=ratio, seed=4)
+    for t in range(3):
+        g = (rng.standard_normal((K, d)) * np.exp(rng.uniform(-3, 0, size=d))).astype(np.float32)
+        p.compare(p.step(g), workers=sorted({0, K - 1}))
+    p.compare_stats()
+    assert p.gpu.check() == 0
+
+
+@pytest.mark.parametrize("levels,ratio", [(1, 0.3), (3, 0.1), (200, 0.01), (200_000, 0.02)])
+def test_ties(levels, ratio):
+    """Few distinct magnitudes: ties at the k-th key from 64 up to all of d."""
+    d, K = 300_003, 3
+    rng = np.random.default_rng(levels)
+    p = Pair(d, K, 0.0, 0.1, ratio=ratio, w0=np.zeros(d, np.float32))
+    for t in range(2):
+        g = rng.integers(1, levels + 1, size=(K, d)).astype(np.float32) * rng.choice([-1.0, 1.0], size=(K, d))
+        p.compare(p.step(g.astype(np.float32)))
+    p.compare_stats()
+
+
+@pytest.mark.parametrize("variant,lam", [("gmc", 0.5), ("server_momentum", None), ("lr_in_residual", None),
+                                         ("local_momentum", 0.3), ("local_momentum_mfm", 0.3)])
+@pytest.mark.parametrize("bf16,offset", [(False, 1), (True, 3)])
+def test_forms_with_detached_rows_and_misaligned_inputs(variant, lam, bf16, offset):
+    import torch
+    d, K = 40_003, 5
+    rng = np.random.default_rng(7)
+    p = Pair(d, K, 0.9, 0.1, ratio=0.01, variant=variant, lam=lam)
+    out = torch.zeros(K * (d + 1) + 8, dtype=torch.float32, device=p.dev)
+    if lam is not None:
+        assert p.gpu.lib.gmc_set_detach_output(p.gpu.h, out.data_ptr() + 4 * offset, d + 1) == 0
+    dt = torch.bfloat16 if bf16 else torch.float32
+    buf = torch.empty(K * d + offset, dtype=dt, device=p.dev)
+    for t in range(3):
+        g = torch.from_numpy(rng.standard_normal((K, d)).astype(np.float32)).to(dt)
+        view = buf[offset:].view(K, d)
+        view.copy_(g)
+        p.compare(p.step(g.float().numpy(), view))
+        if lam is not None:
+            rows = out[offset: offset + K * (d + 1)].view(K, d + 1).cpu().numpy()
+            for k in range(K):
+                assert_fp32_state(rows[k, :d], p.ref.worker_params(k), f"detached row {k}")
+    p.compare_stats()
+
+
+def test_alternating_with_the_dense_engine():
+    """Steps of the one-launch path and of the dense engine continue one another."""
+    d, K = 50_001, 4
+    rng = np.random.default_rng(3)
+    p = Pair(d, K, 0.9, 0.1, ratio=0.01)
+    for t in range(6):
+        assert p.gpu.lib.gmc_set_select_mode(p.gpu.h, t % 2) == 0
+        p.compare(p.step(rng.standard_normal((K, d)).astype(np.float32)))
+    p.compare_stats()
+
+
+def test_captured_in_a_graph():
+    import torch
+    d, K = 65_536, 4
+    rng = np.random.default_rng(5)
+    p = Pair(d, K, 0.9, 0.1, ratio=0.01)
+    g = [rng.standard_normal((K, d)).astype(np.float32) for _ in range(2)]
+    dev = [torch.from_numpy(x).to(p.dev) for x in g]
+    p.step(g[0], dev[0])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        p.gpu.step(dev[1])
+    graph.replay()
+    torch.cuda.synchronize()
+    p.compare(p.ref.step(g[1]))
