@@ -104,15 +104,31 @@ def _check(status: int, what: str) -> None:
         raise GMCError(status, what)
 
 
+_torch = None          # imported on the first use of a tensor: the C ABI needs no torch
+_raw_stream = None     # (device index) -> the current stream's cudaStream_t
+
+
+def _import_torch():
+    global _torch, _raw_stream
+    if _torch is None:
+        import torch
+        # the current stream's handle without building a torch.cuda.Stream:
+        # 0.3 us instead of 3 us a call, on a path that small steps are bound by
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+            lambda dev: torch.cuda.current_stream(dev).cuda_stream)
+        _torch = torch
+    return _torch
+
+
 def _stream_ptr(stream) -> int:
-    import torch
+    torch = _torch or _import_torch()
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return _raw_stream(torch.cuda.current_device())
     return int(stream.cuda_stream)
 
 
 def _dev_ptr(t, dtype, name: str) -> int:
-    import torch
+    torch = _torch or _import_torch()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype or not t.is_contiguous():
@@ -127,8 +143,7 @@ class GMC:
                  ratio: float = 0.01, block: int = 4096, lam: Optional[float] = None,
                  seed: int = 0, per_worker: bool = False, select_mode: str = "sampled",
                  variant: str = "gmc", device=None):
-        import torch
-        self.torch = torch
+        self.torch = torch = _import_torch()
         self.lib = load()
         self.d, self.K = int(d), int(K)
         self.compressor = compressor
