@@ -73,7 +73,6 @@ struct gmc_ctx {
   uint32_t* cand_idx[2] = {nullptr, nullptr};
   float* cand_val[2] = {nullptr, nullptr};
   uint2* chunk[2] = {nullptr, nullptr};
-  uint32_t* mask = nullptr;
   uint32_t* sample_pend = nullptr;  // 3 x sample_stride
   // sample geometry; approximate top-s: its limit and theta blocks
   uint32_t n_sample = 0, sample_stride = 0, limit = 0;
@@ -294,7 +293,6 @@ TopkArgs topk_args_at(gmc_ctx* h, const float* grads, int64_t t) {
   A.cand_idx = h->cand_idx[cur];
   A.cand_val = h->cand_val[cur];
   A.chunk = h->chunk[cur];
-  A.mask = h->mask;
   A.cand_idx_prev = h->cand_idx[prev];
   A.cand_val_prev = h->cand_val[prev];
   A.sample_pend = h->sample_pend;
@@ -463,10 +461,11 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     } else {
       TopkArgs B = A;
       B.a_prev = A.a;
-      B.total_ctr = nullptr;  // k_finalize adds the step's counts to the totals
+      B.finalize = A.server_mom ? 0 : 1;
+      if (A.server_mom) B.total_ctr = nullptr;  // k_finalize adds the step's counts to the totals
+      finalized = !A.server_mom;
       GMC_TRY(timed(h, GMC_KERNEL_AGGREGATE, 24.0 * kk + (B.server_mom ? 20.0 * h->d : 0.0), s, [&] {
-        cudaError_t err = launch_mark(B, h->grid_agg, s);
-        if (err == cudaSuccess) err = launch_owner_sum(B, h->grid_agg, s);
+        cudaError_t err = launch_apply(B, h->grid_agg, s);
         if (err == cudaSuccess && B.server_mom) err = launch_server_update(B, s);  // Alg. 3
         return err;
       }));
@@ -505,8 +504,7 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
   return GMC_OK;
 }
 
-// Apply a pending aggregation on stream s (ordered after the last step):
-// the senders of every coordinate into mask, then k_owner_sum.
+// Apply a pending aggregation on stream s (ordered after the last step).
 int flush(gmc_ctx* h, cudaStream_t s) {
   if (!h->agg_pending) return GMC_OK;
   GMC_TRY(cudaStreamWaitEvent(s, h->ev_step, 0));
@@ -514,8 +512,7 @@ int flush(gmc_ctx* h, cudaStream_t s) {
   A.a_prev = h->a_pending;
   A.step_ctr = h->step_ctr;    // the counts belong to the last step
   A.total_ctr = h->total_ctr;  // which k_finalize has already added up
-  GMC_TRY(launch_mark(A, h->grid_agg, s));
-  GMC_TRY(launch_owner_sum(A, h->grid_agg, s));
+  GMC_TRY(launch_apply(A, h->grid_agg, s));
   GMC_TRY(cudaEventRecord(h->ev_flush, s));
   h->wait_flush = true;
   h->agg_pending = false;
@@ -641,7 +638,8 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
       h->cap = (uint32_t)std::min<double>((double)d, capd);
     }
     h->grid_acc = (int)std::min<int64_t>(h->n_tiles, (int64_t)h->num_sms * accumulate_blocks_per_sm(h->tile));
-    h->grid_agg = 0;  // set below from the candidate regions
+    // k_apply: a warp per sub-tile, as many blocks as are resident at once
+    h->grid_agg = (int)std::min<int64_t>(h->n_tiles, (int64_t)h->num_sms * apply_blocks_per_sm());
     // candidate slots: the bulk pass gives every CTA its own region per worker,
     // one part per consumer warp (twice its share of the expected candidates,
     // plus slack, in whole 128-byte lines); otherwise one region
@@ -661,7 +659,6 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
     h->cap = (uint32_t)std::min<uint64_t>(
         std::max<uint64_t>((uint64_t)h->regions * h->cap_region, h->limit), 0xfffffff0ull);
     const int64_t per = (h->cap + 8191) / 8192;
-    h->grid_agg = h->regions > 1 ? h->regions : (int)std::max<int64_t>(1, 4 * (int64_t)h->num_sms / K);
     // select: on the bulk path a warp walks the candidates of a run of at most
     // 32 parts as one list; the grid is one wave of as many blocks as fit on
     // an SM (each holds kBucketCap keys of shared memory: three on GB300), for
@@ -688,7 +685,6 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
         (err = dalloc(h, &h->sample_keys, (size_t)K * h->sample_stride)) != cudaSuccess ||
         (err = dalloc(h, &h->big_tiles, (size_t)h->n_tiles + 1)) != cudaSuccess ||
         (err = dalloc(h, &h->rcount, (size_t)K * h->regions * kChunksPerTile)) != cudaSuccess ||
-        (err = dalloc(h, &h->mask, (size_t)h->ld)) != cudaSuccess ||
         (err = dalloc(h, &h->sample_pend, (size_t)3 * h->sample_stride)) != cudaSuccess)
       return fail(err);
     if (h->grid_small && (err = dalloc(h, &h->small_scratch, small_scratch_words(K))) != cudaSuccess) return fail(err);
@@ -832,7 +828,6 @@ int reset_state(gmc_ctx* h, cudaStream_t s) {
     for (int p = 0; p < 2; ++p)
       GMC_TRY(cudaMemsetAsync(h->chunk[p], 0, (size_t)h->K * h->n_tiles * kChunksPerTile * sizeof(uint2), s));
     GMC_TRY(cudaMemsetAsync(h->sel, 0, (size_t)h->K * sizeof(WorkerSel), s));
-    GMC_TRY(cudaMemsetAsync(h->mask, 0, (size_t)h->ld * sizeof(uint32_t), s));
     if (h->small_scratch)
       GMC_TRY(cudaMemsetAsync(h->small_scratch, 0, small_scratch_words(h->K) * sizeof(uint32_t), s));
     if (h->blk_cost) GMC_TRY(cudaMemsetAsync(h->blk_cost, 0, (size_t)h->n_blk * sizeof(uint32_t), s));

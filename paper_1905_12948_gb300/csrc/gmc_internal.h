@@ -82,7 +82,6 @@ struct TopkArgs {
   uint32_t* cand_idx;        // current chunks: K x cap
   float* cand_val;
   uint2* chunk;              // sub-chunk (base, count): n_tiles x kChunksPerTile x K, see chunk_at
-  uint32_t* mask;            // d: workers that sent each coordinate (bit k), zero between steps
   int g_direct;              // grads is mapped host memory: read it with loads, not bulk copies
   const uint32_t* cand_idx_prev;    // previous step's sub-chunks
   const float* cand_val_prev;
@@ -111,7 +110,7 @@ struct TopkArgs {
   uint64_t wait_ns;          // bound of the bulk pass's mbarrier waits (kWaitLimitNs)
   int64_t hold_tile;         // test hook: the bulk pass issues no copy for item (hold_tile, hold_k),
   int hold_k;                // so that the waits on it give up; hold_tile = -1: none
-  int finalize;              // k_select_dense ends the step: adds step_ctr (+ pairs_add pairs) to the totals
+  int finalize;              // k_select_dense or k_apply ends the step: adds step_ctr (+ pairs_add pairs) to the totals
   unsigned long long pairs_add;
 };
 
@@ -204,12 +203,11 @@ cudaError_t launch_select_dense(const TopkArgs& A, cudaStream_t s);
 constexpr int kBulkTile = 4096;  // tile of the bulk-copy accumulate pass (k_accumulate_bulk)
 constexpr int kBulkMaxK = 16;    // workers the bulk-copy pass takes (its shared memory grows with K)
 
-// k_mark: the senders of every coordinate into mask (for k_owner_sum).
-cudaError_t launch_mark(const TopkArgs& A, int grid, cudaStream_t s);
 // Sum of the sent pairs into w (with a_prev), residuals to +0 where sent,
-// w_{t+1} - w_t into dlt, mask cleared; counts into step_ctr and total_ctr
-// (either may be null).
-cudaError_t launch_owner_sum(const TopkArgs& A, int grid, cudaStream_t s);
+// w_{t+1} - w_t into dlt; counts into step_ctr and total_ctr (either may be
+// null), or, with finalize, the step's end.
+cudaError_t launch_apply(const TopkArgs& A, int grid, cudaStream_t s);
+int apply_blocks_per_sm();
 cudaError_t launch_gather_selected(const TopkArgs& A, int k, uint32_t* idx_out, float* val_out,
                                    cudaStream_t s);
 cudaError_t launch_rbgs_pick(const RbgsArgs& A, cudaStream_t s);

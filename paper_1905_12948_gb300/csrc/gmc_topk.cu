@@ -17,7 +17,7 @@
 //   aggregate   a candidate is sent iff selected(key, j, T, t_idx): e = +0 where
 //               sent, the sent values summed in ascending worker order from +0,
 //               w -= (eta/K) * sum on the union, w_{t+1} - w_t kept -- in the
-//               next step's bulk pass, or at once (k_mark, k_owner_sum)
+//               next step's bulk pass, or at once (k_apply)
 //
 // Keys are the fp32 bit patterns with the sign cleared (monotone in |v|); the
 // selected set is the first k elements under (key descending, index ascending).
@@ -1914,114 +1914,148 @@ __global__ void __launch_bounds__(1024) k_select_dense(TopkArgs A) {
 }
 
 // ---------------------------------------------------------------------------
-// aggregate + update, over all candidates in parallel (no per-tile order),
-// when it is applied at once (an eager step, or reading the state):
-//   mark  a sent candidate sets its worker's bit in the coordinate's mask
-//   sum   the sent candidate of the lowest worker in the mask (the owner) adds
-//         the workers' values in ascending worker order from +0 -- each value
-//         is still in e[k][j], where the accumulate pass wrote it -- sets those
-//         e to +0, and applies w -= (eta/K) * sum, keeping w_{t+1} - w_t.
-// A candidate is sent iff selected(key, index, T, t_idx) under its worker's
-// selection of that step.
+// aggregate + update when it is applied at once (an eager step, or reading the
+// state): a warp per sub-tile walks the sent candidates of its K sub-chunks in
+// worker order, adds the values that fall on one coordinate in ascending worker
+// order from +0, sets their residuals to +0 and applies w -= (eta/K) * sum,
+// keeping w_{t+1} - w_t. A candidate is sent iff selected(key, index, T, t_idx).
+//
+// Bound by scattered 32-byte accesses: a sub-chunk entry, a pair's index and
+// value, its residual, and w and w_t - w_{t-1} on the union; nothing is read
+// that the sub-chunk lists hold already. (It was two launches: a per-coordinate
+// mask of the senders, then one thread per union coordinate gathering their
+// values from the residuals: d = 138 M, K = 8: 152 -> 72 us; d = 11.2 M, K = 16:
+// 44 -> 24 us.)
 // ---------------------------------------------------------------------------
-// Candidates of worker k, part p of nparts: the dense path's [0, k) when it
-// decided this worker, else a region of the bulk pass or a slice of [0, count).
-__device__ __forceinline__ void sent_part(const TopkArgs& A, int k, int p, int nparts,
-                                          uint32_t* lo, uint32_t* hi) {
-  if (A.sel[k].dense || A.regions == 1) {
-    const uint32_t n = A.sel[k].dense ? (A.approx ? A.sel[k].nsel : A.ksel) : min(A.sel[k].count, A.cap);
-    const uint32_t per = (n + nparts - 1) / nparts;
-    *lo = min(n, (uint32_t)p * per);
-    *hi = min(n, *lo + per);
-  } else {
-    *lo = (uint32_t)p * A.cap_part;
-    *hi = *lo + A.rcount[(int64_t)k * nparts + p];
-  }
-}
-
-__global__ void __launch_bounds__(kThreads) k_mark(TopkArgs A) {
-  griddep_wait();
-  const int k = blockIdx.y;
-  const uint32_t T = A.sel[k].T, tidx = A.sel[k].t_idx;
-  const uint32_t bit = 1u << k;
-  const uint32_t* ci = A.cand_idx + (int64_t)k * A.cap;
-  const float* cv = A.cand_val + (int64_t)k * A.cap;
-  const int nparts = candidate_parts(A);
-  const int lane = threadIdx.x & 31;
-  for (int part = blockIdx.x * kWarps + (threadIdx.x >> 5); part < nparts; part += gridDim.x * kWarps) {
-    uint32_t lo, hi;
-    sent_part(A, k, part, nparts, &lo, &hi);
-    for (uint32_t i0 = lo; i0 < hi; i0 += 4 * 32) {
-      uint32_t jq[4];
-      float vq[4];
+// The position in a list of up to 32 runs (lane l's of length cnt, incl: their
+// inclusive sums): the run that holds element e (the first lane whose sum exceeds it).
+__device__ __forceinline__ int run_of(uint32_t incl, uint32_t e) {
+  int lo = 0, hi = 32;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t i = i0 + q * 32 + lane;
-        jq[q] = i < hi ? ci[i] : kNone;
-        vq[q] = i < hi ? cv[i] : 0.f;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t j = jq[q];
-        if (j < (uint32_t)A.d && selected(mag_key(vq[q]), j, T, tidx)) atomicOr(&A.mask[j], bit);
-      }
+  for (int it = 0; it < 6; ++it) {
+    const int mid = min((lo + hi) >> 1, 31);
+    const uint32_t v = __shfl_sync(0xffffffffu, incl, mid);
+    if (lo < hi) {
+      if (v <= e) lo = mid + 1; else hi = mid;
     }
   }
+  return lo < 32 ? lo : 31;
 }
 
-__global__ void __launch_bounds__(kThreads) k_owner_sum(TopkArgs A) {
+__global__ void __launch_bounds__(kThreads) k_apply(TopkArgs A) {
   griddep_wait();
-  const int k = blockIdx.y;
-  const uint32_t* ci = A.cand_idx + (int64_t)k * A.cap;
-  const float* cv = A.cand_val + (int64_t)k * A.cap;
-  const uint32_t T = A.sel[k].T, tidx = A.sel[k].t_idx;
-  const uint32_t mine = 1u << k, lower = mine - 1u;
-  const int nparts = candidate_parts(A);
-  unsigned long long uni = 0, changed = 0;
-  for (int part = blockIdx.x * kWarps + (threadIdx.x >> 5); part < nparts; part += gridDim.x * kWarps) {
-    uint32_t lo, hi;
-    sent_part(A, k, part, nparts, &lo, &hi);
-    for (uint32_t i = lo + (threadIdx.x & 31); i < hi; i += 32) {
-      const uint32_t j = __ldcg(ci + i);
-      if (j >= (uint32_t)A.d || !selected(mag_key(__ldcg(cv + i)), j, T, tidx)) continue;  // not sent
-      const uint32_t m = A.mask[j];
-      if (!(m & mine) || (m & lower)) continue;  // a lower worker owns j (or done)
-      // every sender's value is still in e[b][j]: load them all at once, then
-      // add in ascending worker order from +0
-      const float wo = A.w[j];
-      float vals[32];
-#pragma unroll
-      for (int b = 0; b < 32; ++b)
-        vals[b] = ((m >> b) & 1u) ? __ldcg(A.e + (int64_t)b * A.ld + j) : 0.f;
-      float sum = 0.f;
-#pragma unroll
-      for (int b = 0; b < 32; ++b) {
-        if ((m >> b) & 1u) {
-          sum = __fadd_rn(sum, vals[b]);
-          A.e[(int64_t)b * A.ld + j] = 0.f;  // e_{t+1,b} = e_{t+1/2,b} - C(.) = +0 where sent
-          if (A.mfm) A.lm[(int64_t)b * A.ld + j] = 0.f;  // momentum factor masking
+  constexpr int kSubMax = kBulkTile / kChunksPerTile;
+  __shared__ float sums[kWarps][kSubMax];             // sub-tiles of more than 32 pairs
+  __shared__ uint32_t seen[kWarps][kSubMax / 32];
+  __shared__ uint32_t Ts[kMaxK], tis[kMaxK];
+  __shared__ uint32_t s_last;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int k = threadIdx.x; k < A.K; k += blockDim.x) {
+    Ts[k] = A.sel[k].T;
+    tis[k] = A.sel[k].t_idx;
+  }
+  __syncthreads();
+  const int sub = A.tile / kChunksPerTile;
+  const int64_t n_sub = A.n_tiles * kChunksPerTile, nw = (int64_t)gridDim.x * kWarps;
+  const uint32_t lt = lanemask_lt();
+  uint32_t uni = 0, changed = 0;
+  // w_{t+1} at union coordinate j (Alg. 3: the sum, for k_server_update)
+  auto update = [&](uint32_t j, float sum, float wo) {
+    ++uni;
+    if (A.server_mom) {
+      A.dlt[j] = sum;
+      return;
+    }
+    const float wn = __fsub_rn(wo, __fmul_rn(A.a_prev, sum));
+    A.w[j] = wn;
+    const float dd = __fsub_rn(wn, wo);
+    A.dlt[j] = dd;
+    changed += dd != 0.f;
+  };
+  const int64_t st0 = (int64_t)blockIdx.x * kWarps + warp;
+  uint2 next = st0 < n_sub && lane < A.K ? A.chunk[st0 * A.K + lane] : make_uint2(0u, 0u);
+  for (int64_t st = st0; st < n_sub; st += nw) {
+    const uint2 bc = next;  // lane k: worker k's sub-chunk
+    next = st + nw < n_sub && lane < A.K ? A.chunk[(st + nw) * A.K + lane] : make_uint2(0u, 0u);
+    uint32_t total;
+    const uint32_t pre = warp_excl_scan(bc.y, &total);
+    if (total == 0) continue;
+    const uint32_t sub0 = (uint32_t)(st * sub);
+    const bool many = total > 32u;
+    if (many) {
+      for (int i = lane; i < sub; i += 32) sums[warp][i] = 0.f;
+      if (lane < kSubMax / 32) seen[warp][lane] = 0u;
+      __syncwarp();
+    }
+    for (uint32_t e0 = 0; e0 < total; e0 += 32) {
+      const uint32_t e = e0 + lane;
+      const int k = run_of(pre + bc.y, e < total ? e : total - 1);
+      const uint32_t at = __shfl_sync(0xffffffffu, bc.x, k) + (e - __shfl_sync(0xffffffffu, pre, k));
+      bool act = e < total && at < A.cap;
+      uint32_t j = kNone;
+      float v = 0.f;
+      if (act) {
+        j = A.cand_idx[(int64_t)k * A.cap + at];
+        v = A.cand_val[(int64_t)k * A.cap + at];
+        act = selected(mag_key(v), j, Ts[k], tis[k]);
+        if (act && (j < sub0 || j - sub0 >= (uint32_t)sub || j >= (uint32_t)A.d)) {
+          atomicOr(A.status, kStatusInternal);
+          act = false;
         }
       }
-      A.mask[j] = 0u;
-      ++uni;
-      if (A.server_mom) {  // Alg. 3: k_server_update applies the sum with the momentum term
-        A.dlt[j] = sum;
-        continue;
+      float wo = 0.f;
+      if (act && !many && !A.server_mom) wo = A.w[j];
+      if (act) {
+        A.e[(int64_t)k * A.ld + j] = 0.f;  // e_{t+1,k} = e_{t+1/2,k} - C(.) = +0 where sent
+        if (A.mfm) A.lm[(int64_t)k * A.ld + j] = 0.f;  // momentum factor masking
       }
-      const float wn = __fsub_rn(wo, __fmul_rn(A.a_prev, sum));
-      A.w[j] = wn;
-      const float dd = __fsub_rn(wn, wo);
-      A.dlt[j] = dd;
-      changed += (dd != 0.f);
+      const uint32_t peers = __match_any_sync(0xffffffffu, act ? j : 0x80000000u + lane);  // d < 2^31
+      const bool lead = act && (peers & lt) == 0u;
+      float sum = many && lead ? sums[warp][j - sub0] : 0.f;
+      uint32_t left = peers;
+      while (__any_sync(0xffffffffu, left != 0u)) {  // in lane (= worker) order
+        const int src = left ? __ffs(left) - 1 : lane;
+        const float x = __shfl_sync(0xffffffffu, v, src);
+        if (left && act) sum = __fadd_rn(sum, x);
+        left &= left - 1u;
+      }
+      if (lead) {
+        if (many) {
+          sums[warp][j - sub0] = sum;
+          atomicOr(&seen[warp][(j - sub0) >> 5], 1u << ((j - sub0) & 31));
+        } else {
+          update(j, sum, wo);
+        }
+      }
+      __syncwarp();
+    }
+    if (many) {
+      for (int q = 0; q < sub / 32; ++q) {
+        if (!((seen[warp][q] >> lane) & 1u)) continue;
+        const uint32_t j = sub0 + q * 32 + lane;
+        update(j, sums[warp][q * 32 + lane], A.server_mom ? 0.f : A.w[j]);
+      }
+      __syncwarp();
     }
   }
-  uni = warp_sum(uni);
-  changed = warp_sum(changed);
-  if ((threadIdx.x & 31) == 0) {
-    for (Counters* c : {A.step_ctr, A.total_ctr}) {
-      if (!c) continue;
-      if (uni) atomicAdd(&c->v[kUnion], uni);
-      if (changed) atomicAdd(&c->v[kChanged], changed);
+  const uint32_t u = __reduce_add_sync(0xffffffffu, uni), c = __reduce_add_sync(0xffffffffu, changed);
+  if (lane == 0) {
+    for (Counters* to : {A.step_ctr, A.total_ctr}) {
+      if (!to || (A.finalize && to == A.total_ctr)) continue;
+      if (u) atomicAdd(&to->v[kUnion], (unsigned long long)u);
+      if (c) atomicAdd(&to->v[kChanged], (unsigned long long)c);
+    }
+  }
+  if (!A.finalize) return;
+  // an eager step ends here: the last block adds the step's counters to the totals
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(&A.sel[0].done[3], 1u) == gridDim.x - 1 ? 1u : 0u;
+    if (s_last) {
+      __threadfence();
+      A.sel[0].done[3] = 0;
+      finalize_counters(A.step_ctr, A.total_ctr, A.pairs_add);
     }
   }
 }
@@ -2223,12 +2257,14 @@ cudaError_t launch_select_dense(const TopkArgs& A, cudaStream_t s) {
   return launch_pdl(k_select_dense, dim3(A.K), dim3(1024), 0, s, A);
 }
 
-cudaError_t launch_mark(const TopkArgs& A, int grid, cudaStream_t s) {
-  return launch_pdl(k_mark, dim3(grid, A.K), dim3(kThreads), 0, s, A);
+cudaError_t launch_apply(const TopkArgs& A, int grid, cudaStream_t s) {
+  return launch_pdl(k_apply, dim3(grid), dim3(kThreads), 0, s, A);
 }
 
-cudaError_t launch_owner_sum(const TopkArgs& A, int grid, cudaStream_t s) {
-  return launch_pdl(k_owner_sum, dim3(grid, A.K), dim3(kThreads), 0, s, A);
+int apply_blocks_per_sm() {
+  int n = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_apply, kThreads, 0) != cudaSuccess) cudaGetLastError();
+  return n > 0 ? n : 1;
 }
 
 cudaError_t launch_server_update(const TopkArgs& A, cudaStream_t s) {
