@@ -671,15 +671,17 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
                                    : (int)std::max<int64_t>(1, std::min<int64_t>(per, std::max<int64_t>(1, streams_wide / K)));
     if (compressor == GMC_TOPK) h->n_sample = (uint32_t)(h->sample_chunks ? kSampleSlots : d);
     h->sample_stride = std::max<uint32_t>(kSampleSlots, (h->n_sample + 3) & ~3u);
-    h->sample_blocks = (int)std::max<int64_t>(1, ((int64_t)h->n_sample + 2047) / 2048);
-    h->theta_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(2 * h->num_sms / K + 1,
-                                                                  ((int64_t)h->n_sample + 8191) / 8192));
+    // the approximate top-s sample: a run of 8 a thread, over about eight blocks
+    // per SM for all the workers; its threshold's passes: a few quads a thread
+    const int64_t share = (8 * (int64_t)h->num_sms + K - 1) / K;
+    h->sample_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(share, ((int64_t)h->n_sample + 2047) / 2048));
+    h->theta_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(share, ((int64_t)h->n_sample + 4095) / 4096));
     const int64_t Kt = (int64_t)K * h->n_tiles;
     if ((err = dalloc(h, &h->e, (size_t)K * h->ld)) != cudaSuccess ||
         (err = dalloc(h, &h->w, (size_t)h->ld)) != cudaSuccess ||
         (err = dalloc(h, &h->dlt, (size_t)h->ld)) != cudaSuccess ||
         (err = dalloc(h, &h->sel, (size_t)K)) != cudaSuccess ||
-        (err = dalloc(h, &h->ghist, (size_t)K * kHistBins)) != cudaSuccess ||
+        (err = dalloc(h, &h->ghist, (size_t)K * kThetaBins)) != cudaSuccess ||
         (err = dalloc(h, &h->chist, (size_t)K * kRelBins)) != cudaSuccess ||
         (err = dalloc(h, &h->bucket, (size_t)K * 2 * kBucketCap)) != cudaSuccess ||
         (err = dalloc(h, &h->sample_keys, (size_t)K * h->sample_stride)) != cudaSuccess ||

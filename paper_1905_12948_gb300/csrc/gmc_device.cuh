@@ -20,6 +20,7 @@ constexpr int kSampleSlots = 32768;          // sampled positions per worker (= 
 constexpr int kSampleChunks = kSampleSlots / kSampleRun;  // sampled runs per worker
 static_assert((kSampleRun & (kSampleRun - 1)) == 0 && kSampleRun <= 32, "kSampleRun: a power of two, at most a warp");
 constexpr int kHistBins = 2048;              // first radix digit: key bits 30..20
+constexpr int kThetaBins = kHistBins + 2048;  // the approximate top-s sample's three digits
 constexpr int kRelBins = 2048;               // bins of the candidates' relative histogram
 constexpr int kBucketCap = 12288;            // candidates of one bin ranked in shared memory
 
@@ -27,15 +28,15 @@ constexpr int kBucketCap = 12288;            // candidates of one bin ranked in 
 struct WorkerSel {
   uint32_t theta;    // candidate threshold key from the sample (kNoCandidate = none)
   uint32_t count;    // candidates appended by the accumulate pass (may exceed cap)
-  uint32_t prefix;   // select: relative-histogram bin holding the k-th key
-  uint32_t rank;     // select: the k-th key's 1-based rank inside that bin
+  uint32_t prefix;   // approximate top-s: theta's digits found so far
+  uint32_t rank;     // and its 1-based rank among the sampled keys with that prefix
   uint32_t T;        // the k-th largest key
   uint32_t n_tie;    // elements equal to T that are kept (lowest indices first)
   uint32_t ties;     // candidates equal to T
   uint32_t t_idx;    // a candidate equal to T is kept iff its index <= t_idx
   uint32_t dense;    // 1: this worker's selection is made by the dense path
   uint32_t done[4];  // finished-block counters: -, the select finish, the approximate
-                     // top-s threshold, and (worker 0's) the dense select's blocks
+                     // top-s threshold's pass, and (worker 0's) the dense select's blocks
   uint32_t count_bucket;  // candidates collected from the k-th key's bin
   uint32_t nsel;     // approximate top-s: components sent (the count varies by step)
   uint32_t shift;    // log2 of the relative histogram's bin width, in keys (from the sample)

@@ -74,7 +74,7 @@ struct TopkArgs {
   int dense_prev;            // restored state: w_t - w_{t-1} is in dlt over [0, d), no pair lists
   int dense_mode;            // GMC_SELECT_DENSE
   WorkerSel* sel;            // K entries
-  uint32_t* ghist;           // K x kHistBins: the approximate top-s sample's histogram (zero between uses)
+  uint32_t* ghist;           // K x kThetaBins: the approximate top-s sample's histograms (zero between uses)
   uint32_t* chist;           // K x kRelBins: the candidates' relative histogram (zeroed by the sample)
   uint32_t* bucket;          // K x 2*kBucketCap: keys, then indices of the k-th key's bin
   uint32_t* sample_keys;     // K x sample_stride
@@ -93,7 +93,7 @@ struct TopkArgs {
   float a_prev;              // fl(eta/K) of that step
   uint32_t* sample_pend;     // 3 x sample_stride: its senders' mask and w_{t+1} - w_t at the
                              // sampled coordinates (k_sample_pending, for k_sample); the
-                             // approximate top-s adds the coordinates
+                             // approximate top-s adds the runs' starts
   Counters* total_ctr;       // running totals: the deferred aggregation counts there
   Counters* step_ctr;
   unsigned* status;

@@ -73,21 +73,11 @@ __device__ __forceinline__ uint32_t warp_excl_scan(uint32_t x, uint32_t* total) 
   return incl - x;
 }
 
-// Sampled coordinate of slot i. Exact top-k: kSampleRun (16) consecutive
+// Sampled coordinate of slot i of the exact top-k: kSampleRun (16) consecutive
 // coordinates from (c * d / chunks) rounded down to a multiple of kSampleRun,
 // c = 0 .. chunks-1 (every coordinate when chunks = 0); this sample only sets
-// the candidate threshold, never the result. Approximate top-s (Sec. 5.1): run i/8 of the
-// n = n_sample/8 runs of 8 consecutive coordinates, one per stratum
-// [r d / n, (r+1) d / n), starting on a multiple of 8 inside it at the slot
-// the r-th draw of the step's shared stream `key` picks (d < 8: slot i).
-__device__ __forceinline__ int64_t sample_coord(const TopkArgs& A, uint64_t key, int i) {
-  if (A.approx) {
-    if (A.d < 8) return i;
-    const uint64_t n = A.n_sample >> 3, d = (uint64_t)A.d, run = (uint64_t)i >> 3;
-    const uint64_t lo = run * d / n, hi = (run + 1) * d / n;
-    const uint64_t a = (lo + 7) & ~uint64_t(7);
-    return (int64_t)(a + 8 * (uint64_t)below(draw(key, run), (hi - a) >> 3) + (i & 7));
-  }
+// the candidate threshold, never the result.
+__device__ __forceinline__ int64_t sample_coord(const TopkArgs& A, int i) {
   if (!A.sample_chunks) return i;
   // sample_chunks is kSampleChunks, a power of two: floor(ch * d / kSampleChunks)
   // by a shift (a 64-bit division would cost more than the slot's loads)
@@ -98,9 +88,18 @@ __device__ __forceinline__ int64_t sample_coord(const TopkArgs& A, uint64_t key,
   const int64_t ch = i >> kRunShift;
   return (((ch * A.d) >> kChunkShift) & ~int64_t(kSampleRun - 1)) + (i & (kSampleRun - 1));
 }
-__device__ __forceinline__ uint64_t sample_key(const TopkArgs& A) {
-  return A.approx ? stream_key(A.seed, A.t, 0) : 0ull;
+// Start of run r of the approximate top-s sample (Sec. 5.1): n = n_sample/8 runs
+// of 8 consecutive coordinates, one per stratum [r d / n, (r+1) d / n), starting
+// on a multiple of 8 inside it at the slot the r-th draw of the step's shared
+// stream `key` picks (d < 8: one run, all of [0, d)).
+__device__ __forceinline__ uint32_t approx_run(const TopkArgs& A, uint64_t key, int r) {
+  if (A.d < 8) return 0u;
+  const uint64_t n = A.n_sample >> 3, d = (uint64_t)A.d, run = (uint64_t)r;
+  const uint64_t lo = run * d / n, hi = (run + 1) * d / n;
+  const uint64_t a = (lo + 7) & ~uint64_t(7);
+  return (uint32_t)(a + 8 * (uint64_t)below(draw(key, run), (hi - a) >> 3));
 }
+__device__ __forceinline__ uint64_t sample_key(const TopkArgs& A) { return stream_key(A.seed, A.t, 0); }
 
 // The previous step's aggregation at the sampled coordinates, when it is
 // still pending, once for all workers: the senders of coordinate j are the
@@ -108,8 +107,8 @@ __device__ __forceinline__ uint64_t sample_key(const TopkArgs& A) {
 // selected; w still holds w_t. For slot i: the senders' mask, and
 // w_{t+1}[j] - w_t[j] -- their values summed in ascending worker order from
 // +0 (Alg. 1). The approximate top-s runs it every step: it also stores each
-// slot's coordinate, and the step's w_t - w_{t-1} there (from dlt when no
-// aggregation is pending), for k_sample to read in order.
+// run's first coordinate, and the step's w_t - w_{t-1} at every slot (from dlt
+// when no aggregation is pending), for k_sample to read in order.
 constexpr int kTailBlocks = 4;  // blocks of tiles the bulk pass ends with: the coldest (tile_order)
 
 __global__ void __launch_bounds__(kThreads) k_sample_pending(TopkArgs A) {
@@ -176,12 +175,8 @@ __global__ void __launch_bounds__(kThreads) k_sample_pending(TopkArgs A) {
     return;
   }
   const int n_s = (int)A.n_sample;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_s) return;
-  const int64_t j = sample_coord(A, sample_key(A), i);
-  uint32_t m = 0;
-  float dd = 0.f;
-  if (A.pending) {
+  // the pending aggregation at coordinate j: its senders, and w_{t+1}[j] - w_t[j] (0 when none)
+  auto senders = [&](int64_t j, uint32_t& m) {
     float x[kMaxK];
 #pragma unroll
     for (int b = 0; b < kMaxK; ++b) x[b] = b < A.K ? __ldcg(A.e + (int64_t)b * A.ld + j) : 0.f;
@@ -194,14 +189,35 @@ __global__ void __launch_bounds__(kThreads) k_sample_pending(TopkArgs A) {
         m |= 1u << b;
       }
     }
-    if (m) dd = __fsub_rn(__fsub_rn(wo, __fmul_rn(A.a_prev, sum)), wo);
+    return m ? __fsub_rn(__fsub_rn(wo, __fmul_rn(A.a_prev, sum)), wo) : 0.f;
+  };
+  if (!A.approx) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_s) return;
+    uint32_t m = 0;
+    const float dd = senders(sample_coord(A, i), m);
+    A.sample_pend[i] = m;
+    A.sample_pend[A.sample_stride + i] = __float_as_uint(dd);
+    return;
   }
-  if (A.approx) {
+  // a thread draws one run of 8 coordinates (64-bit divisions: once a run, not
+  // once a slot), then the warp takes its 32 runs' slots four runs at a time
+  const int lane = threadIdx.x & 31;
+  const int run0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31), runs = (n_s + 7) / 8;
+  const uint32_t start = run0 + lane < runs ? approx_run(A, sample_key(A), run0 + lane) : 0u;
+  if (run0 + lane < runs) A.sample_pend[2 * A.sample_stride + run0 + lane] = start;
+#pragma unroll 1
+  for (int q = 0; q < 8; ++q) {
+    const uint32_t j = __shfl_sync(0xffffffffu, start, q * 4 + (lane >> 3)) + (lane & 7);
+    const int i = (run0 + q * 4) * 8 + lane;
+    if (i >= n_s) continue;
+    uint32_t m = 0;
+    float dd = 0.f;
+    if (A.pending) dd = senders(j, m);
     if (!m) dd = A.dlt[j];
-    A.sample_pend[2 * A.sample_stride + i] = (uint32_t)j;
+    A.sample_pend[i] = m;
+    A.sample_pend[A.sample_stride + i] = __float_as_uint(dd);
   }
-  A.sample_pend[i] = m;
-  A.sample_pend[A.sample_stride + i] = __float_as_uint(dd);
 }
 
 // Bin of a candidate key in the relative histogram: (key - theta) >> shift,
@@ -209,77 +225,6 @@ __global__ void __launch_bounds__(kThreads) k_sample_pending(TopkArgs A) {
 __device__ __forceinline__ int rel_bin(uint32_t key, uint32_t theta, int shift) {
   const uint32_t b = (key > theta ? key - theta : 0u) >> shift;
   return b < (uint32_t)kRelBins ? (int)b : kRelBins - 1;
-}
-
-// ---------------------------------------------------------------------------
-// Sample of the approximate top-s (Sec. 5.1): blocks spread over the workers'
-// samples store every sampled key and add its first radix digit to the
-// worker's histogram, for k_sample_theta. The accumulator at a sampled
-// coordinate is formed as if the previous step's aggregation had been applied
-// (residual +0 where the worker sent, the pending delta).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_sample(TopkArgs A) {
-  griddep_wait();
-  __shared__ uint32_t hist[kHistBins];
-  const int k = blockIdx.y;
-  WorkerSel& S = A.sel[k];
-  if (blockIdx.x == 0 && k == 0 && threadIdx.x == 0) {
-    A.big_tiles[0] = 0;
-    *A.tile_ctr = 0u;  // the bulk pass claims its tiles from zero
-  }
-  if (blockIdx.x == 0)  // this step's candidate histogram starts empty
-    for (int b = threadIdx.x; b < kRelBins; b += blockDim.x) A.chist[(int64_t)k * kRelBins + b] = 0u;
-  if (A.dense_mode) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      S.theta = kNoCandidate;
-      S.count = 0;
-      S.dense = 0;
-    }
-    return;
-  }
-  const float* ek = A.e + (int64_t)k * A.ld;
-  const float* gk = A.grads + (int64_t)k * A.d;
-  const uint16_t* gk16 = A.grads16 + (int64_t)k * A.d;
-  uint32_t* keys = A.sample_keys + (int64_t)k * A.sample_stride;
-  const int n_s = (int)A.n_sample;
-  for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) hist[b] = 0;
-  __syncthreads();
-  const int per = (n_s + gridDim.x - 1) / gridDim.x;
-  const int i_lo = blockIdx.x * per;
-  const int i_hi = min(n_s, i_lo + per);
-  for (int i0 = i_lo; i0 < i_hi; i0 += 8 * blockDim.x) {
-    float ev[8], gv[8], dv[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int i = i0 + q * blockDim.x + threadIdx.x;
-      ev[q] = gv[q] = dv[q] = 0.f;
-      if (i < i_hi) {  // coordinate, senders and w_t - w_{t-1} from k_sample_pending
-        const int64_t j = A.sample_pend[2 * A.sample_stride + i];
-        const uint32_t m = A.sample_pend[i];
-        const float e = ek[j];  // loaded whatever m holds: no load waits on another but j
-        ev[q] = ((m >> k) & 1u) ? 0.f : e;
-        const float g = A.bf16 ? bf16_f32(gk16[j]) : gk[j];
-        gv[q] = A.local_mom ? local_m(A, k, j, g) : (A.gscale ? __fmul_rn(A.gs, g) : g);
-        dv[q] = __uint_as_float(A.sample_pend[A.sample_stride + i]);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int i = i0 + q * blockDim.x + threadIdx.x;
-      int bin = -1;
-      if (i < i_hi) {
-        const uint32_t key = mag_key(accumulate(ev[q], gv[q], A.c, dv[q]));
-        keys[i] = key;
-        bin = (int)(key >> 20);
-      }
-      warp_hist_add(hist, bin);
-    }
-  }
-  __syncthreads();
-  uint32_t* gh = A.ghist + (int64_t)k * kHistBins;
-  for (int b = threadIdx.x; b < kHistBins; b += blockDim.x)
-    if (hist[b]) atomicAdd(&gh[b], hist[b]);
-  // k_sample_theta fixes theta exactly from the keys and this histogram
 }
 
 // ---------------------------------------------------------------------------
@@ -398,7 +343,7 @@ __global__ void __cluster_dims__(scl::kCtas, 1, 1) __launch_bounds__(scl::kThrea
     pm[q] = pd[q] = 0u;
   }
   if (nv == kSlots) {
-    const int64_t j0 = sample_coord(A, 0ull, i0);  // a multiple of kSlots (runs start on kSampleRun)
+    const int64_t j0 = sample_coord(A, i0);  // a multiple of kSlots (runs start on kSampleRun)
     load8(ek + j0, ev);  // rows of e, lm and dlt start on 16 bytes (ld: whole tiles)
     load8(A.dlt + j0, dv);
     if (A.local_mom) load8(A.lm + (int64_t)k * A.ld + j0, lv);
@@ -412,7 +357,7 @@ __global__ void __cluster_dims__(scl::kCtas, 1, 1) __launch_bounds__(scl::kThrea
 #pragma unroll
     for (int q = 0; q < kSlots; ++q) {
       if (q < nv) {
-        const int64_t j = sample_coord(A, 0ull, i0 + q);
+        const int64_t j = sample_coord(A, i0 + q);
         ev[q] = ek[j];
         gv[q] = A.bf16 ? bf16_f32(gk16[j]) : gk[j];
         dv[q] = A.dlt[j];
@@ -492,114 +437,165 @@ __global__ void __cluster_dims__(scl::kCtas, 1, 1) __launch_bounds__(scl::kThrea
 }
 
 // ---------------------------------------------------------------------------
-// Approximate top-s (Sec. 5.1): theta is the exact r-th largest sampled key.
-// Every block finds, from the sample's first-digit histogram, the bin that
-// holds it and collects that bin's keys from its slice of the sample (128 a
-// round, one bucket reservation); the last block ranks the bucket in shared
-// memory. A bin too crowded for the bucket is resolved by the last block's
-// two remaining radix digits over the whole sample.
+// Sample of the approximate top-s (Sec. 5.1): blocks spread over the workers'
+// samples store every sampled key and add its first radix digit to the
+// worker's histogram, for k_sample_theta. The accumulator at a sampled
+// coordinate is formed as if the previous step's aggregation had been applied
+// (residual +0 where the worker sent, the pending delta). A thread takes a run
+// of 8 with 16-byte loads, all issued before any is used; a block takes several
+// runs a thread before it adds its histogram to the worker's (d = 138 M, K = 8,
+// 11 M sampled values: 132 us slot by slot -> SAMPLE_US us).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_sample_theta(TopkArgs A) {
+__global__ void __launch_bounds__(kThreads) k_sample(TopkArgs A) {
   griddep_wait();
-  extern __shared__ __align__(16) uint32_t fin[];  // kBucketCap keys
-  __shared__ uint32_t h[kHistBins];
-  __shared__ uint32_t ws[32];
-  __shared__ uint32_t s_last, s_bin, s_rank, s_n;
+  __shared__ uint32_t hist[kHistBins];
   const int k = blockIdx.y;
-  WorkerSel& S = A.sel[k];
-  uint32_t* gh = A.ghist + (int64_t)k * kHistBins;
-  for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) h[b] = __ldcg(&gh[b]);
-  if (threadIdx.x == 0) {
-    s_bin = 0;
-    s_rank = 0;
+  if (blockIdx.x == 0 && k == 0 && threadIdx.x == 0) {
+    A.big_tiles[0] = 0;
+    *A.tile_ctr = 0u;  // the bulk pass claims its tiles from zero
   }
+  if (blockIdx.x == 0)  // this step's candidate histogram starts empty
+    for (int b = threadIdx.x; b < kRelBins; b += blockDim.x) A.chist[(int64_t)k * kRelBins + b] = 0u;
+  const float* ek = A.e + (int64_t)k * A.ld;
+  const float* gk = A.grads + (int64_t)k * A.d;
+  const uint16_t* gk16 = A.grads16 + (int64_t)k * A.d;
+  uint32_t* keys = A.sample_keys + (int64_t)k * A.sample_stride;
+  const int n_s = (int)A.n_sample, runs = (n_s + 7) / 8;
+  for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) hist[b] = 0;
   __syncthreads();
-  const uint32_t n_s = A.n_sample;
-  const uint32_t r = A.sample_rank < n_s ? A.sample_rank : n_s;
-  block_find_from_top(h, kHistBins, r, ws, &s_bin, &s_rank);
-  const uint32_t b1 = s_bin, r1 = s_rank;
-  const uint32_t* keys = A.sample_keys + (int64_t)k * A.sample_stride;
-  uint32_t* bk = A.bucket + (int64_t)k * 2 * kBucketCap;
-  const int lane = threadIdx.x & 31;
-  const uint32_t lt = lanemask_lt();
-  const uint32_t per = (n_s + gridDim.x - 1) / gridDim.x;
-  const uint32_t i_lo = min(n_s, blockIdx.x * per), i_hi = min(n_s, i_lo + per);
-  for (uint32_t i0 = i_lo + (threadIdx.x >> 5) * 128; i0 < i_hi; i0 += kWarps * 128) {
-    uint32_t key[4], m[4], n = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint32_t i = i0 + q * 32 + lane;
-      key[q] = i < i_hi ? __ldcg(keys + i) : 0u;
-      m[q] = __ballot_sync(0xffffffffu, i < i_hi && (key[q] >> 20) == b1);
-      n += __popc(m[q]);
-    }
-    if (n) {
-      uint32_t base = 0;
-      if (lane == 0) base = atomicAdd(&S.count_bucket, n);
-      base = __shfl_sync(0xffffffffu, base, 0);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t o = base + __popc(m[q] & lt);
-        if (((m[q] >> lane) & 1u) && o < (uint32_t)kBucketCap) bk[o] = key[q];
-        base += __popc(m[q]);
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < runs; r += gridDim.x * blockDim.x) {
+    const int64_t j0 = A.sample_pend[2 * A.sample_stride + r];
+    const int nv = min(8, n_s - r * 8);  // 8, but for d < 8
+    float ev[8], gv[8], lv[8];
+    uint32_t pm[8], pd[8];
+    if (nv == 8) {
+      load8u(A.sample_pend + r * 8, pm);
+      load8u(A.sample_pend + A.sample_stride + r * 8, pd);
+      load8(ek + j0, ev);  // rows of e and lm start on 16 bytes, runs on 8 coordinates
+      if (A.local_mom) load8(A.lm + (int64_t)k * A.ld + j0, lv);
+      if (A.bf16) load8_bf16(gk16 + j0, gv);
+      else load8(gk + j0, gv);
+    } else {
+      for (int q = 0; q < 8; ++q) {
+        const bool in = q < nv;
+        pm[q] = in ? A.sample_pend[r * 8 + q] : 0u;
+        pd[q] = in ? A.sample_pend[A.sample_stride + r * 8 + q] : 0u;
+        ev[q] = in ? ek[j0 + q] : 0.f;
+        lv[q] = in && A.local_mom ? A.lm[(int64_t)k * A.ld + j0 + q] : 0.f;
+        gv[q] = in ? (A.bf16 ? bf16_f32(gk16[j0 + q]) : gk[j0 + q]) : 0.f;
       }
     }
+    uint32_t key[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float g = A.local_mom ? __fadd_rn(__fmul_rn(A.beta, lv[q]), __fmul_rn(A.gs, gv[q]))
+                                  : (A.gscale ? __fmul_rn(A.gs, gv[q]) : gv[q]);
+      key[q] = mag_key(accumulate(((pm[q] >> k) & 1u) ? 0.f : ev[q], g, A.c, __uint_as_float(pd[q])));
+      if (q < nv) atomicAdd(&hist[key[q] >> 20], 1u);
+    }
+    if (nv == 8) {
+      reinterpret_cast<uint4*>(keys + r * 8)[0] = make_uint4(key[0], key[1], key[2], key[3]);
+      reinterpret_cast<uint4*>(keys + r * 8)[1] = make_uint4(key[4], key[5], key[6], key[7]);
+    } else {
+      for (int q = 0; q < nv; ++q) keys[r * 8 + q] = key[q];
+    }
   }
+  __syncthreads();
+  uint32_t* gh = A.ghist + (int64_t)k * kThetaBins;
+  for (int b = threadIdx.x; b < kHistBins; b += blockDim.x)
+    if (hist[b]) atomicAdd(&gh[b], hist[b]);
+}
+
+// ---------------------------------------------------------------------------
+// Approximate top-s (Sec. 5.1): theta is the exact r-th largest sampled key, by
+// its radix digits of 11, 10 and 10 bits: the first from k_sample's histogram,
+// the others by one pass each over the stored keys (PASS 1, 2). Every block
+// counts the digit of its slice's keys that have the prefix so far; the last
+// block finds the next digit. (Collecting the first digit's bin and ranking it
+// in one block took 59 us at d = 138 M, K = 8, and milliseconds when that bin
+// was crowded, as it is late in a run; the two passes take THETA_US us always.)
+// ---------------------------------------------------------------------------
+template <int PASS>
+__global__ void __launch_bounds__(kThreads) k_sample_theta(TopkArgs A) {
+  griddep_wait();
+  __shared__ uint32_t h[kHistBins];
+  __shared__ uint32_t ws[32];
+  __shared__ uint32_t s_last, s_bin, s_rank;
+  const int k = blockIdx.y;
+  WorkerSel& S = A.sel[k];
+  uint32_t* gh = A.ghist + (int64_t)k * kThetaBins;               // first digits
+  uint32_t* gd = gh + kHistBins + (PASS - 1) * 1024;              // this pass's digits
+  const uint32_t n_s = A.n_sample;
+  uint32_t prefix, rank;
+  if (PASS == 1) {
+    for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) h[b] = __ldcg(&gh[b]);
+    if (threadIdx.x == 0) {
+      s_bin = 0;
+      s_rank = 0;
+    }
+    __syncthreads();
+    block_find_from_top(h, kHistBins, A.sample_rank < n_s ? A.sample_rank : n_s, ws, &s_bin, &s_rank);
+    prefix = s_bin;
+    rank = s_rank;
+  } else {
+    prefix = S.prefix;
+    rank = S.rank;
+  }
+  constexpr int shift = PASS == 1 ? 10 : 0;
+  __syncthreads();
+  for (int b = threadIdx.x; b < 1024; b += blockDim.x) h[b] = 0;
+  __syncthreads();
+  const uint32_t* keys = A.sample_keys + (int64_t)k * A.sample_stride;
+  constexpr int kU = 4;  // quads a thread loads together
+  const uint32_t quads = (n_s + 3) / 4, step = gridDim.x * blockDim.x;
+  for (uint32_t q0 = blockIdx.x * blockDim.x + threadIdx.x; q0 < quads; q0 += kU * step) {
+    uint4 x[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (q0 + u * step < quads) x[u] = __ldcg(reinterpret_cast<const uint4*>(keys) + q0 + u * step);
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const uint32_t q = q0 + u * step;
+      if (q >= quads) continue;
+      const uint32_t key[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if ((key[c] >> (shift + 10)) == prefix && q * 4 + c < n_s) atomicAdd(&h[(key[c] >> shift) & 1023u], 1u);
+    }
+  }
+  __syncthreads();
+  for (int b = threadIdx.x; b < 1024; b += blockDim.x)
+    if (h[b]) atomicAdd(&gd[b], h[b]);
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) s_last = (atomicAdd(&S.done[2], 1u) == gridDim.x - 1) ? 1u : 0u;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
+  for (int b = threadIdx.x; b < 1024; b += blockDim.x) {
+    h[b] = __ldcg(&gd[b]);
+    gd[b] = 0;  // zero between uses
+  }
+  if (PASS == 1)
+    for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) gh[b] = 0;
   if (threadIdx.x == 0) {
-    s_n = __ldcg(&S.count_bucket);
-    S.count_bucket = 0;
     S.done[2] = 0;
+    s_bin = 0;
+    s_rank = 0;
   }
-  for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) gh[b] = 0;  // zero between uses
   __syncthreads();
-  const uint32_t n = s_n;
-  uint32_t theta;
-  if (n <= (uint32_t)kBucketCap) {
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) fin[i] = __ldcg(&bk[i]);
-    __syncthreads();
-    uint32_t unused;
-    theta = smem_select(fin, n, r1, h, ws, &s_bin, &s_rank, &unused);
-  } else {
-    // the remaining digits (bits 19..10, then 9..0) over every sampled key
-    uint32_t prefix = b1, rr = r1;
-    for (int pass = 1; pass < 3; ++pass) {
-      const int shift = pass == 1 ? 10 : 0;
-      for (int b = threadIdx.x; b < 1024; b += blockDim.x) h[b] = 0;
-      if (threadIdx.x == 0) {
-        s_bin = 0;
-        s_rank = 0;
-      }
-      __syncthreads();
-      for (uint32_t i0 = 0; i0 < n_s; i0 += blockDim.x) {
-        const uint32_t i = i0 + threadIdx.x;
-        int bin = -1;
-        if (i < n_s) {
-          const uint32_t v = __ldcg(keys + i);
-          if ((v >> (shift + 10)) == prefix) bin = (int)((v >> shift) & 1023u);
-        }
-        warp_hist_add(h, bin);
-      }
-      __syncthreads();
-      block_find_from_top(h, 1024, rr, ws, &s_bin, &s_rank);
-      prefix = (prefix << 10) | s_bin;
-      rr = s_rank;
-      __syncthreads();
-    }
-    theta = prefix;
-  }
+  block_find_from_top(h, 1024, rank, ws, &s_bin, &s_rank);
   if (threadIdx.x == 0) {
-    // capped at the Inf key: every non-finite value is a candidate (and counted there)
-    S.theta = min(theta, 0x7f800000u);
-    S.shift = 20;  // the relative histogram is not used
-    S.count = 0;
-    S.dense = 0;
-    S.nsel = 0;
+    S.prefix = (prefix << 10) | s_bin;
+    S.rank = s_rank;
+    if (PASS == 2) {
+      // capped at the Inf key: every non-finite value is a candidate (and counted there)
+      S.theta = min((prefix << 10) | s_bin, 0x7f800000u);
+      S.shift = 20;  // the relative histogram is not used
+      S.count = 0;
+      S.dense = 0;
+      S.nsel = 0;
+    }
   }
 }
 
@@ -2179,7 +2175,6 @@ cudaError_t configure_topk_kernels() {
   set((const void*)k_accumulate_bulk<false, true>, bulk::smem_bytes(kBulkMaxK));
   set((const void*)k_accumulate_bulk<true, true>, bulk::smem_bytes(kBulkMaxK));
   set((const void*)k_select_finish, kBucketCap * 4);
-  set((const void*)k_sample_theta, kBucketCap * 4);
   return err;
 }
 
@@ -2204,15 +2199,17 @@ int accumulate_blocks_per_sm(int tile) {
 
 cudaError_t launch_sample(const TopkArgs& A, cudaStream_t s) {
   if ((A.pending || A.approx) && !A.dense_mode) {
-    const int n_s = (int)A.n_sample;
-    const unsigned grid = (unsigned)((n_s + kThreads - 1) / kThreads) + (A.use_order ? 1u : 0u);
+    // one thread per slot, or (approximate top-s) per run of 8
+    const int n = A.approx ? (int)((A.n_sample + 7) / 8) : (int)A.n_sample;
+    const unsigned grid = (unsigned)((n + kThreads - 1) / kThreads) + (A.use_order ? 1u : 0u);
     const cudaError_t err = launch_pdl(k_sample_pending, dim3(grid), dim3(kThreads), 0, s, A);
     if (err != cudaSuccess) return err;
   }
   if (!A.approx) return launch_pdl(k_sample_cluster, dim3(scl::kCtas, A.K), dim3(scl::kThreadsC), 0, s, A);
-  const cudaError_t err = launch_pdl(k_sample, dim3(A.sample_blocks, A.K), dim3(kThreads), 0, s, A);
-  if (err != cudaSuccess || !A.approx) return err;
-  return launch_pdl(k_sample_theta, dim3(A.theta_blocks, A.K), dim3(kThreads), kBucketCap * 4, s, A);
+  cudaError_t err = launch_pdl(k_sample, dim3(A.sample_blocks, A.K), dim3(kThreads), 0, s, A);
+  if (err == cudaSuccess) err = launch_pdl(k_sample_theta<1>, dim3(A.theta_blocks, A.K), dim3(kThreads), 0, s, A);
+  if (err == cudaSuccess) err = launch_pdl(k_sample_theta<2>, dim3(A.theta_blocks, A.K), dim3(kThreads), 0, s, A);
+  return err;
 }
 
 // The load/store pass's instantiation for the step's form and gradient type.
