@@ -60,6 +60,7 @@ struct gmc_ctx {
   float* e = nullptr;
   float* w = nullptr;
   float* dlt = nullptr;
+  float* dlt_next = nullptr;  // load/store pass: the aggregate writes here and the two change places
   WorkerSel* sel = nullptr;
   uint32_t* ghist = nullptr;
   uint32_t* chist = nullptr;
@@ -257,7 +258,7 @@ TopkArgs topk_args_at(gmc_ctx* h, const float* grads, int64_t t) {
   A.ld = h->ld;
   A.grads = grads;
   A.d = h->d;
-  A.dlt = h->dlt;
+  A.dlt = A.dlt_out = h->dlt;
   A.w = h->w;
   set_constants(h, &A);
   A.K = h->K;
@@ -436,6 +437,7 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     }
     A.pending = h->agg_pending ? 1 : 0;
     A.a_prev = h->a_pending;
+    if (h->dlt_next && !A.server_mom) A.dlt_out = h->dlt_next;
     // the tile order is built by k_sample_pending, which runs on these steps
     A.use_order = (h->blk_order && (A.pending || approx) && !A.dense_mode) ? 1 : 0;
     const bool defer = h->tile == kBulkTile && !eager && !h->detach_out && !A.server_mom && !A.mfm;
@@ -464,6 +466,7 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
       B.finalize = A.server_mom ? 0 : 1;
       if (A.server_mom) B.total_ctr = nullptr;  // k_finalize adds the step's counts to the totals
       finalized = !A.server_mom;
+      if (A.dlt_out != A.dlt) std::swap(h->dlt, h->dlt_next);
       GMC_TRY(timed(h, GMC_KERNEL_AGGREGATE, 24.0 * kk + (B.server_mom ? 20.0 * h->d : 0.0), s, [&] {
         cudaError_t err = launch_apply(B, h->grid_agg, s);
         if (err == cudaSuccess && B.server_mom) err = launch_server_update(B, s);  // Alg. 3
@@ -637,7 +640,9 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
       const double capd = std::ceil((double)d * (r + 8.0 * std::sqrt(r) + 16.0) / ns) + 4096.0;
       h->cap = (uint32_t)std::min<double>((double)d, capd);
     }
-    h->grid_acc = (int)std::min<int64_t>(h->n_tiles, (int64_t)h->num_sms * accumulate_blocks_per_sm(h->tile));
+    // the bulk pass: a tile at least per CTA; the load/store pass: (sub-tile, worker) items, eight to a block
+    h->grid_acc = (int)std::min<int64_t>(h->tile == kBulkTile ? h->n_tiles : h->n_tiles * K,
+                                         (int64_t)h->num_sms * accumulate_blocks_per_sm(h->tile));
     // k_apply: a warp per sub-tile, as many blocks as are resident at once
     h->grid_agg = (int)std::min<int64_t>(h->n_tiles, (int64_t)h->num_sms * apply_blocks_per_sm());
     // candidate slots: the bulk pass gives every CTA its own region per worker,
@@ -658,7 +663,7 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
     }
     h->cap = (uint32_t)std::min<uint64_t>(
         std::max<uint64_t>((uint64_t)h->regions * h->cap_region, h->limit), 0xfffffff0ull);
-    const int64_t per = (h->cap + 8191) / 8192;
+    const int64_t per = (h->cap + 2047) / 2048;
     // select: on the bulk path a warp walks the candidates of a run of at most
     // 32 parts as one list; the grid is one wave of as many blocks as fit on
     // an SM (each holds kBucketCap keys of shared memory: three on GB300), for
@@ -668,7 +673,7 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
     h->sel_blocks = h->regions > 1 ? (int)std::min<int64_t>(
                                          h->regions, std::max<int64_t>((nparts + 32 * kWarps - 1) / (32 * kWarps),
                                                                        std::max<int64_t>(1, sel_wave / K)))
-                                   : (int)std::max<int64_t>(1, std::min<int64_t>(per, std::max<int64_t>(1, streams_wide / K)));
+                                   : (int)std::max<int64_t>(1, std::min<int64_t>(per, std::max<int64_t>(1, sel_wave / K)));
     if (compressor == GMC_TOPK) h->n_sample = (uint32_t)(h->sample_chunks ? kSampleSlots : d);
     h->sample_stride = std::max<uint32_t>(kSampleSlots, (h->n_sample + 3) & ~3u);
     // the approximate top-s sample: a run of 8 a thread, over about eight blocks
@@ -689,6 +694,7 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
         (err = dalloc(h, &h->rcount, (size_t)K * h->regions * kChunksPerTile)) != cudaSuccess ||
         (err = dalloc(h, &h->sample_pend, (size_t)3 * h->sample_stride)) != cudaSuccess)
       return fail(err);
+    if (h->tile != kBulkTile && (err = dalloc(h, &h->dlt_next, (size_t)h->ld)) != cudaSuccess) return fail(err);
     if (h->grid_small && (err = dalloc(h, &h->small_scratch, small_scratch_words(K))) != cudaSuccess) return fail(err);
     if (h->n_blk >= 8 && ((err = dalloc(h, &h->blk_cost, (size_t)h->n_blk)) != cudaSuccess ||
                           (err = dalloc(h, &h->blk_order, (size_t)h->n_blk)) != cudaSuccess))
@@ -824,6 +830,7 @@ int reset_state(gmc_ctx* h, cudaStream_t s) {
   h->agg_pending = false;  // a pending aggregation of the old state is dropped
   GMC_TRY(cudaMemsetAsync(h->e, 0, (size_t)h->K * h->ld * sizeof(float), s));
   GMC_TRY(cudaMemsetAsync(h->dlt, 0, (size_t)h->ld * sizeof(float), s));
+  if (h->dlt_next) GMC_TRY(cudaMemsetAsync(h->dlt_next, 0, (size_t)h->ld * sizeof(float), s));
   if (h->mom) GMC_TRY(cudaMemsetAsync(h->mom, 0, (size_t)h->ld * sizeof(float), s));
   if (h->lm) GMC_TRY(cudaMemsetAsync(h->lm, 0, (size_t)h->K * h->ld * sizeof(float), s));
   if (h->compressor != GMC_RBGS) {

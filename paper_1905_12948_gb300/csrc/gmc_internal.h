@@ -29,6 +29,7 @@ struct TopkArgs {
   int bf16;
   int64_t d;
   float* dlt;                // w_t - w_{t-1}, dense, zero outside the last union
+  float* dlt_out;            // where the aggregate leaves w_{t+1} - w_t: dlt, or (load/store pass) a second buffer
   float* w;                  // parameters (ld floats)
   float c, a;                // fl(beta/eta), fl(eta/K) (Alg. 4: beta and fl(1/K); Alg. 3: c = 0)
   // The appendix variants: Alg. 4 scales the gradient by eta in the
@@ -224,7 +225,6 @@ cudaError_t launch_finalize(Counters* step, Counters* total, unsigned long long 
 int accumulate_blocks_per_sm(int tile);
 int rbgs_blocks_per_sm();
 int select_blocks_per_sm();  // resident k_select_finish blocks per SM (its grid is one wave)
-int accumulate_smem_bytes(int tile, int K);
 cudaError_t configure_topk_kernels();
 cudaError_t configure_rbgs_kernels();
 

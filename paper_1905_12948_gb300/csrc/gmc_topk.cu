@@ -444,7 +444,7 @@ __global__ void __cluster_dims__(scl::kCtas, 1, 1) __launch_bounds__(scl::kThrea
 // (residual +0 where the worker sent, the pending delta). A thread takes a run
 // of 8 with 16-byte loads, all issued before any is used; a block takes several
 // runs a thread before it adds its histogram to the worker's (d = 138 M, K = 8,
-// 11 M sampled values: 132 us slot by slot -> SAMPLE_US us).
+// 11 M sampled values: 132 us slot by slot -> 79 us).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads) k_sample(TopkArgs A) {
   griddep_wait();
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(kThreads) k_sample(TopkArgs A) {
 // counts the digit of its slice's keys that have the prefix so far; the last
 // block finds the next digit. (Collecting the first digit's bin and ranking it
 // in one block took 59 us at d = 138 M, K = 8, and milliseconds when that bin
-// was crowded, as it is late in a run; the two passes take THETA_US us always.)
+// was crowded, as it is late in a run; the two passes take 34 us always.)
 // ---------------------------------------------------------------------------
 template <int PASS>
 __global__ void __launch_bounds__(kThreads) k_sample_theta(TopkArgs A) {
@@ -815,74 +815,118 @@ __device__ __forceinline__ void write_group(const float v[4], uint32_t j, uint32
   }
 }
 
-// load/store version for small tiles; candidates share one region per worker
+// load/store version, for d below the bulk pass's and above the one-launch
+// step's sizes; candidates share one region per worker. Items are (sub-tile,
+// worker) pairs, taken by the warps of a grid that fills the SMs; a warp loads
+// its next item as soon as this one's v is formed, so that the candidates'
+// slot reservation (an atomic it waits for) and the next item's loads overlap.
+// w_t - w_{t-1} is read as it lies (zero outside the last union) from the
+// buffer the last step wrote; the other buffer, which this step's aggregate
+// will write, is cleared by the items of worker 0. d = 1.3 M, K = 20: 71 us as
+// a loop over the workers per tile -> 53 us (floor 46); K = 32, d = 20 M: step and
+// read of w 1,605 -> 1,431 us (with worker-minor items 1,858: rows of every
+// worker open at once).
 // kLocal: the local-momentum baseline's instantiation (its momentum loads
 // need registers the other forms do without).
 template <int U, bool kLocal, bool kBf16>
 __global__ void __launch_bounds__(kThreads) k_accumulate(TopkArgs A) {
   griddep_wait();
-  constexpr int SUB = 128 * U;       // elements per warp and worker
-  constexpr int T = kWarps * SUB;    // elements per tile
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* dlw = reinterpret_cast<float*>(smem) + warp * SUB;
+  constexpr int SUB = 128 * U;       // elements per item
+  const int lane = threadIdx.x & 31;
   const uint32_t lt = lanemask_lt();
+  // items in blocks of kRun consecutive sub-tiles, worker after worker, so that
+  // neighbouring warps read along one row
+  constexpr uint32_t kRun = 64;
+  const uint32_t n_sub = (uint32_t)(A.n_tiles * kChunksPerTile), nw = gridDim.x * kWarps;
+  const uint32_t items = (n_sub + kRun - 1) / kRun * kRun * (uint32_t)A.K;
+  auto item = [&](uint32_t it, uint32_t& st, uint32_t& k) {
+    const uint32_t sb = it / (kRun * (uint32_t)A.K), r = it - sb * kRun * (uint32_t)A.K;
+    k = r / kRun;
+    st = sb * kRun + r % kRun;
+  };
+  const bool zero_next = A.dlt_out != A.dlt;
   uint32_t nonfinite = 0;
-
-  for (int64_t tile = blockIdx.x; tile < A.n_tiles; tile += gridDim.x) {
-    const uint32_t s0 = (uint32_t)(tile * T) + warp * SUB;
-    stage_delta_warp(A, tile, warp, s0, SUB, dlw, lane);
+  float4 ev[U], gv[U], dv[U], mv[U];
+  uint32_t theta = 0, shift = 0;
+  auto load = [&](uint32_t it) {
+    uint32_t st, k;
+    item(it, st, k);
+    if (st >= n_sub) return;
+    const int64_t s0 = (int64_t)st * SUB;
+    const float* gk = A.grads + (int64_t)k * A.d;
+    const uint16_t* gk16 = A.grads16 + (int64_t)k * A.d;
+    const int gm = g_mode(gk);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t j = s0 + u * 128 + lane * 4;
+      ev[u] = __ldcs(reinterpret_cast<const float4*>(A.e + (int64_t)k * A.ld + j));
+      gv[u] = kBf16 ? load_g4_bf16(gk16, j, A.d) : load_g4(gk, j, A.d, gm);
+      dv[u] = *reinterpret_cast<const float4*>(A.dlt + j);
+      if (kLocal) mv[u] = __ldcs(reinterpret_cast<const float4*>(A.lm + (int64_t)k * A.ld + j));
+    }
+    theta = A.sel[k].theta;
+    shift = A.sel[k].shift;
+  };
+  uint32_t it = blockIdx.x * kWarps + (threadIdx.x >> 5);
+  if (it < items) load(it);
+  for (; it < items; it += nw) {
+    uint32_t st, k;
+    item(it, st, k);
+    if (st >= n_sub) {  // past the last, in its block's run
+      if (it + nw < items) load(it + nw);
+      continue;
+    }
+    const uint32_t s0 = st * SUB, th = theta, sh = shift;
+    float v[U][4];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      float4 g = scale_g(A, gv[u]);
+      if (kLocal) g = local_m4(A, A.lm + (int64_t)k * A.ld + s0 + u * 128 + lane * 4, mv[u], g);
+      v[u][0] = accumulate(ev[u].x, g.x, A.c, dv[u].x);
+      v[u][1] = accumulate(ev[u].y, g.y, A.c, dv[u].y);
+      v[u][2] = accumulate(ev[u].z, g.z, A.c, dv[u].z);
+      v[u][3] = accumulate(ev[u].w, g.w, A.c, dv[u].w);
+    }
+    if (it + nw < items) load(it + nw);
     const int64_t rem = A.d - (int64_t)s0;
     const int lim = rem < SUB ? (int)rem : SUB;
-    for (int k = 0; k < A.K; ++k) {
-      const uint32_t theta = A.sel[k].theta;
-      float* ekt = A.e + (int64_t)k * A.ld + s0;
-      const float* gk = A.grads + (int64_t)k * A.d;
-      const uint16_t* gk16 = A.grads16 + (int64_t)k * A.d;
-      const int gm = g_mode(gk);
-      float4 ev[U], gv[U], mv[U];
+    float* ekt = A.e + (int64_t)k * A.ld + s0;
+    uint32_t bits[U];
+    uint32_t nloc = 0;
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int l = u * 128 + lane * 4;
-        ev[u] = __ldcs(reinterpret_cast<const float4*>(ekt + l));
-        gv[u] = scale_g(A, kBf16 ? load_g4_bf16(gk16, (int64_t)s0 + l, A.d)
-                                 : load_g4(gk, (int64_t)s0 + l, A.d, gm));
-        if (kLocal) mv[u] = __ldcs(reinterpret_cast<const float4*>(A.lm + (int64_t)k * A.ld + s0 + l));
-      }
-      if (kLocal) {
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          gv[u] = local_m4(A, A.lm + (int64_t)k * A.ld + s0 + u * 128 + lane * 4, mv[u], gv[u]);
-      }
-      float v[U][4];
-      uint32_t bits[U];
-      uint32_t nloc = 0;
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int l = u * 128 + lane * 4;
-        const float4 d4 = *reinterpret_cast<const float4*>(dlw + l);
-        v[u][0] = accumulate(ev[u].x, gv[u].x, A.c, d4.x);
-        v[u][1] = accumulate(ev[u].y, gv[u].y, A.c, d4.y);
-        v[u][2] = accumulate(ev[u].z, gv[u].z, A.c, d4.z);
-        v[u][3] = accumulate(ev[u].w, gv[u].w, A.c, d4.w);
-        __stcs(reinterpret_cast<float4*>(ekt + l), make_float4(v[u][0], v[u][1], v[u][2], v[u][3]));
-        bits[u] = cand_bits(v[u], l, lim, theta);
-        nloc += __popc(bits[u]);
-      }
-      const uint32_t cnt = __reduce_add_sync(0xffffffffu, nloc);
-      uint32_t base = 0;
-      if (lane == 0 && cnt) base = atomicAdd(&A.sel[k].count, cnt);
-      base = __shfl_sync(0xffffffffu, base, 0);
-      if (cnt) {
-        uint32_t pos = base;
-        uint32_t* ci = A.cand_idx + (int64_t)k * A.cap;
-        float* cv = A.cand_val + (int64_t)k * A.cap;
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          write_group(v[u], s0 + u * 128 + lane * 4, bits[u], lt, pos, A.cap, ci, cv, nonfinite);
-      }
-      if (lane == 0) A.chunk[chunk_at(A, k, tile, warp)] = make_uint2(base, cnt);
+    for (int u = 0; u < U; ++u) {
+      const int l = u * 128 + lane * 4;
+      __stcs(reinterpret_cast<float4*>(ekt + l), make_float4(v[u][0], v[u][1], v[u][2], v[u][3]));
+      bits[u] = cand_bits(v[u], l, lim, th);
+      nloc += __popc(bits[u]);
     }
+    if (zero_next && k == 0) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        float4* p = reinterpret_cast<float4*>(A.dlt_out + s0 + u * 128 + lane * 4);
+        const float4 x = *p;
+        if ((__float_as_uint(x.x) | __float_as_uint(x.y) | __float_as_uint(x.z) | __float_as_uint(x.w)) != 0u)
+          *p = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+    const uint32_t cnt = __reduce_add_sync(0xffffffffu, nloc);
+    uint32_t base = 0;
+    if (cnt) {
+      if (lane == 0) base = atomicAdd(&A.sel[k].count, cnt);
+      base = __shfl_sync(0xffffffffu, base, 0);
+      uint32_t pos = base;
+      uint32_t* ci = A.cand_idx + (int64_t)k * A.cap;
+      float* cv = A.cand_val + (int64_t)k * A.cap;
+      uint32_t* hk = A.chist + (int64_t)k * kRelBins;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        write_group(v[u], s0 + u * 128 + lane * 4, bits[u], lt, pos, A.cap, ci, cv, nonfinite);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if ((bits[u] >> i) & 1u) atomicAdd(hk + rel_bin(mag_key(v[u][i]), th, (int)sh), 1u);
+      }
+    }
+    if (lane == 0) A.chunk[(int64_t)st * A.K + k] = make_uint2(base, cnt);
   }
   if (nonfinite) {
     atomicOr(A.status, kStatusNonfinite);
@@ -1488,9 +1532,9 @@ __device__ __forceinline__ void candidate_part(const TopkArgs& A, int k, int p, 
 }
 
 // ---------------------------------------------------------------------------
-// exact select among candidates, two passes:
-//   hist    a kRelBins-bin histogram of the candidates' keys above theta, in
-//           bins of 2^shift keys that span the sampled keys around the k-th
+// exact select among candidates:
+//   hist    a kRelBins-bin histogram of the candidates' keys above theta,
+//           counted by the accumulate pass as it writes them, in bins of 2^shift keys that span the sampled keys around the k-th
 //           (k_sample_cluster), so that they follow the data; every block of
 //           the next launch finds the bin holding the k-th key
 //   finish  the candidates of that bin are collected (key, index); the last
@@ -1498,41 +1542,6 @@ __device__ __forceinline__ void candidate_part(const TopkArgs& A, int k, int p, 
 //           equal T are kept, and -- when fewer are kept than there are -- the
 //           largest index kept (ties go to the lower index)
 // ---------------------------------------------------------------------------
-// The candidate histogram of the load/store pass (the bulk pass counts its
-// candidates into chist as they leave its staging lines).
-__global__ void __launch_bounds__(kThreads) k_select_hist(TopkArgs A) {
-  griddep_wait();
-  __shared__ uint32_t h[kRelBins];
-  const int k = blockIdx.y;
-  WorkerSel& S = A.sel[k];
-  if (needs_dense(S, A.ksel, A.cap)) return;
-  const uint32_t theta = S.theta;
-  const int shift = (int)S.shift;
-  for (int b = threadIdx.x; b < kRelBins; b += blockDim.x) h[b] = 0;
-  __syncthreads();
-  const float* cv = A.cand_val + (int64_t)k * A.cap;
-  const int nparts = candidate_parts(A);
-  const int lane = threadIdx.x & 31;
-  for (int part = blockIdx.x * kWarps + (threadIdx.x >> 5); part < nparts; part += gridDim.x * kWarps) {
-    uint32_t lo, hi;
-    candidate_part(A, k, part, nparts, &lo, &hi);
-    for (uint32_t i0 = lo; i0 < hi; i0 += 4 * 32) {
-      uint32_t kv[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t i = i0 + q * 32 + lane;
-        kv[q] = i < hi ? mag_key(cv[i]) : 0xffffffffu;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) warp_hist_add(h, kv[q] != 0xffffffffu ? rel_bin(kv[q], theta, shift) : -1);
-    }
-  }
-  __syncthreads();
-  uint32_t* gh = A.chist + (int64_t)k * kRelBins;
-  for (int b = threadIdx.x; b < kRelBins; b += blockDim.x)
-    if (h[b]) atomicAdd(&gh[b], h[b]);
-}
-
 __global__ void __launch_bounds__(kThreads) k_select_finish(TopkArgs A) {
   griddep_wait();
   // kBucketCap keys (the indices stay in the global bucket): 48 KB, so that
@@ -1921,7 +1930,9 @@ __global__ void __launch_bounds__(1024) k_select_dense(TopkArgs A) {
 // that the sub-chunk lists hold already. (It was two launches: a per-coordinate
 // mask of the senders, then one thread per union coordinate gathering their
 // values from the residuals: d = 138 M, K = 8: 152 -> 72 us; d = 11.2 M, K = 16:
-// 44 -> 24 us.)
+// 44 -> 24 us. Bound by the warps in flight: forms that loaded pairs ahead in
+// registers (95 of them: 107 us), or took heavy sub-tiles by the block through
+// 36 KB of shared memory (92 us), ran slower than this one at 38 registers.)
 // ---------------------------------------------------------------------------
 // The position in a list of up to 32 runs (lane l's of length cnt, incl: their
 // inclusive sums): the run that holds element e (the first lane whose sum exceeds it).
@@ -1965,7 +1976,7 @@ __global__ void __launch_bounds__(kThreads) k_apply(TopkArgs A) {
     const float wn = __fsub_rn(wo, __fmul_rn(A.a_prev, sum));
     A.w[j] = wn;
     const float dd = __fsub_rn(wn, wo);
-    A.dlt[j] = dd;
+    A.dlt_out[j] = dd;
     changed += dd != 0.f;
   };
   const int64_t st0 = (int64_t)blockIdx.x * kWarps + warp;
@@ -2026,10 +2037,15 @@ __global__ void __launch_bounds__(kThreads) k_apply(TopkArgs A) {
       __syncwarp();
     }
     if (many) {
-      for (int q = 0; q < sub / 32; ++q) {
-        if (!((seen[warp][q] >> lane) & 1u)) continue;
-        const uint32_t j = sub0 + q * 32 + lane;
-        update(j, sums[warp][q * 32 + lane], A.server_mom ? 0.f : A.w[j]);
+      for (int q0 = 0; q0 < sub / 32; q0 += 4) {  // four rows of 32: their w loaded together
+        float wq[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          wq[q] = !A.server_mom && ((seen[warp][q0 + q] >> lane) & 1u) ? A.w[sub0 + (q0 + q) * 32 + lane] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if ((seen[warp][q0 + q] >> lane) & 1u)
+            update(sub0 + (q0 + q) * 32 + lane, sums[warp][(q0 + q) * 32 + lane], wq[q]);
       }
       __syncwarp();
     }
@@ -2147,29 +2163,12 @@ bool use_bulk(int tile) { return tile == bulk::kT; }
 
 }  // namespace
 
-// Dynamic shared memory of the accumulate pass for tiles of `tile` and K workers.
-int accumulate_smem_bytes(int tile, int K) {
-  return use_bulk(tile) ? bulk::smem_bytes(K) : tile * 12;
-}
-
 cudaError_t configure_topk_kernels() {
   cudaError_t err = cudaSuccess;
   auto set = [&](const void* f, int bytes) {
     const cudaError_t e2 = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (err == cudaSuccess) err = e2;
   };
-  set((const void*)k_accumulate<1, false, false>, 1024 * 12);
-  set((const void*)k_accumulate<2, false, false>, 2048 * 12);
-  set((const void*)k_accumulate<4, false, false>, 4096 * 12);
-  set((const void*)k_accumulate<1, true, false>, 1024 * 12);
-  set((const void*)k_accumulate<2, true, false>, 2048 * 12);
-  set((const void*)k_accumulate<4, true, false>, 4096 * 12);
-  set((const void*)k_accumulate<1, false, true>, 1024 * 12);
-  set((const void*)k_accumulate<2, false, true>, 2048 * 12);
-  set((const void*)k_accumulate<4, false, true>, 4096 * 12);
-  set((const void*)k_accumulate<1, true, true>, 1024 * 12);
-  set((const void*)k_accumulate<2, true, true>, 2048 * 12);
-  set((const void*)k_accumulate<4, true, true>, 4096 * 12);
   set((const void*)k_accumulate_bulk<false, false>, bulk::smem_bytes(kBulkMaxK));
   set((const void*)k_accumulate_bulk<true, false>, bulk::smem_bytes(kBulkMaxK));
   set((const void*)k_accumulate_bulk<false, true>, bulk::smem_bytes(kBulkMaxK));
@@ -2188,12 +2187,8 @@ int select_blocks_per_sm() {
 int accumulate_blocks_per_sm(int tile) {
   if (use_bulk(tile)) return 1;  // one persistent CTA per SM
   int n = 0;
-  const int smem = accumulate_smem_bytes(tile, kMaxK);
-  switch (tile_u(tile)) {
-    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_accumulate<1, false, false>, kThreads, smem); break;
-    case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_accumulate<2, false, false>, kThreads, smem); break;
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_accumulate<4, false, false>, kThreads, smem); break;
-  }
+  if (tile_u(tile) == 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_accumulate<1, false, false>, kThreads, 0);
+  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_accumulate<2, false, false>, kThreads, 0);
   return n > 0 ? n : 1;
 }
 
@@ -2214,35 +2209,28 @@ cudaError_t launch_sample(const TopkArgs& A, cudaStream_t s) {
 
 // The load/store pass's instantiation for the step's form and gradient type.
 template <int U>
-cudaError_t launch_ls(const TopkArgs& A, int grid, int smem, cudaStream_t s) {
-  if (A.local_mom && A.bf16) return launch_pdl(k_accumulate<U, true, true>, dim3(grid), dim3(kThreads), smem, s, A);
-  if (A.local_mom) return launch_pdl(k_accumulate<U, true, false>, dim3(grid), dim3(kThreads), smem, s, A);
-  if (A.bf16) return launch_pdl(k_accumulate<U, false, true>, dim3(grid), dim3(kThreads), smem, s, A);
-  return launch_pdl(k_accumulate<U, false, false>, dim3(grid), dim3(kThreads), smem, s, A);
+cudaError_t launch_ls(const TopkArgs& A, int grid, cudaStream_t s) {
+  const dim3 g(grid), b(kThreads);
+  if (A.local_mom && A.bf16) return launch_pdl(k_accumulate<U, true, true>, g, b, 0, s, A);
+  if (A.local_mom) return launch_pdl(k_accumulate<U, true, false>, g, b, 0, s, A);
+  if (A.bf16) return launch_pdl(k_accumulate<U, false, true>, g, b, 0, s, A);
+  return launch_pdl(k_accumulate<U, false, false>, g, b, 0, s, A);
 }
 
 cudaError_t launch_accumulate(const TopkArgs& A, int grid, cudaStream_t s) {
-  const int smem = accumulate_smem_bytes(A.tile, A.K);
   if (use_bulk(A.tile)) {
+    const int smem = bulk::smem_bytes(A.K);
     const dim3 g(grid), b(bulk::kThreadsAll);
     if (A.local_mom && A.bf16) return launch_pdl(k_accumulate_bulk<true, true>, g, b, smem, s, A);
     if (A.local_mom) return launch_pdl(k_accumulate_bulk<true, false>, g, b, smem, s, A);
     if (A.bf16) return launch_pdl(k_accumulate_bulk<false, true>, g, b, smem, s, A);
     return launch_pdl(k_accumulate_bulk<false, false>, g, b, smem, s, A);
   }
-  switch (tile_u(A.tile)) {
-    case 1: return launch_ls<1>(A, grid, smem, s);
-    case 2: return launch_ls<2>(A, grid, smem, s);
-    default: return launch_ls<4>(A, grid, smem, s);
-  }
+  return tile_u(A.tile) == 1 ? launch_ls<1>(A, grid, s) : launch_ls<2>(A, grid, s);
 }
 
 cudaError_t launch_select(const TopkArgs& A, int blocks_per_worker, cudaStream_t s) {
   const dim3 grid(blocks_per_worker, A.K);
-  if (A.regions == 1) {  // the bulk pass histogrammed its candidates already
-    const cudaError_t err = launch_pdl(k_select_hist, grid, dim3(kThreads), 0, s, A);
-    if (err != cudaSuccess) return err;
-  }
   return launch_pdl(k_select_finish, grid, dim3(kThreads), kBucketCap * 4, s, A);
 }
 
