@@ -20,9 +20,9 @@
 //
 // Bound by latency and issue: three grid barriers (about 2 us each), a dozen
 // dependent L2 accesses, a few passes over shared memory. Step and read of w,
-// where the step took nine launches: d = 65,536, K = 4: 53 -> 33 us (21 of them
-// this kernel); d = 272 k, K = 8: 70 -> 46 us (36). 512 threads: with 1,024 the
-// accumulator loop spills and the smallest steps take 2 us more.
+// where the step took nine launches: d = 65,536, K = 4: 53 -> 22 us (20 of
+// them this kernel); d = 272 k, K = 8: 70 -> 40 us (34). 768 threads: 512 leave the
+// passes over shared memory short of warps (36 us), 1,024 spill (36).
 #include <algorithm>
 
 #include "gmc_internal.h"
@@ -30,7 +30,7 @@
 namespace gmc {
 namespace {
 
-constexpr int kSmThreads = 512;
+constexpr int kSmThreads = 768;
 constexpr int kSmWarps = kSmThreads / 32;
 constexpr int kMaxK = 32;
 constexpr int kItemMax = kSmallItems;       // (group, worker) items of a block
@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Search sr[kMaxK];
   __shared__ uint32_t cnt[kItemMax];            // per item: sent elements, then its pairs' first slot
+  __shared__ uint32_t imax[kItemMax];           // per item: its largest key
   __shared__ uint16_t smask[kItemMax];          // approximate: sampled blocks of 8 of each own group
   __shared__ unsigned long long red[kSmWarps][5];
   __shared__ uint32_t s_ok, s_active, s_pairs;
@@ -166,13 +167,17 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
       *reinterpret_cast<float4*>(vs + (size_t)i * 128 + lane * 4) = v;
       const float x[4] = {v.x, v.y, v.z, v.w};
       const bool in = !A.approx || ((smask[gi] >> (lane >> 1)) & 1u);
+      uint32_t most = 0;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         if (j + c >= A.d) continue;
         nonfinite += is_nonfinite(x[c]) ? 1u : 0u;
+        most = max(most, mag_key(x[c]));
         const uint32_t bin = mag_key(x[c]) >> 20;
         if (fused && in) atomicAdd(&hs[k * (kHistBins / 2) + (bin >> 1)], (bin & 1) ? 0x10000u : 1u);
       }
+      most = __reduce_max_sync(0xffffffffu, most);
+      if (lane == 0) imax[i] = most;
     }
   }
   // start of a search: the rank-th largest of all keys (or of the sampled ones)
@@ -195,12 +200,14 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
   uint32_t fallbacks = 0;  // thread k: worker k's ties went to index digits, or it exceeded the limit
   // For the items of workers [k_lo, k_hi) that pass `want`: f(k, search, m, key, j)
   // with bit c of m set where value c belongs to the search and has its prefix.
+  // Items whose largest key lies below the prefix are passed over: most, where
+  // layers differ in scale.
   auto each_match = [&](int k_lo, int k_hi, bool sampled, auto&& want, auto&& f) {
     const int nk = k_hi - k_lo, dg = kSmWarps / nk, dk = kSmWarps - dg * nk;
     int gi = warp / nk, k = k_lo + warp % nk;
     while (gi < own) {
       const Search s = sr[k];
-      if (want(s)) {
+      if (want(s) && imax[gi * K + k] >= (s.by_index ? s.T : s.prefix << s.left)) {
         const float4 v = *reinterpret_cast<const float4*>(vs + (size_t)(gi * K + k) * 128 + lane * 4);
         const uint32_t key[4] = {mag_key(v.x), mag_key(v.y), mag_key(v.z), mag_key(v.w)};
         const uint32_t j = (uint32_t)group_of(gi) * 128u + lane * 4;
@@ -226,7 +233,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
   auto flush = [&](uint32_t* gh, int k_lo, int k_hi) {
     const int nw = (k_hi - k_lo) * (kHistBins / 2);
     __syncthreads();
-    for (int q = threadIdx.x; q < nw; q += kSmThreads) {  // whole warps: nw is a multiple of 512
+    for (int q = threadIdx.x; q < nw; q += kSmThreads) {  // whole warps: nw is a multiple of 32
       const uint32_t word = hs[q];
       if (!__any_sync(0xffffffffu, word != 0)) continue;
       const int k = k_lo + q / (kHistBins / 2), bin = (q & (kHistBins / 2 - 1)) * 2;
@@ -475,6 +482,11 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
       const float4 v = *reinterpret_cast<const float4*>(vk);
       float en[4] = {v.x, v.y, v.z, v.w};
       const uint32_t T = sr[k].T, ti = sr[k].t_idx;
+      if (imax[gi * K + k] < T) {  // nothing sent
+        __stcs(reinterpret_cast<float4*>(A.e + (int64_t)k * A.ld + j), v);
+        if (lane == 0) cnt[gi * K + k] = 0;
+        continue;
+      }
       uint32_t n = 0;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {

@@ -32,11 +32,6 @@ namespace {
 
 constexpr int kMaxK = 32;  // workers supported by the top-k kernels (one lane or mask bit each)
 
-// The local momentum of worker k at sampled coordinate j, formed from g
-// (m_{t+1} = beta*m_t + eta*g, Sec. 2.3 eq. (3)) without storing it.
-__device__ __forceinline__ float local_m(const TopkArgs& A, int k, int64_t j, float g) {
-  return __fadd_rn(__fmul_rn(A.beta, A.lm[(int64_t)k * A.ld + j]), __fmul_rn(A.gs, g));
-}
 // The local-momentum baseline: m = beta*m + eta*g over 4 coordinates (m
 // loaded from p beforehand, p 16-byte aligned inside ld), stored back at p;
 // returns it for the accumulator in place of g.
@@ -441,10 +436,10 @@ __global__ void __cluster_dims__(scl::kCtas, 1, 1) __launch_bounds__(scl::kThrea
 // samples store every sampled key and add its first radix digit to the
 // worker's histogram, for k_sample_theta. The accumulator at a sampled
 // coordinate is formed as if the previous step's aggregation had been applied
-// (residual +0 where the worker sent, the pending delta). A thread takes a run
-// of 8 with 16-byte loads, all issued before any is used; a block takes several
-// runs a thread before it adds its histogram to the worker's (d = 138 M, K = 8,
-// 11 M sampled values: 132 us slot by slot -> 79 us).
+// (residual +0 where the worker sent, the pending delta). A thread takes half a
+// run of 8 with 16-byte loads; a block takes many before it adds its histogram
+// to the worker's (d = 138 M, K = 8, 11 M sampled values: 132 us slot by slot,
+// 79 a run a thread -> 73 us).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads) k_sample(TopkArgs A) {
   griddep_wait();
@@ -459,46 +454,33 @@ __global__ void __launch_bounds__(kThreads) k_sample(TopkArgs A) {
   const float* ek = A.e + (int64_t)k * A.ld;
   const float* gk = A.grads + (int64_t)k * A.d;
   const uint16_t* gk16 = A.grads16 + (int64_t)k * A.d;
+  const int gm = g_mode(gk);
   uint32_t* keys = A.sample_keys + (int64_t)k * A.sample_stride;
-  const int n_s = (int)A.n_sample, runs = (n_s + 7) / 8;
+  const int n_s = (int)A.n_sample, quads = (n_s + 3) / 4;
   for (int b = threadIdx.x; b < kHistBins; b += blockDim.x) hist[b] = 0;
   __syncthreads();
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < runs; r += gridDim.x * blockDim.x) {
-    const int64_t j0 = A.sample_pend[2 * A.sample_stride + r];
-    const int nv = min(8, n_s - r * 8);  // 8, but for d < 8
-    float ev[8], gv[8], lv[8];
-    uint32_t pm[8], pd[8];
-    if (nv == 8) {
-      load8u(A.sample_pend + r * 8, pm);
-      load8u(A.sample_pend + A.sample_stride + r * 8, pd);
-      load8(ek + j0, ev);  // rows of e and lm start on 16 bytes, runs on 8 coordinates
-      if (A.local_mom) load8(A.lm + (int64_t)k * A.ld + j0, lv);
-      if (A.bf16) load8_bf16(gk16 + j0, gv);
-      else load8(gk + j0, gv);
-    } else {
-      for (int q = 0; q < 8; ++q) {
-        const bool in = q < nv;
-        pm[q] = in ? A.sample_pend[r * 8 + q] : 0u;
-        pd[q] = in ? A.sample_pend[A.sample_stride + r * 8 + q] : 0u;
-        ev[q] = in ? ek[j0 + q] : 0.f;
-        lv[q] = in && A.local_mom ? A.lm[(int64_t)k * A.ld + j0 + q] : 0.f;
-        gv[q] = in ? (A.bf16 ? bf16_f32(gk16[j0 + q]) : gk[j0 + q]) : 0.f;
-      }
-    }
-    uint32_t key[8];
+  // a thread takes half a run: a pair of lanes reads one 32-byte sector of e and of g
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < quads; q += gridDim.x * blockDim.x) {
+    const int64_t j = (int64_t)A.sample_pend[2 * A.sample_stride + (q >> 1)] + (q & 1) * 4;
+    const int nv = min(4, n_s - q * 4);  // 4, but for d < 8
+    const uint4 pm = *reinterpret_cast<const uint4*>(A.sample_pend + q * 4);
+    const uint4 pd = *reinterpret_cast<const uint4*>(A.sample_pend + A.sample_stride + q * 4);
+    // rows of e and lm start on 16 bytes and reach a whole tile; runs start on 8 coordinates
+    const float4 e4 = *reinterpret_cast<const float4*>(ek + j);
+    float4 l4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (A.local_mom) l4 = *reinterpret_cast<const float4*>(A.lm + (int64_t)k * A.ld + j);
+    const float4 g4 = A.bf16 ? load_g4_bf16(gk16, j, A.d) : load_g4(gk, j, A.d, gm);
+    const float ev[4] = {e4.x, e4.y, e4.z, e4.w}, gv[4] = {g4.x, g4.y, g4.z, g4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
+    const uint32_t m[4] = {pm.x, pm.y, pm.z, pm.w}, dd[4] = {pd.x, pd.y, pd.z, pd.w};
+    uint32_t key[4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float g = A.local_mom ? __fadd_rn(__fmul_rn(A.beta, lv[q]), __fmul_rn(A.gs, gv[q]))
-                                  : (A.gscale ? __fmul_rn(A.gs, gv[q]) : gv[q]);
-      key[q] = mag_key(accumulate(((pm[q] >> k) & 1u) ? 0.f : ev[q], g, A.c, __uint_as_float(pd[q])));
-      if (q < nv) atomicAdd(&hist[key[q] >> 20], 1u);
+    for (int c = 0; c < 4; ++c) {
+      const float g = A.local_mom ? __fadd_rn(__fmul_rn(A.beta, lv[c]), __fmul_rn(A.gs, gv[c]))
+                                  : (A.gscale ? __fmul_rn(A.gs, gv[c]) : gv[c]);
+      key[c] = mag_key(accumulate(((m[c] >> k) & 1u) ? 0.f : ev[c], g, A.c, __uint_as_float(dd[c])));
+      if (c < nv) atomicAdd(&hist[key[c] >> 20], 1u);
     }
-    if (nv == 8) {
-      reinterpret_cast<uint4*>(keys + r * 8)[0] = make_uint4(key[0], key[1], key[2], key[3]);
-      reinterpret_cast<uint4*>(keys + r * 8)[1] = make_uint4(key[4], key[5], key[6], key[7]);
-    } else {
-      for (int q = 0; q < nv; ++q) keys[r * 8 + q] = key[q];
-    }
+    *reinterpret_cast<uint4*>(keys + q * 4) = make_uint4(key[0], key[1], key[2], key[3]);  // (a row holds whole quads)
   }
   __syncthreads();
   uint32_t* gh = A.ghist + (int64_t)k * kThetaBins;
@@ -971,30 +953,35 @@ __global__ void __launch_bounds__(kThreads) k_accumulate(TopkArgs A) {
 // ---------------------------------------------------------------------------
 namespace bulk {
 constexpr int kT = kBulkTile;
-constexpr int kStages = 4;                 // shared-memory ring of (e, g) tiles
-// Each worker-parity warp group has its own kGroupStages of the ring, which it
+// Stages of the shared-memory ring of (e, g) tiles: as many as fit, since the
+// pass is bound by the bytes its ring keeps in flight (an SM's reads of 4 x 32 KB
+// take about 4.9 us under load). bf16 gradients leave room for six stages of
+// 24 KB: d = 138 M, K = 8 step and read of w 2,174 -> 2,161 us.
+__host__ __device__ constexpr int stages(bool bf16) { return bf16 ? 6 : 4; }
+// Each worker-parity warp group has its own half of the ring's stages, which it
 // reads in order: an mbarrier wait by phase parity can only tell the phase it
 // waits for from the one before, so no warp may wait on a stage two phases
 // ahead, as it could if the groups shared stages (an odd K, or a ring whose
 // size is not twice a group's share).
-constexpr int kGroupStages = kStages / 2;
 constexpr int kSubTiles = kChunksPerTile;  // 8 sub-tiles of 512 elements
 constexpr int kSub = kT / kSubTiles;       // 512
 constexpr int kConsumers = 2 * kSubTiles;  // warps 0..15: sub-tile w & 7, workers of parity w >> 3
-constexpr int kGLen = kT + 8;              // g stage: up to 3 leading floats of misalignment
+// g stage: the tile and up to 15 leading bytes of misalignment, in whole 16 bytes
+__host__ __device__ constexpr int g_bytes(bool bf16) { return (kT + 8) * (bf16 ? 2 : 4); }
 constexpr int kProducer = kConsumers;      // warp 16
 constexpr int kThreadsAll = (kConsumers + 1) * 32;
+template <bool kBf16>
 struct Smem {
-  float e[kStages][kT];
-  float g[kStages][kGLen];
+  float e[stages(kBf16)][kT];
+  alignas(16) unsigned char g[stages(kBf16)][g_bytes(kBf16)];
   float dl[kSubTiles][kSub];               // w_t - w_{t-1} of a sub-tile
   uint32_t mk[kSubTiles][kSub];            // senders of the pending aggregation (bit k)
   uint8_t own[kConsumers][32];             // scratch of each consumer warp: worker of each listed pair
   uint32_t upos[kSubTiles][32];            // union coordinates of a sub-tile, one per lane
   uint32_t pflag[kSubTiles];               // per sub-tile: more than 32 pairs (per-element masks)
-  uint64_t full[kStages];                  // e, g landed (1 arrival + tx bytes)
-  uint64_t empty[kStages];                 // all consumer warps read the stage (8 arrivals)
-  int32_t gmeta[kStages];                  // leading floats in the g stage, -1 = not copied
+  uint64_t full[stages(kBf16)];            // e, g landed (1 arrival + tx bytes)
+  uint64_t empty[stages(kBf16)];           // all consumer warps read the stage (8 arrivals)
+  int32_t gmeta[stages(kBf16)];            // leading elements in the g stage, -1 = not copied
   uint32_t theta[kMaxK], shift[kMaxK];     // candidate threshold and relative histogram of each worker
   uint32_t Tp[kMaxK], tip[kMaxK];          // the previous step's selection (T, t_idx) per worker
   uint32_t tq[16];                         // claimed tiles (tile_at)
@@ -1009,17 +996,18 @@ struct Smem {
 // slot is that of tile n + D (D: the pipeline's depth, 3 or 1) during tile n,
 // after it waited on an item of tile n - 1, whose issue followed the
 // producer's publishing of slots up to n - 2 + F: so F = D + 2. The producer
-// runs at most kStages items (tiles, for K <= 2) ahead of the slowest consumer.
+// runs at most a ring of items (tiles, for K <= 2) ahead of the slowest consumer.
 constexpr int kFixedDeep = 5;     // K <= kDeepMaxK: depth 3
 constexpr int kFixedShallow = 3;  // more workers: depth 1
 constexpr int kDeepMaxK = 5;      // from K = 6 the lead warp has three items a tile or more
 constexpr int kQ = 16;
-static_assert(kQ > kStages + kFixedDeep, "the producer may overwrite a claimed tile not yet read");
+static_assert(kQ > stages(true) + kFixedDeep && kQ > stages(false) + kFixedDeep, "the producer may overwrite a claimed tile not yet read");
 // Dynamic shared memory of the bulk pass for K workers.
+template <bool kBf16>
 __host__ __device__ constexpr int smem_bytes(int K) {
-  return (int)((sizeof(Smem) + 127) / 128 * 128) + kSubTiles * K * 64 * 4;
+  return (int)((sizeof(Smem<kBf16>) + 127) / 128 * 128) + kSubTiles * K * 64 * 4;
 }
-static_assert(smem_bytes(kBulkMaxK) <= 232448, "bulk pass shared memory above the 227 KB a block may use");
+static_assert(smem_bytes<false>(kBulkMaxK) <= 232448 && smem_bytes<true>(kBulkMaxK) <= 232448, "bulk pass shared memory above the 227 KB a block may use");
 
 // The first (up to 32) sent pairs of one sub-tile of the previous step, lane e
 // holding pair e of the list that runs through the workers in ascending order.
@@ -1133,7 +1121,9 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
   griddep_wait();
   using namespace bulk;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+  using Sm = Smem<kBf16>;
+  constexpr uint32_t kStages = stages(kBf16), kGroupStages = kStages / 2;
+  Sm& sm = *reinterpret_cast<Sm*>(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // the lead warp's pipeline spans three tiles: for few workers, and for the
   // bf16 and local-momentum forms, where the one-tile pipeline measured slower
@@ -1143,7 +1133,7 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
   const uint32_t* order = A.use_order ? A.blk_order : nullptr;  // the tiles' order (tile_order)
   const uint32_t G = gridDim.x, nbw = (uint32_t)(A.n_tiles / G);  // whole blocks of G tiles
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (uint32_t s = 0; s < kStages; ++s) {
       mbar_init(&sm.full[s], 1);
       mbar_init(&sm.empty[s], kSubTiles);  // the eight warps of the stage's worker parity
     }
@@ -1206,7 +1196,7 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
     // other warp's help. No later phase is armed on their stages, so each
     // parity wait is for exactly that copy.
     for (uint32_t grp = 0; grp < 2; ++grp) {
-      const uint32_t c1 = issued[grp], c0 = c1 > (uint32_t)kGroupStages ? c1 - kGroupStages : 0u;
+      const uint32_t c1 = issued[grp], c0 = c1 > kGroupStages ? c1 - kGroupStages : 0u;
       for (uint32_t c = c0; c < c1; ++c)
         if (((grp << 31) | c) != held &&
             !wait_bounded(&sm.full[grp * kGroupStages + c % kGroupStages], (c / kGroupStages) & 1, kWaitLimitNs))
@@ -1225,10 +1215,10 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
   // the sub-tile's part of the CTA's region, per worker: slots [part0, part0 + cap_part);
   // lane k counts worker k's candidates so far
   const uint32_t part0 = (blockIdx.x * kSubTiles + sw) * A.cap_part;
-  uint32_t* stg = reinterpret_cast<uint32_t*>(smem_raw + (sizeof(Smem) + 127) / 128 * 128) +
+  uint32_t* stg = reinterpret_cast<uint32_t*>(smem_raw + (sizeof(Sm) + 127) / 128 * 128) +
                   sw * A.K * 64;
   uint32_t run = 0;
-  uint32_t taken = 0;  // items of this warp's group read so far (its stages, in order)
+  uint32_t taken = 0;  // the group's stage to read next (its stages, in order), and the phase's parity
   uint32_t nonfinite = 0, uni = 0, chg = 0;
   bool ok = true;  // false after a bounded wait gave up: the items are skipped, the tile loop
                    // still runs (its named barriers need both warps of the sub-tile)
@@ -1312,21 +1302,22 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
     uint2 bc_lane = make_uint2(0u, 0u);
     uint32_t tcnt = 0;  // this warp's candidates of the tile (the block's cost, tile_order)
     for (int k = gp; ok && k < A.K; k += 2) {
-      const uint32_t s = gp * kGroupStages + taken % kGroupStages, r = taken / kGroupStages;
-      ++taken;
+      const uint32_t s = gp * kGroupStages + (taken & 0xffu), parity = taken >> 31;
+      // the group's next stage; its phase's parity in the top bit
+      taken = (taken & 0xffu) + 1u < kGroupStages ? taken + 1u : (taken & 0x80000000u) ^ 0x80000000u;
       float4 mv[kSub / 128];  // the local-momentum baseline: m loaded while the stage lands
       if (kLocal) {
 #pragma unroll
         for (int u = 0; u < kSub / 128; ++u)
           mv[u] = __ldcs(reinterpret_cast<const float4*>(A.lm + (int64_t)k * A.ld + s0 + u * 128 + lane * 4));
       }
-      if (!__all_sync(0xffffffffu, wait_bounded(&sm.full[s], r & 1, A.wait_ns))) {  // warp-uniform
+      if (!__all_sync(0xffffffffu, wait_bounded(&sm.full[s], parity, A.wait_ns))) {  // warp-uniform
         ok = false;
         break;
       }
       const int32_t off = sm.gmeta[s];
       float* se = sm.e[s] + sw * kSub;
-      const float* sg = sm.g[s] + (off > 0 ? off : 0) + sw * kSub;
+      const float* sg = reinterpret_cast<const float*>(sm.g[s]) + (off > 0 ? off : 0) + sw * kSub;
       if (patch) {
         if ((umask >> k) & 1u) {
           se[upos] = 0.f;
@@ -2169,10 +2160,10 @@ cudaError_t configure_topk_kernels() {
     const cudaError_t e2 = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (err == cudaSuccess) err = e2;
   };
-  set((const void*)k_accumulate_bulk<false, false>, bulk::smem_bytes(kBulkMaxK));
-  set((const void*)k_accumulate_bulk<true, false>, bulk::smem_bytes(kBulkMaxK));
-  set((const void*)k_accumulate_bulk<false, true>, bulk::smem_bytes(kBulkMaxK));
-  set((const void*)k_accumulate_bulk<true, true>, bulk::smem_bytes(kBulkMaxK));
+  set((const void*)k_accumulate_bulk<false, false>, bulk::smem_bytes<false>(kBulkMaxK));
+  set((const void*)k_accumulate_bulk<true, false>, bulk::smem_bytes<false>(kBulkMaxK));
+  set((const void*)k_accumulate_bulk<false, true>, bulk::smem_bytes<true>(kBulkMaxK));
+  set((const void*)k_accumulate_bulk<true, true>, bulk::smem_bytes<true>(kBulkMaxK));
   set((const void*)k_select_finish, kBucketCap * 4);
   return err;
 }
@@ -2219,7 +2210,7 @@ cudaError_t launch_ls(const TopkArgs& A, int grid, cudaStream_t s) {
 
 cudaError_t launch_accumulate(const TopkArgs& A, int grid, cudaStream_t s) {
   if (use_bulk(A.tile)) {
-    const int smem = bulk::smem_bytes(A.K);
+    const int smem = A.bf16 ? bulk::smem_bytes<true>(A.K) : bulk::smem_bytes<false>(A.K);
     const dim3 g(grid), b(bulk::kThreadsAll);
     if (A.local_mom && A.bf16) return launch_pdl(k_accumulate_bulk<true, true>, g, b, smem, s, A);
     if (A.local_mom) return launch_pdl(k_accumulate_bulk<true, false>, g, b, smem, s, A);
