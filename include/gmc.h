@@ -196,8 +196,8 @@ int gmc_set_params(gmc_t h, const float* w0_dev, void* stream);
  * synchronises. Non-finite accumulator values still complete the step
  * deterministically and are reported by gmc_check as GMC_ENONFINITE.
  *
- * Deferred aggregation (top-k with d >= 4096 * 2 * SMs, about 1.25 M on GB300):
- * the step selects and records C(e_{t+1/2,k}) but leaves the last line of
+ * Deferred aggregation (top-k on the bulk pass: 2 to 16 workers and d >= 8 *
+ * 4096 * SMs, about 5 M on GB300): the step selects and records C(e_{t+1/2,k}) but leaves the last line of
  * Alg. 1 -- w_{t+1} = w_t - (eta/K) sum_k C_k and the zeroing of the sent
  * residuals -- to the next gmc_step, whose single pass over the tiles applies
  * it before forming its own accumulator. The results are the same, bit for
@@ -346,7 +346,8 @@ int64_t gmc_test_fail_alloc(int64_t fail_at);
  * issue have landed, and gmc_check then reports GMC_ETIMEOUT. GMC_EINVAL when
  * the handle's step has no bulk pass (exact or approximate top-k needs
  * d >= 4096 * 2 * SMs and K <= 16; RBGS d >= 4096 * SMs), or for a tile, worker or
- * limit out of range.
+ * limit out of range. A top-k handle of such a size whose steps take another
+ * pass (see gmc_step) takes the bulk pass from that step on.
  */
 int gmc_test_withhold_copy(gmc_t h, int64_t tile, int32_t k, uint64_t wait_limit_ns);
 

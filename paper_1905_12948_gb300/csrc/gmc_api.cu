@@ -45,12 +45,13 @@ struct gmc_ctx {
   // geometry
   int tile = 0;
   int64_t n_tiles = 0, ld = 0;
-  uint32_t ksel = 0, cap = 0, sample_rank = 0, sample_rank_hi = 0;
+  uint32_t ksel = 0, cap0 = 0, cap = 0, sample_rank = 0, sample_rank_hi = 0;  // cap0: expected candidates, with slack
   int sample_chunks = 0;
   int64_t nb = 0, m = 0;
   uint32_t B_shift = 0xffffffffu;
   int grid_acc = 1, grid_agg = 1, grid_rbgs = 1, sel_blocks = 1;
   bool rbgs_bulk = false;
+  bool bulk_able = false;             // top-k: large enough for the bulk pass (gmc_test_withhold_copy)
   int grid_small = 0;                 // the one-launch top-k step's grid, 0: not taken
   uint32_t* small_scratch = nullptr;
   // state
@@ -66,7 +67,6 @@ struct gmc_ctx {
   uint32_t* chist = nullptr;
   uint32_t* bucket = nullptr;  // K x 2*kBucketCap
   uint32_t* sample_keys = nullptr;
-  uint32_t* big_tiles = nullptr;
   uint32_t* rcount = nullptr;
   int regions = 1;
   uint32_t cap_region = 0, cap_part = 0;
@@ -285,7 +285,6 @@ TopkArgs topk_args_at(gmc_ctx* h, const float* grads, int64_t t) {
   A.t = t;
   A.limit = h->limit;
   A.theta_blocks = h->theta_blocks;
-  A.big_tiles = h->big_tiles;
   A.g_direct = 0;
   A.regions = h->regions;
   A.cap_region = h->cap_region;
@@ -381,6 +380,73 @@ RbgsArgs rbgs_args(gmc_ctx* h, const float* grads) {
   return A;
 }
 
+// The top-k pass of a handle that could take the bulk-copy pass (K <= 16 and
+// two of its 4,096-coordinate tiles per SM): the bulk pass from kBulkTilesPerSm
+// tiles per SM on, and with more than one worker (one worker's items use half of
+// its warps and ring); else the load/store pass, whose items are 16 times finer.
+// Step and read of w, ratio 0.001, load/store against bulk, us: d = 2 M, K = 8
+// 73 / 99, K = 16 108 / 147; 5 M 139 / 152, 220 / 239; 10 M 244 / 241, 406 / 406;
+// 20 M 444 / 408, 750 / 740; K = 1, d = 40 M 224 / 272. Four steps to a read of w
+// (the bulk pass defers the aggregation), K = 8: 3 M 367 / 401; 5 M 562 / 533.
+constexpr int kBulkTilesPerSm = 8;
+
+// Tiles, grids and candidate lists of the top-k pass, and their memory.
+cudaError_t lay_out(gmc_ctx* h, bool bulk) {
+  // a sub-chunk is an eighth of a tile: 512 coordinates, 256, or (small d, and
+  // the one-launch step's groups of) 128
+  h->tile = bulk ? kBulkTile : (h->grid_small || h->d < 4096 * (int64_t)h->num_sms ? 1024 : 2048);
+  h->n_tiles = (h->d + h->tile - 1) / h->tile;
+  // the bulk pass: a tile at least per CTA; the load/store pass: (sub-tile, worker) items, eight to a block
+  h->grid_acc = (int)std::min<int64_t>(h->tile == kBulkTile ? h->n_tiles : h->n_tiles * h->K,
+                                       (int64_t)h->num_sms * accumulate_blocks_per_sm(h->tile));
+  // k_apply: a warp per sub-tile, as many blocks as are resident at once
+  h->grid_agg = (int)std::min<int64_t>(h->n_tiles, (int64_t)h->num_sms * apply_blocks_per_sm());
+  // candidate slots: the bulk pass gives every CTA its own region per worker,
+  // one part per consumer warp: twice its share of the expected candidates --
+  // up to 16 times when there are few tiles, as a layer that holds most of the
+  // candidates then spans few CTAs (1/64 of 1,221 tiles: 8 times the share; with
+  // twice, d = 5 M, K = 8, ratio 0.01 overflowed into the dense path, 7.6 ms a
+  // step) -- plus slack, in whole 128-byte lines. Otherwise one region.
+  const uint32_t cap0 = h->cap0;
+  if (h->tile == kBulkTile) {
+    h->n_blk = (uint32_t)(h->n_tiles / h->grid_acc);
+    h->blk_mul = golden_stride(h->n_blk);
+    h->regions = h->grid_acc;
+    const uint64_t times = std::min<uint64_t>(16, std::max<uint64_t>(2, 128ull * h->num_sms / (uint64_t)h->n_tiles));
+    const uint64_t share = (times * cap0 + h->regions * kChunksPerTile - 1) / (h->regions * kChunksPerTile);
+    h->cap_part = (uint32_t)((share + 128 + 31) & ~31ull);
+    h->cap_region = h->cap_part * kChunksPerTile;
+  } else {
+    h->regions = 1;
+    h->cap_region = (cap0 + 3) & ~3u;
+    h->cap_part = h->cap_region;
+  }
+  h->cap = (uint32_t)std::min<uint64_t>(
+      std::max<uint64_t>((uint64_t)h->regions * h->cap_region, h->limit), 0xfffffff0ull);
+  const int64_t per = (h->cap + 2047) / 2048;
+  // select: on the bulk path a warp walks the candidates of a run of at most
+  // 32 parts as one list; the grid is one wave of as many blocks as fit on
+  // an SM (each holds kBucketCap keys of shared memory: three on GB300), for
+  // all the workers -- a second, partial wave cost about 10 us
+  const int64_t nparts = (int64_t)h->regions * kChunksPerTile;
+  const int64_t sel_wave = (int64_t)select_blocks_per_sm() * h->num_sms;
+  h->sel_blocks = h->regions > 1 ? (int)std::min<int64_t>(
+                                       h->regions, std::max<int64_t>((nparts + 32 * kWarps - 1) / (32 * kWarps),
+                                                                     std::max<int64_t>(1, sel_wave / h->K)))
+                                 : (int)std::max<int64_t>(1, std::min<int64_t>(per, std::max<int64_t>(1, sel_wave / h->K)));
+  cudaError_t err = dalloc(h, &h->rcount, (size_t)h->K * h->regions * kChunksPerTile);
+  if (err == cudaSuccess && bulk && h->n_blk >= 8) {
+    err = dalloc(h, &h->blk_cost, (size_t)h->n_blk);
+    if (err == cudaSuccess) err = dalloc(h, &h->blk_order, (size_t)h->n_blk);
+  }
+  for (int p = 0; p < 2 && err == cudaSuccess; ++p) {
+    err = dalloc(h, &h->cand_idx[p], (size_t)h->K * h->cap);
+    if (err == cudaSuccess) err = dalloc(h, &h->cand_val[p], (size_t)h->K * h->cap);
+    if (err == cudaSuccess) err = dalloc(h, &h->chunk[p], (size_t)h->K * h->n_tiles * kChunksPerTile);
+  }
+  return err;
+}
+
 #define GMC_TRY(expr)                          \
   do {                                         \
     const cudaError_t err_ = (expr);           \
@@ -408,6 +474,14 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
   const uint16_t* grads16 = bf16 ? static_cast<const uint16_t*>(grads_any) : nullptr;
   const double Kd = (double)h->K * (double)h->d;
   GMC_TRY(order_after_flush(h, s, true));
+  if (h->hold_tile >= 0 && h->bulk_able && h->tile != kBulkTile) {
+    // test hook on a handle whose steps take another pass: it takes the bulk
+    // pass from here on (w_t - w_{t-1} is read densely once, as after a restore)
+    h->grid_small = 0;
+    h->dlt_next = nullptr;
+    GMC_TRY(lay_out(h, true));
+    h->restored = h->t > 0;
+  }
   const bool small = h->grid_small && h->select_mode == GMC_SELECT_SAMPLED;
   // the exact top-k's sample kernel and the RBGS pick clear the step's counters
   // themselves (a memset between two kernels would keep the second from starting early)
@@ -596,18 +670,13 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
 
   const int64_t streams_wide = 2 * (int64_t)h->num_sms;
   if (compressor != GMC_RBGS) {
-    // tiles of 4096 take the bulk-copy pass, for up to kBulkMaxK workers (its
-    // shared memory grows with K); otherwise the load/store pass
-    int U = K <= kBulkMaxK ? 4 : 2;
-    if (d < 4096 * streams_wide) U = 2;
-    if (d < 2048 * streams_wide) U = 1;
-    // a problem that fits in the SMs' shared memory takes the one-launch step,
-    // whose sub-chunks are groups of 128 coordinates (tiles of 1024)
-    h->grid_small = U < 4 || K > kBulkMaxK ? small_grid(d, K, h->num_sms) : 0;
-    if (h->grid_small) U = 1;
-    h->tile = 1024 * U;
-    h->n_tiles = (d + h->tile - 1) / h->tile;
-    h->ld = h->n_tiles * h->tile;
+    // the pass: see kBulkTilesPerSm; a problem that fits in the SMs' shared
+    // memory takes the one-launch step
+    h->bulk_able = K <= kBulkMaxK && d >= 4096 * streams_wide;
+    const bool bulk = h->bulk_able && K > 1 && d >= (int64_t)kBulkTilesPerSm * kBulkTile * h->num_sms;
+    h->grid_small = bulk ? 0 : small_grid(d, K, h->num_sms);
+    const int64_t whole = h->bulk_able ? kBulkTile : (d < 2048 * streams_wide ? 1024 : 2048);
+    h->ld = (d + whole - 1) / whole * whole;
     const int64_t ks = std::max<int64_t>(1, (int64_t)std::floor(ratio * (double)d));
     h->ksel = (uint32_t)ks;
     if (compressor == GMC_TOPK_APPROX) {
@@ -640,40 +709,7 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
       const double capd = std::ceil((double)d * (r + 8.0 * std::sqrt(r) + 16.0) / ns) + 4096.0;
       h->cap = (uint32_t)std::min<double>((double)d, capd);
     }
-    // the bulk pass: a tile at least per CTA; the load/store pass: (sub-tile, worker) items, eight to a block
-    h->grid_acc = (int)std::min<int64_t>(h->tile == kBulkTile ? h->n_tiles : h->n_tiles * K,
-                                         (int64_t)h->num_sms * accumulate_blocks_per_sm(h->tile));
-    // k_apply: a warp per sub-tile, as many blocks as are resident at once
-    h->grid_agg = (int)std::min<int64_t>(h->n_tiles, (int64_t)h->num_sms * apply_blocks_per_sm());
-    // candidate slots: the bulk pass gives every CTA its own region per worker,
-    // one part per consumer warp (twice its share of the expected candidates,
-    // plus slack, in whole 128-byte lines); otherwise one region
-    const uint32_t cap0 = h->cap;
-    if (h->tile == kBulkTile) {
-      h->n_blk = (uint32_t)(h->n_tiles / h->grid_acc);
-      h->blk_mul = golden_stride(h->n_blk);
-      h->regions = h->grid_acc;
-      const uint64_t share = (2ull * cap0 + h->regions * kChunksPerTile - 1) / (h->regions * kChunksPerTile);
-      h->cap_part = (uint32_t)((share + 128 + 31) & ~31ull);
-      h->cap_region = h->cap_part * kChunksPerTile;
-    } else {
-      h->regions = 1;
-      h->cap_region = (cap0 + 3) & ~3u;
-      h->cap_part = h->cap_region;
-    }
-    h->cap = (uint32_t)std::min<uint64_t>(
-        std::max<uint64_t>((uint64_t)h->regions * h->cap_region, h->limit), 0xfffffff0ull);
-    const int64_t per = (h->cap + 2047) / 2048;
-    // select: on the bulk path a warp walks the candidates of a run of at most
-    // 32 parts as one list; the grid is one wave of as many blocks as fit on
-    // an SM (each holds kBucketCap keys of shared memory: three on GB300), for
-    // all the workers -- a second, partial wave cost about 10 us
-    const int64_t nparts = (int64_t)h->regions * kChunksPerTile;
-    const int64_t sel_wave = (int64_t)select_blocks_per_sm() * h->num_sms;
-    h->sel_blocks = h->regions > 1 ? (int)std::min<int64_t>(
-                                         h->regions, std::max<int64_t>((nparts + 32 * kWarps - 1) / (32 * kWarps),
-                                                                       std::max<int64_t>(1, sel_wave / K)))
-                                   : (int)std::max<int64_t>(1, std::min<int64_t>(per, std::max<int64_t>(1, sel_wave / K)));
+    h->cap0 = h->cap;
     if (compressor == GMC_TOPK) h->n_sample = (uint32_t)(h->sample_chunks ? kSampleSlots : d);
     h->sample_stride = std::max<uint32_t>(kSampleSlots, (h->n_sample + 3) & ~3u);
     // the approximate top-s sample: a run of 8 a thread, over about eight blocks
@@ -681,7 +717,6 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
     const int64_t share = (8 * (int64_t)h->num_sms + K - 1) / K;
     h->sample_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(share, ((int64_t)h->n_sample + 2047) / 2048));
     h->theta_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(share, ((int64_t)h->n_sample + 4095) / 4096));
-    const int64_t Kt = (int64_t)K * h->n_tiles;
     if ((err = dalloc(h, &h->e, (size_t)K * h->ld)) != cudaSuccess ||
         (err = dalloc(h, &h->w, (size_t)h->ld)) != cudaSuccess ||
         (err = dalloc(h, &h->dlt, (size_t)h->ld)) != cudaSuccess ||
@@ -690,25 +725,15 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
         (err = dalloc(h, &h->chist, (size_t)K * kRelBins)) != cudaSuccess ||
         (err = dalloc(h, &h->bucket, (size_t)K * 2 * kBucketCap)) != cudaSuccess ||
         (err = dalloc(h, &h->sample_keys, (size_t)K * h->sample_stride)) != cudaSuccess ||
-        (err = dalloc(h, &h->big_tiles, (size_t)h->n_tiles + 1)) != cudaSuccess ||
-        (err = dalloc(h, &h->rcount, (size_t)K * h->regions * kChunksPerTile)) != cudaSuccess ||
         (err = dalloc(h, &h->sample_pend, (size_t)3 * h->sample_stride)) != cudaSuccess)
       return fail(err);
-    if (h->tile != kBulkTile && (err = dalloc(h, &h->dlt_next, (size_t)h->ld)) != cudaSuccess) return fail(err);
+    if (!bulk && (err = dalloc(h, &h->dlt_next, (size_t)h->ld)) != cudaSuccess) return fail(err);
     if (h->grid_small && (err = dalloc(h, &h->small_scratch, small_scratch_words(K))) != cudaSuccess) return fail(err);
-    if (h->n_blk >= 8 && ((err = dalloc(h, &h->blk_cost, (size_t)h->n_blk)) != cudaSuccess ||
-                          (err = dalloc(h, &h->blk_order, (size_t)h->n_blk)) != cudaSuccess))
-      return fail(err);
+    if ((err = lay_out(h, bulk)) != cudaSuccess) return fail(err);
     if ((err = cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking)) != cudaSuccess ||
         (err = cudaEventCreateWithFlags(&h->ev_step, cudaEventDisableTiming)) != cudaSuccess ||
         (err = cudaEventCreateWithFlags(&h->ev_flush, cudaEventDisableTiming)) != cudaSuccess)
       return fail(err);
-    for (int p = 0; p < 2; ++p) {
-      if ((err = dalloc(h, &h->cand_idx[p], (size_t)K * h->cap)) != cudaSuccess ||
-          (err = dalloc(h, &h->cand_val[p], (size_t)K * h->cap)) != cudaSuccess ||
-          (err = dalloc(h, &h->chunk[p], (size_t)Kt * kChunksPerTile)) != cudaSuccess)
-        return fail(err);
-    }
   } else {
     h->tile = kRbgsTile;
     h->n_tiles = (d + h->tile - 1) / h->tile;
@@ -1173,8 +1198,9 @@ int gmc_check(gmc_t h) {
 
 int gmc_test_withhold_copy(gmc_t h, int64_t tile, int32_t k, uint64_t wait_limit_ns) {
   if (!h || k < 0 || k >= h->K || wait_limit_ns == 0 || wait_limit_ns > kWaitLimitNs) return GMC_EINVAL;
-  const bool bulk = h->compressor == GMC_RBGS ? h->rbgs_bulk : h->tile == kBulkTile;
-  if (!bulk || tile < 0 || tile >= h->n_tiles) return GMC_EINVAL;
+  const bool bulk = h->compressor == GMC_RBGS ? h->rbgs_bulk : h->bulk_able;
+  if (!bulk || tile < 0 || tile >= (h->d + kBulkTile - 1) / kBulkTile) return GMC_EINVAL;
+  static_assert(kBulkTile == kRbgsTile, "one bound for both passes' tiles");
   h->hold_tile = tile;
   h->hold_k = k;
   h->hold_wait_ns = wait_limit_ns;

@@ -79,7 +79,6 @@ struct TopkArgs {
   uint32_t* chist;           // K x kRelBins: the candidates' relative histogram (zeroed by the sample)
   uint32_t* bucket;          // K x 2*kBucketCap: keys, then indices of the k-th key's bin
   uint32_t* sample_keys;     // K x sample_stride
-  uint32_t* big_tiles;       // [0]: count, then tile ids left to the block aggregate
   uint32_t* cand_idx;        // current chunks: K x cap
   float* cand_val;
   uint2* chunk;              // sub-chunk (base, count): n_tiles x kChunksPerTile x K, see chunk_at

@@ -299,10 +299,7 @@ __global__ void __cluster_dims__(scl::kCtas, 1, 1) __launch_bounds__(scl::kThrea
   const unsigned crank = cl.block_rank();
   WorkerSel& S = A.sel[k];
   if (crank == 0 && k == 0) {  // the step's first kernel that counts: its counters start at zero
-    if (threadIdx.x == 0) {
-      A.big_tiles[0] = 0;
-      *A.tile_ctr = 0u;  // and the bulk pass claims its tiles from zero
-    }
+    if (threadIdx.x == 0) *A.tile_ctr = 0u;  // and the bulk pass claims its tiles from zero
     if (threadIdx.x < 8) A.step_ctr->v[threadIdx.x] = 0ull;
   }
   if (crank == 0)  // this step's candidate histogram starts empty
@@ -445,10 +442,7 @@ __global__ void __launch_bounds__(kThreads) k_sample(TopkArgs A) {
   griddep_wait();
   __shared__ uint32_t hist[kHistBins];
   const int k = blockIdx.y;
-  if (blockIdx.x == 0 && k == 0 && threadIdx.x == 0) {
-    A.big_tiles[0] = 0;
-    *A.tile_ctr = 0u;  // the bulk pass claims its tiles from zero
-  }
+  if (blockIdx.x == 0 && k == 0 && threadIdx.x == 0) *A.tile_ctr = 0u;  // the bulk pass claims its tiles from zero
   if (blockIdx.x == 0)  // this step's candidate histogram starts empty
     for (int b = threadIdx.x; b < kRelBins; b += blockDim.x) A.chist[(int64_t)k * kRelBins + b] = 0u;
   const float* ek = A.e + (int64_t)k * A.ld;

@@ -1,0 +1,54 @@
+"""The bulk top-k pass (2 to 16 workers, d >= 8 * 4096 * SMs: about 5 M) under the
+tests that other files run at smaller sizes, where other passes take the step;
+and single workers, which take the load/store pass at every size."""
+import pytest
+
+import test_gpu_approx
+import test_gpu_bf16
+import test_gpu_checkpoint
+import test_gpu_deferred
+import test_gpu_variants
+
+pytestmark = pytest.mark.gpu
+
+D = 5_100_001
+
+
+@pytest.mark.parametrize("name", ["test_deferred_steps_in_a_row_with_eta_schedule",
+                                  "test_state_read_on_another_stream_between_deferred_steps",
+                                  "test_deferred_steps_mixed_with_host_steps_and_detach",
+                                  "test_dense_sub_tiles_and_ties_on_the_bulk_pass",
+                                  "test_bulk_pass_reports_non_finite_values"])
+def test_deferral(name, monkeypatch):
+    monkeypatch.setattr(test_gpu_deferred, "D_BULK", D)
+    getattr(test_gpu_deferred, name)()
+
+
+@pytest.mark.parametrize("variant,compressor,K", [
+    ("server_momentum", "topk", 3), ("lr_in_residual", "topk_approx", 2), ("local_momentum", "topk", 7),
+    ("local_momentum_mfm", "topk_approx", 2), ("local_momentum", "topk", 1)])
+def test_variants(variant, compressor, K):
+    test_gpu_variants.test_variant_parity(variant, compressor, D, K)
+
+
+@pytest.mark.parametrize("K", [8, 3, 1])
+def test_approximate(K):
+    test_gpu_approx.test_approx_bulk_pass_deferred(D, K)
+
+
+@pytest.mark.parametrize("case", [
+    dict(compressor="topk", d=D, K=4, ratio=0.002), dict(compressor="topk", d=D, K=6, ratio=0.002),
+    dict(compressor="topk", d=D, K=3, ratio=0.002, offset=1), dict(compressor="topk", d=D, K=1, ratio=0.002),
+    dict(compressor="topk_approx", d=D, K=2, ratio=1 / 1024),
+    dict(compressor="topk", d=D, K=3, ratio=0.002, variant="local_momentum")], ids=str)
+def test_bf16(case):
+    test_gpu_bf16.test_bf16_step_parity(case)
+
+
+@pytest.mark.parametrize("case", [
+    dict(compressor="topk", d=D, K=4, ratio=0.002), dict(compressor="topk", d=D, K=6, ratio=0.002),
+    dict(compressor="topk", d=2_500_001, K=4, ratio=0.002),  # load/store pass
+    dict(compressor="topk_approx", d=D, K=2, ratio=1 / 1024),
+    dict(compressor="topk", d=D, K=2, ratio=0.002, variant="local_momentum")], ids=str)
+def test_checkpoint(case):
+    test_gpu_checkpoint.test_resume_continues_the_trajectory(case)

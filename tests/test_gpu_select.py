@@ -12,19 +12,32 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d,K,ratio,width", [
-    (1_300_001, 3, 0.02, 1e-3),    # bulk pass: 26,000 sent within 0.1% (the deep pipeline)
-    (1_300_001, 6, 0.02, 1e-2),    # and the one-tile pipeline
-    (1_300_001, 2, 0.02, 3e-5),    # narrower than the sampled threshold's own step of 2^10 keys
-    (1_300_001, 20, 0.012, 1e-3),  # more workers
-    (400_003, 20, 0.05, 1e-3),     # load/store pass
+    (5_100_001, 3, 0.01, 1e-3),    # bulk pass: 51,000 sent within 0.1% (the deep pipeline)
+    (5_100_001, 6, 0.005, 1e-2),   # and the one-tile pipeline
+    (5_100_001, 2, 0.005, 3e-5),   # narrower than the sampled threshold's own step of 2^10 keys
+    (1_300_001, 20, 0.012, 1e-3),  # load/store pass
+    (400_003, 20, 0.05, 1e-3),
 ])
 def test_crowded_candidates_stay_on_the_fast_path(d, K, ratio, width):
     rng = np.random.default_rng(d + K)
     p = Pair(d, K, 0.9, 0.05, ratio=ratio, seed=3)
     for t in range(3):
         g = (rng.standard_normal((K, d)) * 0.05).astype(np.float32)
-        crowd = rng.random((K, d)) < 1.5 * ratio  # more values in the band than are sent
+        crowd = rng.random((K, d)) < 2.5 * ratio  # more values in the band than the sampled threshold lets through
         band = (1.0 + width * rng.random((K, d))) * np.where(rng.random((K, d)) < 0.5, -1.0, 1.0)
         g = np.where(crowd, band * (2.0 ** t), g).astype(np.float32)
         p.compare(p.step(g), workers=[0, K - 1])
+    assert p.compare_stats()["fallbacks"] == 0
+
+
+def test_candidates_of_one_layer_do_not_overflow_the_bulk_parts():
+    """A layer of 1/64 of the coordinates that holds every sent value: few tiles,
+    so few CTAs' parts take all the candidates."""
+    d, K = 5_100_001, 2
+    rng = np.random.default_rng(1)
+    p = Pair(d, K, 0.9, 0.05, ratio=0.01, seed=3)
+    for t in range(2):
+        g = (rng.standard_normal((K, d)) * 1e-3).astype(np.float32)
+        g[:, 2_000_000:2_080_000] *= 1e3
+        p.compare(p.step(g))
     assert p.compare_stats()["fallbacks"] == 0
