@@ -53,6 +53,7 @@ struct gmc_ctx {
   bool rbgs_bulk = false;
   bool bulk_able = false;             // top-k: large enough for the bulk pass (gmc_test_withhold_copy)
   int grid_small = 0;                 // the one-launch top-k step's grid, 0: not taken
+  bool small_cluster = false;         // as one thread-block cluster
   uint32_t* small_scratch = nullptr;
   // state
   int64_t t = 0;
@@ -495,7 +496,7 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     const DetachArgs D{h->w, h->e, h->ld, h->d, detach_b(h), h->detach_out, h->detach_ld, 0, h->K};
     const double bytes = ((A.local_mom ? 20.0 : 12.0) - (bf16 ? 2.0 : 0.0)) * Kd + (D.out ? 4.0 * Kd : 0.0);
     GMC_TRY(timed(h, GMC_KERNEL_ACCUMULATE, bytes, s,
-                  [&] { return launch_topk_step(A, D, h->grid_small, h->small_scratch, s); }));
+                  [&] { return launch_topk_step(A, D, h->grid_small, h->small_cluster, h->small_scratch, s); }));
     finalized = true;
   } else if (h->compressor != GMC_RBGS) {
     const bool approx = h->compressor == GMC_TOPK_APPROX;
@@ -674,7 +675,7 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
     // memory takes the one-launch step
     h->bulk_able = K <= kBulkMaxK && d >= 4096 * streams_wide;
     const bool bulk = h->bulk_able && K > 1 && d >= (int64_t)kBulkTilesPerSm * kBulkTile * h->num_sms;
-    h->grid_small = bulk ? 0 : small_grid(d, K, h->num_sms);
+    h->grid_small = bulk ? 0 : small_grid(d, K, h->num_sms, &h->small_cluster);
     const int64_t whole = h->bulk_able ? kBulkTile : (d < 2048 * streams_wide ? 1024 : 2048);
     h->ld = (d + whole - 1) / whole * whole;
     const int64_t ks = std::max<int64_t>(1, (int64_t)std::floor(ratio * (double)d));

@@ -233,10 +233,11 @@ constexpr int kSmallItems = 376;
 __host__ __device__ constexpr int kItemMaxBytes(int groups, int grid, int K) {
   return (groups + grid - 1) / grid * K * 512;
 }
-int small_grid(int64_t d, int K, int num_sms);  // its grid, 0 when the problem does not fit
+int small_grid(int64_t d, int K, int num_sms, bool* cluster);  // its grid, 0 when the problem does not fit
 size_t small_scratch_words(int K);
 cudaError_t configure_small_kernels();
-cudaError_t launch_topk_step(const TopkArgs& A, const DetachArgs& D, int grid, uint32_t* scratch, cudaStream_t s);
+cudaError_t launch_topk_step(const TopkArgs& A, const DetachArgs& D, int grid, bool cluster, uint32_t* scratch,
+                             cudaStream_t s);
 
 constexpr int kRbgsTile = 4096;  // elements per tile of the fused RBGS kernel
 

@@ -39,6 +39,8 @@ constexpr int kCoarse = kHistBins / 32;     // sums of 32 bins
 constexpr int kHistWords = kHistBins + kCoarse;
 constexpr uint32_t kDirect = 65536;         // keys of a bin that go straight to the global histogram
 constexpr int kIdxBits = 23;                // an index digit's range: d < 2^23
+constexpr int kClusterMax = 16;             // blocks of a cluster launch (above the portable 8)
+constexpr int kClusterItems = 1024;          // items up to which the step runs as one cluster
 constexpr int kMaxRounds = 16;
 static_assert(kItemMax * 512 + 8 * (kHistBins / 2) * 4 <= 232448 - 6 * 1024, "accumulators and eight histograms");
 
@@ -82,8 +84,14 @@ __device__ __forceinline__ bool sampled_block(const TopkArgs& A, uint64_t key, u
   return false;
 }
 
-template <bool kBf16>
+// kCluster: the grid is one thread-block cluster (co-scheduled by the hardware),
+// whose barrier takes the grid barrier's place (0.8 against 1.8 us) and whose
+// launch overlaps the end of the kernel before it, as a cooperative one does not:
+// steps of up to kClusterItems items (d = 10,000, K = 3: 18.8 -> 14.2 us a step;
+// d = 32,768, K = 4, the largest: 20.8 -> 19.4).
+template <bool kBf16, bool kCluster>
 __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachArgs D, Scratch* S, int hist_k) {
+  if (kCluster) griddep_wait();
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Search sr[kMaxK];
   __shared__ uint32_t cnt[kItemMax];            // per item: sent elements, then its pairs' first slot
@@ -109,6 +117,12 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
     if ((int)threadIdx.x < K) A.sel[threadIdx.x].count = 0;
   }
   uint32_t buf = S->start;  // 0, 1 or 2
+  // every block's writes so far are seen by every block (false: a wait gave up)
+  auto barrier = [&]() -> bool {
+    if (!kCluster) return grid_barrier(&S->bar, &s_ok, A.wait_ns);
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return true;
+  };
 
   if (A.approx) {
     const uint64_t key = stream_key(A.seed, A.t, 0);
@@ -305,7 +319,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
         });
         flush(gh, k_lo, k_hi);
       }
-      ok = grid_barrier(&S->bar, &s_ok, A.wait_ns);
+      ok = barrier();
       if (threadIdx.x == 0) s_active = 0;
       __syncthreads();
       if (!ok) return;
@@ -424,7 +438,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
     }
     __syncthreads();
     if ((int)threadIdx.x < K && cnt[threadIdx.x]) atomicAdd(&S->reach[threadIdx.x], cnt[threadIdx.x]);
-    ok = grid_barrier(&S->bar, &s_ok, A.wait_ns);
+    ok = barrier();
     if (threadIdx.x == 0) s_active = 0;
     __syncthreads();
     if (ok) {
@@ -639,10 +653,17 @@ int small_hist_k(int64_t d, int K, int grid) {
 }  // namespace
 
 // The one-launch step takes the problem: its accumulators fit in `grid` blocks.
-// Returns the grid (0: it does not).
-int small_grid(int64_t d, int K, int num_sms) {
+// Returns the grid (0: it does not); *cluster: as one cluster.
+int small_grid(int64_t d, int K, int num_sms, bool* cluster) {
+  *cluster = false;
   if (d >= (int64_t(1) << kIdxBits)) return 0;
   const int64_t groups = (d + 127) / 128;
+  if (groups * K <= kClusterItems) {
+    int grid = 1;
+    while (grid < kClusterMax && grid < groups) grid *= 2;
+    *cluster = true;
+    return grid;
+  }
   const int grid = (int)std::min<int64_t>(groups, num_sms);
   const int64_t items = (groups + grid - 1) / grid * K;
   if (items > kItemMax) return 0;
@@ -652,25 +673,43 @@ size_t small_scratch_words(int K) {
   return sizeof(Scratch) / 4 + 3 * (size_t)K * kHistWords;
 }
 cudaError_t configure_small_kernels() {
-  const int most = kSmemMost;
-  const cudaError_t a = cudaFuncSetAttribute((const void*)k_topk_step<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  const cudaError_t b = cudaFuncSetAttribute((const void*)k_topk_step<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  return a != cudaSuccess ? a : b;
+  cudaError_t err = cudaSuccess;
+  auto set = [&](const void* f, cudaFuncAttribute a, int v) {
+    const cudaError_t e2 = cudaFuncSetAttribute(f, a, v);
+    if (err == cudaSuccess) err = e2;
+  };
+  set((const void*)k_topk_step<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMost);
+  set((const void*)k_topk_step<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMost);
+  for (const void* f : {(const void*)k_topk_step<false, true>, (const void*)k_topk_step<true, true>}) {
+    set(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMost);
+    set(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  }
+  return err;
 }
-cudaError_t launch_topk_step(const TopkArgs& A, const DetachArgs& D, int grid, uint32_t* scratch, cudaStream_t s) {
+cudaError_t launch_topk_step(const TopkArgs& A, const DetachArgs& D, int grid, bool cluster, uint32_t* scratch,
+                             cudaStream_t s) {
+  const int hist_k = small_hist_k(A.d, A.K, grid);  // at least 8: kSmallItems leaves them room
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kSmThreads);
-  const int hist_k = small_hist_k(A.d, A.K, grid);  // at least 8: kSmallItems leaves them room
   cfg.dynamicSmemBytes = (size_t)kItemMaxBytes((int)((A.d + 127) >> 7), grid, A.K) + hist_k * (kHistBins / 2) * 4;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
+  cfg.attrs = at;
+  Scratch* S = reinterpret_cast<Scratch*>(scratch);
+  if (cluster) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)grid;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, A.bf16 ? k_topk_step<true, true> : k_topk_step<false, true>, A, D, S, hist_k);
+  }
   at[0].id = cudaLaunchAttributeCooperative;  // its blocks meet at grid barriers
   at[0].val.cooperative = 1;
-  cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, A.bf16 ? k_topk_step<true> : k_topk_step<false>, A, D,
-                            reinterpret_cast<Scratch*>(scratch), hist_k);
+  return cudaLaunchKernelEx(&cfg, A.bf16 ? k_topk_step<true, false> : k_topk_step<false, false>, A, D, S, hist_k);
 }
 
 }  // namespace gmc

@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("compressor", ["topk", "topk_approx"])
 @pytest.mark.parametrize("d,K,ratio", [
     (1, 1, 1.0), (5, 2, 0.5), (127, 3, 0.1), (129, 32, 0.05), (1_000, 9, 1.0),
+    (128 * 17, 1, 0.02), (32_768, 4, 0.01), (32_769, 4, 0.01), (4_096, 32, 0.01),  # one cluster, up to its largest
     (128 * 152, 4, 0.01), (128 * 152 + 1, 5, 0.001), (210_001, 32, 0.01), (900_007, 8, 0.002),
     (1_200_003, 1, 0.3), (1_244_159, 6, 0.001),   # the largest slices
 ])
