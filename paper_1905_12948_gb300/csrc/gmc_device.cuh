@@ -48,15 +48,19 @@ struct Counters {
 };
 enum CounterSlot { kSteps = 0, kPairs = 1, kNnz = 2, kUnion = 3, kChanged = 4,
                    kFallbacks = 5, kNonfinite = 6 };
-// The end of a step (one thread, after every kernel of the step that counts):
-// the pairs counted on the host, the step mark, and the step into the totals.
-// The step's counts may come from other blocks of the calling kernel: they
-// are read from L2.
+// The end of a step (a whole warp, after every kernel of the step that counts):
+// the pairs counted on the host, the step mark, and the step into the totals, a
+// lane per counter. The step's counts may come from other blocks of the calling
+// kernel: they are read from L2.
 __device__ __forceinline__ void finalize_counters(Counters* step, Counters* total,
                                                   unsigned long long pairs_add) {
-  step->v[kPairs] = __ldcg(&step->v[kPairs]) + pairs_add;
-  step->v[kSteps] = 1;
-  for (int i = 0; i < 8; ++i) total->v[i] += __ldcg(&step->v[i]);
+  const int i = (int)(threadIdx.x & 31);
+  if (i >= 8) return;
+  unsigned long long x = __ldcg(&step->v[i]);
+  if (i == kPairs) x += pairs_add;
+  if (i == kSteps) x = 1;
+  if (i == kPairs || i == kSteps) step->v[i] = x;
+  total->v[i] += x;
 }
 
 // Device status bits (gmc_check).

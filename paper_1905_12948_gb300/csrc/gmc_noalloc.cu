@@ -12,7 +12,8 @@
 //            the sampled keys give an interval of keys [L, U] that holds the
 //            k-th largest key T but for about 1e-9 of inputs
 //   collect  one pass over x: keys above U counted per chunk, keys inside listed
-//            (key, index); T is the (k - above)-th largest of the list
+//            (key, index) and counted into a histogram over the interval; T is
+//            the (k - above)-th largest of the list, found in its bin
 //   write    a second pass, over the groups of 128 values that hold a key of the
 //            interval or above it: the k pairs in index order, each chunk's
 //            first position from the counts and the list
@@ -44,6 +45,7 @@ constexpr int kNaStage = 2048;   // listed keys a block stages before it reserve
 constexpr int kNaRounds = 16;    // passes at most: a collect, then three histograms and a collect, with slack
 constexpr int kNaUnroll = 4;     // groups of 128 values a warp loads together
 constexpr int kNaQuads = 2;      // quads a thread samples
+constexpr int kNaFew = 512;      // keys of T's histogram bin up to which each is compared with all
 constexpr int kNaBatch = 8;      // listed keys a thread loads together
 static_assert(kNaChunks * 2 <= kNaCap * 4, "the chunk counts fit in the keys' shared memory");
 static_assert(kNaOwn == kNaThreads, "one thread per own chunk");
@@ -255,13 +257,22 @@ __global__ void __launch_bounds__(kNaThreads, 1)
   bool listed = false, found = false;
   uint32_t above = 0, in_list = 0;  // keys above the interval; keys listed
   bool know_above = false;          // `above` is that of [L, U]
-  int hist_round = 0;
+  int hist_round = 0, sh = 0;       // histograms so far; log2 of the last one's bin width in keys
   for (int round = 0; ok && !found && round < kNaRounds; ++round) {
     uint32_t gt = 0, eq = 0;  // this warp's keys above and inside (collect: lane 0, per chunk in gc / ec)
     if (!hist_next) {
       // collect: count above, list inside (or count, when the interval is one key)
       const bool one = L == U;
       uint32_t gc = 0, ec = 0, units = 0;
+      // the listed keys' histogram over the interval, for ranking them
+      sh = 0;
+      while (((uint32_t)(U - L) >> sh) >= (uint32_t)kHistBins) ++sh;
+      uint32_t* gh = S->hist[2 + hist_round % 3];
+      uint32_t* gz = S->hist[2 + (hist_round + 1) % 3];  // last read two histograms ago
+      if (hist_round > 0)
+        for (int b = me * kNaThreads + threadIdx.x; b < kHistBins; b += G * kNaThreads) gz[b] = 0;
+      ++hist_round;
+      clear_hist();
       if (threadIdx.x == 0) s_n = 0;
       C.each(
           X, lane,
@@ -301,6 +312,7 @@ __global__ void __launch_bounds__(kNaThreads, 1)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               if (!((in >> i) & 1u)) continue;
+              if (at < (uint32_t)kNaCap) atomicAdd(&h[(uint32_t)(key[i] - L) >> sh], 1u);  // (past it the list is not used)
               const uint2 p = make_uint2((uint32_t)key[i], (uint32_t)(e + i - X.off));
               if (at < (uint32_t)kNaStage) {
                 stage[at] = p;
@@ -341,7 +353,7 @@ __global__ void __launch_bounds__(kNaThreads, 1)
             S->list.idx[s_base + i] = stage[i].y;
           }
         }
-      ok = grid_barrier(&S->bar, &s_ok, kWaitLimitNs);
+      ok = share_hist(gh);
       know_above = true;
       const uint32_t a_all = block_total(threadIdx.x < G ? __ldcg(&S->above[threadIdx.x]) : 0u);
       const uint32_t q_all = block_total(threadIdx.x < G ? __ldcg(&S->equal[threadIdx.x]) : 0u);
@@ -371,8 +383,8 @@ __global__ void __launch_bounds__(kNaThreads, 1)
     // histogram of the keys of [L, U] in bins of 2^sh keys (the first, on the
     // sampled interval, also counts the keys above it)
     uint32_t* gh = S->hist[2 + hist_round % 3];
-    uint32_t* gz = S->hist[2 + (hist_round + 1) % 3];  // last read two histogram passes ago
-    int sh = 0;
+    uint32_t* gz = S->hist[2 + (hist_round + 1) % 3];  // last read two histograms ago
+    sh = 0;
     while (((uint32_t)(U - L) >> sh) >= (uint32_t)kHistBins) ++sh;
     clear_hist();
     C.each(
@@ -432,55 +444,95 @@ __global__ void __launch_bounds__(kNaThreads, 1)
     // ---- T from the list ----
     for (int o = threadIdx.x; o < kNaOwn; o += kNaThreads) base_gt[o] = base_eq[o] = 0;
     if (listed) {
-      // (kNaBatch loads in flight a thread, here and below)
-      for (uint32_t i0 = threadIdx.x; i0 < in_list; i0 += kNaBatch * kNaThreads) {
-        uint32_t key[kNaBatch];
+      // h: the listed keys' histogram. The bin that holds T, and T's rank there
+      block_find2_from_top(h, kHistBins, k - above, k - above, ws, find);
+      const uint32_t bin = find[0], rank = find[1], in_bin = h[bin];
+      const bool few = in_bin <= (uint32_t)kNaFew;
+      if (threadIdx.x == 0) s_n = 0;
+      if (!few) {
+        // too many to compare with each other: all the listed keys ranked by radix digits
+        for (uint32_t i0 = threadIdx.x; i0 < in_list; i0 += kNaBatch * kNaThreads) {
+          uint32_t key[kNaBatch];
 #pragma unroll
-        for (int q = 0; q < kNaBatch; ++q) {
-          const uint32_t i = i0 + q * kNaThreads;
-          key[q] = i < in_list ? __ldcg(&S->list.key[i]) : 0u;
+          for (int q = 0; q < kNaBatch; ++q) {
+            const uint32_t i = i0 + q * kNaThreads;
+            key[q] = i < in_list ? __ldcg(&S->list.key[i]) : 0u;
+          }
+#pragma unroll
+          for (int q = 0; q < kNaBatch; ++q)
+            if (i0 + q * kNaThreads < in_list) na_keys[i0 + q * kNaThreads] = key[q];
         }
-#pragma unroll
-        for (int q = 0; q < kNaBatch; ++q)
-          if (i0 + q * kNaThreads < in_list) na_keys[i0 + q * kNaThreads] = key[q];
+        int bits = 0;
+        while (bits < 31 && ((uint32_t)(U - L) >> bits) != 0) ++bits;
+        __syncthreads();
+        T = (int32_t)smem_select_bits(na_keys, in_list, k - above, bits, (uint32_t)L, h, ws, &s_bin, &s_rank, &n_tie);
       }
-      int bits = 0;
-      while (bits < 31 && ((uint32_t)(U - L) >> bits) != 0) ++bits;
       __syncthreads();
-      T = (int32_t)smem_select_bits(na_keys, in_list, k - above, bits, (uint32_t)L, h, ws, &s_bin, &s_rank, &n_tie);
-      __syncthreads();
-      // the listed keys that are sent, at the first own chunk after theirs
+      // one pass over the list: the keys known to be sent counted at the first own
+      // chunk after theirs; those of T's bin set aside (kNaBatch loads in flight a thread)
       // (x / G as a product: exact, x < 2^15 and G <= 2^10)
       const uint32_t inv_G = (uint32_t)((0x100000000ull + G - 1) / G);
       const int cg_sh = 31 - __clz(C.cg);
+      auto own_after = [&](uint32_t idx) {
+        const uint32_t c = (idx + X.off) >> (7 + cg_sh);
+        const int j = c < me ? 0 : (G > 1 ? (int)__umulhi(c - me, inv_G) : (int)(c - me)) + 1;
+        return j < C.n_own ? j : -1;
+      };
       for (uint32_t i0 = threadIdx.x & ~31u; i0 < in_list; i0 += kNaBatch * kNaThreads) {
-        int32_t key[kNaBatch];
-        uint32_t idx[kNaBatch];
+        uint32_t key[kNaBatch], idx[kNaBatch];
 #pragma unroll
         for (int q = 0; q < kNaBatch; ++q) {
           const uint32_t i = i0 + lane + q * kNaThreads;
-          key[q] = i < in_list ? (int32_t)na_keys[i] : -1;
-          idx[q] = key[q] >= T ? __ldcg(&S->list.idx[i]) : 0u;
+          key[q] = i < in_list ? __ldcg(&S->list.key[i]) : 0u;
+          idx[q] = i < in_list ? __ldcg(&S->list.idx[i]) : 0u;
         }
 #pragma unroll
         for (int q = 0; q < kNaBatch; ++q) {
           if (i0 + q * kNaThreads >= in_list) break;  // (uniform over the warp)
-          int j = -1;
-          if (key[q] >= T) {
-            const uint32_t c = (idx[q] + X.off) >> (7 + cg_sh);
-            j = c < me ? 0 : (G > 1 ? (int)__umulhi(c - me, inv_G) : (int)(c - me)) + 1;
-            if (j >= C.n_own) j = -1;
-          }
-          const bool up = key[q] > T;
+          const bool in = i0 + lane + q * kNaThreads < in_list;
+          const uint32_t b = in ? (key[q] - (uint32_t)L) >> sh : 0u;
+          const bool up = in && (few ? b > bin : (int32_t)key[q] > T);
+          const bool aside = in && (few ? b == bin : (int32_t)key[q] == T);
+          const int j = up ? own_after(idx[q]) : -1;
           // (most of a warp's keys often fall before one chunk: added at once)
-          const uint32_t any = __ballot_sync(0xffffffffu, j >= 0 && up);
+          const uint32_t any = __ballot_sync(0xffffffffu, j >= 0);
           if (any) {
             const int lead = __ffs(any) - 1, j0 = __shfl_sync(0xffffffffu, j, lead);
-            const uint32_t same = __ballot_sync(0xffffffffu, up && j == j0);
+            const uint32_t same = __ballot_sync(0xffffffffu, j == j0);
             if (lane == lead) atomicAdd(&base_gt[j0], (uint32_t)__popc(same));
-            else if (up && j >= 0 && j != j0) atomicAdd(&base_gt[j], 1u);
+            else if (j >= 0 && j != j0) atomicAdd(&base_gt[j], 1u);
           }
-          if (j >= 0 && !up) atomicAdd(&base_eq[j], 1u);
+          if (aside) {
+            if (few) {
+              stage[atomicAdd(&s_n, 1u)] = make_uint2(key[q], idx[q]);
+            } else {
+              const int t = own_after(idx[q]);
+              if (t >= 0) atomicAdd(&base_eq[t], 1u);
+            }
+          }
+        }
+      }
+      __syncthreads();
+      if (few) {  // T among its bin's few keys, each compared with all
+        uint2 mine = make_uint2(0u, 0u);
+        if (threadIdx.x < in_bin) {
+          mine = stage[threadIdx.x];
+          uint32_t gt = 0, eq = 0;
+          for (uint32_t i = 0; i < in_bin; ++i) {
+            gt += stage[i].x > mine.x ? 1u : 0u;
+            eq += stage[i].x == mine.x ? 1u : 0u;
+          }
+          if (gt < rank && rank <= gt + eq) {  // (every key equal to T writes the same)
+            s_bin = mine.x;
+            s_rank = rank - gt;
+          }
+        }
+        __syncthreads();
+        T = (int32_t)s_bin;
+        n_tie = s_rank;
+        if (threadIdx.x < in_bin && (int32_t)mine.x >= T) {
+          const int t = own_after(mine.y);
+          if (t >= 0) atomicAdd((int32_t)mine.x > T ? &base_gt[t] : &base_eq[t], 1u);
         }
       }
     }

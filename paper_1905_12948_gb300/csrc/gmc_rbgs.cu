@@ -153,12 +153,12 @@ __device__ __forceinline__ void end_step(const RbgsArgs& A, unsigned long long* 
   if (lane == 0) {
     __threadfence();
     last = atomicAdd(A.tile_ctr + 1, 1u) == gridDim.x - 1 ? 1u : 0u;
-    if (last) {
-      __threadfence();
-      finalize_counters(A.step_ctr, A.total_ctr, 0ull);
-    }
   }
   last = __shfl_sync(0xffffffffu, last, 0);
+  if (last) {
+    __threadfence();
+    finalize_counters(A.step_ctr, A.total_ctr, 0ull);
+  }
   if (last && A.clear_flags)
     for (int64_t b = lane * 4; b < A.nb; b += 128)  // allocated in whole words
       *reinterpret_cast<uint32_t*>(A.uflag_prev + b) = 0u;
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kThreads) k_copy_row(const float* __restrict__
 
 __global__ void k_finalize(Counters* step, Counters* total, unsigned long long pairs_add) {
   griddep_wait();
-  if (threadIdx.x == 0) finalize_counters(step, total, pairs_add);
+  finalize_counters(step, total, pairs_add);  // one warp
 }
 
 

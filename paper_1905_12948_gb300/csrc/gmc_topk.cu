@@ -1896,9 +1896,9 @@ __global__ void __launch_bounds__(1024) k_select_dense(TopkArgs A) {
     s_last = atomicAdd(&A.sel[0].done[3], 1u) == gridDim.x - 1 ? 1u : 0u;
   }
   __syncthreads();
-  if (s_last && threadIdx.x == 0) {
+  if (s_last && threadIdx.x < 32) {
     __threadfence();
-    A.sel[0].done[3] = 0;
+    if (threadIdx.x == 0) A.sel[0].done[3] = 0;
     finalize_counters(A.step_ctr, A.total_ctr, A.pairs_add);
   }
 }
@@ -2049,11 +2049,12 @@ __global__ void __launch_bounds__(kThreads) k_apply(TopkArgs A) {
   if (threadIdx.x == 0) {
     __threadfence();
     s_last = atomicAdd(&A.sel[0].done[3], 1u) == gridDim.x - 1 ? 1u : 0u;
-    if (s_last) {
-      __threadfence();
-      A.sel[0].done[3] = 0;
-      finalize_counters(A.step_ctr, A.total_ctr, A.pairs_add);
-    }
+  }
+  __syncthreads();
+  if (s_last && threadIdx.x < 32) {
+    __threadfence();
+    if (threadIdx.x == 0) A.sel[0].done[3] = 0;
+    finalize_counters(A.step_ctr, A.total_ctr, A.pairs_add);
   }
 }
 
