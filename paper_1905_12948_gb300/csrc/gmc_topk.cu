@@ -580,10 +580,10 @@ __global__ void __launch_bounds__(kThreads) k_sample_theta(TopkArgs A) {
 // tile; for each worker it writes v over e and appends its candidates as one
 // index-sorted sub-chunk, reserved at once -- warps never wait for each other.
 // ---------------------------------------------------------------------------
-// A restored state (gmc_load_state): w_t - w_{t-1} is in dlt over the whole
-// range, with no pair lists of the step before. Read it densely for one warp's
-// sub-tile [sub0, sub0 + n) (n a multiple of 4, sub0 16-byte aligned, inside
-// ld) and clear it, as the listed path does.
+// w_t - w_{t-1} of one warp's sub-tile [sub0, sub0 + n) (n a multiple of 4, sub0
+// 16-byte aligned, inside ld) read densely from dlt and cleared: a restored
+// state (gmc_load_state), which has no pair lists of the step before, and a
+// sub-tile with more pairs than one round takes.
 __device__ __forceinline__ void stage_delta_dense(const TopkArgs& A, uint32_t sub0, int n, float* dlw,
                                                   int lane) {
   for (int i = lane; i < n / 4; i += 32) {
@@ -596,61 +596,19 @@ __device__ __forceinline__ void stage_delta_dense(const TopkArgs& A, uint32_t su
   __syncwarp();
 }
 
-// w_t - w_{t-1} on one warp's sub-tile [sub0, sub0 + n) into dlw: non-zero only
-// where the previous step sent pairs, listed by its sub-chunks (k', tile, w).
-__device__ __forceinline__ void stage_delta_warp(const TopkArgs& A, int64_t tile, int w,
-                                                 uint32_t sub0, int n, float* dlw, int lane) {
-  if (A.dense_prev) {
-    stage_delta_dense(A, sub0, n, dlw, lane);
-    return;
-  }
-  for (int i = lane; i < n / 4; i += 32)
-    reinterpret_cast<float4*>(dlw)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  __syncwarp();
-  if (A.has_prev) {
-    for (int k0 = 0; k0 < A.K; k0 += 32) {
-      const int kk = k0 + lane;
-      uint32_t base = 0, cnt = 0;
-      if (kk < A.K) {
-        const uint2 bc = A.chunk_prev[chunk_at(A, kk, tile, w)];
-        base = bc.x;
-        cnt = bc.y;
-      }
-      uint32_t total;
-      const uint32_t pre = warp_excl_scan(cnt, &total);
-      for (uint32_t e0 = 0; e0 < total; e0 += 32) {
-        const uint32_t e = e0 + lane;
-        int src = 0;  // the last lane whose non-empty sub-chunk starts at or before e
-#pragma unroll 1
-        for (int l = 1; l < 32; ++l) {
-          const uint32_t pl = __shfl_sync(0xffffffffu, pre, l);
-          const uint32_t cl = __shfl_sync(0xffffffffu, cnt, l);
-          if (cl && pl <= e) src = l;
-        }
-        const uint32_t b = __shfl_sync(0xffffffffu, base, src);
-        const uint32_t p = __shfl_sync(0xffffffffu, pre, src);
-        if (e < total) {
-          const uint32_t at = b + (e - p);
-          if (at < A.cap) {
-            const int64_t q = (int64_t)(k0 + src) * A.cap + at;
-            const uint32_t j = A.cand_idx_prev[q];
-            const WorkerSel& Sp = A.sel[k0 + src];  // the previous step's selection
-            if (selected(mag_key(A.cand_val_prev[q]), j, Sp.T, Sp.t_idx)) {
-              const int64_t l = (int64_t)j - sub0;
-              if (l >= 0 && l < n) dlw[l] = A.dlt[j];
-              else atomicOr(A.status, kStatusInternal);
-            }
-          }
-        }
-      }
+// The position in a list of up to 32 runs (lane l's of length cnt, incl: their
+// inclusive sums): the run that holds element e (the first lane whose sum exceeds it).
+__device__ __forceinline__ int run_of(uint32_t incl, uint32_t e) {
+  int lo = 0, hi = 32;
+#pragma unroll
+  for (int it = 0; it < 6; ++it) {
+    const int mid = min((lo + hi) >> 1, 31);
+    const uint32_t v = __shfl_sync(0xffffffffu, incl, mid);
+    if (lo < hi) {
+      if (v <= e) lo = mid + 1; else hi = mid;
     }
-    __syncwarp();
-    // w_t - w_{t-1} has been read for this sub-tile; clear it here (this step's
-    // aggregate writes w_{t+1} - w_t)
-    for (int l = lane; l < n; l += 32)
-      if (dlw[l] != 0.f) A.dlt[sub0 + l] = 0.f;
   }
-  __syncwarp();
+  return lo < 32 ? lo : 31;
 }
 
 // The previous step's aggregation (Alg. 1: w_{t+1} = w_t - (eta/K) sum_k C_k(.),
@@ -669,48 +627,43 @@ __device__ __forceinline__ void stage_pending_warp(const TopkArgs& A, int64_t ti
   }
   __syncwarp();
   const uint32_t lt = lanemask_lt();
-  for (int k0 = 0; k0 < A.K; k0 += 32) {
-    const int kk = k0 + lane;
-    uint32_t base = 0, cnt = 0;
-    if (kk < A.K) {
-      const uint2 bc = A.chunk_prev[chunk_at(A, kk, tile, w)];
-      base = bc.x;
-      cnt = bc.y;
-    }
-    uint32_t total;
-    const uint32_t pre = warp_excl_scan(cnt, &total);
-    // entries run through the workers in ascending order, 32 per round
-    for (uint32_t e0 = 0; e0 < total; e0 += 32) {
-      const uint32_t e = e0 + lane;
-      int src = 0;
-#pragma unroll 1
-      for (int l = 1; l < 32; ++l) {
-        const uint32_t pl = __shfl_sync(0xffffffffu, pre, l);
-        const uint32_t cl = __shfl_sync(0xffffffffu, cnt, l);
-        if (cl && pl <= e) src = l;
+  const uint2 bc = lane < A.K ? A.chunk_prev[chunk_at(A, lane, tile, w)] : make_uint2(0u, 0u);
+  uint32_t total;
+  const uint32_t pre = warp_excl_scan(bc.y, &total);
+  // pairs run through the workers in ascending order, 32 per round, the rounds'
+  // loads kAhead at a time
+  constexpr int kAhead = 2;
+  for (uint32_t e0 = 0; e0 < total; e0 += kAhead * 32) {
+    int kq[kAhead];
+    uint32_t jq[kAhead];
+    float vq[kAhead];
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) {
+      const uint32_t e = e0 + q * 32 + lane;
+      kq[q] = run_of(pre + bc.y, e < total ? e : total - 1);
+      const uint32_t at = __shfl_sync(0xffffffffu, bc.x, kq[q]) + (e - __shfl_sync(0xffffffffu, pre, kq[q]));
+      jq[q] = kNone;
+      vq[q] = 0.f;
+      if (e < total && at < A.cap) {
+        const int64_t i = (int64_t)kq[q] * A.cap + at;
+        jq[q] = A.cand_idx_prev[i];
+        vq[q] = A.cand_val_prev[i];
       }
-      const uint32_t b = __shfl_sync(0xffffffffu, base, src);
-      const uint32_t p = __shfl_sync(0xffffffffu, pre, src);
+    }
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) {
       bool act = false;
       uint32_t l = 0;
-      float v = 0.f;
-      if (e < total) {
-        const uint32_t at = b + (e - p);
-        if (at < A.cap) {
-          const int64_t q = (int64_t)(k0 + src) * A.cap + at;
-          const uint32_t j = A.cand_idx_prev[q];
-          const float vq = A.cand_val_prev[q];
-          const WorkerSel& Sp = A.sel[k0 + src];  // the previous step's selection
-          if (selected(mag_key(vq), j, Sp.T, Sp.t_idx)) {
-            const int64_t ll = (int64_t)j - sub0;
-            if (ll >= 0 && ll < n) {
-              act = true;
-              l = (uint32_t)ll;
-              v = vq;
-              atomicOr(&mkw[l], 1u << (k0 + src));
-            } else {
-              atomicOr(A.status, kStatusInternal);
-            }
+      if (jq[q] != kNone) {
+        const WorkerSel& Sp = A.sel[kq[q]];  // the previous step's selection
+        if (selected(mag_key(vq[q]), jq[q], Sp.T, Sp.t_idx)) {
+          const int64_t ll = (int64_t)jq[q] - sub0;
+          if (ll >= 0 && ll < n) {
+            act = true;
+            l = (uint32_t)ll;
+            atomicOr(&mkw[l], 1u << kq[q]);
+          } else {
+            atomicOr(A.status, kStatusInternal);
           }
         }
       }
@@ -719,7 +672,7 @@ __device__ __forceinline__ void stage_pending_warp(const TopkArgs& A, int64_t ti
       const uint32_t r = __popc(peers & lt);
       const uint32_t rmax = __reduce_max_sync(0xffffffffu, act ? r : 0u);
       for (uint32_t turn = 0; turn <= rmax; ++turn) {
-        if (act && r == turn) dlw[l] = __fadd_rn(dlw[l], v);
+        if (act && r == turn) dlw[l] = __fadd_rn(dlw[l], vq[q]);
         __syncwarp();
       }
     }
@@ -934,7 +887,7 @@ __global__ void __launch_bounds__(kThreads) k_accumulate(TopkArgs A) {
 // entries of tile n+3. With more workers a tile lasts long enough for the
 // whole chain of tile n+1: its entries at the start of tile n, its pairs
 // after the warp's first item, w after its second. A sub-tile with more than
-// 32 pairs takes the direct path (stage_pending_warp / stage_delta_warp).
+// 32 pairs takes the direct path (stage_pending_warp / stage_delta_dense).
 //
 // A CTA's first tiles are fixed and every later one is claimed from a counter
 // (tile_at_n, tile_claim_n), so that CTAs whose streams run faster take more
@@ -1253,8 +1206,8 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
       } else if (A.pending) {
         stage_pending_warp(A, tile, sw, s0, kSub, dlw, mkw, lane, uni, chg);
         many = true;
-      } else {
-        stage_delta_warp(A, tile, sw, s0, kSub, dlw, lane);
+      } else {  // more pairs than lanes: dlt holds w_t - w_{t-1} densely all the same
+        stage_delta_dense(A, s0, kSub, dlw, lane);
       }
       sm.upos[sw][lane] = up;
       if (lane == 0) sm.pflag[sw] = many ? 1u : 0u;
@@ -1919,21 +1872,6 @@ __global__ void __launch_bounds__(1024) k_select_dense(TopkArgs A) {
 // registers (95 of them: 107 us), or took heavy sub-tiles by the block through
 // 36 KB of shared memory (92 us), ran slower than this one at 38 registers.)
 // ---------------------------------------------------------------------------
-// The position in a list of up to 32 runs (lane l's of length cnt, incl: their
-// inclusive sums): the run that holds element e (the first lane whose sum exceeds it).
-__device__ __forceinline__ int run_of(uint32_t incl, uint32_t e) {
-  int lo = 0, hi = 32;
-#pragma unroll
-  for (int it = 0; it < 6; ++it) {
-    const int mid = min((lo + hi) >> 1, 31);
-    const uint32_t v = __shfl_sync(0xffffffffu, incl, mid);
-    if (lo < hi) {
-      if (v <= e) lo = mid + 1; else hi = mid;
-    }
-  }
-  return lo < 32 ? lo : 31;
-}
-
 __global__ void __launch_bounds__(kThreads) k_apply(TopkArgs A) {
   griddep_wait();
   constexpr int kSubMax = kBulkTile / kChunksPerTile;
