@@ -1,6 +1,7 @@
 """The bulk top-k pass (2 to 16 workers, d >= 8 * 4096 * SMs: about 5 M) under the
 tests that other files run at smaller sizes, where other passes take the step;
 and single workers, which take the load/store pass at every size."""
+import numpy as np
 import pytest
 
 import test_gpu_approx
@@ -8,6 +9,7 @@ import test_gpu_bf16
 import test_gpu_checkpoint
 import test_gpu_deferred
 import test_gpu_variants
+from parity_util import Pair
 
 pytestmark = pytest.mark.gpu
 
@@ -52,3 +54,22 @@ def test_bf16(case):
     dict(compressor="topk", d=D, K=2, ratio=0.002, variant="local_momentum")], ids=str)
 def test_checkpoint(case):
     test_gpu_checkpoint.test_resume_continues_the_trajectory(case)
+
+
+@pytest.mark.parametrize("read_between", [False, True])
+@pytest.mark.parametrize("K", [2, 5, 16])
+def test_sent_pairs_concentrated_in_one_region(K, read_between):
+    """Gradients whose scale falls along the coordinates: sub-tiles of 512 hold
+    every number of sent pairs from none to some hundreds, so the counts cross 32
+    (one round) and 64 (two rounds), for a pending aggregation and an applied one."""
+    rng = np.random.default_rng(60 + K)
+    p = Pair(D, K, 0.9, 0.1, ratio=0.004, seed=11)
+    scale = np.exp(-np.arange(D) / (0.05 * D)).astype(np.float32)
+    for t in range(3):
+        r = p.step(rng.standard_normal((K, D), dtype=np.float32) * scale)
+        p.compare(r, state=read_between or t == 2)
+    per_sub = np.bincount(np.concatenate(r.supports) // 512)
+    assert per_sub.min() <= 32 < 64 < per_sub.max()
+    p.compare_stats()
+    assert p.gpu.check() == 0
+    p.gpu.close()
