@@ -91,7 +91,7 @@ struct gmc_ctx {
   int32_t* blocks = nullptr;
   uint8_t* uflag[2] = {nullptr, nullptr};
   float* slab = nullptr;
-  Counters* step_ctr = nullptr;
+  Counters* step_ctr = nullptr;  // [1]: an RBGS step's counts while its blocks add them up
   uint32_t* tile_ctr = nullptr;  // tiles claimed by the persistent passes
   uint32_t* blk_cost = nullptr;  // the bulk top-k pass's tile order (tile_order): costs, order
   uint32_t* blk_order = nullptr;
@@ -374,6 +374,7 @@ RbgsArgs rbgs_args(gmc_ctx* h, const float* grads) {
   A.det_b = detach_b(h);
   A.step_ctr = h->step_ctr;
   A.total_ctr = h->total_ctr;
+  A.acc_ctr = h->step_ctr + 1;
   A.tile_ctr = h->tile_ctr;
   A.wait_ns = kWaitLimitNs;
   A.hold_tile = -1;
@@ -561,9 +562,10 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     }
     // restored state: w_t - w_{t-1} may be non-zero in any block (zero outside
     // the last union, where dlt holds it): flag every block as the last union's
-    if (h->restored && h->t > 0) GMC_TRY(cudaMemsetAsync(A.uflag_prev, 1, (size_t)h->nb, s));
-    if (!A.clear_flags) GMC_TRY(cudaMemsetAsync(A.uflag_cur, 0, (size_t)h->nb, s));
-    GMC_TRY(timed(h, GMC_KERNEL_RBGS_PICK, 0.0, s, [&] { return launch_rbgs_pick(A, s); }));
+    if (A.bulk && h->restored && h->t > 0) GMC_TRY(cudaMemsetAsync(A.uflag_prev, 1, (size_t)h->nb, s));
+    if (A.bulk && !A.clear_flags) GMC_TRY(cudaMemsetAsync(A.uflag_cur, 0, (size_t)h->nb, s));
+    if (!rbgs_picks_in_step(A))
+      GMC_TRY(timed(h, GMC_KERNEL_RBGS_PICK, 0.0, s, [&] { return launch_rbgs_pick(A, s); }));
     const double det_bytes = A.det ? 4.0 * Kd + 4.0 * h->d : 0.0;  // the detached rows, and w
     GMC_TRY(timed(h, GMC_KERNEL_RBGS_STEP, (bf16 ? 10.0 : 12.0) * Kd + det_bytes, s,
                   [&] { return launch_rbgs_step(A, h->grid_rbgs, s); }));
@@ -763,7 +765,7 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
         (err = dalloc(h, &h->slab, (size_t)K * h->m * block)) != cudaSuccess)
       return fail(err);
   }
-  if ((err = dalloc(h, &h->step_ctr, 1)) != cudaSuccess ||
+  if ((err = dalloc(h, &h->step_ctr, 2)) != cudaSuccess ||
       (err = dalloc(h, &h->tile_ctr, 2)) != cudaSuccess ||
       (err = dalloc(h, &h->total_ctr, 1)) != cudaSuccess ||
       (err = dalloc(h, &h->status, 1)) != cudaSuccess)

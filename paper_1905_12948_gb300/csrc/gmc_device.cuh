@@ -202,6 +202,17 @@ __device__ __forceinline__ uint64_t draw(uint64_t key, uint64_t i) {
 __device__ __forceinline__ uint32_t below(uint64_t x, uint64_t n) {
   return (uint32_t)(((x >> 32) * n) >> 32);
 }
+__device__ __forceinline__ uint32_t warp_excl_scan(uint32_t x, uint32_t* total) {
+  const int lane = threadIdx.x & 31;
+  uint32_t incl = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  *total = __shfl_sync(0xffffffffu, incl, 31);
+  return incl - x;
+}
 // Membership of a candidate in C(v): above the k-th key, or equal to it with
 // an index no larger than the last tie kept (ties go to the lower index).
 __device__ __forceinline__ bool selected(uint32_t key, uint32_t j, uint32_t T, uint32_t t_idx) {

@@ -145,12 +145,12 @@ struct RbgsArgs {
   int32_t* blocks;           // streams x m: chosen blocks ascending
   uint8_t* uflag_prev;       // nb: union of the previous step's blocks
   uint8_t* uflag_cur;        // nb: union of this step's blocks (zero before the pick)
-  int clear_flags;           // the step's last warp clears uflag_prev, the next step's uflag_cur
+  int clear_flags;           // the step's last warp clears uflag_prev, the next step's uflag_cur (bulk; k_rbgs_step reads none)
   float* slab;               // K x (m*B): C(e_{t+1/2,k}) values, block slot major
   int has_prev;
   int bulk;                  // k_rbgs_bulk (bulk copies through shared memory), else k_rbgs_step
   int g_direct;              // grads is mapped host memory: read it with loads, not bulk copies
-  uint32_t* tile_ctr;        // tiles claimed by k_rbgs_bulk, warps that ended the step (zeroed by k_rbgs_pick)
+  uint32_t* tile_ctr;        // tiles claimed by k_rbgs_bulk (zeroed by k_rbgs_pick), blocks that ended the step
   uint64_t wait_ns;          // bound of the bulk pass's mbarrier waits (kWaitLimitNs)
   int64_t hold_tile;         // test hook, as in TopkArgs: no copy for item (hold_tile, hold_k)
   int hold_k;
@@ -159,6 +159,7 @@ struct RbgsArgs {
   float det_b;
   Counters* step_ctr;
   Counters* total_ctr;       // the step's last warp adds step_ctr to them
+  Counters* acc_ctr;         // the step's counts while its blocks add them up, zero between steps
   unsigned* status;
 };
 
@@ -210,6 +211,7 @@ cudaError_t launch_apply(const TopkArgs& A, int grid, cudaStream_t s);
 int apply_blocks_per_sm();
 cudaError_t launch_gather_selected(const TopkArgs& A, int k, uint32_t* idx_out, float* val_out,
                                    cudaStream_t s);
+bool rbgs_picks_in_step(const RbgsArgs& A);
 cudaError_t launch_rbgs_pick(const RbgsArgs& A, cudaStream_t s);
 cudaError_t launch_rbgs_step(const RbgsArgs& A, int grid, cudaStream_t s);
 cudaError_t launch_rbgs_expand(const RbgsArgs& A, int k, uint32_t* idx_out, float* val_out,

@@ -16,7 +16,8 @@
 //          w_{t+1} - b*e_{t+1,k}: 4 bytes a value on top of the step's 12,
 //          where a pass of its own read e back as well (d = 25.6 M, K = 32:
 //          step and rows 3,249 -> 2,040 us). The last block ends the step
-//          (end_step): two launches a step in all, where there were five.
+//          (end_step): two launches a step in all, where there were five; one
+//          where a small step's blocks each make the choice (pick_here).
 #include "gmc_internal.h"
 
 namespace gmc {
@@ -46,8 +47,8 @@ constexpr int kFirstWords = 16384;  // first-draw table kept in shared memory up
 __global__ void __launch_bounds__(kPickThreads) k_rbgs_pick(RbgsArgs A) {
   griddep_wait();
   if (blockIdx.x == 0) {
+    if (threadIdx.x < 8) A.acc_ctr->v[threadIdx.x] = 0ull;
     if (threadIdx.x < 2) A.tile_ctr[threadIdx.x] = 0u;  // tiles claimed by the fused pass, its warps done
-    if (threadIdx.x < 8) A.step_ctr->v[threadIdx.x] = 0ull;
   }
   extern __shared__ uint32_t pick_s[];
   __shared__ uint32_t ws[32];
@@ -107,7 +108,7 @@ __global__ void __launch_bounds__(kPickThreads) k_rbgs_pick(RbgsArgs A) {
         rank[b] = on ? (int32_t)q : -1;
         if (on) {
           blk[q] = (int32_t)b;
-          A.uflag_cur[b] = 1;
+          if (A.bulk) A.uflag_cur[b] = 1;
         }
       }
     }
@@ -118,9 +119,9 @@ __global__ void __launch_bounds__(kPickThreads) k_rbgs_pick(RbgsArgs A) {
 // ---------------------------------------------------------------------------
 // The end of the fused step, by the `warps` consumer warps of every block (red:
 // shared memory, 5 words a warp; they meet at named barrier 1): the block's
-// counts into step_ctr with one atomic each, and the last block out adds them
-// to the totals and clears the flags of the step before, which the next step's
-// pick sets again. (With a set of atomics per warp the d = 272 k step's 2,129
+// counts into acc_ctr with one atomic each, and the last block out moves them to
+// step_ctr, adds them to the totals, leaves acc_ctr zero for the next step, and
+// clears the flags of the step before, which the next step's pick sets again. (With a set of atomics per warp the d = 272 k step's 2,129
 // warps queued at one line.)
 // ---------------------------------------------------------------------------
 constexpr int kEndWords = 5;
@@ -143,7 +144,7 @@ __device__ __forceinline__ void end_step(const RbgsArgs& A, unsigned long long* 
 #pragma unroll
     for (int i = 1; i < kEndWords; ++i) at = lane == i ? slot[i] : at;
     if (x) {
-      atomicAdd(&A.step_ctr->v[at], x);
+      atomicAdd(&A.acc_ctr->v[at], x);
       if (lane == kEndWords - 1) atomicOr(A.status, kStatusNonfinite);
     }
     __threadfence();
@@ -157,9 +158,14 @@ __device__ __forceinline__ void end_step(const RbgsArgs& A, unsigned long long* 
   last = __shfl_sync(0xffffffffu, last, 0);
   if (last) {
     __threadfence();
+    if (lane < 8) {
+      A.step_ctr->v[lane] = __ldcg(&A.acc_ctr->v[lane]);
+      A.acc_ctr->v[lane] = 0ull;
+    }
+    if (lane == 0) A.tile_ctr[1] = 0u;
     finalize_counters(A.step_ctr, A.total_ctr, 0ull);
   }
-  if (last && A.clear_flags)
+  if (last && A.bulk && A.clear_flags)
     for (int64_t b = lane * 4; b < A.nb; b += 128)  // allocated in whole words
       *reinterpret_cast<uint32_t*>(A.uflag_prev + b) = 0u;
 }
@@ -180,9 +186,103 @@ __device__ __forceinline__ float4 detached4(float4 w, float b, float4 e) {
 constexpr int kLsSub = 128;  // elements per warp
 constexpr int kWk = 4;       // workers loaded together
 
-template <bool kBf16, bool kDetach>
+// With kPick the step is one launch: every block makes the step's whole choice
+// for itself in shared memory (pick_here), before it waits for the kernel ahead
+// of it, and looks the slots up there. The choice costs each block what the
+// launch of k_rbgs_pick and the wait for it cost the step, or less, while there
+// are few streams and the block has little else to do (us a step, shared unless
+// noted, k_rbgs_pick and step against one launch):
+//   d = 65,536, K = 4             10.4 -> 7.0     d = 272,474, K = 8, per worker  14.9 -> 12.1
+//   d = 600,000, K = 12, per w.   23.1 -> 22.6    d = 600,000, K = 16             27.5 -> 27.3
+// and past the lines below:
+//   d = 1,700, K = 16, per worker 17.7 -> 19.0    d = 600,000, K = 16, per worker 27.5 -> 28.2
+//   d = 600,000, K = 32           52.4 -> 53.0    d = 2,310, K = 32, per worker   25.5 -> 29.0
+constexpr int kPickHereStreams = 12;
+constexpr int64_t kPickHereValues = 10 << 20;  // K * d
+constexpr int kPickHereWords = 11264;  // shared words: a first-draw table, bitmap and its prefix per stream (44 KB)
+constexpr int kPickHereDraws = 1024;   // draws of all streams: four a thread (K = 4, m = nb = 1,024: 14.4 -> 11.7)
+
+// Words of shared memory that pick_here needs.
+__host__ __device__ __forceinline__ int64_t pick_here_words(const RbgsArgs& A) {
+  return (A.per_worker ? A.K : 1) * (A.nb + 2 * ((A.nb + 31) / 32));
+}
+
+struct Choice {
+  const uint32_t* bm;   // streams x nbw: the chosen blocks
+  const uint32_t* pre;  // streams x nbw: chosen blocks before the word's first
+  int nbw;
+  __device__ __forceinline__ int32_t slot(int s, uint32_t b) const {
+    const int at = s * nbw + (int)(b >> 5);
+    const uint32_t word = bm[at];
+    return (word >> (b & 31)) & 1u ? (int32_t)(pre[at] + __popc(word & ((1u << (b & 31)) - 1u))) : -1;
+  }
+};
+
+// The choice of k_rbgs_pick, of every stream, by one block of kThreads.
+__device__ __forceinline__ Choice pick_here(const RbgsArgs& A, uint32_t* sm) {
+  const int streams = A.per_worker ? A.K : 1;
+  const int nb = (int)A.nb, m = (int)A.m, nbw = (nb + 31) / 32;
+  int32_t* first = reinterpret_cast<int32_t*>(sm);
+  uint32_t* bm = sm + streams * nb;
+  uint32_t* pre = bm + streams * nbw;
+  for (int i = threadIdx.x; i < streams * nb; i += kThreads) first[i] = 0x7fffffff;
+  for (int i = threadIdx.x; i < streams * nbw; i += kThreads) bm[i] = 0u;
+  __syncthreads();
+  const int top0 = nb - m;
+  auto drawn = [&](uint64_t key, int i) { return below(draw(key, (uint64_t)i), (uint64_t)(top0 + i) + 1); };
+  auto key_of = [&](int s) { return stream_key(A.seed, A.t, A.per_worker ? (uint64_t)s + 1 : 0ull); };
+  for (int x = threadIdx.x; x < streams * m; x += kThreads) {
+    const int s = x / m, i = x - s * m;
+    atomicMin(&first[s * nb + (int)drawn(key_of(s), i)], i);
+  }
+  __syncthreads();
+  for (int x = threadIdx.x; x < streams * m; x += kThreads) {
+    const int s = x / m, i = x - s * m;
+    const uint64_t key = key_of(s);
+    const uint32_t r0 = drawn(key, i);
+    bool taken = false;
+    int at = i, b = (int)r0;
+    for (;;) {  // `at` decreases at every turn
+      if (first[s * nb + b] < at) {
+        taken = true;
+        break;
+      }
+      if (b < top0 || b - top0 >= at) break;
+      at = b - top0;
+      b = (int)drawn(key, at);
+    }
+    const uint32_t pick = taken ? (uint32_t)(top0 + i) : r0;
+    atomicOr(&bm[s * nbw + (int)(pick >> 5)], 1u << (pick & 31));
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int s = threadIdx.x >> 5; s < streams; s += kWarps) {
+    uint32_t carry = 0;
+    for (int w0 = 0; w0 < nbw; w0 += 32) {
+      const uint32_t n = w0 + lane < nbw ? (uint32_t)__popc(bm[s * nbw + w0 + lane]) : 0u;
+      uint32_t tot;
+      const uint32_t exc = warp_excl_scan(n, &tot);
+      if (w0 + lane < nbw) pre[s * nbw + w0 + lane] = carry + exc;
+      carry += tot;
+    }
+  }
+  __syncthreads();
+  return Choice{bm, pre, nbw};
+}
+
+template <bool kBf16, bool kDetach, bool kPick>
 __global__ void __launch_bounds__(kThreads) k_rbgs_step(RbgsArgs A) {
+  extern __shared__ uint32_t pick_sm[];
+  Choice choice = {};
+  if (kPick) choice = pick_here(A, pick_sm);
   griddep_wait();
+  if (kPick) {  // the lists of chosen blocks, a stream a block (gmc_selected reads them)
+    for (int s = blockIdx.x; s < (A.per_worker ? A.K : 1); s += gridDim.x)
+      for (int b = threadIdx.x; b < (int)A.nb; b += kThreads) {
+        const int32_t q = choice.slot(s, (uint32_t)b);
+        if (q >= 0) A.blocks[(int64_t)s * A.m + q] = b;
+      }
+  }
   __shared__ unsigned long long red[kWarps * kEndWords];
   const int lane = threadIdx.x & 31;
   uint32_t nonfinite = 0, pairs = 0, nnz = 0, uni = 0, changed = 0;
@@ -214,7 +314,8 @@ __global__ void __launch_bounds__(kThreads) k_rbgs_step(RbgsArgs A) {
           gv[q] = kBf16 ? load_g4_bf16(A.grads16 + (int64_t)k * A.d, j, A.d) : load_g4(gk, j, A.d, g_mode(gk));
           const int32_t* rk = A.rank + (A.per_worker ? (int64_t)k * A.nb : 0);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) at[q][i] = lane * 4 + i < lim ? rk[bid[i]] : -1;
+          for (int i = 0; i < 4; ++i)
+            at[q][i] = lane * 4 + i < lim ? (kPick ? choice.slot(A.per_worker ? k : 0, bid[i]) : rk[bid[i]]) : -1;
         }
       }
 #pragma unroll
@@ -601,8 +702,15 @@ cudaError_t configure_rbgs_kernels() {
 
 int rbgs_blocks_per_sm() {
   int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rbgs_step<false, true>, kThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rbgs_step<false, true, false>, kThreads, 0);
   return n > 0 ? n : 1;
+}
+
+// Whether the load/store step makes its choice itself.
+bool rbgs_picks_in_step(const RbgsArgs& A) {
+  const int streams = A.per_worker ? A.K : 1;
+  return !A.bulk && streams <= kPickHereStreams && A.K * A.d <= kPickHereValues &&
+         pick_here_words(A) <= kPickHereWords && streams * A.m <= kPickHereDraws;
 }
 
 cudaError_t launch_rbgs_pick(const RbgsArgs& A, cudaStream_t s) {
@@ -618,8 +726,14 @@ cudaError_t launch_rbgs_step(const RbgsArgs& A, int grid, cudaStream_t s) {
     if (A.det) return launch_pdl(A.bf16 ? k_rbgs_bulk<true, true> : k_rbgs_bulk<false, true>, g, b, sm, s, A);
     return launch_pdl(A.bf16 ? k_rbgs_bulk<true, false> : k_rbgs_bulk<false, false>, g, b, sm, s, A);
   }
-  if (A.det) return launch_pdl(A.bf16 ? k_rbgs_step<true, true> : k_rbgs_step<false, true>, dim3(grid), dim3(kThreads), 0, s, A);
-  return launch_pdl(A.bf16 ? k_rbgs_step<true, false> : k_rbgs_step<false, false>, dim3(grid), dim3(kThreads), 0, s, A);
+  const dim3 g(grid), b(kThreads);
+  if (rbgs_picks_in_step(A)) {
+    const size_t sm = (size_t)pick_here_words(A) * 4;
+    if (A.det) return launch_pdl(A.bf16 ? k_rbgs_step<true, true, true> : k_rbgs_step<false, true, true>, g, b, sm, s, A);
+    return launch_pdl(A.bf16 ? k_rbgs_step<true, false, true> : k_rbgs_step<false, false, true>, g, b, sm, s, A);
+  }
+  if (A.det) return launch_pdl(A.bf16 ? k_rbgs_step<true, true, false> : k_rbgs_step<false, true, false>, g, b, 0, s, A);
+  return launch_pdl(A.bf16 ? k_rbgs_step<true, false, false> : k_rbgs_step<false, false, false>, g, b, 0, s, A);
 }
 
 cudaError_t launch_rbgs_expand(const RbgsArgs& A, int k, uint32_t* idx_out, float* val_out,

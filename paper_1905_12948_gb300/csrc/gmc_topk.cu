@@ -56,18 +56,6 @@ __device__ __forceinline__ float4 scale_g(const TopkArgs& A, float4 g) {
   return g;
 }
 
-__device__ __forceinline__ uint32_t warp_excl_scan(uint32_t x, uint32_t* total) {
-  const int lane = threadIdx.x & 31;
-  uint32_t incl = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  *total = __shfl_sync(0xffffffffu, incl, 31);
-  return incl - x;
-}
-
 // Sampled coordinate of slot i of the exact top-k: kSampleRun (16) consecutive
 // coordinates from (c * d / chunks) rounded down to a multiple of kSampleRun,
 // c = 0 .. chunks-1 (every coordinate when chunks = 0); this sample only sets

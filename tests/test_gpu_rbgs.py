@@ -25,6 +25,35 @@ def test_pick(d, B, ratio, per_worker):
     p.compare_stats()
 
 
+@pytest.mark.parametrize("d,K,B,ratio,per_worker", [
+    (1_024, 2, 1, 1.0, False), (1_025, 2, 1, 1.0, False),       # the most draws a step makes itself, one more
+    (10_600, 1, 1, 0.05, False), (10_601, 1, 1, 0.05, False),   # its largest table, one more
+    (6_174, 12, 7, 0.09, True), (6_181, 12, 7, 0.09, True),     # the same with a stream per worker
+    (130, 12, 1, 0.1, True), (130, 13, 1, 0.1, True), (129, 32, 1, 0.1, False),  # the most streams
+    (590_000, 17, 4096, 0.05, False), (590_000, 18, 4096, 0.05, False),          # the most values
+    (272_474, 8, 256, 0.05, True), (33, 3, 1, 0.04, True),
+])
+def test_choice_within_the_step(d, K, B, ratio, per_worker):
+    rng = np.random.default_rng(d)
+    p = Pair(d, K, 0.9, 0.1, compressor="rbgs", ratio=ratio, block=B, lam=0.5, seed=6, per_worker=per_worker)
+    for t in range(3):
+        p.compare(p.step(rng.standard_normal((K, d)).astype(np.float32)))
+    p.compare_stats()
+
+
+def test_choice_within_and_before_the_step_in_turn():
+    """One handle whose shared choice is made in the step and whose per-worker
+    choice (too many draws) by a kernel of its own."""
+    d, K = 9_000, 4
+    rng = np.random.default_rng(77)
+    p = Pair(d, K, 0.9, 0.1, compressor="rbgs", ratio=0.5, block=10, lam=0.5, seed=7)
+    for t in range(6):
+        assert p.gpu.lib.gmc_set_rbgs_mode(p.gpu.h, t & 1) == 0
+        p.ref.per_worker = bool(t & 1)
+        p.compare(p.step(rng.standard_normal((K, d)).astype(np.float32)))
+    p.compare_stats()
+
+
 @pytest.mark.parametrize("d,K,B,offset,pad", [
     (127, 1, 10, 0, 0), (128, 5, 128, 1, 1), (1_025, 9, 100, 2, 3), (50_001, 32, 333, 3, 0),  # load/store pass
     (4096 * 160 + 130, 3, 1000, 1, 2), (4096 * 152 + 4095, 2, 4096, 3, 1),                     # bulk pass
