@@ -479,46 +479,48 @@ __device__ __forceinline__ bool wait_bounded(uint64_t* bar, uint32_t parity, uin
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
-// Grid barrier of a cooperative launch (every block resident). `bar` is a word
-// that is zero when the launch begins; the blocks' arrivals of one barrier add
-// up to 2^31, so its top bit flips when the last one arrives. A wait is bounded
-// (limit_ns): false, for the whole block, when it gave up -- the block then
-// leaves. The word is put back to zero by the last block to leave (leave_grid),
-// also after a wait that gave up.
+// Barriers of a cooperative launch (every block resident): one word counts the
+// blocks' arrivals and is never put back. The launch's b-th barrier ends when the
+// count has grown by b * gridDim.x since the launch began, told by the sign of
+// the difference, so that the word may wrap. An arrival needs no answer (a
+// reduction with release), so a barrier costs the word's way to L2 and back once,
+// for the blocks that poll it. A wait is bounded: wait() is false, for the whole
+// block, when it gave up, and from then on (the block does not arrive again: it
+// would stand for the one that is missing). The count then no longer matches what
+// the next launch expects: it must be cleared first.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t* s_ok, uint64_t limit_ns) {
-  const uint32_t n = gridDim.x;
-  if (n == 1) {
+struct GridBarrier {
+  uint32_t* count;    // arrivals
+  uint32_t reached;   // what the count has reached after the barriers passed so far (at launch: its value)
+  uint64_t limit_ns;
+  uint32_t* s_ok;     // a word of shared memory
+  bool alive = true;  // no wait gave up yet
+  __device__ __forceinline__ bool wait() {
+    if (!alive) return false;
+    reached += gridDim.x;
     __syncthreads();
-    return true;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const uint32_t old = atomicAdd(bar, blockIdx.x == 0 ? 0x80000000u - (n - 1) : 1u);
-    uint32_t ok = 1;
-    uint64_t t0 = 0;
-    for (uint32_t spins = 0; ((old ^ ld_acquire(bar)) & 0x80000000u) == 0; ++spins) {
-      if ((spins & 1023u) == 1023u) {
+    if (gridDim.x == 1) return true;
+    if (threadIdx.x == 0) {
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+      uint64_t since = 0;
+      bool here = false;
+      for (uint32_t polls = 1; !(here = (int32_t)(ld_acquire(count) - reached) >= 0); ++polls) {
+        if (polls & 1023u) continue;  // the clock now and then
         const uint64_t now = global_ns();
-        if (t0 == 0) t0 = now;
-        if (now - t0 > limit_ns) {
-          ok = 0;
-          break;
-        }
+        if (since == 0) since = now;
+        if (now - since > limit_ns) break;
       }
+      *s_ok = here ? 1u : 0u;
     }
-    __threadfence();
-    *s_ok = ok;
+    __syncthreads();
+    return alive = *s_ok != 0u;
   }
-  __syncthreads();
-  return *s_ok != 0;
-}
+};
 // Every block, as its last act: true for the last one of the grid to call it
 // (all its threads), which then resets what the next launch finds zeroed.
 __device__ __forceinline__ bool leave_grid(uint32_t* left, uint32_t* s_last) {

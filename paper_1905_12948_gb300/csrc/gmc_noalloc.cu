@@ -54,7 +54,7 @@ constexpr int64_t kNaBlockMin = 8192;  // values per block below which fewer blo
 // The shared scratch, about 270 KB per device. Zero when a call begins (but
 // for what a collect pass writes first); the last block of a call leaves it so.
 struct NaScratch {
-  uint32_t bar, left;                   // grid_barrier, leave_grid
+  uint32_t arrivals, left;              // GridBarrier, leave_grid
   uint32_t pad[30];
   uint32_t count[kNaRounds];            // keys listed by each collect pass
   uint32_t hist[5][kHistBins];          // the sample's two digits; three in turn for the narrowing passes
@@ -168,13 +168,14 @@ __global__ void __launch_bounds__(kNaThreads, 1)
   C.n_own = (uint32_t)C.n_chunks > me ? (int)((C.n_chunks - 1 - me) / G) + 1 : 0;
   C.claim = &s_claim;
   bool ok = true;
+  GridBarrier grid{&S->arrivals, 0u, kWaitLimitNs, &s_ok};
 
   // A histogram in shared memory added to a global one, and read back after a barrier.
   auto share_hist = [&](uint32_t* gh) {
     __syncthreads();
     for (int b = threadIdx.x; b < kHistBins; b += kNaThreads)
       if (h[b]) atomicAdd(&gh[b], h[b]);
-    const bool good = grid_barrier(&S->bar, &s_ok, kWaitLimitNs);
+    const bool good = grid.wait();
     for (int b = threadIdx.x; b < kHistBins; b += kNaThreads) h[b] = __ldcg(&gh[b]);
     if (threadIdx.x < 4) find[threadIdx.x] = 0;
     __syncthreads();
@@ -639,7 +640,7 @@ __global__ void __launch_bounds__(kNaThreads, 1)
   if (leave_grid(&S->left, &s_ok)) {  // the next call finds the scratch zeroed
     for (int b = threadIdx.x; b < 5 * kHistBins; b += kNaThreads) S->hist[0][b] = 0;
     if (threadIdx.x < kNaRounds) S->count[threadIdx.x] = 0;
-    if (threadIdx.x == 0) S->bar = S->left = 0;
+    if (threadIdx.x == 0) S->arrivals = S->left = 0;
   }
 }
 

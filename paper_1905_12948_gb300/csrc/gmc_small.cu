@@ -46,8 +46,9 @@ static_assert(kItemMax * 512 + 8 * (kHistBins / 2) * 4 <= 232448 - 6 * 1024, "ac
 
 // The launch's global scratch (words; zero when the state is reset).
 struct Scratch {
-  uint32_t bar, start;        // grid_barrier; the first round's histogram of the three
-  uint32_t pad[30];
+  uint32_t arrivals, base;    // GridBarrier's count, and its value when a launch begins
+  uint32_t start;             // the first round's histogram of the three
+  uint32_t pad[29];
   uint32_t listed[kMaxK];     // elements listed
   uint32_t reach[kMaxK];      // approximate top-s: elements that reach theta
   uint2 list[kMaxK][kListCap];
@@ -117,9 +118,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
     if ((int)threadIdx.x < K) A.sel[threadIdx.x].count = 0;
   }
   uint32_t buf = S->start;  // 0, 1 or 2
+  GridBarrier grid{&S->arrivals, S->base, A.wait_ns, &s_ok};
   // every block's writes so far are seen by every block (false: a wait gave up)
   auto barrier = [&]() -> bool {
-    if (!kCluster) return grid_barrier(&S->bar, &s_ok, A.wait_ns);
+    if (!kCluster) return grid.wait();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     return true;
   };
@@ -464,7 +466,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
     return;
   }
   if (me == 0) {
-    if (threadIdx.x == 0) S->start = buf;
+    if (threadIdx.x == 0) {
+      S->start = buf;
+      if (!kCluster) S->base = grid.reached;
+    }
     if ((int)threadIdx.x < K) {
       WorkerSel& W = A.sel[threadIdx.x];
       const Search& s = sr[threadIdx.x];
