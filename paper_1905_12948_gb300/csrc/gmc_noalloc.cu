@@ -58,8 +58,11 @@ struct NaScratch {
   uint32_t pad[30];
   uint32_t count[kNaRounds];            // keys listed by each collect pass
   uint32_t hist[5][kHistBins];          // the sample's two digits; three in turn for the narrowing passes
-  uint32_t above[kNaMaxBlocks];         // per block: keys above the interval
-  uint32_t equal[kNaMaxBlocks];         // per block: keys inside it
+  // per block: keys above the interval, and inside it. Two of each, used in turn:
+  // a pass is separated from the one before by a single barrier, after which
+  // some blocks still read that pass's counts while others write this one's
+  uint32_t above[2][kNaMaxBlocks];
+  uint32_t equal[2][kNaMaxBlocks];
   uint16_t above_c[kNaChunks];          // per chunk: keys above the interval
   union {
     struct {                            // the keys inside, and their indices
@@ -342,8 +345,8 @@ __global__ void __launch_bounds__(kNaThreads, 1)
       eq = block_total(eq);
       const uint32_t staged = min(s_n, (uint32_t)kNaStage);
       if (threadIdx.x == 0) {
-        S->above[me] = gt;
-        S->equal[me] = eq;
+        S->above[round & 1][me] = gt;
+        S->equal[round & 1][me] = eq;
         s_base = (!one && staged) ? atomicAdd(&S->count[round], staged) : 0u;
       }
       __syncthreads();
@@ -356,8 +359,8 @@ __global__ void __launch_bounds__(kNaThreads, 1)
         }
       ok = share_hist(gh);
       know_above = true;
-      const uint32_t a_all = block_total(threadIdx.x < G ? __ldcg(&S->above[threadIdx.x]) : 0u);
-      const uint32_t q_all = block_total(threadIdx.x < G ? __ldcg(&S->equal[threadIdx.x]) : 0u);
+      const uint32_t a_all = block_total(threadIdx.x < G ? __ldcg(&S->above[round & 1][threadIdx.x]) : 0u);
+      const uint32_t q_all = block_total(threadIdx.x < G ? __ldcg(&S->equal[round & 1][threadIdx.x]) : 0u);
       above = a_all;
       if (a_all >= k) {  // T lies above the interval
         L = U + 1;       // U < 2^31 - 1, since keys lie above it
@@ -410,11 +413,11 @@ __global__ void __launch_bounds__(kNaThreads, 1)
       for (int b = me * kNaThreads + threadIdx.x; b < kHistBins; b += G * kNaThreads) gz[b] = 0;
     ++hist_round;
     gt = block_total(gt);
-    if (threadIdx.x == 0) S->above[me] = gt;
+    if (threadIdx.x == 0) S->above[round & 1][me] = gt;
     ok = share_hist(gh);
     if (!know_above) {
       know_above = true;
-      above = block_total(threadIdx.x < G ? __ldcg(&S->above[threadIdx.x]) : 0u);
+      above = block_total(threadIdx.x < G ? __ldcg(&S->above[round & 1][threadIdx.x]) : 0u);
       for (int b = threadIdx.x; b < kHistBins; b += kNaThreads) eq += h[b];
       eq = block_total(eq);
       if (above >= k) {  // T lies above the interval

@@ -63,3 +63,17 @@ def test_alignment(n, offset):
     x = rng.standard_normal(n).astype(np.float32)
     for k in {1, (n + 1) // 2, n}:
         _run(x, k, offset)
+
+
+def test_passes_in_quick_succession():
+    """A few blocks whose passes last a microsecond or two and are many (more keys in
+    the interval than the list takes, so that it is narrowed again): a block's
+    counts of one pass stand until every other block has read them."""
+    rng = np.random.default_rng(77)
+    for n in (24_577, 60_001):
+        for width in (1e-5, 3e-4):
+            x = np.ascontiguousarray(_band(rng, n, 1.0, 1.0 + width))
+            x[rng.integers(0, n, n // 3)] = 1.0
+            for k in (n // 3, n // 2, n - 1):
+                for _ in range(10):
+                    _run(x, k)
