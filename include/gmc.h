@@ -352,6 +352,15 @@ int64_t gmc_test_fail_alloc(int64_t fail_at);
 int gmc_test_withhold_copy(gmc_t h, int64_t tile, int32_t k, uint64_t wait_limit_ns);
 
 /*
+ * gmc_test_leave_barrier -- process-wide, the next gmc_topk_noalloc only: one of
+ * its blocks leaves at once, so the other blocks' waits for it give up after
+ * wait_limit_ns (1 .. 2e9; 0 disarms the hook) instead of about two seconds, and
+ * the call reports that as described there. Without effect on a call of one
+ * block (n <= 8192). GMC_EINVAL for a limit out of range.
+ */
+int gmc_test_leave_barrier(uint64_t wait_limit_ns);
+
+/*
  * gmc_topk_noalloc -- the top-k compressor of one vector without allocating.
  * The paper has no counterpart: this is a library convenience for callers
  * that cannot call cudaMalloc, e.g. code whose device memory is all owned by
@@ -362,11 +371,16 @@ int gmc_test_withhold_copy(gmc_t h, int64_t tile, int32_t k, uint64_t wait_limit
  * GMC_TOPK -- to idx_dev / val_dev (device, k entries each) in ascending index
  * order. x_dev is device memory, fp32, read-only. Requires 1 <= k <= n
  * (else GMC_EINVAL) and n <= 2^26 (else GMC_ETOOBIG).
- * It allocates nothing: its scratch is one fixed array of about 270 KB in the
+ * It allocates nothing: its scratch is one fixed array of about 280 KB in the
  * library's device memory, which every GPU that loads the library holds until
  * the process exits. All calls share that array, so calls that overlap on the
  * GPU (on different streams, or from different threads) race; serialise
- * them. The first call on each device (and the first after the device's
+ * them (calls that overlapped all the same spoil their own results only). It
+ * runs as one kernel whose blocks wait for one another. Should such a wait give
+ * up (about two seconds without progress), entries of idx_dev are left as
+ * 0xffffffff, which no index is: a result without such an entry is complete. The
+ * next call is not affected.
+ * The first call on each device (and the first after the device's
  * context was replaced, e.g. by cudaDeviceReset) looks up the array's device
  * address and the SM count; make that first call before any stream capture.
  * A NaN in x ranks above every finite value and Inf (its magnitude bit pattern

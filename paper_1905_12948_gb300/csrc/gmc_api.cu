@@ -1210,6 +1210,12 @@ int gmc_test_withhold_copy(gmc_t h, int64_t tile, int32_t k, uint64_t wait_limit
   return GMC_OK;
 }
 
+int gmc_test_leave_barrier(uint64_t wait_limit_ns) {
+  if (wait_limit_ns > kWaitLimitNs) return GMC_EINVAL;
+  noalloc_leave_barrier(wait_limit_ns);
+  return GMC_OK;
+}
+
 int64_t gmc_test_fail_alloc(int64_t fail_at) {
   g_fail_countdown.store(fail_at < 0 ? -1 : fail_at);
   return g_live_allocations.load();

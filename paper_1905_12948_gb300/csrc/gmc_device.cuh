@@ -521,19 +521,6 @@ struct GridBarrier {
     return alive = *s_ok != 0u;
   }
 };
-// Every block, as its last act: true for the last one of the grid to call it
-// (all its threads), which then resets what the next launch finds zeroed.
-__device__ __forceinline__ bool leave_grid(uint32_t* left, uint32_t* s_last) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    *s_last = atomicAdd(left, 1u) == gridDim.x - 1 ? 1u : 0u;
-    __threadfence();
-  }
-  __syncthreads();
-  return *s_last != 0;
-}
-
 // Tiles of a persistent streaming pass. A CTA's first kFixed tiles are fixed,
 // blockIdx.x + n * gridDim.x; every later one is claimed from a counter that
 // the step's previous kernel zeroed, kFixed - 1 tiles before the CTA starts

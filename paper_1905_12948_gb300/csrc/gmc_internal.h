@@ -241,6 +241,10 @@ cudaError_t configure_small_kernels();
 cudaError_t launch_topk_step(const TopkArgs& A, const DetachArgs& D, int grid, bool cluster, uint32_t* scratch,
                              cudaStream_t s);
 
+// Test hook: the next gmc_topk_noalloc's last block leaves before its first
+// barrier, and its waits are bounded by wait_limit_ns.
+void noalloc_leave_barrier(uint64_t wait_limit_ns);
+
 constexpr int kRbgsTile = 4096;  // elements per tile of the fused RBGS kernel
 
 }  // namespace gmc

@@ -26,6 +26,8 @@
 // at k = n/1000), by its four grid barriers below a few million values. n = 25.6 M, k = n/1000: 304 us with five
 // passes of 4-byte loads in seven launches -> 70 us (14 for the sample, 24 the
 // pass over x, 12 ranking the list in every block, 6 the write).
+#include <atomic>
+#include <cstddef>
 #include <mutex>
 
 #include "gmc.h"
@@ -51,11 +53,13 @@ static_assert(kNaChunks * 2 <= kNaCap * 4, "the chunk counts fit in the keys' sh
 static_assert(kNaOwn == kNaThreads, "one thread per own chunk");
 constexpr int64_t kNaBlockMin = 8192;  // values per block below which fewer blocks run
 
-// The shared scratch, about 270 KB per device. Zero when a call begins (but
-// for what a collect pass writes first); the last block of a call leaves it so.
+// The shared scratch, about 280 KB per device. A call begins with a memset of
+// what comes before `above`, so that nothing an earlier call left behind (one
+// whose waits gave up, or that overlapped another) reaches it; the rest is
+// written before it is read.
 struct NaScratch {
-  uint32_t arrivals, left;              // GridBarrier, leave_grid
-  uint32_t pad[30];
+  uint32_t arrivals;                    // GridBarrier
+  uint32_t pad[31];
   uint32_t count[kNaRounds];            // keys listed by each collect pass
   uint32_t hist[5][kHistBins];          // the sample's two digits; three in turn for the narrowing passes
   // per block: keys above the interval, and inside it. Two of each, used in turn:
@@ -145,7 +149,9 @@ struct NaChunks {
 };
 
 __global__ void __launch_bounds__(kNaThreads, 1)
-    k_na_topk(const float* __restrict__ x, int64_t n, uint32_t k, NaScratch* S, uint32_t* idx_out, float* val_out) {
+    k_na_topk(const float* __restrict__ x, int64_t n, uint32_t k, NaScratch* S, uint32_t* idx_out, float* val_out,
+              uint64_t wait_ns, int leave) {
+  if (leave && blockIdx.x == gridDim.x - 1) return;  // test hook: the others' waits give up
   extern __shared__ __align__(16) uint32_t na_keys[];  // kNaCap
   __shared__ uint32_t h[kHistBins];
   __shared__ uint2 stage[kNaStage];
@@ -171,7 +177,7 @@ __global__ void __launch_bounds__(kNaThreads, 1)
   C.n_own = (uint32_t)C.n_chunks > me ? (int)((C.n_chunks - 1 - me) / G) + 1 : 0;
   C.claim = &s_claim;
   bool ok = true;
-  GridBarrier grid{&S->arrivals, 0u, kWaitLimitNs, &s_ok};
+  GridBarrier grid{&S->arrivals, 0u, wait_ns, &s_ok};
 
   // A histogram in shared memory added to a global one, and read back after a barrier.
   auto share_hist = [&](uint32_t* gh) {
@@ -444,7 +450,12 @@ __global__ void __launch_bounds__(kNaThreads, 1)
   }
   ok = ok && found;
 
-  if (ok) {
+  if (!ok) {
+    // a wait gave up: no selection, and every index says so. (Blocks whose waits
+    // all ended write their pairs meanwhile: what ends up with an index is one of
+    // theirs, and valid; this block's pairs keep the mark.)
+    for (uint32_t i = threadIdx.x; i < k; i += kNaThreads) idx_out[i] = kNone;
+  } else {
     // ---- T from the list ----
     for (int o = threadIdx.x; o < kNaOwn; o += kNaThreads) base_gt[o] = base_eq[o] = 0;
     if (listed) {
@@ -640,11 +651,6 @@ __global__ void __launch_bounds__(kNaThreads, 1)
       }
     }
   }
-  if (leave_grid(&S->left, &s_ok)) {  // the next call finds the scratch zeroed
-    for (int b = threadIdx.x; b < 5 * kHistBins; b += kNaThreads) S->hist[0][b] = 0;
-    if (threadIdx.x < kNaRounds) S->count[threadIdx.x] = 0;
-    if (threadIdx.x == 0) S->arrivals = S->left = 0;
-  }
 }
 
 // Set-up of one device: the scratch array's device address and the grid,
@@ -654,6 +660,8 @@ struct DeviceSetup {
   NaScratch* scratch = nullptr;
   int blocks = 1;                 // resident blocks of k_na_topk
 };
+// Test hook (gmc_test_leave_barrier): the next call's wait limit, 0 = off.
+std::atomic<uint64_t> g_leave_ns{0};
 std::mutex g_setup_mutex;
 DeviceSetup g_setup[kNaMaxDevices];
 
@@ -722,6 +730,9 @@ cudaError_t device_setup(DeviceSetup* out) {
 }
 
 }  // namespace
+
+void noalloc_leave_barrier(uint64_t wait_limit_ns) { g_leave_ns.store(wait_limit_ns); }
+
 }  // namespace gmc
 
 extern "C" int gmc_topk_noalloc(const float* x_dev, int64_t n, int64_t k, uint32_t* idx_dev,
@@ -743,7 +754,11 @@ extern "C" int gmc_topk_noalloc(const float* x_dev, int64_t n, int64_t k, uint32
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  const uint64_t leave_ns = g_leave_ns.exchange(0);
   // the launch's own error: earlier, unrelated work's is neither read nor cleared
-  const cudaError_t err = cudaLaunchKernelEx(&cfg, k_na_topk, x_dev, n, (uint32_t)k, dv.scratch, idx_dev, val_dev);
+  cudaError_t err = cudaMemsetAsync(dv.scratch, 0, offsetof(NaScratch, above), cfg.stream);
+  if (err == cudaSuccess)
+    err = cudaLaunchKernelEx(&cfg, k_na_topk, x_dev, n, (uint32_t)k, dv.scratch, idx_dev, val_dev,
+                             leave_ns ? leave_ns : kWaitLimitNs, leave_ns ? 1 : 0);
   return err == cudaSuccess ? GMC_OK : GMC_ECUDA;
 }

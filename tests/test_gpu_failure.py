@@ -3,7 +3,8 @@
 * A bounded wait that runs out: the test hook withholds one item's copy in a
   bulk pass, so the waits on it give up after a short limit; the kernel
   returns, gmc_check reports GMC_ETIMEOUT, and a reset (or a new handle) steps
-  exactly as the oracle again.
+  exactly as the oracle again. Likewise a block that leaves before a grid
+  barrier of gmc_topk_noalloc.
 * A device allocation that fails: the allocation hook makes the n-th
   allocation of gmc_create / gmc_set_variant fail as cudaMalloc does when
   memory runs out; the call returns GMC_ENOMEM, leaks nothing, and leaves an
@@ -75,6 +76,32 @@ def test_withheld_copy_times_out_and_is_reported(compressor, d, K, hold):
     assert p.gpu.check() == GMC_OK and p2.gpu.check() == GMC_OK
     p.gpu.close()
     p2.gpu.close()
+
+
+@pytest.mark.parametrize("n,k", [(20_000, 300), (3_000_001, 3_000), (100_000, 100_000)])
+def test_noalloc_wait_that_gives_up_marks_its_output(n, k):
+    """A block that never comes to the barrier: the call returns, its indices say
+    that there is no selection, and the next call is as if it had not been."""
+    import oracle
+    import torch
+    lib = _lib()
+    x_np = np.random.default_rng(n).standard_normal(n).astype(np.float32)
+    x = torch.from_numpy(x_np).cuda()
+    idx = torch.zeros(k, dtype=torch.int32, device="cuda")
+    val = torch.zeros(k, dtype=torch.float32, device="cuda")
+
+    def call():
+        assert lib.gmc_topk_noalloc(x.data_ptr(), n, k, idx.data_ptr(), val.data_ptr(),
+                                    torch.cuda.current_stream().cuda_stream) == GMC_OK
+        torch.cuda.synchronize()
+        return idx.cpu().numpy()
+
+    want = oracle.top_s_support(x_np, k)
+    assert np.array_equal(call(), want)
+    assert lib.gmc_test_leave_barrier(5_000_000_000) == GMC_EINVAL
+    assert lib.gmc_test_leave_barrier(20_000_000) == GMC_OK
+    assert np.all(call() == -1)
+    assert np.array_equal(call(), want)
 
 
 def test_withhold_refused_without_a_bulk_pass():
