@@ -297,8 +297,10 @@ int gmc_load_state(gmc_t h, const void* host_in, int64_t bytes);
  * (or gmc_load_state), most severe first: GMC_ECUDA (a CUDA error, e.g. a failed
  * kernel), GMC_EINTERNAL (an internal consistency check failed), GMC_ETIMEOUT (a
  * bounded wait of a bulk pass gave up, about two seconds without progress, and the
- * pass skipped the rest of that CTA's tiles: w and the residuals are not Alg. 1's
- * and the handle must be reset with gmc_set_params or gmc_load_state), or
+ * pass skipped the rest of that CTA's tiles, or one of the one-launch step of small
+ * problems, and blocks skipped the rest of the step: w and the residuals are not
+ * Alg. 1's and the handle must be reset with gmc_set_params or gmc_load_state; the
+ * one-launch step leaves the state alone until then), or
  * GMC_ENONFINITE (a NaN or Inf accumulator value, Sec. 3.1's step otherwise
  * completed). GMC_OK when none. The status is not cleared by reading it.
  * The recorded state is Alg. 1's (Sec. 3.1): the step runs to completion or
@@ -352,13 +354,16 @@ int64_t gmc_test_fail_alloc(int64_t fail_at);
 int gmc_test_withhold_copy(gmc_t h, int64_t tile, int32_t k, uint64_t wait_limit_ns);
 
 /*
- * gmc_test_leave_barrier -- process-wide, the next gmc_topk_noalloc only: one of
- * its blocks leaves at once, so the other blocks' waits for it give up after
- * wait_limit_ns (1 .. 2e9; 0 disarms the hook) instead of about two seconds, and
- * the call reports that as described there. Without effect on a call of one
- * block (n <= 8192). GMC_EINVAL for a limit out of range.
+ * gmc_test_leave_barrier -- the next gmc_step of h, or with h = NULL the next
+ * gmc_topk_noalloc of the process (only that one): one of its blocks leaves at
+ * once, so the other blocks' waits for it give up after wait_limit_ns (1 .. 2e9;
+ * 0 disarms the hook) instead of about two seconds, and that is reported
+ * (gmc_check, or as gmc_topk_noalloc describes). GMC_EINVAL for a limit out of
+ * range, and for a handle whose steps are not one launch of blocks that wait for
+ * one another (top-k, sampled, K x d from about 131,000 to 7 M). Without effect
+ * on a gmc_topk_noalloc of one block (n <= 8192).
  */
-int gmc_test_leave_barrier(uint64_t wait_limit_ns);
+int gmc_test_leave_barrier(gmc_t h, uint64_t wait_limit_ns);
 
 /*
  * gmc_topk_noalloc -- the top-k compressor of one vector without allocating.

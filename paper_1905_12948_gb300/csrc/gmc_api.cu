@@ -103,6 +103,7 @@ struct gmc_ctx {
   int64_t hold_tile = -1;
   int hold_k = 0;
   uint64_t hold_wait_ns = 0;
+  uint64_t leave_ns = 0;  // test hook (gmc_test_leave_barrier): the next one-launch step's wait limit, 0 = off
   float* gstage = nullptr;
   std::vector<void*> allocations;
   // profiling
@@ -494,6 +495,11 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     TopkArgs A = topk_args(h, grads);
     A.grads16 = grads16;
     A.bf16 = bf16 ? 1 : 0;
+    if (h->leave_ns) {
+      A.hold_tile = 0;
+      A.wait_ns = h->leave_ns;
+      h->leave_ns = 0;
+    }
     const DetachArgs D{h->w, h->e, h->ld, h->d, detach_b(h), h->detach_out, h->detach_ld, 0, h->K};
     const double bytes = ((A.local_mom ? 20.0 : 12.0) - (bf16 ? 2.0 : 0.0)) * Kd + (D.out ? 4.0 * Kd : 0.0);
     GMC_TRY(timed(h, GMC_KERNEL_ACCUMULATE, bytes, s,
@@ -1210,9 +1216,14 @@ int gmc_test_withhold_copy(gmc_t h, int64_t tile, int32_t k, uint64_t wait_limit
   return GMC_OK;
 }
 
-int gmc_test_leave_barrier(uint64_t wait_limit_ns) {
+int gmc_test_leave_barrier(gmc_t h, uint64_t wait_limit_ns) {
   if (wait_limit_ns > kWaitLimitNs) return GMC_EINVAL;
-  noalloc_leave_barrier(wait_limit_ns);
+  if (!h) {
+    noalloc_leave_barrier(wait_limit_ns);
+    return GMC_OK;
+  }
+  if (h->grid_small < 2 || h->small_cluster || h->select_mode != GMC_SELECT_SAMPLED) return GMC_EINVAL;
+  h->leave_ns = wait_limit_ns;
   return GMC_OK;
 }
 

@@ -109,7 +109,8 @@ struct TopkArgs {
   int use_order;             // this step's pass follows blk_order (it was built this step)
   uint64_t wait_ns;          // bound of the bulk pass's mbarrier waits (kWaitLimitNs)
   int64_t hold_tile;         // test hook: the bulk pass issues no copy for item (hold_tile, hold_k),
-  int hold_k;                // so that the waits on it give up; hold_tile = -1: none
+  int hold_k;                // so that the waits on it give up; hold_tile = -1: none (the one-launch
+                             // step: >= 0: its last block leaves at once)
   int finalize;              // k_select_dense or k_apply ends the step: adds step_ctr (+ pairs_add pairs) to the totals
   unsigned long long pairs_add;
 };

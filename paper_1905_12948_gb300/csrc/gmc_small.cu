@@ -48,7 +48,8 @@ static_assert(kItemMax * 512 + 8 * (kHistBins / 2) * 4 <= 232448 - 6 * 1024, "ac
 struct Scratch {
   uint32_t arrivals, base;    // GridBarrier's count, and its value when a launch begins
   uint32_t start;             // the first round's histogram of the three
-  uint32_t pad[29];
+  uint32_t dead;              // a launch's wait gave up: later launches do nothing until the state is reset
+  uint32_t pad[28];
   uint32_t listed[kMaxK];     // elements listed
   uint32_t reach[kMaxK];      // approximate top-s: elements that reach theta
   uint2 list[kMaxK][kListCap];
@@ -93,6 +94,8 @@ __device__ __forceinline__ bool sampled_block(const TopkArgs& A, uint64_t key, u
 template <bool kBf16, bool kCluster>
 __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachArgs D, Scratch* S, int hist_k) {
   if (kCluster) griddep_wait();
+  const uint32_t dead = S->dead;
+  if (A.hold_tile >= 0 && blockIdx.x == gridDim.x - 1) return;  // test hook: the other blocks' waits give up
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Search sr[kMaxK];
   __shared__ uint32_t cnt[kItemMax];            // per item: sent elements, then its pairs' first slot
@@ -111,12 +114,6 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
   auto group_of = [&](int gi) { return me + gi * G; };
   const uint32_t lt = lanemask_lt();
 
-  if (me == 0 && threadIdx.x < kMaxK) {  // used after the first barrier
-    if (threadIdx.x < 8) A.step_ctr->v[threadIdx.x] = 0ull;
-    S->listed[threadIdx.x] = 0;
-    S->reach[threadIdx.x] = 0;
-    if ((int)threadIdx.x < K) A.sel[threadIdx.x].count = 0;
-  }
   uint32_t buf = S->start;  // 0, 1 or 2
   GridBarrier grid{&S->arrivals, S->base, A.wait_ns, &s_ok};
   // every block's writes so far are seen by every block (false: a wait gave up)
@@ -141,6 +138,13 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
   if (fused)
     for (int q = threadIdx.x; q < K * (kHistBins / 2); q += kSmThreads) hs[q] = 0;
   __syncthreads();
+  if (dead) return;  // (every block: set by a launch before, or by this one, whose waits then give up)
+  if (me == 0 && threadIdx.x < kMaxK) {  // used after the first barrier
+    if (threadIdx.x < 8) A.step_ctr->v[threadIdx.x] = 0ull;
+    S->listed[threadIdx.x] = 0;
+    S->reach[threadIdx.x] = 0;
+    if ((int)threadIdx.x < K) A.sel[threadIdx.x].count = 0;
+  }
 
   // ---- form v ----
   unsigned long long nonfinite = 0;
@@ -462,7 +466,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
     }
   }
   if (!ok) {
-    if (threadIdx.x == 0) atomicOr(A.status, kStatusTimeout);
+    if (threadIdx.x == 0) {
+      atomicOr(A.status, kStatusTimeout);
+      S->dead = 1;
+    }
     return;
   }
   if (me == 0) {

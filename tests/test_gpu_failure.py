@@ -4,7 +4,7 @@
   bulk pass, so the waits on it give up after a short limit; the kernel
   returns, gmc_check reports GMC_ETIMEOUT, and a reset (or a new handle) steps
   exactly as the oracle again. Likewise a block that leaves before a grid
-  barrier of gmc_topk_noalloc.
+  barrier of gmc_topk_noalloc or of the one-launch top-k step.
 * A device allocation that fails: the allocation hook makes the n-th
   allocation of gmc_create / gmc_set_variant fail as cudaMalloc does when
   memory runs out; the call returns GMC_ENOMEM, leaks nothing, and leaves an
@@ -78,6 +78,46 @@ def test_withheld_copy_times_out_and_is_reported(compressor, d, K, hold):
     p2.gpu.close()
 
 
+@pytest.mark.parametrize("compressor,d,K", [("topk", 50_003, 4), ("topk", 900_007, 7), ("topk_approx", 300_001, 3)])
+def test_one_launch_step_whose_wait_gives_up(compressor, d, K):
+    """A block that never comes to the barrier: the step is reported, the steps
+    after it leave the state alone, and a reset handle steps as the oracle does."""
+    import torch
+    lib = _lib()
+    rng = np.random.default_rng(d)
+    p = Pair(d, K, 0.9, 0.1, compressor=compressor, ratio=0.01, seed=3)
+    p.compare(p.step(_grads(rng, K, d)))
+    assert lib.gmc_test_leave_barrier(p.gpu.h, 20_000_000) == GMC_OK
+    g = torch.from_numpy(_grads(rng, K, d)).cuda()
+    p.gpu.step(g)
+    assert p.gpu.check() == GMC_ETIMEOUT
+    state = [p.gpu.residual(k).clone() for k in range(K)] + [p.gpu.params().clone()]
+    for _ in range(3):
+        p.gpu.step(g)
+    assert p.gpu.check() == GMC_ETIMEOUT
+    after = [p.gpu.residual(k) for k in range(K)] + [p.gpu.params()]
+    assert all(torch.equal(a, b) for a, b in zip(state, after))
+    w0 = (np.random.default_rng(5).standard_normal(d) * 0.01).astype(np.float32)
+    p.gpu.set_params(torch.from_numpy(w0).cuda())
+    p.ref.set_params(w0)
+    assert p.gpu.check() == GMC_OK
+    for _ in range(3):
+        p.compare(p.step(_grads(rng, K, d)))
+    p.compare_stats()
+    assert p.gpu.check() == GMC_OK
+
+
+def test_leave_barrier_refused_without_a_grid_barrier():
+    import torch
+    from paper_1905_12948_gb300 import GMC
+    lib = _lib()
+    for d, K in [(1_000, 2), (1_300_001, 20)]:  # one cluster; load/store pass
+        h = GMC(d, K, 0.9, 0.1, compressor="topk", ratio=0.01)
+        h.set_params(torch.zeros(d, device="cuda"))
+        assert lib.gmc_test_leave_barrier(h.h, 1_000_000) == GMC_EINVAL
+        h.close()
+
+
 @pytest.mark.parametrize("n,k", [(20_000, 300), (3_000_001, 3_000), (100_000, 100_000)])
 def test_noalloc_wait_that_gives_up_marks_its_output(n, k):
     """A block that never comes to the barrier: the call returns, its indices say
@@ -98,8 +138,7 @@ def test_noalloc_wait_that_gives_up_marks_its_output(n, k):
 
     want = oracle.top_s_support(x_np, k)
     assert np.array_equal(call(), want)
-    assert lib.gmc_test_leave_barrier(5_000_000_000) == GMC_EINVAL
-    assert lib.gmc_test_leave_barrier(20_000_000) == GMC_OK
+    assert lib.gmc_test_leave_barrier(None, 20_000_000) == GMC_OK
     assert np.all(call() == -1)
     assert np.array_equal(call(), want)
 
