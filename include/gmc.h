@@ -197,15 +197,21 @@ int gmc_set_params(gmc_t h, const float* w0_dev, void* stream);
  * deterministically and are reported by gmc_check as GMC_ENONFINITE.
  *
  * Deferred aggregation (top-k on the bulk pass: 2 to 16 workers and d >= 8 *
- * 4096 * SMs, about 5 M on GB300): the step selects and records C(e_{t+1/2,k}) but leaves the last line of
- * Alg. 1 -- w_{t+1} = w_t - (eta/K) sum_k C_k and the zeroing of the sent
- * residuals -- to the next gmc_step, whose single pass over the tiles applies
- * it before forming its own accumulator. The results are the same, bit for
- * bit: every call that reads the state (gmc_get_params, gmc_get_residual,
- * gmc_get_worker_params, gmc_get_stats) first applies a pending aggregation,
- * on its own stream after the step. gmc_step_host and a set detach output
- * apply it within the step. Because a getter writes the state, a getter on
- * one stream and a later gmc_step on another are ordered by the library. */
+ * 4096 * SMs, about 5 M on GB300): the step selects and records
+ * C(e_{t+1/2,k}) but leaves the last line of Alg. 1 -- w_{t+1} = w_t -
+ * (eta/K) sum_k C_k and the zeroing of the sent residuals -- to the next
+ * gmc_step, whose single pass over the tiles applies it before forming its own
+ * accumulator. The results are the same, bit for bit: every call that reads the
+ * state (gmc_get_params, gmc_get_residual, gmc_get_worker_params, gmc_get_stats)
+ * first applies a pending aggregation, on its own stream after the step.
+ * gmc_step_host and a set detach output apply it within the step.
+ *
+ * Order across streams (top-k with up to 16 workers and d >= 2 * 4096 * SMs,
+ * about 1.25 M on GB300): gmc_get_params, gmc_get_residual and
+ * gmc_get_worker_params run after the last gmc_step, and a later gmc_step after
+ * them, whatever streams they take (a step captured into a graph excepted,
+ * unless its aggregation is pending). Other handles' calls, and steps on
+ * several streams, are ordered by the caller. */
 int gmc_step(gmc_t h, const float* grads_dev, void* stream);
 
 /* gmc_step_host -- gmc_step from host memory grads_host (K x d fp32,

@@ -86,6 +86,12 @@ struct gmc_ctx {
   cudaStream_t aux = nullptr;  // library stream for flushes outside a caller stream
   cudaEvent_t ev_step = nullptr, ev_flush = nullptr;
   bool wait_flush = false;     // the next launch waits for ev_flush
+  // Reads of the state are ordered with the steps across streams where they
+  // were when such sizes deferred their aggregation (bulk_able): ev_step follows
+  // the last step on stream step_id (unless that was being captured), ev_flush
+  // the last read, on stream read_id.
+  bool step_marked = false;
+  unsigned long long step_id = 0, read_id = 0;
   uint32_t* bitmap = nullptr;
   int32_t* rank = nullptr;
   int32_t* blocks = nullptr;
@@ -456,12 +462,28 @@ cudaError_t lay_out(gmc_ctx* h, bool bulk) {
     if (err_ != cudaSuccess) return status_of(err_); \
   } while (0)
 
-// Work on s that reads or writes the state waits for a flush that may have
-// been enqueued on another stream since the last step; a step (clear = true)
-// resets the flag, later work is ordered after that step by the caller.
+// A stream's id, unique over the process's life (a handle may be given again
+// to a later stream); 0 where there is none.
+unsigned long long stream_id(cudaStream_t s) {
+  unsigned long long id = 0;
+  if (cudaStreamGetId(s, &id) == cudaSuccess) return id;
+  cudaGetLastError();
+  return 0;
+}
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &c) == cudaSuccess) return c != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // the default stream while another is captured
+  return true;
+}
+
+// Work on s that reads or writes the state waits for a read or a flush that may
+// have been enqueued on another stream since the last step; a step (clear =
+// true) resets the flag, later work is ordered after that step by the caller.
 cudaError_t order_after_flush(gmc_ctx* h, cudaStream_t s, bool clear) {
   if (!h->wait_flush) return cudaSuccess;
   if (clear) h->wait_flush = false;
+  if (h->read_id && h->read_id == stream_id(s)) return cudaSuccess;
   return cudaStreamWaitEvent(s, h->ev_flush, 0);
 }
 
@@ -584,24 +606,60 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
   if (!finalized)
     GMC_TRY(timed(h, GMC_KERNEL_OTHER, 0.0, s,
                   [&] { return launch_finalize(h->step_ctr, h->total_ctr, pairs_add, s); }));
-  if (h->agg_pending) GMC_TRY(cudaEventRecord(h->ev_step, s));  // a flush on another stream waits for it
+  // a flush or a read on another stream waits for it
+  h->step_marked = h->agg_pending || (h->bulk_able && !capturing(s));
+  if (h->step_marked) {
+    GMC_TRY(cudaEventRecord(h->ev_step, s));
+    h->step_id = stream_id(s);
+  }
   h->t += 1;
   h->restored = false;
   return GMC_OK;
 }
 
+// A read of the state on s runs after the last step, whatever stream that took.
+cudaError_t order_after_step(gmc_ctx* h, cudaStream_t s) {
+  if (!h->step_marked || (h->step_id && h->step_id == stream_id(s)) || (!h->agg_pending && capturing(s)))
+    return cudaSuccess;
+  return cudaStreamWaitEvent(s, h->ev_step, 0);
+}
+
+// What was enqueued on s is done before the next step or read on another stream.
+cudaError_t mark_read(gmc_ctx* h, cudaStream_t s) {
+  const cudaError_t err = cudaEventRecord(h->ev_flush, s);
+  if (err != cudaSuccess) return err;
+  h->read_id = stream_id(s);
+  h->wait_flush = true;
+  return cudaSuccess;
+}
+
 // Apply a pending aggregation on stream s (ordered after the last step).
 int flush(gmc_ctx* h, cudaStream_t s) {
   if (!h->agg_pending) return GMC_OK;
-  GMC_TRY(cudaStreamWaitEvent(s, h->ev_step, 0));
+  GMC_TRY(order_after_step(h, s));
   TopkArgs A = topk_args_at(h, nullptr, h->t - 1);
   A.a_prev = h->a_pending;
   A.step_ctr = h->step_ctr;    // the counts belong to the last step
   A.total_ctr = h->total_ctr;  // which k_finalize has already added up
   GMC_TRY(launch_apply(A, h->grid_agg, s));
-  GMC_TRY(cudaEventRecord(h->ev_flush, s));
-  h->wait_flush = true;
+  GMC_TRY(mark_read(h, s));
   h->agg_pending = false;
+  return GMC_OK;
+}
+
+// A getter's read of the state on s: `read` after what writes it, and before
+// the next step, whatever streams these take.
+template <typename F>
+int read_state(gmc_ctx* h, cudaStream_t s, F&& read) {
+  const bool flushed = h->agg_pending;
+  const int st = flush(h, s);
+  if (st != GMC_OK) return st;
+  if (!flushed) {
+    GMC_TRY(order_after_flush(h, s, false));
+    GMC_TRY(order_after_step(h, s));
+  }
+  GMC_TRY(read());
+  if (h->bulk_able && (flushed || !capturing(s))) GMC_TRY(mark_read(h, s));
   return GMC_OK;
 }
 
@@ -956,20 +1014,16 @@ int gmc_get_params(gmc_t h, float* w_dev_out, void* stream) {
   if (!h || !w_dev_out) return GMC_EINVAL;
   if (!h->initialized) return GMC_ESTATE;
   DeviceGuard g(h->device);
-  GMC_TRY_ST(flush(h, static_cast<cudaStream_t>(stream)));
-  GMC_TRY(order_after_flush(h, static_cast<cudaStream_t>(stream), false));
-  GMC_TRY(launch_copy_row(h->w, w_dev_out, h->d, static_cast<cudaStream_t>(stream)));
-  return GMC_OK;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  return read_state(h, s, [&] { return launch_copy_row(h->w, w_dev_out, h->d, s); });
 }
 
 int gmc_get_residual(gmc_t h, int32_t k, float* e_dev_out, void* stream) {
   if (!h || !e_dev_out || k < 0 || k >= h->K) return GMC_EINVAL;
   if (!h->initialized) return GMC_ESTATE;
   DeviceGuard g(h->device);
-  GMC_TRY_ST(flush(h, static_cast<cudaStream_t>(stream)));
-  GMC_TRY(order_after_flush(h, static_cast<cudaStream_t>(stream), false));
-  GMC_TRY(launch_copy_row(h->e + (int64_t)k * h->ld, e_dev_out, h->d, static_cast<cudaStream_t>(stream)));
-  return GMC_OK;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  return read_state(h, s, [&] { return launch_copy_row(h->e + (int64_t)k * h->ld, e_dev_out, h->d, s); });
 }
 
 int64_t gmc_selected_capacity(gmc_t h) {
@@ -984,6 +1038,7 @@ int gmc_get_selected(gmc_t h, int32_t k, uint32_t* idx_dev, float* val_dev, int6
   if (!h->initialized || h->t == 0 || h->restored) return GMC_ESTATE;
   DeviceGuard g(h->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  GMC_TRY(order_after_step(h, s));
   if (h->compressor != GMC_RBGS) {
     int64_t count = h->ksel;
     if (h->compressor == GMC_TOPK_APPROX) {  // the count varies by step: read it
@@ -1016,11 +1071,9 @@ int gmc_get_worker_params(gmc_t h, int32_t k, float* out_dev, void* stream) {
   if (!h || !out_dev || k < 0 || k >= h->K) return GMC_EINVAL;
   if (!h->initialized) return GMC_ESTATE;
   DeviceGuard g(h->device);
-  GMC_TRY_ST(flush(h, static_cast<cudaStream_t>(stream)));
-  GMC_TRY(order_after_flush(h, static_cast<cudaStream_t>(stream), false));
-  DetachArgs D{h->w, h->e, h->ld, h->d, detach_b(h), out_dev, h->d, k, k + 1};
-  GMC_TRY(launch_detach(D, static_cast<cudaStream_t>(stream)));
-  return GMC_OK;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const DetachArgs D{h->w, h->e, h->ld, h->d, detach_b(h), out_dev, h->d, k, k + 1};
+  return read_state(h, s, [&] { return launch_detach(D, s); });
 }
 
 int gmc_get_stats(gmc_t h, uint64_t* counters_host, int32_t n, double* rcc_host) {

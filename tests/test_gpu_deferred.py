@@ -13,7 +13,7 @@ import math
 import numpy as np
 import pytest
 
-from parity_util import Pair
+from parity_util import Pair, bits
 
 pytestmark = pytest.mark.gpu
 
@@ -57,6 +57,65 @@ def test_state_read_on_another_stream_between_deferred_steps():
                                           p.ref.w.astype(np.float32).view(np.uint32))
     p.compare(r)
     p.compare_stats()
+
+
+@pytest.mark.parametrize("compressor,d,K,ratio", [
+    ("topk", 1_300_001, 3, 0.01),         # the one-launch step
+    ("topk", 1_300_001, 8, 0.01),         # load/store pass
+    ("topk", 8_000_001, 1, 0.002),        # load/store pass, one worker
+    ("topk_approx", 2_000_003, 16, 0.002),
+    ("topk", 5_100_001, 2, 0.002),        # bulk pass, deferred
+])
+def test_reads_on_another_stream_enqueued_right_behind_the_step(compressor, d, K, ratio):
+    """Nothing waits on the host between a step, reads of the state on another
+    stream and the next step: each read sees the state between the two steps,
+    though the first stream is held up before its step, the other before its reads."""
+    import torch
+    rng = np.random.default_rng(d + K)
+    p = Pair(d, K, 0.8, 0.05, compressor=compressor, ratio=ratio, seed=5)
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    hold = 4_000_000  # clock cycles: about 2 ms
+    grads = [_grads(rng, K, d) for _ in range(4)]
+    dev = [torch.from_numpy(g).to(p.dev) for g in grads]
+    outs = []
+    torch.cuda.synchronize()
+    for g in dev:
+        with torch.cuda.stream(a):
+            torch.cuda._sleep(hold)
+            p.gpu.step(g)
+        with torch.cuda.stream(b):
+            torch.cuda._sleep(hold)
+            outs.append([p.gpu.params(), p.gpu.residual(K - 1), p.gpu.worker_params(0)])
+    torch.cuda.synchronize()
+    for g, o in zip(grads, outs):
+        p.ref.step(g)
+        for x, want in zip(o, (p.ref.w, p.ref.e[K - 1], p.ref.worker_params(0))):
+            assert np.array_equal(bits(x.cpu().numpy()), bits(want))
+    p.compare_stats()
+    assert p.gpu.check() == 0
+
+
+def test_read_and_next_step_on_different_streams():
+    """A read on the step's own stream, and the next step on another one behind it."""
+    import torch
+    d, K = 1_300_001, 8
+    rng = np.random.default_rng(9)
+    p = Pair(d, K, 0.8, 0.05, ratio=0.01, seed=5)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    grads = [_grads(rng, K, d) for _ in range(4)]
+    dev = [torch.from_numpy(g).to(p.dev) for g in grads]
+    outs = []
+    torch.cuda.synchronize()
+    for t, g in enumerate(dev):
+        s = streams[t % 2]
+        with torch.cuda.stream(s):
+            p.gpu.step(g)
+            torch.cuda._sleep(4_000_000)
+            outs.append(p.gpu.residual(2))
+    torch.cuda.synchronize()
+    for g, o in zip(grads, outs):
+        p.ref.step(g)
+        assert np.array_equal(bits(o.cpu().numpy()), bits(p.ref.e[2]))
 
 
 def test_deferred_steps_mixed_with_host_steps_and_detach():
