@@ -116,8 +116,8 @@ __device__ __forceinline__ float4 load_g4_bf16(const uint16_t* g, int64_t j, int
 }
 
 // Elements j .. j+3 of an fp32 row of d, zeros past d; mode: g_mode of the row.
-__device__ __forceinline__ float4 load_g4(const float* __restrict__ g, int64_t j, int64_t d,
-                                          int mode) {
+// (Not __restrict__: the kernel that writes the row may end only after this one began.)
+__device__ __forceinline__ float4 load_g4(const float* g, int64_t j, int64_t d, int mode) {
   if (j + 3 < d) {
     if (mode == 4) return __ldcs(reinterpret_cast<const float4*>(g + j));
     if (mode == 2) {
@@ -549,7 +549,7 @@ __device__ __forceinline__ int64_t tile_order(int64_t i, int64_t n_tiles, const 
   const uint32_t G = gridDim.x, nb = (uint32_t)(n_tiles / G);
   if ((uint64_t)i >= (uint64_t)nb * G) return i;
   const uint32_t b = (uint32_t)i / G, o = (uint32_t)i - b * G;
-  const uint32_t ob = __ldg(order + b);
+  const uint32_t ob = order[b];  // (a plain load: a kernel just before wrote it)
   return (int64_t)(ob < nb ? ob : b) * G + o;
 }
 template <int kFixed, int kQ>

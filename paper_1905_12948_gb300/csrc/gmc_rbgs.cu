@@ -412,8 +412,10 @@ __global__ void __launch_bounds__(kThreads) k_detach(DetachArgs A, int per) {
 // dst[0..n) = src[0..n), src 16-byte aligned and readable to the next 128
 // floats. As fast as cudaMemcpyAsync at every size (138.4 M floats: 169 against
 // 170 us) and begins while the kernel before it ends (d = 272 k: 1.8 against
-// 5.4 us on the device, 11.4 against 17 us a call on the host).
-__global__ void __launch_bounds__(kThreads) k_copy_row(const float* __restrict__ src, float* dst, int64_t n) {
+// 5.4 us on the device, 11.4 against 17 us a call on the host). src is not
+// __restrict__: the kernel before, which writes it, may still run when this one
+// begins, so its loads must not be taken for loads of constant memory.
+__global__ void __launch_bounds__(kThreads) k_copy_row(const float* src, float* dst, int64_t n) {
   griddep_wait();
   const int lane = threadIdx.x & 31;
   const int64_t nw = (int64_t)gridDim.x * kWarps;
