@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachA
   // every block's writes so far are seen by every block (false: a wait gave up)
   auto barrier = [&]() -> bool {
     if (!kCluster) return grid.wait();
+    __syncwarp();  // (.aligned: a whole warp at once)
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     return true;
   };
