@@ -1015,7 +1015,7 @@ int gmc_get_params(gmc_t h, float* w_dev_out, void* stream) {
   if (!h->initialized) return GMC_ESTATE;
   DeviceGuard g(h->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  return read_state(h, s, [&] { return launch_copy_row(h->w, w_dev_out, h->d, s); });
+  return read_state(h, s, [&] { return launch_copy_row(h->w, w_dev_out, h->d, h->device, s); });
 }
 
 int gmc_get_residual(gmc_t h, int32_t k, float* e_dev_out, void* stream) {
@@ -1023,7 +1023,7 @@ int gmc_get_residual(gmc_t h, int32_t k, float* e_dev_out, void* stream) {
   if (!h->initialized) return GMC_ESTATE;
   DeviceGuard g(h->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  return read_state(h, s, [&] { return launch_copy_row(h->e + (int64_t)k * h->ld, e_dev_out, h->d, s); });
+  return read_state(h, s, [&] { return launch_copy_row(h->e + (int64_t)k * h->ld, e_dev_out, h->d, h->device, s); });
 }
 
 int64_t gmc_selected_capacity(gmc_t h) {

@@ -218,8 +218,8 @@ cudaError_t launch_rbgs_step(const RbgsArgs& A, int grid, cudaStream_t s);
 cudaError_t launch_rbgs_expand(const RbgsArgs& A, int k, uint32_t* idx_out, float* val_out,
                                cudaStream_t s);
 cudaError_t launch_detach(const DetachArgs& A, cudaStream_t s);
-// dst = src over n floats; src 16-byte aligned, allocated to a whole tile past n.
-cudaError_t launch_copy_row(const float* src, float* dst, int64_t n, cudaStream_t s);
+// dst = src over n floats; src 16-byte aligned, allocated on `device` to a whole tile past n.
+cudaError_t launch_copy_row(const float* src, float* dst, int64_t n, int device, cudaStream_t s);
 cudaError_t launch_finalize(Counters* step, Counters* total, unsigned long long pairs_add,
                             cudaStream_t s);
 

@@ -757,8 +757,14 @@ cudaError_t launch_detach(const DetachArgs& A, cudaStream_t s) {
   return launch_pdl(k_detach, grid, dim3(kThreads), 0, s, A, per);
 }
 
-cudaError_t launch_copy_row(const float* src, float* dst, int64_t n, cudaStream_t s) {
-  if (reinterpret_cast<uintptr_t>(dst) & 3u)
+cudaError_t launch_copy_row(const float* src, float* dst, int64_t n, int device, cudaStream_t s) {
+  // the kernel writes this device's memory; what else dst may be (host memory,
+  // another device's, no memory at all) is cudaMemcpyAsync's to copy to or refuse
+  cudaPointerAttributes at;
+  const cudaError_t err = cudaPointerGetAttributes(&at, dst);
+  if (err != cudaSuccess) cudaGetLastError();
+  if (err != cudaSuccess || at.type != cudaMemoryTypeDevice || at.device != device ||
+      (reinterpret_cast<uintptr_t>(dst) & 3u))
     return cudaMemcpyAsync(dst, src, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, s);
   const int64_t blocks = (n + 128 * kWarps - 1) / (128 * kWarps);
   return launch_pdl(k_copy_row, dim3((unsigned)blocks), dim3(kThreads), 0, s, src, dst, n);

@@ -16,7 +16,7 @@ import gc
 import numpy as np
 import pytest
 
-from parity_util import Pair
+from parity_util import Pair, bits
 
 pytestmark = pytest.mark.gpu
 
@@ -105,6 +105,29 @@ def test_one_launch_step_whose_wait_gives_up(compressor, d, K):
         p.compare(p.step(_grads(rng, K, d)))
     p.compare_stats()
     assert p.gpu.check() == GMC_OK
+
+
+@pytest.mark.parametrize("compressor,d", [("topk", 5_003), ("rbgs", 5_003)])
+def test_getters_leave_other_destinations_to_the_copy_call(compressor, d):
+    """Host memory as a getter's destination: copied to or refused by the CUDA
+    copy call, as it decides, and never written by a kernel; pinned memory is
+    copied to. (The header asks for device memory.)"""
+    import torch
+    lib = _lib()
+    K = 2
+    p = Pair(d, K, 0.9, 0.1, compressor=compressor, ratio=0.05, block=64)
+    p.step(_grads(np.random.default_rng(2), K, d))
+    s = torch.cuda.current_stream().cuda_stream
+    for pinned in (True, False):
+        for read, want in ((lambda q: lib.gmc_get_params(p.gpu.h, q, s), p.ref.w),
+                           (lambda q: lib.gmc_get_residual(p.gpu.h, 1, q, s), p.ref.e[1])):
+            out = torch.zeros(d, pin_memory=pinned)
+            st = read(out.data_ptr())
+            torch.cuda.synchronize()
+            assert st == GMC_OK if pinned else st in (GMC_OK, 3)
+            if st == GMC_OK:
+                assert np.array_equal(bits(out.numpy()), bits(want))
+    p.compare(p.step(_grads(np.random.default_rng(3), K, d)))
 
 
 def test_leave_barrier_refused_without_a_grid_barrier():
