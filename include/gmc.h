@@ -206,6 +206,12 @@ int gmc_set_params(gmc_t h, const float* w0_dev, void* stream);
  * first applies a pending aggregation, on its own stream after the step.
  * gmc_step_host and a set detach output apply it within the step.
  *
+ * A small top-k problem (K x d up to about 7 M on GB300, sampled engine) is one
+ * launch whose blocks wait for one another: it begins when every SM it takes (up
+ * to all of them) has room for a block of up to 227 KB of shared memory, and where
+ * the context may use fewer SMs than that, the handle takes several launches a
+ * step instead, with the same results.
+ *
  * Order across streams (top-k with up to 16 workers and d >= 2 * 4096 * SMs,
  * about 1.25 M on GB300): gmc_get_params, gmc_get_residual and
  * gmc_get_worker_params run after the last gmc_step, and a later gmc_step after
@@ -372,6 +378,14 @@ int gmc_test_withhold_copy(gmc_t h, int64_t tile, int32_t k, uint64_t wait_limit
 int gmc_test_leave_barrier(gmc_t h, uint64_t wait_limit_ns);
 
 /*
+ * gmc_test_refuse_cooperative -- process-wide: the next `launches` launches whose
+ * blocks wait for one another (the one-launch step of small top-k problems,
+ * gmc_topk_noalloc) are answered as CUDA answers one that is too large for its
+ * context; 0 disarms the hook. GMC_EINVAL for a negative count.
+ */
+int gmc_test_refuse_cooperative(int64_t launches);
+
+/*
  * gmc_topk_noalloc -- the top-k compressor of one vector without allocating.
  * The paper has no counterpart: this is a library convenience for callers
  * that cannot call cudaMalloc, e.g. code whose device memory is all owned by
@@ -387,7 +401,8 @@ int gmc_test_leave_barrier(gmc_t h, uint64_t wait_limit_ns);
  * the process exits. All calls share that array, so calls that overlap on the
  * GPU (on different streams, or from different threads) race; serialise
  * them (calls that overlapped all the same spoil their own results only). It
- * runs as one kernel whose blocks wait for one another. Should such a wait give
+ * runs as one kernel whose blocks wait for one another, one to an SM (fewer where
+ * the context may use fewer), and begins when they all have room. Should a wait give
  * up (about two seconds without progress), entries of idx_dev are left as
  * 0xffffffff, which no index is: a result without such an entry is complete. The
  * next call is not affected.

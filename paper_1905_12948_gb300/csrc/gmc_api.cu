@@ -144,6 +144,8 @@ class DeviceGuard {
 std::atomic<int64_t> g_fail_countdown{-1};
 std::atomic<int64_t> g_live_allocations{0};  // device allocations held by all handles
 
+std::atomic<int64_t> g_refuse{0};  // test hook (gmc_test_refuse_cooperative): launches still to be refused
+
 bool injected_alloc_failure() {
   int64_t c = g_fail_countdown.load();
   while (c >= 0 && !g_fail_countdown.compare_exchange_weak(c, c - 1)) {
@@ -456,6 +458,17 @@ cudaError_t lay_out(gmc_ctx* h, bool bulk) {
   return err;
 }
 
+}  // namespace
+
+bool gmc::refuse_cooperative() {
+  int64_t c = g_refuse.load();
+  while (c > 0 && !g_refuse.compare_exchange_weak(c, c - 1)) {
+  }
+  return c > 0;
+}
+
+namespace {
+
 #define GMC_TRY(expr)                          \
   do {                                         \
     const cudaError_t err_ = (expr);           \
@@ -507,12 +520,7 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     GMC_TRY(lay_out(h, true));
     h->restored = h->t > 0;
   }
-  const bool small = h->grid_small && h->select_mode == GMC_SELECT_SAMPLED;
-  // the exact top-k's sample kernel and the RBGS pick clear the step's counters
-  // themselves (a memset between two kernels would keep the second from starting early)
-  if (h->compressor == GMC_TOPK_APPROX && !small) GMC_TRY(cudaMemsetAsync(h->step_ctr, 0, sizeof(Counters), s));
-  unsigned long long pairs_add = 0;
-  bool finalized = false;  // the step's counters already added up by its last kernel
+  bool small = h->grid_small && h->select_mode == GMC_SELECT_SAMPLED;
   if (small) {
     TopkArgs A = topk_args(h, grads);
     A.grads16 = grads16;
@@ -524,8 +532,23 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     }
     const DetachArgs D{h->w, h->e, h->ld, h->d, detach_b(h), h->detach_out, h->detach_ld, 0, h->K};
     const double bytes = ((A.local_mom ? 20.0 : 12.0) - (bf16 ? 2.0 : 0.0)) * Kd + (D.out ? 4.0 * Kd : 0.0);
-    GMC_TRY(timed(h, GMC_KERNEL_ACCUMULATE, bytes, s,
-                  [&] { return launch_topk_step(A, D, h->grid_small, h->small_cluster, h->small_scratch, s); }));
+    const cudaError_t err = timed(h, GMC_KERNEL_ACCUMULATE, bytes, s, [&] {
+      return launch_topk_step(A, D, h->grid_small, h->small_cluster, h->small_scratch, s);
+    });
+    if (too_large_here(err)) {  // not in this context: the load/store pass, which is laid out, from here on
+      cudaGetLastError();
+      h->grid_small = 0;
+      small = false;
+    } else {
+      GMC_TRY(err);
+    }
+  }
+  // the exact top-k's sample kernel and the RBGS pick clear the step's counters
+  // themselves (a memset between two kernels would keep the second from starting early)
+  if (h->compressor == GMC_TOPK_APPROX && !small) GMC_TRY(cudaMemsetAsync(h->step_ctr, 0, sizeof(Counters), s));
+  unsigned long long pairs_add = 0;
+  bool finalized = false;  // the step's counters already added up by its last kernel
+  if (small) {
     finalized = true;
   } else if (h->compressor != GMC_RBGS) {
     const bool approx = h->compressor == GMC_TOPK_APPROX;
@@ -1277,6 +1300,12 @@ int gmc_test_leave_barrier(gmc_t h, uint64_t wait_limit_ns) {
   }
   if (h->grid_small < 2 || h->small_cluster || h->select_mode != GMC_SELECT_SAMPLED) return GMC_EINVAL;
   h->leave_ns = wait_limit_ns;
+  return GMC_OK;
+}
+
+int gmc_test_refuse_cooperative(int64_t launches) {
+  if (launches < 0) return GMC_EINVAL;
+  g_refuse.store(launches);
   return GMC_OK;
 }
 

@@ -193,6 +193,15 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// The answer to a cooperative or cluster launch whose blocks cannot all be
+// resident in this context (an MPS share, a green context, a partitioned GPU).
+inline bool too_large_here(cudaError_t e) {
+  return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize ||
+         e == cudaErrorLaunchOutOfResources || e == cudaErrorInvalidConfiguration || e == cudaErrorNotSupported;
+}
+// Test hook (gmc_test_refuse_cooperative): true for the launches it refuses.
+bool refuse_cooperative();
+
 // Launch wrappers (each returns the cudaGetLastError of its launches).
 cudaError_t launch_sample(const TopkArgs& A, cudaStream_t s);
 cudaError_t launch_accumulate(const TopkArgs& A, int grid, cudaStream_t s);

@@ -5,7 +5,7 @@
 // the library holds that array until the process exits.
 //
 // One cooperative launch, a block per SM. x is cut into chunks of 512 to 2,048
-// values, dealt to the blocks in turn (the selected values of a layered
+// values (up to 32,768 where only a few blocks may run), dealt to the blocks in turn (the selected values of a layered
 // gradient lie close together: with a contiguous slice a block, one block wrote
 // most of them), and within a block taken by the warps as they come:
 //   sample   8,192 values a block (all of x up to 1.2 M): two radix digits of
@@ -757,8 +757,18 @@ extern "C" int gmc_topk_noalloc(const float* x_dev, int64_t n, int64_t k, uint32
   const uint64_t leave_ns = g_leave_ns.exchange(0);
   // the launch's own error: earlier, unrelated work's is neither read nor cleared
   cudaError_t err = cudaMemsetAsync(dv.scratch, 0, offsetof(NaScratch, above), cfg.stream);
-  if (err == cudaSuccess)
-    err = cudaLaunchKernelEx(&cfg, k_na_topk, x_dev, n, (uint32_t)k, dv.scratch, idx_dev, val_dev,
-                             leave_ns ? leave_ns : kWaitLimitNs, leave_ns ? 1 : 0);
+  if (err != cudaSuccess) return GMC_ECUDA;
+  // fewer blocks where the context may use fewer SMs than the device has, as long
+  // as kNaOwn chunks of at most 2^15 values (16-bit counts) a block cover x
+  const unsigned least = (unsigned)((n + 3 + kNaOwn * 32768ll - 1) / (kNaOwn * 32768ll));
+  for (;;) {
+    err = refuse_cooperative()
+              ? cudaErrorCooperativeLaunchTooLarge
+              : cudaLaunchKernelEx(&cfg, k_na_topk, x_dev, n, (uint32_t)k, dv.scratch, idx_dev, val_dev,
+                                   leave_ns ? leave_ns : kWaitLimitNs, leave_ns ? 1 : 0);
+    if (!too_large_here(err) || cfg.gridDim.x <= least) break;
+    cudaGetLastError();  // this launch's
+    cfg.gridDim.x = cfg.gridDim.x / 2 > least ? cfg.gridDim.x / 2 : least;
+  }
   return err == cudaSuccess ? GMC_OK : GMC_ECUDA;
 }

@@ -701,6 +701,7 @@ cudaError_t configure_small_kernels() {
 }
 cudaError_t launch_topk_step(const TopkArgs& A, const DetachArgs& D, int grid, bool cluster, uint32_t* scratch,
                              cudaStream_t s) {
+  if (refuse_cooperative()) return cudaErrorCooperativeLaunchTooLarge;
   const int hist_k = small_hist_k(A.d, A.K, grid);  // at least 8: kSmallItems leaves them room
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);

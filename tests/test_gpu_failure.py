@@ -130,6 +130,57 @@ def test_getters_leave_other_destinations_to_the_copy_call(compressor, d):
     p.compare(p.step(_grads(np.random.default_rng(3), K, d)))
 
 
+@pytest.mark.parametrize("compressor,d,K,ratio", [
+    ("topk", 1, 1, 1.0), ("topk", 4_099, 3, 0.01), ("topk", 32_768, 8, 0.01), ("topk", 65_537, 4, 0.01),
+    ("topk", 900_007, 7, 0.002), ("topk", 1_300_001, 3, 0.01),
+    ("topk_approx", 5, 2, 0.5), ("topk_approx", 40_001, 5, 0.01), ("topk_approx", 300_001, 3, 0.01),
+])
+@pytest.mark.parametrize("variant,lam", [("gmc", 0.5), ("server_momentum", None), ("local_momentum_mfm", 0.3)])
+def test_one_launch_step_refused_by_its_context(compressor, d, K, ratio, variant, lam):
+    """A context with fewer SMs than the one-launch step's blocks: the step that is
+    refused and those after it take the load/store pass and give the same."""
+    import torch
+    lib = _lib()
+    rng = np.random.default_rng(d)
+    p = Pair(d, K, 0.9, 0.1, compressor=compressor, ratio=ratio, seed=3, variant=variant, lam=lam)
+    out = torch.zeros(K, d, device="cuda")
+    if lam is not None:
+        assert lib.gmc_set_detach_output(p.gpu.h, out.data_ptr(), d) == GMC_OK
+    for t in range(5):
+        if t == 2:
+            assert lib.gmc_test_refuse_cooperative(1) == GMC_OK
+        r = p.step(_grads(rng, K, d))
+        p.compare(r, workers=sorted({0, K - 1}))
+        if lam is not None:
+            assert np.array_equal(bits(out[K - 1].cpu().numpy()), bits(p.ref.worker_params(K - 1)))
+    p.compare_stats()
+    assert p.gpu.check() == GMC_OK
+    p.gpu.profile()
+    p.step(_grads(rng, K, d))
+    assert "dense_select" in p.gpu.profile_read()  # the load/store pass
+
+
+@pytest.mark.parametrize("n,k,refused", [(20_000, 300, 1), (3_000_001, 3_000, 2), (3_000_001, 2_000_000, 7),
+                                         (30_000_000, 30_000, 8), ((1 << 26) - 3, 60_000, 6)])
+def test_noalloc_refused_by_its_context(n, k, refused):
+    """Fewer SMs than blocks: the call is repeated with half the blocks, down to one."""
+    import oracle
+    import torch
+    lib = _lib()
+    x_np = np.random.default_rng(n).standard_normal(n, dtype=np.float32)
+    x = torch.from_numpy(x_np).cuda()
+    idx = torch.zeros(k, dtype=torch.int32, device="cuda")
+    val = torch.zeros(k, dtype=torch.float32, device="cuda")
+    assert lib.gmc_test_refuse_cooperative(refused) == GMC_OK
+    assert lib.gmc_topk_noalloc(x.data_ptr(), n, k, idx.data_ptr(), val.data_ptr(),
+                                torch.cuda.current_stream().cuda_stream) == GMC_OK
+    assert lib.gmc_test_refuse_cooperative(0) == GMC_OK
+    torch.cuda.synchronize()
+    want = oracle.top_s_support(x_np, k)
+    assert np.array_equal(idx.cpu().numpy(), want)
+    assert np.array_equal(bits(val.cpu().numpy()), bits(x_np[want]))
+
+
 def test_leave_barrier_refused_without_a_grid_barrier():
     import torch
     from paper_1905_12948_gb300 import GMC
