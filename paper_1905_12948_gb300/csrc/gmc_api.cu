@@ -417,15 +417,23 @@ cudaError_t lay_out(gmc_ctx* h, bool bulk) {
   // up to 16 times when there are few tiles, as a layer that holds most of the
   // candidates then spans few CTAs (1/64 of 1,221 tiles: 8 times the share; with
   // twice, d = 5 M, K = 8, ratio 0.01 overflowed into the dense path, 7.6 ms a
-  // step) -- plus slack, in whole 128-byte lines. Otherwise one region.
+  // step) -- plus slack, in whole 128-byte lines. Not more than such a layer can
+  // bring: cap0 candidates fill at least cap0 / 4,096 tiles, consecutive ones go
+  // to different CTAs, and a part gets 512 coordinates of each of its CTA's (two
+  // tiles more for CTAs that claim faster; without this bound d = 5.1 M, K = 16
+  // took 19.6 GB of candidate slots at ratio 1, 2.5 at 0.1; with it 2.7 and 0.7).
+  // Otherwise one region.
   const uint32_t cap0 = h->cap0;
   if (h->tile == kBulkTile) {
     h->n_blk = (uint32_t)(h->n_tiles / h->grid_acc);
     h->blk_mul = golden_stride(h->n_blk);
     h->regions = h->grid_acc;
     const uint64_t times = std::min<uint64_t>(16, std::max<uint64_t>(2, 128ull * h->num_sms / (uint64_t)h->n_tiles));
-    const uint64_t share = (times * cap0 + h->regions * kChunksPerTile - 1) / (h->regions * kChunksPerTile);
-    h->cap_part = (uint32_t)((share + 128 + 31) & ~31ull);
+    const uint64_t parts = (uint64_t)h->regions * kChunksPerTile;
+    auto share = [&](uint64_t f) { return (f * cap0 + parts - 1) / parts; };
+    const uint64_t layer = (cap0 / ((uint64_t)kBulkTile * h->regions) + 3) * (kBulkTile / kChunksPerTile);
+    const uint64_t part = std::max(share(2), std::min(share(times), layer));
+    h->cap_part = (uint32_t)((part + 128 + 31) & ~31ull);
     h->cap_region = h->cap_part * kChunksPerTile;
   } else {
     h->regions = 1;

@@ -41,3 +41,18 @@ def test_candidates_of_one_layer_do_not_overflow_the_bulk_parts():
         g[:, 2_000_000:2_080_000] *= 1e3
         p.compare(p.step(g))
     assert p.compare_stats()["fallbacks"] == 0
+
+
+@pytest.mark.parametrize("ratio,most", [(1.0, 0.6e9), (0.1, 0.25e9), (0.01, 0.2e9)])
+def test_candidate_memory_at_large_ratios(ratio, most):
+    """Bulk pass, d = 5.1 M, K = 2: e, w and the like take 0.12 GB; the candidates'
+    parts at most twice the expected candidates, or what one layer can bring."""
+    import torch
+    from paper_1905_12948_gb300 import GMC
+    GMC(5_100_001, 2, 0.9, 0.1, compressor="topk", ratio=0.001).close()  # the library's kernels are loaded
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    h = GMC(5_100_001, 2, 0.9, 0.1, compressor="topk", ratio=ratio)
+    used = before - torch.cuda.mem_get_info()[0]
+    h.close()
+    assert used <= most, f"{used / 1e9:.2f} GB"
