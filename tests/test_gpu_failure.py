@@ -161,7 +161,7 @@ def test_one_launch_step_refused_by_its_context(compressor, d, K, ratio, variant
 
 
 @pytest.mark.parametrize("n,k,refused", [(20_000, 300, 1), (3_000_001, 3_000, 2), (3_000_001, 2_000_000, 7),
-                                         (30_000_000, 30_000, 8), ((1 << 26) - 3, 60_000, 6)])
+                                         (30_000_000, 30_000, 7), ((1 << 26) - 3, 60_000, 6)])
 def test_noalloc_refused_by_its_context(n, k, refused):
     """Fewer SMs than blocks: the call is repeated with half the blocks, down to one."""
     import oracle
