@@ -215,9 +215,10 @@ int gmc_set_params(gmc_t h, const float* w0_dev, void* stream);
  * Order across streams (top-k with up to 16 workers and d >= 2 * 4096 * SMs,
  * about 1.25 M on GB300): gmc_get_params, gmc_get_residual and
  * gmc_get_worker_params run after the last gmc_step, and a later gmc_step after
- * them, whatever streams they take (a step captured into a graph excepted,
- * unless its aggregation is pending). Other handles' calls, and steps on
- * several streams, are ordered by the caller. */
+ * them, whatever streams they take. All else is ordered by the caller: other
+ * sizes, steps on several streams, and reads after gmc_step_host, a step with a
+ * detach output set, one under Alg. 3 or momentum factor masking, or one captured
+ * into a graph (unless its aggregation is pending). */
 int gmc_step(gmc_t h, const float* grads_dev, void* stream);
 
 /* gmc_step_host -- gmc_step from host memory grads_host (K x d fp32,

@@ -86,10 +86,10 @@ struct gmc_ctx {
   cudaStream_t aux = nullptr;  // library stream for flushes outside a caller stream
   cudaEvent_t ev_step = nullptr, ev_flush = nullptr;
   bool wait_flush = false;     // the next launch waits for ev_flush
-  // Reads of the state are ordered with the steps across streams where they
-  // were when such sizes deferred their aggregation (bulk_able): ev_step follows
-  // the last step on stream step_id (unless that was being captured), ev_flush
-  // the last read, on stream read_id.
+  // Reads of the state are ordered with the steps across streams where the
+  // aggregation is deferred, or would be on the bulk pass (bulk_able, and a form
+  // that defers): ev_step follows the last step on stream step_id (unless that
+  // was being captured), ev_flush the last read, on stream read_id.
   bool step_marked = false;
   unsigned long long step_id = 0, read_id = 0;
   uint32_t* bitmap = nullptr;
@@ -556,6 +556,9 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
   if (h->compressor == GMC_TOPK_APPROX && !small) GMC_TRY(cudaMemsetAsync(h->step_ctr, 0, sizeof(Counters), s));
   unsigned long long pairs_add = 0;
   bool finalized = false;  // the step's counters already added up by its last kernel
+  // the step's form defers its aggregation on the bulk pass: reads on other streams are ordered with it
+  const bool ordered = h->bulk_able && !eager && !h->detach_out && h->variant != GMC_VARIANT_SERVER_MOMENTUM &&
+                       h->variant != GMC_VARIANT_LOCAL_MOMENTUM_MFM;
   if (small) {
     finalized = true;
   } else if (h->compressor != GMC_RBGS) {
@@ -575,7 +578,7 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     if (h->dlt_next && !A.server_mom) A.dlt_out = h->dlt_next;
     // the tile order is built by k_sample_pending, which runs on these steps
     A.use_order = (h->blk_order && (A.pending || approx) && !A.dense_mode) ? 1 : 0;
-    const bool defer = h->tile == kBulkTile && !eager && !h->detach_out && !A.server_mom && !A.mfm;
+    const bool defer = h->tile == kBulkTile && ordered;
     const double kk = (double)h->K * (double)h->ksel;
     pairs_add = approx ? 0ull : (unsigned long long)h->K * h->ksel;  // approximate: counted on the device
     // deferred: the dense select is the step's last launch and ends it
@@ -638,7 +641,7 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     GMC_TRY(timed(h, GMC_KERNEL_OTHER, 0.0, s,
                   [&] { return launch_finalize(h->step_ctr, h->total_ctr, pairs_add, s); }));
   // a flush or a read on another stream waits for it
-  h->step_marked = h->agg_pending || (h->bulk_able && !capturing(s));
+  h->step_marked = h->agg_pending || (ordered && !capturing(s));
   if (h->step_marked) {
     GMC_TRY(cudaEventRecord(h->ev_step, s));
     h->step_id = stream_id(s);
@@ -690,7 +693,7 @@ int read_state(gmc_ctx* h, cudaStream_t s, F&& read) {
     GMC_TRY(order_after_step(h, s));
   }
   GMC_TRY(read());
-  if (h->bulk_able && (flushed || !capturing(s))) GMC_TRY(mark_read(h, s));
+  if (flushed || (h->step_marked && !capturing(s))) GMC_TRY(mark_read(h, s));
   return GMC_OK;
 }
 
