@@ -134,7 +134,6 @@ __device__ __forceinline__ void end_step(const RbgsArgs& A, unsigned long long* 
   if (lane == 0)
 #pragma unroll
     for (int i = 0; i < kEndWords; ++i) red[warp * kEndWords + i] = c[i];
-  __syncwarp();  // (bar.sync: a whole warp at once)
   asm volatile("bar.sync 1, %0;" ::"r"(warps * 32) : "memory");
   if (warp != 0) return;
   if (lane < kEndWords) {

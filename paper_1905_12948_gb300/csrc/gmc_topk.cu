@@ -1206,7 +1206,6 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
       sm.upos[sw][lane] = up;
       if (lane == 0) sm.pflag[sw] = many ? 1u : 0u;
     }
-    __syncwarp();  // (bar.sync: a whole warp at once)
     asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
     const bool many = sm.pflag[sw] != 0u;
     const uint32_t upos = sm.upos[sw][lane];
@@ -1219,7 +1218,6 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
       sm.next[sw] = (!ok || n + 1 >= (uint64_t)A.n_tiles) ? (uint32_t)A.n_tiles
                                                           : (uint32_t)tile_n(n + 1);
     // the lead warp rewrites the sub-tile's buffers for the next tile only after this
-    __syncwarp();
     asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
     float wn = 0.f;
     Pairs pnn{kNone, 0.f, 0, 0u};
@@ -1409,10 +1407,7 @@ __global__ void __launch_bounds__(bulk::kThreadsAll, 1) k_accumulate_bulk(TopkAr
       }
     }
     // the per-element masks of a many-sender sub-tile stay in use until both warps are done
-    if (many) {
-      __syncwarp();
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-    }
+    if (many) asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
     tile = (int64_t)sm.next[sw];  // written before this tile's second barrier, rewritten after the next one's first
   }
   if (!ok) atomicOr(A.status, kStatusTimeout);
