@@ -367,6 +367,13 @@ int64_t gmc_test_fail_alloc(int64_t fail_at);
 int gmc_test_withhold_copy(gmc_t h, int64_t tile, int32_t k, uint64_t wait_limit_ns);
 
 /*
+ * gmc_test_pass -- the pass that the next gmc_step of h takes by the sizes of its
+ * problem: 0 the load/store pass, 1 the bulk pass, 2 the one-launch step of small
+ * top-k problems; -1 for a NULL handle. For tests of one pass to say so.
+ */
+int gmc_test_pass(gmc_t h);
+
+/*
  * gmc_test_leave_barrier -- the next gmc_step of h, or with h = NULL the next
  * gmc_topk_noalloc of the process (only that one): one of its blocks leaves at
  * once, so the other blocks' waits for it give up after wait_limit_ns (1 .. 2e9;

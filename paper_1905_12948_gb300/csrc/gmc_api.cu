@@ -1303,6 +1303,13 @@ int gmc_test_withhold_copy(gmc_t h, int64_t tile, int32_t k, uint64_t wait_limit
   return GMC_OK;
 }
 
+int gmc_test_pass(gmc_t h) {
+  if (!h) return -1;
+  if (h->compressor == GMC_RBGS) return h->rbgs_bulk ? 1 : 0;
+  if (h->grid_small && h->select_mode == GMC_SELECT_SAMPLED) return 2;
+  return h->tile == kBulkTile ? 1 : 0;
+}
+
 int gmc_test_leave_barrier(gmc_t h, uint64_t wait_limit_ns) {
   if (wait_limit_ns > kWaitLimitNs) return GMC_EINVAL;
   if (!h) {

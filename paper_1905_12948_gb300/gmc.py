@@ -68,6 +68,7 @@ _SIGNATURES = {
     "gmc_topk_noalloc": (ctypes.c_int, [_c_p, _i64, _i64, _c_p, _c_p, _c_p]),
     "gmc_test_fail_alloc": (_i64, [_i64]),
     "gmc_test_withhold_copy": (ctypes.c_int, [_c_p, _i64, _i32, _u64]),
+    "gmc_test_pass": (ctypes.c_int, [_c_p]),
     "gmc_test_leave_barrier": (ctypes.c_int, [_c_p, _u64]),
     "gmc_test_refuse_cooperative": (ctypes.c_int, [_i64]),
 }

@@ -46,6 +46,10 @@ class Pair:
         self.gpu.set_params(torch.from_numpy(w0).to(self.dev))
         self.ref.set_params(w0)
 
+    def route(self):
+        """The pass that the handle's steps take."""
+        return {0: "load/store", 1: "bulk", 2: "one launch"}[self.gpu.lib.gmc_test_pass(self.gpu.h)]
+
     def step(self, g, grads_dev=None):
         if grads_dev is None:
             grads_dev = self.torch.from_numpy(np.ascontiguousarray(g)).to(self.dev)

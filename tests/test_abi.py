@@ -68,6 +68,7 @@ def test_failure_hooks_without_gpu(lib):
     assert lib.gmc_strerror(8).startswith(b"a bounded wait")
     assert lib.gmc_strerror(9) == b"unknown status"
     assert lib.gmc_test_withhold_copy(None, 0, 0, 1000) == 1
+    assert lib.gmc_test_pass(None) == -1
     assert lib.gmc_test_leave_barrier(None, 2_000_000_001) == 1
     assert lib.gmc_test_refuse_cooperative(-1) == 1
     assert lib.gmc_test_refuse_cooperative(0) == 0

@@ -25,7 +25,7 @@ def _check_counts(p, r):
 @pytest.mark.parametrize("d,K,ratio", [(50_000, 4, 0.01), (100, 2, 0.5), (99, 3, 0.01),
                                        (333_337, 5, 1 / 1024)])
 def test_approx_load_store_pass(d, K, ratio):
-    """Below the bulk pass's size: the load/store pass, aggregate each step."""
+    """Small problems: the one-launch step."""
     rng = np.random.default_rng(d + K)
     p = Pair(d, K, 0.9, 0.1, compressor="topk_approx", ratio=ratio, seed=7)
     for t in range(5):
@@ -38,7 +38,8 @@ def test_approx_load_store_pass(d, K, ratio):
 
 @pytest.mark.parametrize("d,K", [(1_300_001, 8), (4096 * 200, 3), (1_250_003, 1)])
 def test_approx_bulk_pass_deferred(d, K):
-    """The bulk pass with the aggregation deferred into the next step; the
+    """Steps in a row with only the selections read in between; on the bulk pass
+    (test_gpu_bulk_sizes.py) the aggregation is deferred into the next step; the
     selections are compared every step, the state at the end."""
     rng = np.random.default_rng(3 + K)
     p = Pair(d, K, 0.9, 0.05, compressor="topk_approx", ratio=1 / 1024, seed=11)
@@ -69,7 +70,7 @@ def test_approx_many_workers_and_eta_schedule():
 def test_approx_limit_takes_exact_top(d):
     """All-zero accumulators: theta is the zero key and every component
     reaches it, so the limit applies and the exact top (the lowest indices)
-    is sent, through the dense path, on both passes."""
+    is sent; on the load/store and bulk passes through the dense path."""
     import torch
     K = 2
     p = Pair(d, K, 0.9, 0.1, compressor="topk_approx", ratio=0.001, seed=1,
@@ -90,9 +91,10 @@ def test_approx_limit_takes_exact_top(d):
     del torch
 
 
-def test_approx_ties_all_sent():
+@pytest.mark.parametrize("d", [1_300_001])
+def test_approx_ties_all_sent(d):
     """Values from a small set: many components equal theta; all are sent."""
-    d, K = 1_300_001, 3
+    K = 3
     rng = np.random.default_rng(8)
     p = Pair(d, K, 0.0, 0.1, compressor="topk_approx", ratio=0.001, seed=5,
              w0=np.zeros(d, np.float32))
@@ -106,10 +108,11 @@ def test_approx_ties_all_sent():
     assert p.gpu.check() == 0
 
 
-def test_approx_host_steps_and_gmcplus_detach():
+@pytest.mark.parametrize("d", [1_300_001])
+def test_approx_host_steps_and_gmcplus_detach(d):
     """Host gradients (in place when page-locked) and the GMC+ detach output."""
     import torch
-    d, K = 1_300_001, 4
+    K = 4
     rng = np.random.default_rng(9)
     p = Pair(d, K, 0.9, 0.05, compressor="topk_approx", ratio=1 / 1024, seed=3, lam=0.5)
     out = torch.empty((K, d), dtype=torch.float32, device=p.dev)

@@ -22,9 +22,9 @@ def _fresh(p, **kw):
 
 
 CASES = [
-    dict(compressor="topk", d=1_300_001, K=4, ratio=0.002),               # bulk pass, deferred
-    dict(compressor="topk", d=1_300_001, K=6, ratio=0.002),               # and its one-tile pipeline
-    dict(compressor="topk", d=50_003, K=3, ratio=0.01),                   # load/store pass
+    dict(compressor="topk", d=1_300_001, K=4, ratio=0.002),               # one launch (the bulk pass: test_gpu_bulk_sizes.py)
+    dict(compressor="topk", d=1_300_001, K=6, ratio=0.002),               # load/store pass
+    dict(compressor="topk", d=50_003, K=3, ratio=0.01),
     dict(compressor="topk_approx", d=1_300_001, K=3, ratio=1 / 1024),
     dict(compressor="rbgs", d=4096 * 160 + 3, K=5, ratio=0.05, block=4096, lam=0.5),
     dict(compressor="rbgs", d=70_001, K=3, ratio=0.1, block=1000, lam=0.5, per_worker=True),

@@ -17,7 +17,10 @@ from parity_util import Pair, bits
 
 pytestmark = pytest.mark.gpu
 
-D_BULK = 1_300_001  # above the bulk-pass size; odd, so rows start at every alignment
+# Odd, so rows start at every alignment. At this size the one-launch step and the
+# load/store pass take these tests; test_gpu_bulk_sizes.py repeats them on the bulk
+# pass, which is the one that defers.
+D_BULK = 1_300_001
 
 
 def _grads(rng, K, d):

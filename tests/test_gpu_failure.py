@@ -34,7 +34,8 @@ def _grads(rng, K, d):
 
 
 @pytest.mark.parametrize("compressor,d,K,hold", [
-    ("topk", 1_300_001, 3, (5, 1)),      # bulk top-k pass (d >= 4096 * 2 * SMs), an odd worker
+    ("topk", 5_100_001, 6, (1_000, 3)),  # bulk top-k pass, the one-tile pipeline
+    ("topk", 1_300_001, 3, (5, 1)),      # moved to the bulk pass by the hook (d >= 4096 * 2 * SMs), an odd worker
     ("topk", 1_300_001, 4, (0, 0)),      # the first fixed tile of CTA 0, the lead warps' worker
     ("topk_approx", 1_300_001, 2, (317, 1)),  # the last tile, ragged
     ("rbgs", 700_001, 3, (40, 2)),       # bulk RBGS pass (d >= 4096 * SMs)
@@ -221,7 +222,7 @@ def test_withhold_refused_without_a_bulk_pass():
     import torch
     from paper_1905_12948_gb300 import GMC
     lib = _lib()
-    small = GMC(100_000, 2, 0.9, 0.1, compressor="topk", ratio=0.01)  # load/store pass
+    small = GMC(100_000, 2, 0.9, 0.1, compressor="topk", ratio=0.01)  # one launch, too small for the bulk pass
     small.set_params(torch.zeros(100_000, device="cuda"))
     assert lib.gmc_test_withhold_copy(small.h, 0, 0, 1_000_000) == GMC_EINVAL
     small.close()
@@ -234,8 +235,8 @@ def test_withhold_refused_without_a_bulk_pass():
 
 
 @pytest.mark.parametrize("d,K,compressor", [
-    (100_000, 4, 0),      # top-k, load/store pass
-    (1_300_001, 3, 0),    # top-k, bulk pass (candidate regions per CTA)
+    (100_000, 4, 0),      # top-k, one-launch step (the other passes: test_gpu_bulk_sizes.py)
+    (1_300_001, 3, 0),
     (700_001, 5, 1),      # RBGS
     (300_000, 2, 2),      # approximate top-s
 ])

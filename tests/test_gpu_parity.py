@@ -54,14 +54,14 @@ def test_topk_sampled_and_dense_agree_ragged_large():
     assert pairs[1].gpu.stats()["fallbacks"] == 4 * K
 
 
+@pytest.mark.parametrize("d,K", [(1_300_001, 3), (1_300_001, 8)])
 @pytest.mark.parametrize("offset", [0, 1])
-def test_topk_bulk_copy_path(offset):
-    """d large enough for the bulk-copy dense pass (tiles of 4096); odd d gives
-    rows at every alignment, and offset 1 makes the first row start 4 bytes
-    past an aligned address so its bulk copy would begin before the buffer
-    (that row is then loaded directly)."""
+def test_topk_bulk_copy_path(offset, d, K):
+    """Odd d gives rows at every alignment, and offset 1 makes the first row
+    start 4 bytes past an aligned address so that on the bulk pass its copy would
+    begin before the buffer (that row is then loaded directly). Here the one-launch
+    step and the load/store pass; test_gpu_bulk_sizes.py has the bulk pass."""
     import torch
-    d, K = 1_300_001, 3
     rng = np.random.default_rng(15 + offset)
     p = Pair(d, K, 0.9, 0.05, ratio=0.002, seed=2)
     for t in range(3):

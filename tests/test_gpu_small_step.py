@@ -14,16 +14,27 @@ pytestmark = pytest.mark.gpu
     (1, 1, 1.0), (5, 2, 0.5), (127, 3, 0.1), (129, 32, 0.05), (1_000, 9, 1.0),
     (128 * 17, 1, 0.02), (32_768, 4, 0.01), (32_769, 4, 0.01), (4_096, 32, 0.01),  # one cluster, up to its largest
     (128 * 152, 4, 0.01), (128 * 152 + 1, 5, 0.001), (210_001, 32, 0.01), (900_007, 8, 0.002),
-    (1_200_003, 1, 0.3), (1_244_159, 6, 0.001),   # the largest slices
+    (1_200_003, 1, 0.3), (128 * 152 * 94, 4, 0.001), (128 * 152 * 47 - 1, 8, 0.001),  # all of a block's 376 items
+    (128 * 152 * 376 - 3, 1, 0.001),
 ])
 def test_sizes(d, K, ratio, compressor):
     rng = np.random.default_rng(d + K)
     p = Pair(d, K, 0.9, 0.1, compressor=compressor, ratio=ratio, seed=4)
+    assert p.route() == "one launch"
     for t in range(3):
         g = (rng.standard_normal((K, d)) * np.exp(rng.uniform(-3, 0, size=d))).astype(np.float32)
         p.compare(p.step(g), workers=sorted({0, K - 1}))
     p.compare_stats()
     assert p.gpu.check() == 0
+
+
+@pytest.mark.parametrize("d,K", [(128 * 152 * 94 + 1, 4), (128 * 152 * 376 + 1, 1)])
+def test_one_coordinate_past_the_largest(d, K):
+    p = Pair(d, K, 0.9, 0.1, ratio=0.001)
+    assert p.route() == "load/store"
+    for t in range(2):
+        p.compare(p.step(np.random.default_rng(t).standard_normal((K, d), dtype=np.float32)))
+    p.compare_stats()
 
 
 @pytest.mark.parametrize("levels,ratio", [(1, 0.3), (3, 0.1), (200, 0.01), (200_000, 0.02)])
