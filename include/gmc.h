@@ -109,15 +109,16 @@ typedef struct gmc_ctx* gmc_t;
 #define GMC_STAT_COUNT      8 /* array length to pass */
 
 /* Kernel ids for gmc_profile_read. */
-#define GMC_KERNEL_ACCUMULATE  0 /* fused accumulator + candidate filter (top-k), one dense pass */
+#define GMC_KERNEL_ACCUMULATE  0 /* fused accumulator + candidate filter (top-k), one dense pass;
+                                    or the whole one-launch step of small problems */
 #define GMC_KERNEL_RBGS_STEP   1 /* fused accumulator + RBGS compress + aggregate + update */
 #define GMC_KERNEL_SAMPLE      2 /* sampled threshold per worker */
-#define GMC_KERNEL_SELECT      3 /* exact select among candidates (2 launches per step) */
+#define GMC_KERNEL_SELECT      3 /* exact select among candidates */
 #define GMC_KERNEL_DENSE       4 /* exact dense select for workers that fell back */
 #define GMC_KERNEL_COMPACT     5 /* reserved: no launch (the dense pass writes C(v) as
                                     index-ordered sub-chunks) */
-#define GMC_KERNEL_AGGREGATE   6 /* marks the sent pairs; when the aggregation is not
-                                    deferred also the worker-ordered aggregate + update */
+#define GMC_KERNEL_AGGREGATE   6 /* worker-ordered aggregate + update, when the aggregation is
+                                    not deferred */
 #define GMC_KERNEL_RBGS_PICK   7 /* RBGS block choice (Floyd sampling) */
 #define GMC_KERNEL_DETACH      8 /* GMC+ detached points */
 #define GMC_KERNEL_OTHER       9 /* counters and small bookkeeping */

@@ -1,7 +1,7 @@
 // C ABI of libgmc (declared in include/gmc.h): handle lifecycle, argument
 // validation, device state, and the orchestration of one GMC / GMC+ step on a
 // caller-given stream. Only host code lives here; the kernels are in
-// gmc_topk.cu and gmc_rbgs.cu.
+// gmc_topk.cu, gmc_small.cu, gmc_rbgs.cu and (gmc_topk_noalloc) gmc_noalloc.cu.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -793,7 +793,7 @@ int gmc_create(gmc_t* out, int64_t d, int32_t K, float beta, float eta, int32_t 
       const double r = (double)h->sample_rank;
       const double capd = std::ceil((double)ks * (1.0 + 5.0 / std::sqrt(r))) + 4096.0;
       h->cap = (uint32_t)std::min<double>((double)d, capd);
-    } else if (d <= kSampleAll) {
+    } else if (d <= kSampleAll) {  // (used where the context refuses the one-launch step)
       h->sample_chunks = 0;
       h->sample_rank = h->sample_rank_hi = h->ksel;
       h->cap = (uint32_t)d;

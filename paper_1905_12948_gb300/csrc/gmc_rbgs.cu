@@ -41,6 +41,19 @@ __device__ __forceinline__ uint32_t block_of(int64_t j, const RbgsArgs& A) {
 // thread of its own: a chain of a few shared-memory reads, where the serial
 // form cost about 50 ns a draw (m = 62: 9.9 us, m = 3,906: 200 us).
 // ---------------------------------------------------------------------------
+// Draw i's block: `first(b)` the first draw that gave block b, `drawn(i)` draw i. I: an index type.
+template <typename I, typename First, typename Drawn>
+__device__ __forceinline__ uint32_t floyd_pick(I i, I top0, First&& first, Drawn&& drawn) {
+  const uint32_t r0 = drawn(i);
+  I at = i, b = (I)r0;
+  while (first(b) >= (int32_t)at) {      // no draw before `at` gave block b
+    if (b < top0 || b - top0 >= at) return r0;  // nor is it an earlier step's top
+    at = b - top0;                       // taken iff that step took its top (`at` decreases at every turn)
+    b = (I)drawn(at);
+  }
+  return (uint32_t)(top0 + i);
+}
+
 constexpr int kPickThreads = 1024;
 constexpr int kFirstWords = 16384;  // first-draw table kept in shared memory up to this many blocks
 
@@ -71,19 +84,8 @@ __global__ void __launch_bounds__(kPickThreads) k_rbgs_pick(RbgsArgs A) {
   for (int64_t i = threadIdx.x; i < A.m; i += blockDim.x) atomicMin(&first[drawn(i)], (int32_t)i);
   __syncthreads();
   for (int64_t i = threadIdx.x; i < A.m; i += blockDim.x) {
-    const uint32_t r0 = drawn(i);
-    bool taken = false;
-    int64_t at = i, x = r0;
-    for (;;) {  // `at` decreases at every turn
-      if ((first_smem ? first[x] : __ldcg(first + x)) < (int32_t)at) {
-        taken = true;
-        break;
-      }
-      if (x < top0 || x - top0 >= at) break;
-      at = x - top0;  // taken iff that step took its top
-      x = drawn(at);
-    }
-    const uint32_t pick = taken ? (uint32_t)(top0 + i) : r0;
+    const uint32_t pick =
+        floyd_pick<int64_t>(i, top0, [&](int64_t b) { return first_smem ? first[b] : __ldcg(first + b); }, drawn);
     atomicOr(&bm[pick >> 5], 1u << (pick & 31));
   }
   __syncthreads();
@@ -121,8 +123,9 @@ __global__ void __launch_bounds__(kPickThreads) k_rbgs_pick(RbgsArgs A) {
 // shared memory, 5 words a warp; they meet at named barrier 1): the block's
 // counts into acc_ctr with one atomic each, and the last block out moves them to
 // step_ctr, adds them to the totals, leaves acc_ctr zero for the next step, and
-// clears the flags of the step before, which the next step's pick sets again. (With a set of atomics per warp the d = 272 k step's 2,129
-// warps queued at one line.)
+// clears the flags of the step before, which the next step's pick sets again.
+// (With a set of atomics per warp the d = 272 k step's 2,129 warps queued at one
+// line.)
 // ---------------------------------------------------------------------------
 constexpr int kEndWords = 5;
 __device__ __forceinline__ void end_step(const RbgsArgs& A, unsigned long long* red, int warp, int warps, int lane,
@@ -239,19 +242,8 @@ __device__ __forceinline__ Choice pick_here(const RbgsArgs& A, uint32_t* sm) {
   for (int x = threadIdx.x; x < streams * m; x += kThreads) {
     const int s = x / m, i = x - s * m;
     const uint64_t key = key_of(s);
-    const uint32_t r0 = drawn(key, i);
-    bool taken = false;
-    int at = i, b = (int)r0;
-    for (;;) {  // `at` decreases at every turn
-      if (first[s * nb + b] < at) {
-        taken = true;
-        break;
-      }
-      if (b < top0 || b - top0 >= at) break;
-      at = b - top0;
-      b = (int)drawn(key, at);
-    }
-    const uint32_t pick = taken ? (uint32_t)(top0 + i) : r0;
+    const uint32_t pick = floyd_pick<int>(i, top0, [&](int b) { return first[s * nb + b]; },
+                                          [&](int q) { return drawn(key, q); });
     atomicOr(&bm[s * nbw + (int)(pick >> 5)], 1u << (pick & 31));
   }
   __syncthreads();

@@ -58,8 +58,9 @@ __device__ __forceinline__ float4 scale_g(const TopkArgs& A, float4 g) {
 
 // Sampled coordinate of slot i of the exact top-k: kSampleRun (16) consecutive
 // coordinates from (c * d / chunks) rounded down to a multiple of kSampleRun,
-// c = 0 .. chunks-1 (every coordinate when chunks = 0); this sample only sets
-// the candidate threshold, never the result.
+// c = 0 .. chunks-1 (every coordinate when chunks = 0: d <= kSampleAll, whose
+// steps come here where the context refuses the one-launch step); this sample
+// only sets the candidate threshold, never the result.
 __device__ __forceinline__ int64_t sample_coord(const TopkArgs& A, int i) {
   if (!A.sample_chunks) return i;
   // sample_chunks is kSampleChunks, a power of two: floor(ch * d / kSampleChunks)
@@ -705,9 +706,8 @@ __device__ __forceinline__ uint32_t cand_bits(const float v[4], int l, int lim, 
 
 // Write one group's candidates (index order: lane-major, element-minor) at
 // pos; counts the non-finite ones (theta never exceeds the Inf key).
-__device__ __forceinline__ void write_group(const float v[4], uint32_t j, uint32_t bits, uint32_t lt,
-                                            uint32_t& pos, uint32_t end, uint32_t* ci, float* cv,
-                                            uint32_t& nonfinite) {
+__device__ __forceinline__ void write_group(const float v[4], uint32_t j, uint32_t bits, uint32_t& pos,
+                                            uint32_t end, uint32_t* ci, float* cv, uint32_t& nonfinite) {
   const uint32_t n = __popc(bits);
   if (!__any_sync(0xffffffffu, n != 0)) return;
   uint32_t incl = n;
@@ -718,7 +718,6 @@ __device__ __forceinline__ void write_group(const float v[4], uint32_t j, uint32
   }
   uint32_t o = pos + incl - n;
   pos += __shfl_sync(0xffffffffu, incl, 31);
-  (void)lt;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     if ((bits >> i) & 1u) {
@@ -750,7 +749,6 @@ __global__ void __launch_bounds__(kThreads) k_accumulate(TopkArgs A) {
   griddep_wait();
   constexpr int SUB = 128 * U;       // elements per item
   const int lane = threadIdx.x & 31;
-  const uint32_t lt = lanemask_lt();
   // items in blocks of kRun consecutive sub-tiles, worker after worker, so that
   // neighbouring warps read along one row
   constexpr uint32_t kRun = 64;
@@ -837,7 +835,7 @@ __global__ void __launch_bounds__(kThreads) k_accumulate(TopkArgs A) {
       uint32_t* hk = A.chist + (int64_t)k * kRelBins;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        write_group(v[u], s0 + u * 128 + lane * 4, bits[u], lt, pos, A.cap, ci, cv, nonfinite);
+        write_group(v[u], s0 + u * 128 + lane * 4, bits[u], pos, A.cap, ci, cv, nonfinite);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
           if ((bits[u] >> i) & 1u) atomicAdd(hk + rel_bin(mag_key(v[u][i]), th, (int)sh), 1u);
@@ -1466,7 +1464,8 @@ __device__ __forceinline__ void candidate_part(const TopkArgs& A, int k, int p, 
 // ---------------------------------------------------------------------------
 // exact select among candidates:
 //   hist    a kRelBins-bin histogram of the candidates' keys above theta,
-//           counted by the accumulate pass as it writes them, in bins of 2^shift keys that span the sampled keys around the k-th
+//           counted by the accumulate pass as it writes them, in bins of
+//           2^shift keys that span the sampled keys around the k-th
 //           (k_sample_cluster), so that they follow the data; every block of
 //           the next launch finds the bin holding the k-th key
 //   finish  the candidates of that bin are collected (key, index); the last
@@ -1477,7 +1476,7 @@ __device__ __forceinline__ void candidate_part(const TopkArgs& A, int k, int p, 
 __global__ void __launch_bounds__(kThreads) k_select_finish(TopkArgs A) {
   griddep_wait();
   // kBucketCap keys (the indices stay in the global bucket): 48 KB, so that
-  // four blocks fit on an SM and the grid runs in one wave
+  // three blocks fit on an SM and the grid runs in one wave
   extern __shared__ __align__(16) uint32_t fin[];
   __shared__ uint32_t h[kHistBins];
   __shared__ uint32_t ws[32];
@@ -1563,16 +1562,7 @@ __global__ void __launch_bounds__(kThreads) k_select_finish(TopkArgs A) {
       for (int q = 0; q < kQ; ++q) {
         const uint32_t i = i0 + q * 32 + lane;
         in[q] = i < total;
-        int lo = 0, hi = 32;  // the first lane whose inclusive count exceeds i (six halvings of 32)
-#pragma unroll
-        for (int it = 0; it < 6; ++it) {
-          const int mid = min((lo + hi) >> 1, 31);
-          const uint32_t v = __shfl_sync(0xffffffffu, incl, mid);
-          if (lo < hi) {
-            if (v <= i) lo = mid + 1; else hi = mid;
-          }
-        }
-        const int L = lo < 32 ? lo : 31;
+        const int L = run_of(incl, i);  // the lane whose part holds candidate i
         const uint32_t before = __shfl_sync(0xffffffffu, incl - cnt, L);
         slot[q] = in[q] ? (uint32_t)(p_lo + L) * A.cap_part + (i - before) : 0u;
       }
