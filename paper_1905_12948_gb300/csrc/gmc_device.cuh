@@ -549,7 +549,9 @@ __device__ __forceinline__ int64_t tile_order(int64_t i, int64_t n_tiles, const 
   const uint32_t G = gridDim.x, nb = (uint32_t)(n_tiles / G);
   if ((uint64_t)i >= (uint64_t)nb * G) return i;
   const uint32_t b = (uint32_t)i / G, o = (uint32_t)i - b * G;
-  const uint32_t ob = __ldcg(order + b);  // (not read-only: the step's first kernel writes it)
+  // (constant for the kernel's life: k_sample_pending, two kernels or more ahead,
+  // ended before the kernel between them did, and this one began after that)
+  const uint32_t ob = __ldg(order + b);
   return (int64_t)(ob < nb ? ob : b) * G + o;
 }
 template <int kFixed, int kQ>
