@@ -100,3 +100,46 @@ def test_captured_in_a_graph():
     graph.replay()
     torch.cuda.synchronize()
     p.compare(p.ref.step(g[1]))
+
+
+def test_handles_and_calls_on_streams_of_their_own():
+    """Two handles and the bare compressor, each a launch that wants every SM at
+    once, on three streams with other work between them: none waits for another
+    beyond its turn, and each gives what it gives alone."""
+    import torch
+    from paper_1905_12948_gb300 import gmc
+    import oracle
+    steps = 12
+    shapes = [(272_474, 8), (900_007, 7)]
+    rng = np.random.default_rng(12)
+    pairs = [Pair(d, K, 0.9, 0.1, ratio=0.005, seed=2) for d, K in shapes]
+    assert all(p.route() == "one launch" for p in pairs)
+    grads = [[rng.standard_normal((K, d)).astype(np.float32) for _ in range(steps)] for d, K in shapes]
+    dev = [[torch.from_numpy(g).cuda() for g in gs] for gs in grads]
+    n, k = 3_000_001, 3_000
+    x_np = rng.standard_normal(n).astype(np.float32)
+    x = torch.from_numpy(x_np).cuda()
+    idx = torch.zeros(k, dtype=torch.int32, device="cuda")
+    val = torch.zeros(k, device="cuda")
+    a = torch.randn(2048, 2048, device="cuda")
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    torch.cuda.synchronize()
+    for t in range(steps):
+        for p, gs, s in zip(pairs, dev, streams):
+            with torch.cuda.stream(s):
+                p.gpu.step(gs[t])
+        assert gmc.load().gmc_topk_noalloc(x.data_ptr(), n, k, idx.data_ptr(), val.data_ptr(),
+                                           streams[2].cuda_stream) == 0
+        with torch.cuda.stream(streams[3]):
+            a = torch.tanh(a @ a)
+        if t == 0:
+            torch.cuda.synchronize()
+            assert all(p.gpu.check() == 0 for p in pairs)
+    torch.cuda.synchronize()
+    for p, gs in zip(pairs, grads):
+        for g in gs:
+            r = p.ref.step(g)
+        p.compare(r)
+        p.compare_stats()
+        assert p.gpu.check() == 0
+    assert np.array_equal(idx.cpu().numpy(), oracle.top_s_support(x_np, k))
