@@ -164,7 +164,10 @@ cudaError_t dalloc(gmc_ctx* h, T** p, size_t count) {
   h->allocations.push_back(q);
   g_live_allocations.fetch_add(1);
   *p = static_cast<T*>(q);
-  return cudaMemset(q, 0, bytes);
+  // the memset runs on the default stream, with which a caller's stream need not
+  // be ordered: it is over before the memory is used
+  err = cudaMemset(q, 0, bytes);
+  return err == cudaSuccess ? cudaStreamSynchronize(nullptr) : err;
 }
 
 void free_all(gmc_ctx* h) {
@@ -917,8 +920,7 @@ int gmc_set_variant(gmc_t h, int32_t variant) {
   if (h->initialized && h->t > 0) return GMC_ESTATE;  // the residuals mean another thing
   if (variant == GMC_VARIANT_SERVER_MOMENTUM && !h->mom) {
     DeviceGuard g(h->device);
-    cudaError_t err = dalloc(h, &h->mom, (size_t)h->ld);
-    if (err == cudaSuccess) err = cudaMemset(h->mom, 0, (size_t)h->ld * sizeof(float));
+    const cudaError_t err = dalloc(h, &h->mom, (size_t)h->ld);
     if (err != cudaSuccess) return status_of(err);
   }
   if ((variant == GMC_VARIANT_LOCAL_MOMENTUM || variant == GMC_VARIANT_LOCAL_MOMENTUM_MFM) && !h->lm) {

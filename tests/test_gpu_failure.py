@@ -297,3 +297,29 @@ def _handle_allocations(d, K):
     lib.gmc_destroy(h)
     assert lib.gmc_test_fail_alloc(-1) == before
     return n
+
+
+@pytest.mark.parametrize("variant", ["gmc", "local_momentum"])
+def test_memory_allocated_on_the_way_is_ready_on_any_stream(variant):
+    """The staging buffer of pageable host gradients and a variant's momentum are
+    allocated by a call and cleared on the default stream: the work of that call
+    on another stream comes after, however busy the default stream is."""
+    import torch
+    d, K = 200_003, 3
+    rng = np.random.default_rng(8)
+    p = Pair(d, K, 0.9, 0.1, ratio=0.01)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    g = [_grads(rng, K, d) for _ in range(2)]
+    torch.cuda._sleep(20_000_000)  # the default stream, about 10 ms
+    if variant != "gmc":
+        assert _lib().gmc_set_variant(p.gpu.h, 3) == GMC_OK
+        p.ref = type(p.ref)(d, K, 0.9, 0.1, compressor="topk", ratio=0.01, variant=variant)
+        p.ref.set_params(p.gpu.params().cpu().numpy())
+        torch.cuda.synchronize()
+        torch.cuda._sleep(20_000_000)
+    for x in g:
+        p.gpu.step_host(torch.from_numpy(x), stream=s)
+        r = p.ref.step(x)
+    torch.cuda.synchronize()
+    p.compare(r)
