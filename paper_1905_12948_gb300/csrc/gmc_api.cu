@@ -398,10 +398,13 @@ RbgsArgs rbgs_args(gmc_ctx* h, const float* grads) {
 // two of its 4,096-coordinate tiles per SM): the bulk pass from kBulkTilesPerSm
 // tiles per SM on, and with more than one worker (one worker's items use half of
 // its warps and ring); else the load/store pass, whose items are 16 times finer.
-// Step and read of w, ratio 0.001, load/store against bulk, us: d = 2 M, K = 8
-// 73 / 99, K = 16 108 / 147; 5 M 139 / 152, 220 / 239; 10 M 244 / 241, 406 / 406;
-// 20 M 444 / 408, 750 / 740; K = 1, d = 40 M 224 / 272. Four steps to a read of w
-// (the bulk pass defers the aggregation), K = 8: 3 M 367 / 401; 5 M 562 / 533.
+// Ratio 0.001, load/store against bulk, us, a step and a read of w (and four steps
+// to a read, where the bulk pass defers the aggregation):
+//   K = 4    3 M  65 /  69 (254 / 255)   4 M  83 /  87 (319 / 314)   5 M  98 /  94 (378 / 347)   10 M 166 / 144 ( 683 / 526)
+//   K = 8    3 M  91 /  99 (353 / 364)   4 M 115 / 119 (448 / 453)   5 M 138 / 133 (548 / 497)   10 M 241 / 215 ( 985 / 806)
+//   K = 16   3 M 145 / 150 (581 / 581)   4 M 183 / 186 (732 / 742)   5 M 219 / 211 (892 / 821)   10 M 403 / 364 (1667 / 1402)
+//   K = 1    8 M  71 /  81 (238 / 300)  40 M 227 / 261 (781 / 977)   138 M 696 / 797 (2360 / 3009)
+// (K = 2 crosses between 5 and 8 M: 68 / 71, 94 / 94.)
 constexpr int kBulkTilesPerSm = 8;
 
 // Tiles, grids and candidate lists of the top-k pass, and their memory.

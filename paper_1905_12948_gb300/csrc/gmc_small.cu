@@ -2,9 +2,9 @@
 // appendix variants) as ONE cooperative launch, for problems whose K x d
 // accumulator fits in the SMs' shared memory (about 7 M values).
 //
-// A block owns every sixteenth-or-so group of 128 coordinates (group g of block
-// g mod grid) for all K workers, and keeps their accumulators v in shared memory
-// from the moment they are formed until the residuals are written:
+// A block owns the groups of 128 coordinates g with g mod grid its index, for all
+// K workers, and keeps their accumulators v in shared memory from the moment they
+// are formed until the residuals are written:
 //   form     v = (e + g) - c*(w_t - w_{t-1}); e, g and w_t - w_{t-1} read once
 //   select   radix rounds over all blocks: each round a histogram of 2,048 bins
 //            per worker of the digit in question, a grid barrier, and every
@@ -18,11 +18,13 @@
 // The approximate top-s ranks the sampled coordinates' keys the same way, then
 // counts what reaches theta, and ranks all keys when that exceeds its limit.
 //
-// Bound by latency and issue: three grid barriers (about 2 us each), a dozen
-// dependent L2 accesses, a few passes over shared memory. Step and read of w,
-// where the step took nine launches: d = 65,536, K = 4: 53 -> 22 us (20 of
-// them this kernel); d = 272 k, K = 8: 70 -> 40 us (34). 768 threads: 512 leave the
-// passes over shared memory short of warps (36 us), 1,024 spill (36).
+// Bound by latency and issue: three grid barriers, a dozen dependent L2 accesses,
+// a few passes over shared memory. Step and read of w, where the step took nine
+// launches: d = 65,536, K = 4: 53 -> 22 us; d = 272 k, K = 8: 70 -> 36 us (steps
+// alone, back to back: 21.3 and 35.0; 21.7 and 37.5 when a barrier's arrival was
+// an atomic whose answer its block waited for). 768 threads, 80 registers (28 to
+// 68 bytes of spills): with 512 the passes over shared memory are short of warps,
+// with 1,024 more is spilled; either took 2 us more at d = 272 k, K = 8.
 #include <algorithm>
 
 #include "gmc_internal.h"
@@ -87,10 +89,12 @@ __device__ __forceinline__ bool sampled_block(const TopkArgs& A, uint64_t key, u
 }
 
 // kCluster: the grid is one thread-block cluster (co-scheduled by the hardware),
-// whose barrier takes the grid barrier's place (0.8 against 1.8 us) and whose
-// launch overlaps the end of the kernel before it, as a cooperative one does not:
-// steps of up to kClusterItems items (d = 10,000, K = 3: 18.8 -> 14.2 us a step;
-// d = 32,768, K = 4, the largest: 20.8 -> 19.4).
+// whose barrier takes the grid barrier's place and whose launch overlaps the end
+// of the kernel before it, as a cooperative one does not: steps of up to
+// kClusterItems items. Step and read of w, cluster against cooperative, us, at
+// 256 items (K = 4) 21.2 / 24.6, 512 21.2 / 24.0, 1,024 20.9 / 24.2, 1,536 22.4 /
+// 23.1 (K = 8: 24.5 / 23.8), 2,048 28.1 / 23.8, 4,096 41.2 / 24.7: past the line a
+// cluster's 16 blocks have too much each.
 template <bool kBf16, bool kCluster>
 __global__ void __launch_bounds__(kSmThreads, 1) k_topk_step(TopkArgs A, DetachArgs D, Scratch* S, int hist_k) {
   if (kCluster) griddep_wait();
