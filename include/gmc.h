@@ -218,8 +218,8 @@ int gmc_set_params(gmc_t h, const float* w0_dev, void* stream);
  * gmc_get_worker_params run after the last gmc_step, and a later gmc_step after
  * them, whatever streams they take. All else is ordered by the caller: other
  * sizes, steps on several streams, and reads after gmc_step_host, a step with a
- * detach output set, one under Alg. 3 or momentum factor masking, or one captured
- * into a graph (unless its aggregation is pending). */
+ * detach output set, or one under Alg. 3 or momentum factor masking; and a graph's
+ * steps and reads with those outside it. */
 int gmc_step(gmc_t h, const float* grads_dev, void* stream);
 
 /* gmc_step_host -- gmc_step from host memory grads_host (K x d fp32,

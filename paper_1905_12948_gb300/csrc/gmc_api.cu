@@ -91,6 +91,7 @@ struct gmc_ctx {
   // that defers): ev_step follows the last step on stream step_id (unless that
   // was being captured), ev_flush the last read, on stream read_id.
   bool step_marked = false;
+  bool step_captured = false, read_captured = false;  // ev_step, ev_flush recorded in a capture
   unsigned long long step_id = 0, read_id = 0;
   uint32_t* bitmap = nullptr;
   int32_t* rank = nullptr;
@@ -489,19 +490,20 @@ namespace {
     if (err_ != cudaSuccess) return status_of(err_); \
   } while (0)
 
-// A stream's id, unique over the process's life (a handle may be given again
-// to a later stream); 0 where there is none.
-unsigned long long stream_id(cudaStream_t s) {
-  unsigned long long id = 0;
-  if (cudaStreamGetId(s, &id) == cudaSuccess) return id;
-  cudaGetLastError();
-  return 0;
-}
 bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &c) == cudaSuccess) return c != cudaStreamCaptureStatusNone;
   cudaGetLastError();  // the default stream while another is captured
   return true;
+}
+// A stream's id, unique over the process's life (a handle may be given again to a
+// later stream); 0 while it is being captured, when CUDA does not tell it.
+unsigned long long stream_id(cudaStream_t s) {
+  unsigned long long id = 0;
+  if (capturing(s)) return 0;
+  if (cudaStreamGetId(s, &id) == cudaSuccess) return id;
+  cudaGetLastError();
+  return 0;
 }
 
 // Work on s that reads or writes the state waits for a read or a flush that may
@@ -511,6 +513,7 @@ cudaError_t order_after_flush(gmc_ctx* h, cudaStream_t s, bool clear) {
   if (!h->wait_flush) return cudaSuccess;
   if (clear) h->wait_flush = false;
   if (h->read_id && h->read_id == stream_id(s)) return cudaSuccess;
+  if (h->read_captured != capturing(s)) return cudaSuccess;  // a graph's work is ordered with the rest by the caller
   return cudaStreamWaitEvent(s, h->ev_flush, 0);
 }
 
@@ -647,7 +650,8 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     GMC_TRY(timed(h, GMC_KERNEL_OTHER, 0.0, s,
                   [&] { return launch_finalize(h->step_ctr, h->total_ctr, pairs_add, s); }));
   // a flush or a read on another stream waits for it
-  h->step_marked = h->agg_pending || (ordered && !capturing(s));
+  h->step_captured = ordered && capturing(s);
+  h->step_marked = h->agg_pending || (ordered && !h->step_captured);
   if (h->step_marked) {
     GMC_TRY(cudaEventRecord(h->ev_step, s));
     h->step_id = stream_id(s);
@@ -659,8 +663,8 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
 
 // A read of the state on s runs after the last step, whatever stream that took.
 cudaError_t order_after_step(gmc_ctx* h, cudaStream_t s) {
-  if (!h->step_marked || (h->step_id && h->step_id == stream_id(s)) || (!h->agg_pending && capturing(s)))
-    return cudaSuccess;
+  if (!h->step_marked || (h->step_id && h->step_id == stream_id(s))) return cudaSuccess;
+  if (h->step_captured != capturing(s)) return cudaSuccess;  // (see order_after_flush)
   return cudaStreamWaitEvent(s, h->ev_step, 0);
 }
 
@@ -669,6 +673,7 @@ cudaError_t mark_read(gmc_ctx* h, cudaStream_t s) {
   const cudaError_t err = cudaEventRecord(h->ev_flush, s);
   if (err != cudaSuccess) return err;
   h->read_id = stream_id(s);
+  h->read_captured = capturing(s);
   h->wait_flush = true;
   return cudaSuccess;
 }

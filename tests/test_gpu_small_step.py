@@ -102,6 +102,30 @@ def test_captured_in_a_graph():
     p.compare(p.ref.step(g[1]))
 
 
+@pytest.mark.parametrize("d,K", [(65_536, 4), (1_300_001, 3), (1_300_001, 8), (5_100_001, 2)])
+def test_step_and_read_captured_after_a_read(d, K):
+    """A step and a read of w captured on another stream than the read before them,
+    replayed once, and read and stepped on from outside; also at sizes whose reads
+    are ordered across streams."""
+    import torch
+    rng = np.random.default_rng(5)
+    p = Pair(d, K, 0.9, 0.1, ratio=0.01)
+    g = [torch.from_numpy(rng.standard_normal((K, d)).astype(np.float32)).to(p.dev) for _ in range(3)]
+    w = torch.empty(d, device=p.dev)
+    p.compare(p.step(g[0].cpu().numpy(), g[0]))
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        p.gpu.step(g[1])
+        assert p.gpu.lib.gmc_get_params(p.gpu.h, w.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+    graph.replay()
+    torch.cuda.synchronize()
+    r = p.ref.step(g[1].cpu().numpy())
+    assert_fp32_state(w.cpu().numpy(), p.ref.w, "w")
+    p.compare(r)
+    p.compare(p.step(g[2].cpu().numpy(), g[2]))
+
+
 def test_handles_and_calls_on_streams_of_their_own():
     """Two handles and the bare compressor, each a launch that wants every SM at
     once, on three streams with other work between them: none waits for another
