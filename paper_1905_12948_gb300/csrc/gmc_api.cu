@@ -165,9 +165,14 @@ cudaError_t dalloc(gmc_ctx* h, T** p, size_t count) {
   h->allocations.push_back(q);
   g_live_allocations.fetch_add(1);
   *p = static_cast<T*>(q);
-  // the memset runs on the default stream, with which a caller's stream need not
-  // be ordered: it is over before the memory is used
-  err = cudaMemset(q, 0, bytes);
+  return cudaMemset(q, 0, bytes);
+}
+// The same by a call other than gmc_create (which ends in a synchronisation): the
+// memset runs on the default stream, with which a caller's stream need not be
+// ordered, so it is waited for before the memory is used.
+template <typename T>
+cudaError_t dalloc_ready(gmc_ctx* h, T** p, size_t count) {
+  const cudaError_t err = dalloc(h, p, count);
   return err == cudaSuccess ? cudaStreamSynchronize(nullptr) : err;
 }
 
@@ -535,6 +540,7 @@ int enqueue_step(gmc_ctx* h, const void* grads_any, cudaStream_t s, bool eager, 
     h->grid_small = 0;
     h->dlt_next = nullptr;
     GMC_TRY(lay_out(h, true));
+    GMC_TRY(cudaStreamSynchronize(nullptr));  // its memory is cleared
     h->restored = h->t > 0;
   }
   bool small = h->grid_small && h->select_mode == GMC_SELECT_SAMPLED;
@@ -928,12 +934,12 @@ int gmc_set_variant(gmc_t h, int32_t variant) {
   if (h->initialized && h->t > 0) return GMC_ESTATE;  // the residuals mean another thing
   if (variant == GMC_VARIANT_SERVER_MOMENTUM && !h->mom) {
     DeviceGuard g(h->device);
-    const cudaError_t err = dalloc(h, &h->mom, (size_t)h->ld);
+    const cudaError_t err = dalloc_ready(h, &h->mom, (size_t)h->ld);
     if (err != cudaSuccess) return status_of(err);
   }
   if ((variant == GMC_VARIANT_LOCAL_MOMENTUM || variant == GMC_VARIANT_LOCAL_MOMENTUM_MFM) && !h->lm) {
     DeviceGuard g(h->device);
-    cudaError_t err = dalloc(h, &h->lm, (size_t)h->K * h->ld);
+    const cudaError_t err = dalloc_ready(h, &h->lm, (size_t)h->K * h->ld);
     if (err != cudaSuccess) return status_of(err);
   }
   h->variant = variant;
@@ -1001,7 +1007,7 @@ int step_host(gmc_ctx* h, const void* grads_host, uint64_t* step_stats_host, cud
     cudaGetLastError();
     const size_t n = (size_t)h->K * (size_t)h->d;
     if (!h->gstage) {
-      cudaError_t err = dalloc(h, &h->gstage, n);
+      const cudaError_t err = dalloc_ready(h, &h->gstage, n);
       if (err != cudaSuccess) return status_of(err);
     }
     GMC_TRY(cudaMemcpyAsync(h->gstage, grads_host, n * (bf16 ? 2 : 4), cudaMemcpyHostToDevice, s));
