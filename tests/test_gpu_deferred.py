@@ -182,8 +182,8 @@ def test_host_steps_pinned_and_pageable(pinned):
 
 def test_dense_sub_tiles_and_ties_on_the_bulk_pass():
     """Many sent pairs per 512-coordinate sub-tile (more than one per lane:
-    the per-element sender masks), K = 1, an odd K and K = 12, ties across
-    tiles, deferred and host (applied at once) steps alternating."""
+    the per-element sender masks), an odd K and K = 12 (K = 1 takes the
+    one-launch step), ties across tiles, deferred and host (applied at once) steps alternating."""
     import torch
     for K, ratio in ((1, 0.05), (7, 0.02), (12, 0.01)):
         rng = np.random.default_rng(40 + K)
@@ -226,8 +226,7 @@ def test_claimed_tiles_and_odd_worker_counts(K, tail):
     """Several tiles per CTA beyond its fixed ones, so the bulk pass claims
     the rest from its tile counter; the worker-parity warp groups each read
     their own stages of the ring, in order, for every K (odd K gives the two
-    groups different item counts per tile, K = 1 leaves one group without
-    items). K <= 5 runs the three-tile pipeline of w_t - w_{t-1}, K >= 6 the
+    groups different item counts per tile; K = 1 takes the one-launch step). K <= 5 runs the three-tile pipeline of w_t - w_{t-1}, K >= 6 the
     one-tile pipeline with two tiles claimed ahead. The ragged last tile's
     last four sub-tiles lie past d (tail 1001) or hold its last 953
     coordinates (tail 3001)."""
